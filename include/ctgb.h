@@ -234,13 +234,12 @@ int ct_set_stream(ct_handle *h, void *cuda_stream);
  * Pick launch shapes for this handle's geometry by timing the candidates on
  * its stream: images per lane (1, 2, 4, 8), warps per ray (1, 2, 4, 8) and
  * neighbouring views per CTA (1, 2, 4, 8) for the forward projection at
- * max_batch, images per thread and view groups per pixel tile (1, 2, 4) for
+ * max_batch, sinograms per thread and CTAs per pixel tile (1, 2, 4) for
  * the transpose, warps per ray and views per CTA for the Jacobian kernels
  * (and, for max_batch > 1, images per lane of the batched ones),
  * and (FP32 handles) the staged forms: the forward and Jacobian kernels
  * with 4 or 8 views per CTA, 4 or 8 rows per shared-memory block and 1, 2
- * or 4 CTAs per ray, the transpose with 8 or 16 views per block and 1, 2 or
- * 4 CTAs per tile.  Synchronises; allocates and frees scratch buffers; must not run
+ * or 4 CTAs per ray.  Synchronises; allocates and frees scratch buffers; must not run
  * during stream capture.  Results of every operator are independent of the
  * chosen shapes up to floating-point summation order.
  */
@@ -249,10 +248,13 @@ int ct_autotune(ct_handle *h);
 /*
  * Read / set the launch shapes, CT_TUNING_COUNT values:
  *   [0] forward images per lane, [1] forward warps per ray (row segments),
- *   [2] forward views per CTA, [3] transpose images per thread,
- *   [4] transpose view groups per pixel tile, [5] Jacobian warps per ray,
- *   [6] Jacobian views per CTA, [7] forward staging, [8] Jacobian staging,
- *   [9] transpose staging, [10] images per lane of the batched Jacobian
+ *   [2] forward views per CTA, [3] transpose sinograms per thread,
+ *   [4] least number of CTAs (view subsets) per transpose pixel tile (the
+ *   launch takes more, up to 8, where the tiles alone leave SMs idle; for the
+ *   fan beam and for images of side up to 64, thread groups of a CTA),
+ *   [5] Jacobian warps per ray, [6] Jacobian views per CTA, [7] forward
+ *   staging, [8] Jacobian staging, [9] 0, 8 or 16 (kept with the shape; the
+ *   transpose has one form), [10] images per lane of the batched Jacobian
  *   products (1, 2 or 4; the staged and fan-beam forms take 1), [11] forward
  *   image layout: 0 pair images (each pixel stored beside its neighbour), 1
  *   images interleaved in groups of 4 (FP32 parallel-beam handles, forward
@@ -264,14 +266,11 @@ int ct_autotune(ct_handle *h);
  * [0]..[6] are powers of two, at most 8 (view groups at most 4), warps per
  * ray x views per CTA at most 16 (unstaged kernels).  Forward / Jacobian
  * staging is 0 (gathers through L1) or 4 / 8 (rows per shared-memory block of
- * the band-staged march, which needs 4 or 8 views per CTA).  Transpose
- * staging is 0 or 8 / 16 (views per shared-memory block of the staged
- * transpose).  Staging applies to FP32 handles only.  With forward staging,
- * [1] is the number of CTAs sharing one ray (row segments, at most 4); with
- * transpose staging, [4] is the number of CTAs sharing one pixel tile (view
- * subsets).  A value above 1 there allocates a workspace of
- * 3 x max_batch x max(V x B, F x N x N) floats the first time (CT_ERR_OOM if
- * that fails).  The Jacobian kernels ignore [5] when staged.  CT_ERR_ARG for
+ * the band-staged march, which needs 4 or 8 views per CTA).  Staging applies
+ * to FP32 handles only.  With forward staging, [1] is the number of CTAs
+ * sharing one ray (row segments, at most 4); a value above 1 there allocates a
+ * workspace of 3 x max_batch x max(V x B, F x N x N) floats the first time
+ * (CT_ERR_OOM if that fails).  The Jacobian kernels ignore [5] when staged.  CT_ERR_ARG for
  * any other value.
  */
 #define CT_TUNING_COUNT 12

@@ -45,6 +45,7 @@ void free_all(ctgb::Handle &h)
     cudaFree(h.d_px);
     cudaFree(h.d_pt);
     cudaFree(h.d_yp);
+    cudaFree(h.d_rowflag);
     cudaFree(h.d_partial);
     cudaFree(h.d_segpart);
     cudaFree(h.d_rays);
@@ -59,6 +60,7 @@ void free_all(ctgb::Handle &h)
     h.d_views = nullptr;
     h.d_fov = h.d_fstart = h.d_fcount = h.d_flag = h.d_order = nullptr;
     h.d_px = h.d_pt = h.d_yp = nullptr;
+    h.d_rowflag = nullptr;
     h.d_partial = nullptr;
     h.d_segpart = nullptr;
 }
@@ -110,8 +112,9 @@ int do_forward(ctgb::Handle &h, const double *theta, const double *delta, const 
 template <typename T>
 int do_adjoint(ctgb::Handle &h, const double *theta, const double *delta, const void *Y, void *X, int batch)
 {
-    CT_CUDA(ctgb::launch_pairs_sino<T>(h, (const T *)Y, batch, nullptr, theta, delta));
-    CT_CUDA(ctgb::launch_adjoint<T>(h, (T *)X, batch, h.tune.adj_kb, h.tune.adj_split, h.tune.adj_stage));
+    h.adj_kb_laid = h.tune.adj_kb;
+    CT_CUDA(ctgb::launch_sino_layout<T>(h, (const T *)Y, batch, h.tune.adj_kb, nullptr, theta, delta));
+    CT_CUDA(ctgb::launch_adjoint<T>(h, (T *)X, batch, h.tune.adj_kb, h.tune.adj_split, batch));
     return CT_OK;
 }
 
@@ -213,10 +216,10 @@ void default_tuning(ctgb::Handle &h)
 {
     const int kb = h.max_batch >= 8 ? 8 : (h.max_batch >= 4 ? 4 : (h.max_batch >= 2 ? 2 : 1));
     h.tune.fwd_kb = std::min(kb, 4);
-    h.tune.adj_kb = std::min(kb, 4);
+    h.tune.adj_kb = h.precision ? std::min(kb, 4) : kb;
     const long long rays = (long long)h.V * h.nchunks;  // warps per image
     h.tune.fwd_split = rays >= 16LL * h.num_sms ? 2 : 4;
-    h.tune.adj_split = 2;
+    h.tune.adj_split = 1;  // the launch raises it where the tiles alone leave SMs idle
     h.tune.der_split = rays >= 32LL * h.num_sms ? 2 : 4;
     h.tune.fwd_vw = 2;
     h.tune.der_vw = 2;
@@ -367,20 +370,15 @@ template <typename T> int autotune_impl(ctgb::Handle &h)
         best = 1e30f;
         for (int kb : {1, 2, 4, 8}) {
             if (kb > K) continue;
-            for (int st : {0, 8, 16}) {
-                for (int sp : {1, 2, 4}) {
-                    if (st > 0 && (!fp32 || !ctgb::adj_band_ok(h, st, sp)))
-                        continue;
-                    const float ms = time_config(h.stream, [&] {
-                        ctgb::launch_pairs_sino<T>(h, X, K);
-                        ctgb::launch_adjoint<T>(h, (T *)d_out, K, kb, sp, st);
-                    });
-                    if (ms < best) {
-                        best = ms;
-                        t.adj_kb = kb;
-                        t.adj_split = sp;
-                        t.adj_stage = st;
-                    }
+            for (int sp : {1, 2, 4}) {
+                const float ms = time_config(h.stream, [&] {
+                    ctgb::launch_sino_layout<T>(h, X, K, kb);
+                    ctgb::launch_adjoint<T>(h, (T *)d_out, K, kb, sp, K);
+                });
+                if (ms < best) {
+                    best = ms;
+                    t.adj_kb = kb;
+                    t.adj_split = sp;
                 }
             }
         }
@@ -533,6 +531,7 @@ int ct_init(const ct_geom *g, void *cuda_stream, ct_handle **out)
                   cudaMalloc(&h.d_px, img_pairs * pair_bytes) == cudaSuccess &&
                   cudaMalloc(&h.d_pt, img_pairs * pair_bytes) == cudaSuccess &&
                   cudaMalloc(&h.d_yp, sino_pairs * pair_bytes) == cudaSuccess &&
+                  (h.precision != 0 || cudaMalloc(&h.d_rowflag, sizeof(int) * (size_t)h.max_batch * h.V) == cudaSuccess) &&
                   cudaMalloc(&h.d_partial, sizeof(double) * 4 * (size_t)h.max_batch * h.V * h.nchunks) ==
                       cudaSuccess &&
                   (h.fan_D == 0.0 ||
@@ -609,9 +608,9 @@ int ct_adjoint_repeat(ct_handle *H, void *X, int batch)
     if (!H || !X || batch < 1 || batch > H->h.adj_ready) return CT_ERR_ARG;
     ctgb::Handle &h = H->h;
     if (h.precision)
-        CT_CUDA(ctgb::launch_adjoint<double>(h, (double *)X, batch, h.tune.adj_kb, h.tune.adj_split, h.tune.adj_stage));
+        CT_CUDA(ctgb::launch_adjoint<double>(h, (double *)X, batch, h.adj_kb_laid, h.tune.adj_split, h.adj_ready));
     else
-        CT_CUDA(ctgb::launch_adjoint<float>(h, (float *)X, batch, h.tune.adj_kb, h.tune.adj_split, h.tune.adj_stage));
+        CT_CUDA(ctgb::launch_adjoint<float>(h, (float *)X, batch, h.adj_kb_laid, h.tune.adj_split, h.adj_ready));
     return CT_OK;
 }
 

@@ -21,10 +21,17 @@
 // r holds (X[r][c], X[r][c+1]) for c = -2 .. N+1 (stored at c + 2, pitch
 // Pp = N + 4 pairs), zero outside the image.  One 8-byte load then fetches
 // both interpolation taps, and clamping the cell to [-2, N] keeps every load
-// in bounds while rays outside the image read exact zeros.  The transpose
-// operator reads sinograms the same way: pair b of view v holds
+// in bounds while rays outside the image read exact zeros.  The FP64
+// transpose reads sinograms the same way: pair b of view v holds
 // (Y[v][b], Y[v][b+1]) for b = -2 .. B+1 (stored at b + 2, pitch Pb = B + 4
-// rounded up to even, so that rows start on 16-byte boundaries).
+// rounded up to even).
+//
+// Interleaved sinograms (FP32 transpose).  The batch is cut into groups of
+// kb sinograms, the last one of the smallest power of two that holds the
+// rest (its missing sinograms are zero); element (v, b) of a group holds the
+// group's sinograms at that bin side by side, rows of sino_pitch(B) bins (a
+// multiple of 4: 16-byte copies), zero from B on.  The group of sinogram k0
+// starts k0 * V * sino_pitch(B) floats into the buffer.
 //
 // Interleaved images (FP32 forward, fwd_layout 1).  The forward of a batch
 // may read its images from a second layout without the pair duplication:
@@ -49,6 +56,7 @@ constexpr double kFixScale = 281474976710656.0;  // 2^48
 constexpr int kMaxN = 4096;                      // keeps |q| * 2^48 inside int64
 constexpr int kChunk = 32;                       // bins per warp work item
 constexpr int kTile = 16;                        // transpose-operator pixel tile side
+constexpr int kAdjFrac = 26;                     // fractional bits of the FP32 transpose's in-tile coordinate
 constexpr double kAllRowsBelow = 4e-3;           // |qr| below this: march every row
 
 enum ViewFlags : int { kAllRows = 1, kValid = 2 };
@@ -71,6 +79,7 @@ struct __align__(16) ViewGeo {
     int flags;
     int n0;                // integer part of the bin-centre offset -(B-1)/2 + delta
     int gen;               // incremented at every rebuild (tables derived per view compare it)
+    int aC, aS;            // c and s with kAdjFrac fractional bits (FP32 transpose)
 };
 
 // Launch shapes.  kb: images (or sinograms) per lane; split: warps sharing
@@ -81,16 +90,15 @@ struct __align__(16) ViewGeo {
 // stage: 0 = gather through L1; 4 or 8 = rows per block of the band-staged
 // FP32 march (vw 4 or 8).  There the forward's split is the number of CTAs
 // that share one ray (row segments, combined by a second kernel); the
-// derivative kernels march whole rays.  The staged transpose's split is the
-// number of CTAs per pixel tile, one thread-block cluster.
+// derivative kernels march whole rays.  The parallel-beam transpose's split is
+// the least number of CTAs per pixel tile, one thread-block cluster.
 struct Tuning {
     int fwd_kb = 8, fwd_split = 2, fwd_vw = 1;  // forward projection of a batch
     int adj_kb = 8, adj_split = 2;              // transpose of a batch
     int der_split = 4, der_vw = 1;              // JVP / VJP / Gauss-Newton terms
     int der_kb = 1;                             // images per lane of the batched derivative modes
     int fwd_stage = 0, der_stage = 0;
-    int adj_stage = 0;  // 0: gather through L1; 8 or 16: views per shared-memory block of the
-                        // staged FP32 transpose, whose adj_split is then CTAs per tile
+    int adj_stage = 0;  // kept with the shape; the transpose has one form
     int fwd_layout = 0; // 1: the FP32 L1-gather forward (fwd_stage 0, fwd_kb 4 or 8, parallel
                         // beam) reads the interleaved images; 0: the pair images
 };
@@ -111,6 +119,28 @@ __host__ __device__ inline void interleave_group(int k, int K, int &k0, int &w)
     }
 }
 
+// Groups of the interleaved sinogram layout of `batch` sinograms at kb per
+// group: up to two runs of `count` groups of one width, run q starting at
+// sinogram k0 and group number `first`.  Returns the number of runs.
+struct SinoGroup {
+    int k0, width, count, first;
+};
+inline int sino_groups(int batch, int kb, SinoGroup *g)
+{
+    const int full = batch / kb, rem = batch - full * kb;
+    int w = 1;
+    while (w < rem) w *= 2;
+    if (rem && w == kb) {  // the rest makes one more group of the same width
+        g[0] = {0, kb, full + 1, 0};
+        return 1;
+    }
+    int n = 0;
+    if (full) g[n++] = {0, kb, full, 0};
+    if (rem) g[n++] = {full * kb, w, 1, full};
+    return n;
+}
+inline int sino_pitch(int B) { return (B + 3) & ~3; }
+
 struct Handle {
     int N = 0, B = 0, V = 0, F = 1, max_batch = 1, precision = 0, device = 0;
     int Pp = 0, Pb = 0;  // pair pitches
@@ -124,7 +154,8 @@ struct Handle {
     int *d_order = nullptr;   // view order of the ray kernels (sorted by axis and slope)
     void *d_px = nullptr;     // pair images, rows of X:   (max_batch + 1) * F * N * Pp pairs
     void *d_pt = nullptr;     // pair images, rows of X^T: (max_batch + 1) * F * N * Pp pairs
-    void *d_yp = nullptr;     // pair sinograms: max_batch * V * Pb pairs
+    void *d_yp = nullptr;     // sinograms of the transpose: pairs (FP64) or interleaved (FP32), max_batch * V * Pb pairs
+    int *d_rowflag = nullptr; // FP32 transpose: [group][V], the row of the group holds a non-finite value
     float *d_qx = nullptr;    // interleaved images, rows of X and of X^T: max_batch * F * N * Pp
     float *d_qt = nullptr;    // floats each, allocated when fwd_layout 1 is set (FP32 handles)
     double *d_partial = nullptr;  // per (image, view, chunk) reduction partials, 4 per item, max_batch images
@@ -141,6 +172,7 @@ struct Handle {
     // (ct_adjoint_repeat) may rerun the projection kernel alone.  Any other
     // call that may change the view table or the pair layouts clears them.
     int fwd_ready = 0, adj_ready = 0;
+    int adj_kb_laid = 1;  // sinograms per group of the layout behind adj_ready
     // Images (of F frames) whose pair layouts are current from the last
     // operator call that took images: a later call may pass X = null to use
     // them again (its batch at most this).  The solvers and the autotuner,
@@ -169,9 +201,11 @@ cudaError_t launch_view_setup_wide(const Handle &h, const double *theta, const d
 template <typename T>
 cudaError_t launch_pairs_img(const Handle &h, const T *X, int nimg, const int *skip = nullptr,
                              const double *theta = nullptr, const double *delta = nullptr);
+// Sinograms in the layout the handle's transpose reads at kb sinograms per
+// group (pairs in FP64, interleaved in FP32, fan-beam blocks of 8).
 template <typename T>
-cudaError_t launch_pairs_sino(const Handle &h, const T *Y, int nsino, const int *skip = nullptr,
-                              const double *theta = nullptr, const double *delta = nullptr);
+cudaError_t launch_sino_layout(const Handle &h, const T *Y, int nsino, int kb, const int *skip = nullptr,
+                               const double *theta = nullptr, const double *delta = nullptr);
 // Layout the forward projection reads (pair images of X and X^T).
 template <typename T>
 cudaError_t launch_prep_forward(const Handle &h, const T *X, int nimg, const int *skip = nullptr,
@@ -191,12 +225,10 @@ cudaError_t launch_interleaved_to_pairs(const Handle &h, int batch);
 template <typename T>
 cudaError_t launch_forward(const Handle &h, T *Y, int batch, int kb, int split, int vw, int stage,
                            const int *skip = nullptr, bool interleaved = false, int layout_batch = 0);
+// The first `batch` of the layout_batch sinograms laid out at kb per group.
 template <typename T>
-cudaError_t launch_adjoint(const Handle &h, T *X, int batch, int kb, int split, int stage,
+cudaError_t launch_adjoint(const Handle &h, T *X, int batch, int kb, int split, int layout_batch,
                            const int *skip = nullptr);
-// Staged FP32 transpose (ct_adj_band.cu); adj_band_ok tells whether a shape can run on this handle.
-bool adj_band_ok(const Handle &h, int stage, int segs);
-cudaError_t launch_adjoint_band(const Handle &h, float *X, int batch, int kb, int segs, int stage, const int *skip);
 // Derivative modes on `batch` images laid out in the pair buffers (kb images
 // per lane: 1, 2 or 4), one launch of the ray kernel plus (VJP, GN) the
 // per-view reduction.  JVP: image k uses dtheta + k * dir_stride (0: one

@@ -3,7 +3,7 @@
 //   k_view_prep   per-view constants from (theta, delta), FP64 -> fixed point,
 //                 and the view order of the ray kernels
 //   k_pairs_img   X -> pair layouts of X and X^T (zero padded)
-//   k_pairs_sino  Y -> pair layout of the sinogram (zero padded)
+//   k_pairs_sino, k_interleave_sino  Y -> the layout of the FP64 / FP32 transpose
 //   k_ray         one warp per 32 consecutive rays of one view (optionally
 //                 SPLIT warps per ray group, each marching a row segment):
 //                   FWD  Y = H X for KB images at once
@@ -119,6 +119,8 @@ __device__ bool view_setup_one(int v, const double *__restrict__ theta, const do
     g.beta0 = h * (s - c) - dl + 0.5 * (B - 1);
     g.c = c;
     g.s = s;
+    g.aC = __double2int_rn(c * (double)(1 << kAdjFrac));
+    g.aS = __double2int_rn(s * (double)(1 << kAdjFrac));
     g.th = th_in;
     g.dl = dl_in;
     g.frame = fov ? fov[v] : 0;
@@ -356,10 +358,9 @@ __global__ void k_interleaved_to_pairs(const float *__restrict__ QX, const float
     }
 }
 
-// YP[row][bp] = (Y[row][bp - 2], Y[row][bp - 1]), zero outside [0, B).
+// FP64: YP[row][bp] = (Y[row][bp - 2], Y[row][bp - 1]), zero outside [0, B).
 // With p.on, the last CTA runs the view-table step of the call instead.
-template <typename T>
-__global__ void k_pairs_sino(const T *__restrict__ Y, pair_t<T> *__restrict__ YP, int B, int Pb, long long total,
+__global__ void k_pairs_sino(const double *__restrict__ Y, double2 *__restrict__ YP, int B, int Pb, long long total,
                              ViewPrep p, const int *__restrict__ skip)
 {
     extern __shared__ unsigned long long prep_key[];
@@ -374,11 +375,60 @@ __global__ void k_pairs_sino(const T *__restrict__ Y, pair_t<T> *__restrict__ YP
         const long long row = idx / Pb;
         const int bp = (int)(idx - row * Pb);
         const int b0 = bp - 2, b1 = bp - 1;
-        const T *y = Y + row * B;
-        pair_t<T> p;
-        p.x = (b0 >= 0 && b0 < B) ? y[b0] : T(0);
-        p.y = (b1 >= 0 && b1 < B) ? y[b1] : T(0);
+        const double *y = Y + row * B;
+        double2 p;
+        p.x = (b0 >= 0 && b0 < B) ? y[b0] : 0.0;
+        p.y = (b1 >= 0 && b1 < B) ? y[b1] : 0.0;
         YP[idx] = p;
+    }
+}
+
+// FP32: the interleaved sinograms of the transpose (ct_internal.cuh).  A CTA
+// takes rows (group, view): each thread reads its bin of the group's sinograms
+// (coalesced over the bins) and writes them side by side; the row's flag says
+// whether it holds a non-finite value.  With p.on, the last CTA runs the
+// view-table step of the call instead.
+__global__ void __launch_bounds__(256) k_interleave_sino(const float *__restrict__ Y, float *__restrict__ YI,
+                                                         int *__restrict__ rowflag, int B, int Pq, int V, int nsino,
+                                                         int kb, long long rows, ViewPrep p,
+                                                         const int *__restrict__ skip)
+{
+    extern __shared__ unsigned long long prep_key[];
+    if (skip && *skip) return;
+    const int nblk = gridDim.x - (p.on ? 1 : 0);
+    if (p.on && blockIdx.x == nblk) {
+        view_prep_block(p, prep_key);
+        return;
+    }
+    for (long long row = blockIdx.x; row < rows; row += nblk) {
+        const int grp = (int)(row / V), v = (int)(row - (long long)grp * V);
+        const int k0 = grp * kb, live = min(kb, nsino - k0);
+        int w = 1;
+        while (w < live) w *= 2;
+        float *out = YI + ((size_t)k0 * V + (size_t)v * w) * Pq;
+        const float *in = Y + ((size_t)k0 * V + v) * B;
+        int bad = 0;
+        auto value = [&](int k, int b) {
+            const float y = (k < live && b < B) ? in[(size_t)k * V * B + b] : 0.0f;
+            bad |= !isfinite(y);
+            return y;
+        };
+        for (int b = threadIdx.x; b < Pq; b += blockDim.x) {
+            if (w == 1) {
+                out[b] = value(0, b);
+            } else if (w == 2) {
+                reinterpret_cast<float2 *>(out)[b] = make_float2(value(0, b), value(1, b));
+            } else {
+                float y[8];
+#pragma unroll
+                for (int k = 0; k < 8; ++k) y[k] = k < w ? value(k, b) : 0.0f;
+                float4 *o = reinterpret_cast<float4 *>(out + (size_t)b * w);
+                o[0] = make_float4(y[0], y[1], y[2], y[3]);
+                if (w == 8) o[1] = make_float4(y[4], y[5], y[6], y[7]);
+            }
+        }
+        bad = __syncthreads_or(bad);
+        if (threadIdx.x == 0) rowflag[row] = bad;
     }
 }
 
@@ -846,26 +896,37 @@ cudaError_t launch_interleaved_to_pairs(const Handle &h, int batch)
 }
 
 template <typename T>
-cudaError_t launch_pairs_sino(const Handle &h, const T *Y, int nsino, const int *skip, const double *theta,
-                              const double *delta)
+cudaError_t launch_sino_layout(const Handle &h, const T *Y, int nsino, int kb, const int *skip, const double *theta,
+                               const double *delta)
 {
     const ViewPrep p = view_prep_args(h, theta, delta);
-    cudaError_t e = allow_prep_smem<k_pairs_sino<T>>();
-    if (e != cudaSuccess) return e;
-    const long long total = (long long)nsino * h.V * h.Pb;
-    const int threads = 256;
-    const long long blocks = std::min<long long>((total + threads - 1) / threads, (long long)h.num_sms * 16);
     if (h.fan_D > 0.0) {
-        // fan beam: the transpose reads the interleaved layout instead; the view-table
-        // step (when the angles come with the call) runs on its own
+        // fan beam: the view-table step (when the angles come with the call) runs on its own
         if (p.on) {
-            e = launch_view_setup(h, theta, delta, skip);
+            cudaError_t e = launch_view_setup(h, theta, delta, skip);
             if (e != cudaSuccess) return e;
         }
         return launch_fan_sino<T>(h, Y, nsino, skip);
     }
-    k_pairs_sino<T><<<(int)std::max<long long>(1, blocks) + (p.on ? 1 : 0), threads, prep_smem(p), h.stream>>>(
-        Y, (pair_t<T> *)h.d_yp, h.B, h.Pb, total, p, skip);
+    if constexpr (std::is_same<T, float>::value) {
+        SinoGroup g[2];
+        const int ng = sino_groups(nsino, kb, g);
+        const int groups = g[ng - 1].first + g[ng - 1].count;
+        cudaError_t e = allow_prep_smem<k_interleave_sino>();
+        if (e != cudaSuccess) return e;
+        const long long rows = (long long)groups * h.V;
+        const int blocks = (int)std::min<long long>(rows, (long long)h.num_sms * 16);
+        k_interleave_sino<<<blocks + (p.on ? 1 : 0), 256, prep_smem(p), h.stream>>>(
+            Y, (float *)h.d_yp, h.d_rowflag, h.B, sino_pitch(h.B), h.V, nsino, kb, rows, p, skip);
+    } else {
+        cudaError_t e = allow_prep_smem<k_pairs_sino>();
+        if (e != cudaSuccess) return e;
+        const long long total = (long long)nsino * h.V * h.Pb;
+        const int threads = 256;
+        const long long blocks = std::min<long long>((total + threads - 1) / threads, (long long)h.num_sms * 16);
+        k_pairs_sino<<<(int)std::max<long long>(1, blocks) + (p.on ? 1 : 0), threads, prep_smem(p), h.stream>>>(
+            Y, (double2 *)h.d_yp, h.B, h.Pb, total, p, skip);
+    }
     return cudaGetLastError();
 }
 
@@ -1020,8 +1081,8 @@ cudaError_t launch_gn(const Handle &h, const T *bdata, T *res, double *grad, dou
 #define CTGB_RAY_INSTANTIATE(T)                                                                             \
     template cudaError_t launch_pairs_img<T>(const Handle &, const T *, int, const int *, const double *,   \
                                              const double *);                                              \
-    template cudaError_t launch_pairs_sino<T>(const Handle &, const T *, int, const int *, const double *,  \
-                                              const double *);                                             \
+    template cudaError_t launch_sino_layout<T>(const Handle &, const T *, int, int, const int *,            \
+                                               const double *, const double *);                            \
     template cudaError_t launch_prep_forward<T>(const Handle &, const T *, int, const int *, const double *, \
                                                 const double *);                                           \
     template cudaError_t launch_forward<T>(const Handle &, T *, int, int, int, int, int, const int *, bool, int); \

@@ -339,8 +339,8 @@ template <typename T> struct Solver {
     // out = H(theta)^T yin  (n vector)
     int backproject(const double *theta, const T *yin, T *out, const int *stop)
     {
-        SV_CUDA(launch_pairs_sino<T>(h, yin, 1, stop, theta, delta));
-        SV_CUDA(launch_adjoint<T>(h, out, 1, h.tune.adj_kb, h.tune.adj_split, h.tune.adj_stage, stop));
+        SV_CUDA(launch_sino_layout<T>(h, yin, 1, h.tune.adj_kb, stop, theta, delta));
+        SV_CUDA(launch_adjoint<T>(h, out, 1, h.tune.adj_kb, h.tune.adj_split, 1, stop));
         return CT_OK;
     }
 
