@@ -84,18 +84,34 @@ cudaError_t prep_images(ctgb::Handle &h, const T *X, int nimg, const double *the
     return ctgb::launch_view_setup(h, theta, delta);
 }
 
-// Whether a forward that takes images lays them out interleaved (the tuning
-// asks for it and the handle can: FP32, parallel beam, workspace present).
-bool forward_interleaves(const ctgb::Handle &h)
+// Whether a product that takes `batch` images lays them out interleaved (the
+// tuning asks for it and the handle can: FP32, parallel beam, workspace
+// present).  One image keeps the pair images, which fetch both taps in one
+// load: 58.8 against 77 us for the forward of 16 frames of 256^2 / 1200 views.
+bool can_interleave(const ctgb::Handle &h, int batch)
 {
-    return h.tune.fwd_layout == 1 && h.precision == 0 && h.fan_D == 0.0 && h.d_qx;
+    return h.tune.fwd_layout == 1 && h.precision == 0 && h.fan_D == 0.0 && h.d_qx && batch >= 2;
+}
+
+// The layout of a batched derivative call and the view table; *inter: the
+// interleaved images hold the call's batch (512^2 / 360 views, 4 images, J^T with
+// offsets: 207 us a call against 221 on pair images), else the pair images do.
+template <typename T>
+cudaError_t prep_batch(ctgb::Handle &h, const T *X, int batch, const double *theta, const double *delta, bool *inter)
+{
+    *inter = can_interleave(h, batch) && h.tune.der_stage == 0 && h.tune.der_kb == 4 &&
+             (X || (h.img_kind == 1 && h.img_ready == batch));
+    if (!*inter) return prep_images<T>(h, X, batch * h.F, theta, delta);
+    if (!X) return ctgb::launch_view_setup(h, theta, delta);
+    h.img_kind = 1;
+    return ctgb::launch_interleave_img(h, (const float *)X, batch, theta, delta);
 }
 
 template <typename T>
 int do_forward(ctgb::Handle &h, const double *theta, const double *delta, const void *X, void *Y, int batch)
 {
     // X == null reads whichever layout the previous call left
-    const bool inter = X ? forward_interleaves(h) : h.img_kind == 1;
+    const bool inter = X ? can_interleave(h, batch) : h.img_kind == 1;
     if (inter && X) {
         CT_CUDA(ctgb::launch_interleave_img(h, (const float *)X, batch, theta, delta));
         h.img_kind = 1;
@@ -141,9 +157,10 @@ int do_jac_batch(ctgb::Handle &h, const double *theta, const double *delta, cons
                  const double *ddelta, void *dY, int batch, int flags)
 {
     const long long dstride = (flags & CT_BATCH_PER_IMAGE_DIRECTION) ? h.V : 0;
-    CT_CUDA(prep_images<T>(h, (const T *)X, batch * h.F, theta, delta));
+    bool inter;
+    CT_CUDA(prep_batch<T>(h, (const T *)X, batch, theta, delta, &inter));
     CT_CUDA(ctgb::launch_jvp<T>(h, dtheta, ddelta, (T *)dY, h.tune.der_split, h.tune.der_vw, h.tune.der_stage, batch,
-                                h.tune.der_kb, dstride));
+                                h.tune.der_kb, dstride, inter));
     return CT_OK;
 }
 
@@ -152,9 +169,10 @@ int do_jacT_batch(ctgb::Handle &h, const double *theta, const double *delta, con
                   double *gtheta, double *gdelta, int batch, int flags)
 {
     const long long rstride = (flags & CT_BATCH_SHARED_R) ? 0 : (long long)h.V * h.B;
-    CT_CUDA(prep_images<T>(h, (const T *)X, batch * h.F, theta, delta));
+    bool inter;
+    CT_CUDA(prep_batch<T>(h, (const T *)X, batch, theta, delta, &inter));
     CT_CUDA(ctgb::launch_vjp<T>(h, (const T *)R, gtheta, gdelta, h.tune.der_split, h.tune.der_vw, h.tune.der_stage,
-                                batch, h.tune.der_kb, rstride, (flags & CT_BATCH_SUM) ? 1 : 0));
+                                batch, h.tune.der_kb, rstride, (flags & CT_BATCH_SUM) ? 1 : 0, inter));
     return CT_OK;
 }
 
@@ -162,9 +180,10 @@ template <typename T>
 int do_gn_batch(ctgb::Handle &h, const double *theta, const double *delta, const void *X, const void *bdata,
                 void *res, double *grad, double *jnorm2, double *fval, int batch)
 {
-    CT_CUDA(prep_images<T>(h, (const T *)X, batch * h.F, theta, delta));
+    bool inter;
+    CT_CUDA(prep_batch<T>(h, (const T *)X, batch, theta, delta, &inter));
     CT_CUDA(ctgb::launch_gn<T>(h, (const T *)bdata, (T *)res, grad, jnorm2, fval, h.tune.der_split, h.tune.der_vw,
-                               h.tune.der_stage, nullptr, nullptr, batch, h.tune.der_kb));
+                               h.tune.der_stage, nullptr, nullptr, batch, h.tune.der_kb, nullptr, inter));
     return CT_OK;
 }
 
@@ -222,7 +241,14 @@ void default_tuning(ctgb::Handle &h)
     h.tune.adj_split = 1;  // the launch raises it where the tiles alone leave SMs idle
     h.tune.der_split = rays >= 32LL * h.num_sms ? 2 : 4;
     h.tune.fwd_vw = 2;
-    h.tune.der_vw = 2;
+    if (h.precision) {
+        // the FP64 pipe is the bound: no warp waits for its neighbours, and finer segments
+        // even out the rays (255^2, 181 views, 4 images: 278 -> 255 us); small images keep
+        // theirs (and with them the order of their sums)
+        h.tune.fwd_vw = 1;
+        if (h.N > 64 && rays < 16LL * h.num_sms) h.tune.fwd_split = 8;
+    }
+    h.tune.der_vw = rays >= 32LL * h.num_sms ? 2 : 1;
     h.tune.der_kb = std::min(kb, 4);
     if (h.fan_D > 0.0) {
         // fan-beam transpose: one candidate search per pixel and view serves
@@ -567,6 +593,9 @@ int ct_init(const ct_geom *g, void *cuda_stream, ct_handle **out)
         return rc;
     }
     default_tuning(h);
+    // batches read the interleaved images where their workspace can be had
+    if (h.tune.fwd_kb >= 4 && h.precision == 0 && h.fan_D == 0.0 && ensure_interleaved(h) == CT_OK)
+        h.tune.fwd_layout = 1;
     *out = H;
     return CT_OK;
 }

@@ -33,8 +33,8 @@
 // multiple of 4: 16-byte copies), zero from B on.  The group of sinogram k0
 // starts k0 * V * sino_pitch(B) floats into the buffer.
 //
-// Interleaved images (FP32 forward, fwd_layout 1).  The forward of a batch
-// may read its images from a second layout without the pair duplication:
+// Interleaved images (FP32, fwd_layout 1).  The products of a batch of two or
+// more may read its images from a second layout without the pair duplication:
 // the batch is cut into groups of 4 images (a remainder of 2 or 3 gives one
 // group of 2, an odd remainder one group of 1, in that order), and element
 // c + 2 of row r holds X_k[r][c] of the group's w images side by side, for
@@ -99,8 +99,9 @@ struct Tuning {
     int der_kb = 1;                             // images per lane of the batched derivative modes
     int fwd_stage = 0, der_stage = 0;
     int adj_stage = 0;  // kept with the shape; the transpose has one form
-    int fwd_layout = 0; // 1: the FP32 L1-gather forward (fwd_stage 0, fwd_kb 4 or 8, parallel
-                        // beam) reads the interleaved images; 0: the pair images
+    int fwd_layout = 0; // 1: the FP32 L1-gather products of a batch (fwd_stage 0 with fwd_kb 4 or 8,
+                        // der_stage 0 with der_kb 4, parallel beam) read the interleaved images;
+                        // 0: the pair images
 };
 
 // Group of image k in the interleaved layout of a batch of K: first image k0, width w.
@@ -237,16 +238,19 @@ cudaError_t launch_adjoint(const Handle &h, T *X, int batch, int kb, int split, 
 // one [V] vector summing the images in order.  GN: image k reads
 // bdata + k * V * B and writes [k][V] outputs; rscale (nullable) receives
 // sum_b |r_b| (|(H x)_b| + |b_b|) per view, the rounding scale of the misfit.
+// interleaved (FP32, parallel beam, stage 0): the images are in the interleaved
+// layout of a batch of `batch`, read 4 (then 2, 1) per lane whatever kb is.
 template <typename T>
 cudaError_t launch_jvp(const Handle &h, const double *dtheta, const double *ddelta, T *dY, int split, int vw,
-                       int stage, int batch = 1, int kb = 1, long long dir_stride = 0);
+                       int stage, int batch = 1, int kb = 1, long long dir_stride = 0, bool interleaved = false);
 template <typename T>
 cudaError_t launch_vjp(const Handle &h, const T *R, double *gtheta, double *gdelta, int split, int vw, int stage,
-                       int batch = 1, int kb = 1, long long r_stride = 0, int sum = 0);
+                       int batch = 1, int kb = 1, long long r_stride = 0, int sum = 0,
+                       bool interleaved = false);
 template <typename T>
 cudaError_t launch_gn(const Handle &h, const T *bdata, T *res, double *grad, double *jnorm2, double *fval,
                       int split, int vw, int stage, const int *view_mask = nullptr, const int *skip = nullptr,
-                      int batch = 1, int kb = 1, double *rscale = nullptr);
+                      int batch = 1, int kb = 1, double *rscale = nullptr, bool interleaved = false);
 
 // Fan beam (ct_fan.cu).  launch_fan_rays rebuilds the per-ray table from the
 // view table; every launcher that brings the view table up to date runs it

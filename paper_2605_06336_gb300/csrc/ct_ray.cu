@@ -467,13 +467,48 @@ __device__ __forceinline__ void taps_interleaved(const float *__restrict__ q, lo
     }
 }
 
-// QL (FP32 forward only): the images come from the interleaved layout; the
-// taps, the fractions and the order of the sums are those of the pair form,
-// so both give the same bits.
+// Element indices (cell + 2, clamped to the row's zero padding) and fractions
+// of U consecutive rows from the exact line value Q at the first.  FP32: the
+// rows are walked relative to the first one's cell with 55 fractional bits (the
+// 48 of the line, shifted), so the high word holds the cell offset in its top
+// 9 bits and the 23 bits of the fraction below them: one shift, one logic
+// operation and one add-and-clamp a row, where the full-range line needs a
+// two-word shift, two clamps and a second shift (the integer pipe was the bound
+// of one image per lane: 74 % busy, now 58).  The same bits as cell_of and
+// frac_of.  One image of 2048^2, 120 views: 362 -> 282 us; 256^2 / 180 views:
+// 18.6 -> 16.3.
+template <typename T, int U>
+__device__ __forceinline__ void ray_cells(long long Q, long long dQ, unsigned lim, unsigned (&idx)[U], T (&f)[U])
+{
+    if constexpr (std::is_same<T, float>::value) {
+        static_assert(kFracBits == 48 && U <= 16, "cell offsets of a block fit 9 bits");
+        const unsigned base = (unsigned)(cell_of(Q) + 2);
+        const long long L0 = (long long)(((unsigned long long)Q << 16) >> 9), dL = dQ << 7;
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int hi = (int)((L0 + (long long)u * dL) >> 32);
+            // (a negative index is a large unsigned one)
+            idx[u] = __viaddmin_u32((unsigned)(hi >> 23), base, lim);
+            f[u] = __int_as_float((hi & 0x7FFFFF) | 0x3F800000) - 1.0f;
+        }
+    } else {
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const long long Qu = Q + (long long)u * dQ;
+            idx[u] = min((unsigned)(cell_of(Qu) + 2), lim);
+            f[u] = frac_of(Qu, T());
+        }
+    }
+}
+
+// QL (FP32): the images come from the interleaved layout; the taps, the
+// fractions and the order of the sums are those of the pair form, so both
+// give the same bits.
 template <typename T, int MODE, bool OFFS, int KB, int SPLIT, bool QL = false>
 __global__ void __launch_bounds__(512) k_ray(RayArgs<T> a)
 {
     using P2 = pair_t<T>;
+    constexpr bool F32 = std::is_same<T, float>::value;
     constexpr int NACC = (MODE == kFwd) ? KB : 3 * KB;
     extern __shared__ unsigned char ray_smem[];
     T *red = reinterpret_cast<T *>(ray_smem);  // [VW][SPLIT][NACC][32], only when SPLIT > 1
@@ -510,100 +545,59 @@ __global__ void __launch_bounds__(512) k_ray(RayArgs<T> a)
             const int r1 = min(rhi, r0 + per - 1);
             long long Q = line_at(g, b, r0, N);
             const long long dQ = 2 * g.Qh;
-            const P2 *img = (g.mode ? a.PT : a.PX) + (size_t)g.frame * N * a.Pp + (size_t)k0 * a.pimg_stride +
-                            (size_t)r0 * a.Pp + 2;
+            constexpr int QW = KB >= 4 ? 4 : KB;  // floats per element of the group's interleaved layout
+            const unsigned pp = (unsigned)a.Pp, lim = (unsigned)(N + 2);
+            const P2 *img = nullptr;
+            const float *qimg = nullptr;
+            if constexpr (QL)
+                qimg = (g.mode ? a.QT : a.QX) + (size_t)k0 * a.qimg_stride + ((size_t)g.frame * N + r0) * pp * QW;
+            else
+                img = (g.mode ? a.PT : a.PX) + ((size_t)g.frame * N + r0) * pp + (size_t)k0 * a.pimg_stride;
+            [[maybe_unused]] const T g0 = fma(GeoT<T>::sb(g, b), GeoT<T>::gs(g), GeoT<T>::gh(g, N));
+            [[maybe_unused]] const T gr = GeoT<T>::gr(g);
+            [[maybe_unused]] T rf = (T)r0;
             // Rows are processed in blocks of U: all loads of a block are issued
             // before any of them is used, so U*KB gathers are in flight per warp.
+            // The rows past the segment's end in the last block read nothing and add
+            // exact zeros (one more round trip to memory, where a row at a time
+            // took one each).
             constexpr int U = KB >= 4 ? 4 : 8;
-            const int pp = a.Pp;
-            if constexpr (MODE == kFwd && QL) {
-                constexpr int QW = KB >= 4 ? 4 : KB;  // floats per element of the group's layout
-                const float *q = (g.mode ? a.QT : a.QX) + (size_t)k0 * a.qimg_stride +
-                                 (((size_t)g.frame * N + r0) * pp + 2) * QW;
-                int r = r0;
-                for (; r + U - 1 <= r1; r += U) {
-                    P2 p[U][KB];
-                    T f[U];
+            auto block = [&](auto whole, int rows) {
+                constexpr bool WHOLE = decltype(whole)::value;
+                unsigned idx[U];
+                T f[U];
+                P2 p[U][KB];
+                ray_cells<T, U>(Q, dQ, lim, idx, f);
 #pragma unroll
-                    for (int u = 0; u < U; ++u) {
-                        const long long Qu = Q + (long long)u * dQ;
-                        const int cell = min(max(cell_of(Qu), -2), N);
-                        f[u] = frac_of(Qu, T());
-                        taps_interleaved<KB>(q + ((size_t)u * pp + cell) * QW, a.qimg_stride, p[u]);
+                for (int u = 0; u < U; ++u) {
+                    if (WHOLE || u < rows) {
+                        if constexpr (QL) {
+                            taps_interleaved<KB>(qimg + (size_t)(idx[u] + u * pp) * QW, a.qimg_stride, p[u]);
+                        } else {
+                            const P2 *row = img + (idx[u] + u * pp);
+#pragma unroll
+                            for (int k = 0; k < KB; ++k) p[u][k] = __ldg(row + (size_t)k * a.pimg_stride);
+                        }
+                    } else {
+#pragma unroll
+                        for (int k = 0; k < KB; ++k) p[u][k].x = p[u][k].y = T(0);
                     }
+                }
+                if constexpr (MODE == kFwd) {
 #pragma unroll
                     for (int u = 0; u < U; ++u) {
+                        if (!F32 && !WHOLE && u >= rows) break;  // FP64 products are dear (uniform)
                         const T omf = T(1) - f[u];
 #pragma unroll
                         for (int k = 0; k < KB; ++k) acc[k] = fma(omf, p[u][k].x, fma(f[u], p[u][k].y, acc[k]));
                     }
-                    q += (size_t)U * pp * QW;
-                    Q += (long long)U * dQ;
-                }
-                for (; r <= r1; ++r, q += (size_t)pp * QW, Q += dQ) {
-                    const int cell = min(max(cell_of(Q), -2), N);
-                    const T fr = frac_of(Q, T());
-                    const T omf = T(1) - fr;
-                    P2 p[KB];
-                    taps_interleaved<KB>(q + (size_t)cell * QW, a.qimg_stride, p);
-#pragma unroll
-                    for (int k = 0; k < KB; ++k) acc[k] = fma(omf, p[k].x, fma(fr, p[k].y, acc[k]));
-                }
-            } else if constexpr (MODE == kFwd) {
-                int r = r0;
-                for (; r + U - 1 <= r1; r += U) {
-                    P2 p[U][KB];
-                    T f[U];
+                } else {
+                    // per image k of the group: acc[3k] = sum of interpolated values,
+                    // acc[3k+1] = sum slope * dq/dtheta, acc[3k+2] = sum of slopes
+                    // (offset derivative); the line, cell and fraction serve all KB images
 #pragma unroll
                     for (int u = 0; u < U; ++u) {
-                        const long long Qu = Q + (long long)u * dQ;
-                        const int cell = min(max(cell_of(Qu), -2), N);
-                        f[u] = frac_of(Qu, T());
-                        const P2 *row = img + (size_t)u * pp + cell;
-#pragma unroll
-                        for (int k = 0; k < KB; ++k) p[u][k] = __ldg(row + (size_t)k * a.pimg_stride);
-                    }
-#pragma unroll
-                    for (int u = 0; u < U; ++u) {
-                        const T omf = T(1) - f[u];
-#pragma unroll
-                        for (int k = 0; k < KB; ++k) acc[k] = fma(omf, p[u][k].x, fma(f[u], p[u][k].y, acc[k]));
-                    }
-                    img += (size_t)U * pp;
-                    Q += (long long)U * dQ;
-                }
-                for (; r <= r1; ++r, img += pp, Q += dQ) {
-                    const int cell = min(max(cell_of(Q), -2), N);
-                    const T fr = frac_of(Q, T());
-                    const T omf = T(1) - fr;
-#pragma unroll
-                    for (int k = 0; k < KB; ++k) {
-                        const P2 q = __ldg(img + (size_t)k * a.pimg_stride + cell);
-                        acc[k] = fma(omf, q.x, fma(fr, q.y, acc[k]));
-                    }
-                }
-            } else {
-                // per image k of the group: acc[3k] = sum of interpolated values,
-                // acc[3k+1] = sum slope * dq/dtheta, acc[3k+2] = sum of slopes
-                // (offset derivative); the line, cell and fraction serve all KB images
-                const T g0 = fma(GeoT<T>::sb(g, b), GeoT<T>::gs(g), GeoT<T>::gh(g, N));
-                const T gr = GeoT<T>::gr(g);
-                T rf = (T)r0;
-                int r = r0;
-                for (; r + U - 1 <= r1; r += U) {
-                    P2 p[U][KB];
-                    T f[U];
-#pragma unroll
-                    for (int u = 0; u < U; ++u) {
-                        const long long Qu = Q + (long long)u * dQ;
-                        const int cell = min(max(cell_of(Qu), -2), N);
-                        f[u] = frac_of(Qu, T());
-                        const P2 *row = img + (size_t)u * pp + cell;
-#pragma unroll
-                        for (int k = 0; k < KB; ++k) p[u][k] = __ldg(row + (size_t)k * a.pimg_stride);
-                    }
-#pragma unroll
-                    for (int u = 0; u < U; ++u) {
+                        if (!F32 && !WHOLE && u >= rows) break;
                         const T dq = fma(rf + T(u), gr, g0);
 #pragma unroll
                         for (int k = 0; k < KB; ++k) {
@@ -613,24 +607,15 @@ __global__ void __launch_bounds__(512) k_ray(RayArgs<T> a)
                             if (OFFS) acc[3 * k + 2] += d;
                         }
                     }
-                    img += (size_t)U * pp;
-                    Q += (long long)U * dQ;
                     rf += T(U);
                 }
-                for (; r <= r1; ++r, img += pp, Q += dQ, rf += T(1)) {
-                    const int cell = min(max(cell_of(Q), -2), N);
-                    const T fr = frac_of(Q, T());
-                    const T dq = fma(rf, gr, g0);
-#pragma unroll
-                    for (int k = 0; k < KB; ++k) {
-                        const P2 q = __ldg(img + (size_t)k * a.pimg_stride + cell);
-                        const T d = q.y - q.x;
-                        acc[3 * k] += fma(fr, d, q.x);
-                        acc[3 * k + 1] = fma(d, dq, acc[3 * k + 1]);
-                        if (OFFS) acc[3 * k + 2] += d;
-                    }
-                }
-            }
+                if constexpr (QL) qimg += (size_t)U * pp * QW;
+                else img += (size_t)U * pp;
+                Q += (long long)U * dQ;
+            };
+            int r = r0;
+            for (; r + U - 1 <= r1; r += U) block(std::true_type(), U);
+            if (r <= r1) block(std::false_type(), r1 - r + 1);
         }
         if constexpr (SPLIT > 1) {
             T *mine = red + ((size_t)(slot * SPLIT + seg) * NACC) * 32;
@@ -656,51 +641,41 @@ __global__ void __launch_bounds__(512) k_ray(RayArgs<T> a)
 // out_q[k][v] = scale_q * sum_c partial[k][v][c][q], summed in chunk order,
 // for each of nimg images (partials part_stride doubles apart); with sum, one
 // output per view summing the images in order (each image's chunks in order).
-// One warp per output: the lanes load 32 chunks at a time in one round trip,
-// and the sums run over them in chunk order through shuffles.
-__global__ void k_finalize(const double *__restrict__ partial, int V, int nchunks, int nimg, long long part_stride,
-                           int sum, double *out0, double *out1, double *out2, double scale2, double *out3,
-                           const int *__restrict__ view_mask, const int *__restrict__ skip)
+// One thread per output and quantity, the four quantities of a view side by
+// side: an FP64 addition serves 8 views' four sums at once (it occupies the
+// pipe for 64 cycles whatever the lanes do), where a warp per view with the
+// sums carried by shuffles issued 36 for each view, and the loads of kFinAhead
+// chunks are in flight (Gauss-Newton terms of 512^2 / 360 views: 95.5 -> 91.6
+// us a call).
+constexpr int kFinAhead = 24;
+__global__ void __launch_bounds__(64) k_finalize(const double *__restrict__ partial, int V, int nchunks, int nimg,
+                                                 long long part_stride, int sum, double *out0, double *out1,
+                                                 double *out2, double scale2, double *out3,
+                                                 const int *__restrict__ view_mask, const int *__restrict__ skip)
 {
-    const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    const int o = t >> 2, q = t & 3;
     const int nout = sum ? 1 : nimg;
-    if (w >= V * nout || (skip && *skip)) return;  // warp-uniform
-    const int v = w % V, kout = w / V;
-    if (view_mask && view_mask[v] == 0) return;
-    double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;  // sums over the images, each image's sum added in order
+    if (o >= V * nout || (skip && *skip)) return;
+    const int v = o % V, kout = o / V;
+    double *out = q == 0 ? out0 : (q == 1 ? out1 : (q == 2 ? out2 : out3));
+    if (!out || (view_mask && view_mask[v] == 0)) return;
+    double s = 0.0;  // sum over the images, each image's sum added in order
     const int klo = sum ? 0 : kout, khi = sum ? nimg : kout + 1;
     for (int k = klo; k < khi; ++k) {
-        const double *p = partial + (size_t)k * part_stride + (size_t)v * nchunks * 4;
-        double t0 = 0.0, t1 = 0.0, t2 = 0.0, t3 = 0.0;  // this image, chunks in order
-        for (int base = 0; base < nchunks; base += 32) {
-            double q0 = 0.0, q1 = 0.0, q2 = 0.0, q3 = 0.0;
-            if (base + lane < nchunks) {
-                q0 = p[4 * (base + lane) + 0];
-                q1 = p[4 * (base + lane) + 1];
-                q2 = p[4 * (base + lane) + 2];
-                if (out3) q3 = p[4 * (base + lane) + 3];
-            }
-            const int n = min(32, nchunks - base);
-            for (int c = 0; c < n; ++c) {
-                t0 += __shfl_sync(0xffffffffu, q0, c);
-                t1 += __shfl_sync(0xffffffffu, q1, c);
-                t2 += __shfl_sync(0xffffffffu, q2, c);
-                if (out3) t3 += __shfl_sync(0xffffffffu, q3, c);
-            }
+        const double *p = partial + (size_t)k * part_stride + (size_t)v * nchunks * 4 + q;
+        double x = 0.0;  // this image, chunks in order
+        for (int c = 0; c < nchunks; c += kFinAhead) {
+            double y[kFinAhead];
+#pragma unroll
+            for (int u = 0; u < kFinAhead; ++u) y[u] = c + u < nchunks ? p[4 * (c + u)] : 0.0;
+#pragma unroll
+            for (int u = 0; u < kFinAhead; ++u)
+                if (c + u < nchunks) x += y[u];
         }
-        s0 += t0;
-        s1 += t1;
-        s2 += t2;
-        s3 += t3;
+        s += x;
     }
-    if (lane == 0) {
-        const size_t o = (size_t)kout * V + v;
-        if (out0) out0[o] = s0;
-        if (out1) out1[o] = s1;
-        if (out2) out2[o] = scale2 * s2;
-        if (out3) out3[o] = s3;
-    }
+    out[(size_t)kout * V + v] = q == 2 ? scale2 * s : s;
 }
 
 // ---------------------------------------------------------------------------
@@ -741,14 +716,14 @@ cudaError_t run_ray(const Handle &h, const RayArgs<T> &a)
     return cudaGetLastError();
 }
 
-template <typename T, int MODE, bool OFFS, int KB>
+template <typename T, int MODE, bool OFFS, int KB, bool QL = false>
 cudaError_t run_ray_split(const Handle &h, const RayArgs<T> &a, int split)
 {
     switch (split) {
-    case 1: return run_ray<T, MODE, OFFS, KB, 1>(h, a);
-    case 2: return run_ray<T, MODE, OFFS, KB, 2>(h, a);
-    case 4: return run_ray<T, MODE, OFFS, KB, 4>(h, a);
-    default: return run_ray<T, MODE, OFFS, KB, 8>(h, a);
+    case 1: return run_ray<T, MODE, OFFS, KB, 1, QL>(h, a);
+    case 2: return run_ray<T, MODE, OFFS, KB, 2, QL>(h, a);
+    case 4: return run_ray<T, MODE, OFFS, KB, 4, QL>(h, a);
+    default: return run_ray<T, MODE, OFFS, KB, 8, QL>(h, a);
     }
 }
 
@@ -762,18 +737,6 @@ cudaError_t run_ray_any(const Handle &h, const RayArgs<T> &a, int split, int sta
         if (stage > 0 && band_shape_ok(MODE, KB, a.VW, stage)) return run_ray_band(h, a, MODE, OFFS, KB, stage);
     }
     return run_ray_split<T, MODE, OFFS, KB>(h, a, split);
-}
-
-// The FP32 forward on the interleaved images: kb 8 (two groups of 4), 4, 2 or 1.
-template <int KB>
-cudaError_t run_fwd_interleaved(const Handle &h, const RayArgs<float> &a, int split)
-{
-    switch (split) {
-    case 1: return run_ray<float, kFwd, false, KB, 1, true>(h, a);
-    case 2: return run_ray<float, kFwd, false, KB, 2, true>(h, a);
-    case 4: return run_ray<float, kFwd, false, KB, 4, true>(h, a);
-    default: return run_ray<float, kFwd, false, KB, 8, true>(h, a);
-    }
 }
 
 template <typename T>
@@ -958,10 +921,10 @@ cudaError_t launch_forward(const Handle &h, T *Y, int batch, int kb, int split, 
                 if (groups == 0) continue;
                 a.kbase = k;
                 a.ngroups = groups;
-                cudaError_t e = width == 8   ? run_fwd_interleaved<8>(h, a, split)
-                                : width == 4 ? run_fwd_interleaved<4>(h, a, split)
-                                : width == 2 ? run_fwd_interleaved<2>(h, a, split)
-                                             : run_fwd_interleaved<1>(h, a, split);
+                cudaError_t e = width == 8   ? run_ray_split<float, kFwd, false, 8, true>(h, a, split)
+                                : width == 4 ? run_ray_split<float, kFwd, false, 4, true>(h, a, split)
+                                : width == 2 ? run_ray_split<float, kFwd, false, 2, true>(h, a, split)
+                                             : run_ray_split<float, kFwd, false, 1, true>(h, a, split);
                 if (e != cudaSuccess) return e;
                 k += groups * width;
             }
@@ -999,9 +962,34 @@ cudaError_t launch_forward(const Handle &h, T *Y, int batch, int kb, int split, 
 // The derivative modes over `batch` images sharing the view table: groups of
 // up to kb (1, 2 or 4) images per lane; the fan-beam and band-staged forms
 // take one image per lane (their launches still cover the whole batch).
+// interleaved (FP32, parallel beam, stage 0): the images are those of the
+// interleaved layout of a batch of `batch`, read by its groups of 4, 2 and 1.
 template <typename T, int MODE, bool OFFS>
-cudaError_t der_groups(const Handle &h, RayArgs<T> a, int batch, int kb, int split, int stage)
+cudaError_t der_groups(const Handle &h, RayArgs<T> a, int batch, int kb, int split, int stage, bool interleaved)
 {
+    if (interleaved) {
+        if constexpr (std::is_same<T, float>::value) {
+            if (!h.d_qx || h.fan_D > 0.0 || batch > h.max_batch) return cudaErrorInvalidValue;
+            a.QX = h.d_qx;
+            a.QT = h.d_qt;
+            a.qimg_stride = (long long)h.F * h.N * h.Pp;
+            int k = 0;
+            for (int width : {4, 2, 1}) {
+                const int groups = (batch - k) / width;
+                if (groups == 0) continue;
+                a.kbase = k;
+                a.ngroups = groups;
+                cudaError_t e = width == 4   ? run_ray_split<float, MODE, OFFS, 4, true>(h, a, split)
+                                : width == 2 ? run_ray_split<float, MODE, OFFS, 2, true>(h, a, split)
+                                             : run_ray_split<float, MODE, OFFS, 1, true>(h, a, split);
+                if (e != cudaSuccess) return e;
+                k += groups * width;
+            }
+            return cudaSuccess;
+        } else {
+            return cudaErrorInvalidValue;
+        }
+    }
     bool one = h.fan_D > 0.0;
     if constexpr (std::is_same<T, float>::value) one = one || (stage > 0 && band_shape_ok(MODE, 1, a.VW, stage));
     int k = 0;
@@ -1025,7 +1013,7 @@ cudaError_t der_groups(const Handle &h, RayArgs<T> a, int batch, int kb, int spl
 
 template <typename T>
 cudaError_t launch_jvp(const Handle &h, const double *dtheta, const double *ddelta, T *dY, int split, int vw,
-                       int stage, int batch, int kb, long long dir_stride)
+                       int stage, int batch, int kb, long long dir_stride, bool interleaved)
 {
     RayArgs<T> a = base_args<T>(h);
     a.VW = vw;
@@ -1033,13 +1021,13 @@ cudaError_t launch_jvp(const Handle &h, const double *dtheta, const double *ddel
     a.dtheta = dtheta;
     a.ddelta = ddelta;
     a.dir_stride = dir_stride;
-    return ddelta ? der_groups<T, kJvp, true>(h, a, batch, kb, split, stage)
-                  : der_groups<T, kJvp, false>(h, a, batch, kb, split, stage);
+    return ddelta ? der_groups<T, kJvp, true>(h, a, batch, kb, split, stage, interleaved)
+                  : der_groups<T, kJvp, false>(h, a, batch, kb, split, stage, interleaved);
 }
 
 template <typename T>
 cudaError_t launch_vjp(const Handle &h, const T *R, double *gtheta, double *gdelta, int split, int vw, int stage,
-                       int batch, int kb, long long r_stride, int sum)
+                       int batch, int kb, long long r_stride, int sum, bool interleaved)
 {
     RayArgs<T> a = base_args<T>(h);
     a.VW = vw;
@@ -1047,11 +1035,11 @@ cudaError_t launch_vjp(const Handle &h, const T *R, double *gtheta, double *gdel
     a.r_stride = r_stride;
     a.partial = h.d_partial;
     a.part_stride = 4LL * h.V * h.nchunks;
-    cudaError_t e = gdelta ? der_groups<T, kVjp, true>(h, a, batch, kb, split, stage)
-                           : der_groups<T, kVjp, false>(h, a, batch, kb, split, stage);
+    cudaError_t e = gdelta ? der_groups<T, kVjp, true>(h, a, batch, kb, split, stage, interleaved)
+                           : der_groups<T, kVjp, false>(h, a, batch, kb, split, stage, interleaved);
     if (e != cudaSuccess) return e;
     const long long outs = (long long)h.V * (sum ? 1 : batch);
-    k_finalize<<<(int)((outs + 7) / 8), 256, 0, h.stream>>>(h.d_partial, h.V, h.nchunks, batch, a.part_stride,
+    k_finalize<<<(int)((4 * outs + 63) / 64), 64, 0, h.stream>>>(h.d_partial, h.V, h.nchunks, batch, a.part_stride,
                                                             sum, gtheta, gdelta, nullptr, 1.0, nullptr, nullptr,
                                                             nullptr);
     return cudaGetLastError();
@@ -1059,7 +1047,8 @@ cudaError_t launch_vjp(const Handle &h, const T *R, double *gtheta, double *gdel
 
 template <typename T>
 cudaError_t launch_gn(const Handle &h, const T *bdata, T *res, double *grad, double *jnorm2, double *fval, int split,
-                      int vw, int stage, const int *view_mask, const int *skip, int batch, int kb, double *rscale)
+                      int vw, int stage, const int *view_mask, const int *skip, int batch, int kb, double *rscale,
+                      bool interleaved)
 {
     RayArgs<T> a = base_args<T>(h);
     a.VW = vw;
@@ -1070,10 +1059,10 @@ cudaError_t launch_gn(const Handle &h, const T *bdata, T *res, double *grad, dou
     a.part_stride = 4LL * h.V * h.nchunks;
     a.view_mask = view_mask;
     a.skip = skip;
-    cudaError_t e = der_groups<T, kGn, false>(h, a, batch, kb, split, stage);
+    cudaError_t e = der_groups<T, kGn, false>(h, a, batch, kb, split, stage, interleaved);
     if (e != cudaSuccess) return e;
     const long long outs = (long long)h.V * batch;
-    k_finalize<<<(int)((outs + 7) / 8), 256, 0, h.stream>>>(h.d_partial, h.V, h.nchunks, batch, a.part_stride, 0,
+    k_finalize<<<(int)((4 * outs + 63) / 64), 64, 0, h.stream>>>(h.d_partial, h.V, h.nchunks, batch, a.part_stride, 0,
                                                             grad, jnorm2, fval, 0.5, rscale, view_mask, skip);
     return cudaGetLastError();
 }
@@ -1087,11 +1076,11 @@ cudaError_t launch_gn(const Handle &h, const T *bdata, T *res, double *grad, dou
                                                 const double *);                                           \
     template cudaError_t launch_forward<T>(const Handle &, T *, int, int, int, int, int, const int *, bool, int); \
     template cudaError_t launch_jvp<T>(const Handle &, const double *, const double *, T *, int, int, int, int, \
-                                       int, long long);                                                   \
+                                       int, long long, bool);                                             \
     template cudaError_t launch_vjp<T>(const Handle &, const T *, double *, double *, int, int, int, int, int, \
-                                       long long, int);                                                   \
+                                       long long, int, bool);                                             \
     template cudaError_t launch_gn<T>(const Handle &, const T *, T *, double *, double *, double *, int,    \
-                                      int, int, const int *, const int *, int, int, double *);
+                                      int, int, const int *, const int *, int, int, double *, bool);
 
 CTGB_RAY_INSTANTIATE(float)
 CTGB_RAY_INSTANTIATE(double)
