@@ -252,9 +252,9 @@ void default_tuning(ctgb::Handle &h)
     h.tune.der_kb = std::min(kb, 4);
     if (h.fan_D > 0.0) {
         // fan-beam transpose: one candidate search per pixel and view serves
-        // every sinogram of a thread; two view groups per pixel keep the warps up
+        // every sinogram of a thread; in FP64 two view groups per pixel keep the warps up
         h.tune.adj_kb = kb;
-        h.tune.adj_split = 2;
+        h.tune.adj_split = h.precision ? 2 : 1;
     }
 }
 
@@ -469,6 +469,8 @@ template <typename T> int autotune_impl(ctgb::Handle &h)
     cudaFree(d_in);
     // the view table now holds the tuning angles; force a rebuild on the next call
     cudaMemsetAsync(h.d_views, 0, sizeof(ctgb::ViewGeo) * h.V, h.stream);
+    // (and with it the fan-beam tables, whose stamps count from the view table's)
+    if (h.d_fanview) cudaMemsetAsync(h.d_fanview, 0, ctgb::fan_view_bytes() * (size_t)h.V, h.stream);
     return rc;
 }
 
@@ -578,7 +580,7 @@ int ct_init(const ct_geom *g, void *cuda_stream, ct_handle **out)
         if (e == cudaSuccess) e = cudaMemset(h.d_px, 0, img_pairs * pair_bytes);
         if (e == cudaSuccess) e = cudaMemset(h.d_pt, 0, img_pairs * pair_bytes);
         if (e == cudaSuccess) e = cudaMemset(h.d_yp, 0, sino_pairs * pair_bytes);
-        // fan beam: generation 0 marks every ray and view entry as not built (views start at 1)
+        // fan beam: generation 0 marks every view record as not built (views start at 1)
         if (e == cudaSuccess && h.d_rays)
             e = cudaMemset(h.d_rays, 0, ctgb::fan_ray_bytes(h.precision) * (size_t)h.V * h.B);
         if (e == cudaSuccess && h.d_fanview) e = cudaMemset(h.d_fanview, 0, ctgb::fan_view_bytes() * (size_t)h.V);

@@ -37,7 +37,6 @@ namespace {
 
 namespace cg = cooperative_groups;
 
-constexpr int kMaxSegs = 8;  // CTAs per tile: the portable cluster size
 
 // ---------------------------------------------------------------------------
 // FP32
@@ -74,38 +73,6 @@ struct __align__(16) AdjView {
     int row;        // view
     float w2, c1;   // KB >= 4: w^2 and w - w^2
 };
-
-__device__ __forceinline__ void cp_async16_zfill(void *smem, const void *gmem, bool valid)
-{
-    const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
-    const int bytes = valid ? 16 : 0;  // 0: the destination is zero-filled, the source is not read
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(s), "l"(gmem), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait0() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
-
-// Two floats in a register pair, for the packed multiply-adds (fma.rn.f32x2:
-// one issue slot for two).
-typedef unsigned long long f32x2;
-__device__ __forceinline__ f32x2 pack2(float x, float y)
-{
-    f32x2 r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
-    return r;
-}
-__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c)
-{
-    f32x2 r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-    return r;
-}
-__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b)
-{
-    f32x2 r;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ float half2f(f32x2 v, int i) { return __uint_as_float((unsigned)(v >> (32 * i))); }
 
 // Sums of a thread's 2 x 2 pixels (index 2 * y + x) for KB sinograms.
 // KB <= 2: each pixel reads its own two bins, the kernel being bound by the
@@ -785,53 +752,6 @@ template <typename T> SmallArgs<T> small_args(const Handle &h, T *X, int k0, int
 // ---------------------------------------------------------------------------
 // launches
 // ---------------------------------------------------------------------------
-// CTAs per tile: at least `split` (the launch shape), at most kMaxSegs, such
-// that the SM with most CTAs has least to do: ceil(tiles * segs / SMs) CTAs of
-// (views / segs) views plus `fixed` views' worth of prologue and epilogue
-// each (8 in FP32; 3 in FP64, whose views take longer); an SM with one CTA does not hide its latency and counts as two.  More
-// than 2 CTAs only where each keeps 8 views: below that the prologue is all
-// there is (64^2, 22 views: 6.1 us at any size).
-// Clusters of odd size measured slower (256^2, 180 views, 8 sinograms: 30.7 us
-// at 4 or 6, 34.8 at 5 and 34.9 at 7; one CTA per tile 65.5).
-int adj_segs(const Handle &h, long long tiles, int split, int fixed)
-{
-    const int views = std::max(1, h.V / h.F);
-    int best = 1;
-    double best_cost = 1e300;
-    for (int segs : {1, 2, 4, 6, 8}) {
-        if (segs < split) continue;
-        if (segs > 2 && views < 8 * segs) break;
-        const long long ctas = std::max<long long>(2, (tiles * segs + h.num_sms - 1) / h.num_sms);
-        const double cost = (double)ctas * ((views + segs - 1) / segs + fixed);
-        if (cost < best_cost) {
-            best_cost = cost;
-            best = segs;
-        }
-    }
-    return best;
-}
-
-template <typename A> cudaError_t launch_cluster(void (*kern)(A), const A &a, const Handle &h, size_t smem)
-{
-    if (smem > 48 * 1024) return cudaErrorInvalidValue;  // no kernel here needs more
-    const long long items = (long long)a.ngroups * a.F * a.tps * a.tps * a.segs;
-    int grid = persistent_grid(kern, 256, smem, items, h.num_sms);
-    grid -= grid % a.segs;  // whole clusters (items is a multiple of segs, so grid >= segs)
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(256);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = h.stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = a.segs;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kern, a);
-}
-
 cudaError_t adjoint32(const Handle &h, float *X, int batch, int kb, int split, int layout_batch, const int *skip)
 {
     AdjArgs a{};

@@ -7,6 +7,7 @@
 #include <map>
 #include <mutex>
 #include <tuple>
+#include <type_traits>
 
 #include "ct_internal.cuh"
 
@@ -148,6 +149,40 @@ __device__ __forceinline__ void warp_rows(const ViewGeo &g, int b, bool active, 
     rhi = __reduce_max_sync(0xffffffffu, u);
 }
 
+// Element indices (cell + 2, clamped to the row's zero padding) and fractions
+// of U consecutive rows from the exact line value Q at the first.  FP32: the
+// rows are walked relative to the first one's cell with 55 fractional bits (the
+// 48 of the line, shifted), so the high word holds the cell offset in its top
+// 9 bits and the 23 bits of the fraction below them: one shift, one logic
+// operation and one add-and-clamp a row, where the full-range line needs a
+// two-word shift, two clamps and a second shift (the integer pipe was the bound
+// of one image per lane: 74 % busy, now 58).  The same bits as cell_of and
+// frac_of.  One image of 2048^2, 120 views: 362 -> 282 us; 256^2 / 180 views:
+// 18.6 -> 16.3.
+template <typename T, int U>
+__device__ __forceinline__ void ray_cells(long long Q, long long dQ, unsigned lim, unsigned (&idx)[U], T (&f)[U])
+{
+    if constexpr (std::is_same<T, float>::value) {
+        static_assert(kFracBits == 48 && U <= 16, "cell offsets of a block fit 9 bits");
+        const unsigned base = (unsigned)(cell_of(Q) + 2);
+        const long long L0 = (long long)(((unsigned long long)Q << 16) >> 9), dL = dQ << 7;
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int hi = (int)((L0 + (long long)u * dL) >> 32);
+            // (a negative index is a large unsigned one)
+            idx[u] = __viaddmin_u32((unsigned)(hi >> 23), base, lim);
+            f[u] = __int_as_float((hi & 0x7FFFFF) | 0x3F800000) - 1.0f;
+        }
+    } else {
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const long long Qu = Q + (long long)u * dQ;
+            idx[u] = min((unsigned)(cell_of(Qu) + 2), lim);
+            f[u] = frac_of(Qu, T());
+        }
+    }
+}
+
 // Per-ray output of a march: the forward stores w * sum for each image, the
 // JVP stores the directional derivative, the VJP and Gauss-Newton modes write
 // per-(view, chunk) partial sums reduced over the warp in a fixed order.
@@ -268,5 +303,90 @@ inline int persistent_grid(K kernel, int threads, size_t smem, long long work_bl
     const long long cap = 64LL * per_sm * num_sms;
     return (int)std::max<long long>(1, std::min(work_blocks, cap));
 }
+
+// ---------------------------------------------------------------------------
+// transpose kernels (ct_backproject.cu, ct_fan.cu)
+// ---------------------------------------------------------------------------
+constexpr int kMaxSegs = 8;  // CTAs per tile: the portable cluster size
+
+// CTAs per tile: at least `split` (the launch shape), at most kMaxSegs, such
+// that the SM with most CTAs has least to do: ceil(tiles * segs / SMs) CTAs of
+// (views / segs) views plus `fixed` views' worth of prologue and epilogue
+// each (8 in FP32; 3 in FP64, whose views take longer); an SM with one CTA does not hide its latency and counts as two.  More
+// than 2 CTAs only where each keeps 8 views: below that the prologue is all
+// there is (64^2, 22 views: 6.1 us at any size).
+// Clusters of odd size measured slower (256^2, 180 views, 8 sinograms: 30.7 us
+// at 4 or 6, 34.8 at 5 and 34.9 at 7; one CTA per tile 65.5).
+inline int adj_segs(const Handle &h, long long tiles, int split, int fixed)
+{
+    const int views = std::max(1, h.V / h.F);
+    int best = 1;
+    double best_cost = 1e300;
+    for (int segs : {1, 2, 4, 6, 8}) {
+        if (segs < split) continue;
+        if (segs > 2 && views < 8 * segs) break;
+        const long long ctas = std::max<long long>(2, (tiles * segs + h.num_sms - 1) / h.num_sms);
+        const double cost = (double)ctas * ((views + segs - 1) / segs + fixed);
+        if (cost < best_cost) {
+            best_cost = cost;
+            best = segs;
+        }
+    }
+    return best;
+}
+
+// Launch of a transpose kernel: 256 threads, the a.segs CTAs of a tile one cluster.
+template <typename A> inline cudaError_t launch_cluster(void (*kern)(A), const A &a, const Handle &h, size_t smem)
+{
+    if (smem > 48 * 1024) return cudaErrorInvalidValue;  // no kernel here needs more
+    const long long items = (long long)a.ngroups * a.F * a.tps * a.tps * a.segs;
+    int grid = persistent_grid(kern, 256, smem, items, h.num_sms);
+    grid -= grid % a.segs;  // whole clusters (items is a multiple of segs, so grid >= segs)
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(256);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = h.stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = a.segs;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, a);
+}
+
+__device__ __forceinline__ void cp_async16_zfill(void *smem, const void *gmem, bool valid)
+{
+    const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
+    const int bytes = valid ? 16 : 0;  // 0: the destination is zero-filled, the source is not read
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(s), "l"(gmem), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
+__device__ __forceinline__ void cp_async_wait0() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
+
+// Two floats in a register pair, for the packed multiply-adds (fma.rn.f32x2:
+// one issue slot for two).
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pack2(float x, float y)
+{
+    f32x2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
+    return r;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c)
+{
+    f32x2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b)
+{
+    f32x2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ float half2f(f32x2 v, int i) { return __uint_as_float((unsigned)(v >> (32 * i))); }
 
 }  // namespace ctgb

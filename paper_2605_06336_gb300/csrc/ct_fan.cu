@@ -20,22 +20,23 @@
 // along e (ds_b/ddelta = 1, the source stays): dq/ddelta = s0 + r sr with
 // sr = -dC/ds, s0 = +-dA/ds + h dC/ds, and dw/ddelta = C dC/ds / w.
 //
-//   k_fan_rays   per-ray table (fixed-point line, weight, derivative
-//                constants, march range) from the view table, for the views
-//                rebuilt since (generation stamps)
-//   k_fan_views  per-view record of the transpose (FP32 constants, bin
-//                ranges of row- and column-marched rays)
+//   k_fan_table  per-ray table (fixed-point line, weight, derivative
+//                constants, march range) and per-view record of the transpose
+//                (FP32 constants, bin ranges of row- and column-marched rays)
+//                from the view table, for the views rebuilt since
 //   k_ray_fan    SPLIT warps (row segments) per 32 bins of one view: forward
 //                (KB images), JVP, VJP and Gauss-Newton terms, each lane on
 //                its own line
 //   k_fan_sino   sinograms interleaved in blocks of 8 for the transpose
-//   k_adj_fan    exact transpose in gather form: a pixel takes, per view,
+//   k_adj_fan_tile, k_adj_fan (FP32, FP64)
+//                exact transpose in gather form: a pixel takes, per view,
 //                the rays whose fixed-point sample at its row (row-marched
 //                rays) or column (column-marched rays) falls in its
 //                interpolation cell; the candidates come from the projective
 //                inverse of the pixel's neighbourhood and are then tested
 //                with the very values the forward uses, so the matrix
 //                entries are those of the forward.
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -53,7 +54,7 @@ template <typename T> struct __align__(16) FanRay {
     T w, dw, g0, gr;   // weight, d w / d theta, dq/dtheta = g0 + r gr
     float rlo, rhi;    // march indices with -1 < q < N lie in [rlo, rhi] (two indices of margin)
     int mode;          // 0: rows of X, 1: rows of X^T (columns)
-    int gen;           // generation of the view record the entry was built from (0: never)
+    int pad;
     T dws, s0, sr;     // d w / d delta, dq/ddelta = s0 + r sr
 };
 
@@ -78,111 +79,97 @@ struct __align__(16) FanView {
     int mode0, split, gen, pad;
 };
 
+// One CTA per view: nothing when the view record it was built from is current
+// (one generation stamp per view; a stamp per ray made every call read the
+// whole table), else the view's rays and its record.
 template <typename T>
-__global__ void __launch_bounds__(256) k_fan_rays(const ViewGeo *__restrict__ vg, int V, int B, int N, double D,
-                                                  FanRay<T> *__restrict__ out, FanLine<T> *__restrict__ lines,
-                                                  const int *__restrict__ skip)
+__global__ void __launch_bounds__(128) k_fan_table(const ViewGeo *__restrict__ vg, int V, int B, int N, double D,
+                                                   FanRay<T> *__restrict__ rays, FanLine<T> *__restrict__ lines,
+                                                   FanView *__restrict__ views, const int *__restrict__ skip)
 {
     if (skip && *skip) return;
+    __shared__ int s_mode0, s_split;
     const double h = 0.5 * (N - 1);
-    for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < (long long)V * B;
-         idx += (long long)gridDim.x * blockDim.x) {
-        const int v = (int)(idx / B), b = (int)(idx - (long long)v * B);
+    for (int v = blockIdx.x; v < V; v += gridDim.x) {
         const ViewGeo &g = vg[v];
-        if (out[idx].gen == g.gen) continue;  // built from this view record already
-        const double c = g.c, sn = g.s, s = g.sb0d + (double)b;
-        const double rx = s * c - D * sn, ry = s * sn + D * c;
-        const double px = s * c, py = s * sn, dpx = -s * sn, dpy = s * c;
-        double C, A, dC, dA, qh, g0, dCs, s0;
-        int mode;
-        if (fabs(rx) <= fabs(ry)) {
-            mode = 0;
-            C = rx / ry;
-            A = px - py * C;
-            dC = -(1.0 + C * C);
-            dA = dpx - C * dpy - py * dC;
-            qh = h + A;
-            g0 = dA + h * dC;
-            dCs = (c * ry - sn * rx) / (ry * ry);  // d/ds of C and A: P_b and r move by e
-            s0 = (c - C * sn - py * dCs) + h * dCs;
-        } else {
-            mode = 1;
-            C = ry / rx;
-            A = py - px * C;
-            dC = 1.0 + C * C;
-            dA = dpy - C * dpx - px * dC;
-            qh = h - A;
-            g0 = -dA + h * dC;
-            dCs = (sn * rx - c * ry) / (rx * rx);
-            s0 = -(sn - C * c - px * dCs) + h * dCs;
+        if (views[v].gen == g.gen) continue;  // uniform
+        __syncthreads();  // every thread has read the stamp and the previous view's record is written
+        if (threadIdx.x == 0) s_split = B;
+        for (int b = threadIdx.x; b < B; b += blockDim.x) {
+            const size_t idx = (size_t)v * B + b;
+            const double c = g.c, sn = g.s, s = g.sb0d + (double)b;
+            const double rx = s * c - D * sn, ry = s * sn + D * c;
+            const double px = s * c, py = s * sn, dpx = -s * sn, dpy = s * c;
+            double C, A, dC, dA, qh, g0, dCs, s0;
+            int mode;
+            if (fabs(rx) <= fabs(ry)) {
+                mode = 0;
+                C = rx / ry;
+                A = px - py * C;
+                dC = -(1.0 + C * C);
+                dA = dpx - C * dpy - py * dC;
+                qh = h + A;
+                g0 = dA + h * dC;
+                dCs = (c * ry - sn * rx) / (ry * ry);  // d/ds of C and A: P_b and r move by e
+                s0 = (c - C * sn - py * dCs) + h * dCs;
+            } else {
+                mode = 1;
+                C = ry / rx;
+                A = py - px * C;
+                dC = 1.0 + C * C;
+                dA = dpy - C * dpx - px * dC;
+                qh = h - A;
+                g0 = -dA + h * dC;
+                dCs = (sn * rx - c * ry) / (rx * rx);
+                s0 = -(sn - C * c - px * dCs) + h * dCs;
+            }
+            const double qr = -C;
+            const double w = sqrt(1.0 + C * C);
+            FanRay<T> R;
+            R.Qc = __double2ll_rn(qh * kFixScale);
+            R.Qh = __double2ll_rn(qr * 0.5 * kFixScale);
+            R.w = (T)w;
+            R.dw = (T)(C * dC / w);
+            R.g0 = (T)g0;
+            R.gr = (T)(-dC);
+            R.dws = (T)(C * dCs / w);
+            R.s0 = (T)s0;
+            R.sr = (T)(-dCs);
+            R.mode = mode;
+            R.pad = 0;
+            if (fabs(qr) < 1e-12) {
+                const bool in = qh > -1.0 && qh < (double)N;
+                R.rlo = in ? 0.0f : (float)N;
+                R.rhi = in ? (float)(N - 1) : -1.0f;
+            } else {
+                const double ra = h + (-1.0 - qh) / qr, rb = h + ((double)N - qh) / qr;
+                R.rlo = (float)fmin(fmax(fmin(ra, rb) - 2.0, 0.0), (double)N);
+                R.rhi = (float)fmax(fmin(fmax(ra, rb) + 2.0, (double)(N - 1)), -1.0);
+            }
+            rays[idx] = R;
+            FanLine<T> L;
+            L.Qc = R.Qc;
+            L.Qh = R.Qh;
+            L.w = R.w;
+            lines[idx] = L;
+            if (b == 0) s_mode0 = R.mode;
         }
-        const double qr = -C;
-        const double w = sqrt(1.0 + C * C);
-        FanRay<T> R;
-        R.Qc = __double2ll_rn(qh * kFixScale);
-        R.Qh = __double2ll_rn(qr * 0.5 * kFixScale);
-        R.w = (T)w;
-        R.dw = (T)(C * dC / w);
-        R.g0 = (T)g0;
-        R.gr = (T)(-dC);
-        R.dws = (T)(C * dCs / w);
-        R.s0 = (T)s0;
-        R.sr = (T)(-dCs);
-        R.mode = mode;
-        R.gen = g.gen;
-        if (fabs(qr) < 1e-12) {
-            const bool in = qh > -1.0 && qh < (double)N;
-            R.rlo = in ? 0.0f : (float)N;
-            R.rhi = in ? (float)(N - 1) : -1.0f;
-        } else {
-            const double ra = h + (-1.0 - qh) / qr, rb = h + ((double)N - qh) / qr;
-            R.rlo = (float)fmin(fmax(fmin(ra, rb) - 2.0, 0.0), (double)N);
-            R.rhi = (float)fmax(fmin(fmax(ra, rb) + 2.0, (double)(N - 1)), -1.0);
+        __syncthreads();
+        for (int b = threadIdx.x; b < B; b += blockDim.x)  // the thread's own rays, written above
+            if (rays[(size_t)v * B + b].mode != s_mode0) atomicMin(&s_split, b);
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            FanView f;
+            f.c = (float)g.c;
+            f.sn = (float)g.s;
+            f.sb0 = (float)g.sb0d;
+            f.iD = (float)(1.0 / D);
+            f.mode0 = s_mode0;
+            f.split = s_split;
+            f.gen = g.gen;
+            f.pad = 0;
+            views[v] = f;
         }
-        out[idx] = R;
-        FanLine<T> L;
-        L.Qc = R.Qc;
-        L.Qh = R.Qh;
-        L.w = R.w;
-        lines[idx] = L;
-    }
-}
-
-// One warp per view: the per-view record of the transpose, rebuilt when the
-// view record changed (after k_fan_rays has rebuilt its rays).
-template <typename T>
-__global__ void __launch_bounds__(256) k_fan_views(const ViewGeo *__restrict__ vg, int V, int B, double D,
-                                                   const FanRay<T> *__restrict__ rays, FanView *__restrict__ out,
-                                                   const int *__restrict__ skip)
-{
-    if (skip && *skip) return;
-    const int v = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    if (v >= V) return;  // warp-uniform
-    const ViewGeo &g = vg[v];
-    if (out[v].gen == g.gen) return;
-    const FanRay<T> *rv = rays + (size_t)v * B;
-    const int mode0 = rv[0].mode;
-    int split = B;
-    for (int base = 0; base < B; base += 32) {
-        const int b = base + lane;
-        const unsigned other = __ballot_sync(0xffffffffu, b < B && rv[b].mode != mode0);
-        if (other) {
-            split = base + __ffs(other) - 1;
-            break;
-        }
-    }
-    if (lane == 0) {
-        FanView f;
-        f.c = (float)g.c;
-        f.sn = (float)g.s;
-        f.sb0 = (float)g.sb0d;
-        f.iD = (float)(1.0 / D);
-        f.mode0 = mode0;
-        f.split = split;
-        f.gen = g.gen;
-        f.pad = 0;
-        out[v] = f;
     }
 }
 
@@ -219,75 +206,48 @@ __global__ void __launch_bounds__(32 * SPLIT) k_ray_fan(RayArgs<T> a, const FanR
         T acc[NACC];
 #pragma unroll
         for (int k = 0; k < NACC; ++k) acc[k] = T(0);
-        const P2 *img = (R.mode ? a.PT : a.PX) + (size_t)a.vg[v].frame * N * a.Pp + (size_t)k0 * a.pimg_stride + 2;
+        const P2 *img = (R.mode ? a.PT : a.PX) + ((size_t)a.vg[v].frame * N + r0) * a.Pp + (size_t)k0 * a.pimg_stride;
         const long long dQ = 2 * R.Qh;
         long long Q = R.Qc + (long long)(2 * r0 - (N - 1)) * R.Qh;
+        const unsigned pp = (unsigned)a.Pp, lim = (unsigned)(N + 2);
         constexpr int U = 4;
-        int r = r0;
-        if constexpr (MODE == kFwd) {
-            for (; r + U - 1 <= r1; r += U) {
-                P2 p[U][KB];
-                T f[U];
+        // rows in blocks of U whose loads are all issued first; the last block's
+        // missing rows read nothing and add exact zeros
+        auto block = [&](auto whole, int r, int rows) {
+            constexpr bool WHOLE = decltype(whole)::value;
+            unsigned idx[U];
+            T f[U];
+            P2 p[U][KB];
+            ray_cells<T, U>(Q, dQ, lim, idx, f);
 #pragma unroll
-                for (int u = 0; u < U; ++u) {
-                    const long long Qu = Q + (long long)u * dQ;
-                    const int cell = min(max(cell_of(Qu), -2), N);
-                    f[u] = frac_of(Qu, T());
-                    const P2 *row = img + (size_t)(r + u) * a.Pp + cell;
+            for (int u = 0; u < U; ++u) {
 #pragma unroll
-                    for (int k = 0; k < KB; ++k) p[u][k] = __ldg(row + (size_t)k * a.pimg_stride);
+                for (int k = 0; k < KB; ++k) {
+                    if (WHOLE || u < rows) p[u][k] = __ldg(img + (idx[u] + u * pp) + (size_t)k * a.pimg_stride);
+                    else p[u][k].x = p[u][k].y = T(0);
                 }
+            }
 #pragma unroll
-                for (int u = 0; u < U; ++u) {
+            for (int u = 0; u < U; ++u) {
+                if constexpr (MODE == kFwd) {
                     const T omf = T(1) - f[u];
 #pragma unroll
                     for (int k = 0; k < KB; ++k) acc[k] = fma(omf, p[u][k].x, fma(f[u], p[u][k].y, acc[k]));
-                }
-                Q += (long long)U * dQ;
-            }
-            for (; r <= r1; ++r, Q += dQ) {
-                const int cell = min(max(cell_of(Q), -2), N);
-                const T fr = frac_of(Q, T());
-                const T omf = T(1) - fr;
-#pragma unroll
-                for (int k = 0; k < KB; ++k) {
-                    const P2 q = __ldg(img + (size_t)r * a.Pp + (size_t)k * a.pimg_stride + cell);
-                    acc[k] = fma(omf, q.x, fma(fr, q.y, acc[k]));
-                }
-            }
-        } else {
-            // acc[0] = sum of interpolated values, acc[1] = sum slope * dq/dtheta,
-            // acc[2] (offsets) = sum slope * dq/ddelta; rows in blocks of U whose
-            // loads are all issued first
-            for (; r + U - 1 <= r1; r += U) {
-                P2 p[U];
-                T f[U];
-#pragma unroll
-                for (int u = 0; u < U; ++u) {
-                    const long long Qu = Q + (long long)u * dQ;
-                    const int cell = min(max(cell_of(Qu), -2), N);
-                    f[u] = frac_of(Qu, T());
-                    p[u] = __ldg(img + (size_t)(r + u) * a.Pp + cell);
-                }
-#pragma unroll
-                for (int u = 0; u < U; ++u) {
-                    const T d = p[u].y - p[u].x;
-                    acc[0] += fma(f[u], d, p[u].x);
+                } else {
+                    // acc[0] = sum of interpolated values, acc[1] = sum slope * dq/dtheta,
+                    // acc[2] (offsets) = sum slope * dq/ddelta
+                    const T d = p[u][0].y - p[u][0].x;
+                    acc[0] += fma(f[u], d, p[u][0].x);
                     acc[1] = fma(d, fma((T)(r + u), R.gr, R.g0), acc[1]);
                     if constexpr (OFFS) acc[NACC - 1] = fma(d, fma((T)(r + u), R.sr, R.s0), acc[NACC - 1]);
                 }
-                Q += (long long)U * dQ;
             }
-            for (; r <= r1; ++r, Q += dQ) {
-                const int cell = min(max(cell_of(Q), -2), N);
-                const T fr = frac_of(Q, T());
-                const P2 q = __ldg(img + (size_t)r * a.Pp + cell);
-                const T d = q.y - q.x;
-                acc[0] += fma(fr, d, q.x);
-                acc[1] = fma(d, fma((T)r, R.gr, R.g0), acc[1]);
-                if constexpr (OFFS) acc[NACC - 1] = fma(d, fma((T)r, R.sr, R.s0), acc[NACC - 1]);
-            }
-        }
+            img += (size_t)U * pp;
+            Q += (long long)U * dQ;
+        };
+        int r = r0;
+        for (; r + U - 1 <= r1; r += U) block(std::true_type(), r, U);
+        if (r <= r1) block(std::false_type(), r, r1 - r + 1);
         if constexpr (SPLIT > 1) {
 #pragma unroll
             for (int k = 0; k < NACC; ++k) red[seg][k][lane] = acc[k];
@@ -388,6 +348,270 @@ __global__ void k_fan_sino(const T *__restrict__ Y, T *__restrict__ YI, long lon
     }
 }
 
+// ---------------------------------------------------------------------------
+// FP32 transpose
+// ---------------------------------------------------------------------------
+constexpr int kFanWin = 64;      // rays of a view staged at a time
+constexpr int kFanVB = 4;        // views per staged block: one staged ray per thread
+constexpr int kFanCap = 128;     // views whose tile constants are staged at a time
+constexpr int kFanFrac = 25;     // fractional bits of a ray's in-tile coordinate
+
+struct FanTileArgs {
+    const FanLine<float> *lines;
+    const FanView *views;
+    const int *fstart, *fcount;
+    int N, B, F, tps;
+    const float *YI;             // [k / 8][V][B][8]
+    long long yi_stride;         // floats per block of 8 sinograms
+    int kbase, ngroups;
+    float *X;
+    long long img_stride;
+    int segs;
+    const int *skip;
+};
+
+struct __align__(16) FanTileView {
+    float c, sn, sb0, iD;
+    int mode0, split, start, count;  // rays [start, start + count) can touch the tile
+    int v, pad[3];
+};
+
+// A ray near the tile: its coordinate at the tile's centre row (column, for
+// column-marched rays) relative to the centre pixel, its slope, its weight.
+struct __align__(16) FanTileRay {
+    int P, S;
+    float w;
+    int pad;
+};
+
+template <int KB> struct FanSums {
+    float v[KB];
+    __device__ void clear()
+    {
+#pragma unroll
+        for (int k = 0; k < KB; ++k) v[k] = 0.0f;
+    }
+    __device__ float get(int k) const { return v[k]; }
+    __device__ __forceinline__ void add(float w, const float *y)
+    {
+#pragma unroll
+        for (int k = 0; k < KB; ++k) v[k] = fmaf(w, y[k], v[k]);
+    }
+};
+template <int KB> struct FanSumsPacked {
+    f32x2 v[KB / 2];
+    __device__ void clear()
+    {
+#pragma unroll
+        for (int k = 0; k < KB / 2; ++k) v[k] = 0ull;
+    }
+    __device__ float get(int k) const { return half2f(v[k >> 1], k & 1); }
+    __device__ __forceinline__ void add(float w, const float *y)
+    {
+        const f32x2 ww = pack2(w, w);
+#pragma unroll
+        for (int g = 0; g < KB / 4; ++g) {
+            const ulonglong2 u = *reinterpret_cast<const ulonglong2 *>(y + 4 * kFanWin * g);
+            v[2 * g] = fma2(ww, u.x, v[2 * g]);
+            v[2 * g + 1] = fma2(ww, u.y, v[2 * g + 1]);
+        }
+    }
+};
+template <> struct FanSums<4> : FanSumsPacked<4> {};
+template <> struct FanSums<8> : FanSumsPacked<8> {};
+
+// One CTA = one 16 x 16 pixel tile of one frame, one of `segs` view subsets
+// and KB sinograms.  What bounds the transpose is the search: per pixel and
+// view two projective bounds and two or three candidate rays, each tested with
+// its own line.  With the rays' full-range lines read from global memory it
+// took 250 instructions per warp and view, waiting on loads (152 us for 256^2 /
+// 180 views, 8 sinograms).  Here the rays that can touch the tile (between the
+// projections of the corners of its one-pixel neighbourhood) are staged once
+// per tile and view with their lines reduced to 32-bit in-tile coordinates
+// (from the table's fixed-point line, to 2^-25 pixel: closer than the forward's
+// 23-bit fractions), their sinogram bins beside them; the next block's lines
+// are loaded and its bins copied while the current one is read: 92 us.
+template <int KB>
+__global__ void __launch_bounds__(256) k_adj_fan_tile(FanTileArgs a)
+{
+    namespace cg = cooperative_groups;
+    __shared__ FanTileView s_view[kFanCap];
+    __shared__ FanTileRay s_ray[2][kFanVB][kFanWin];
+    // (8 sinograms as two arrays of 4, so that a quarter-warp's 16-byte loads meet no bank twice)
+    constexpr int W = KB >= 4 ? 4 : KB;
+    __shared__ __align__(16) float s_y[2][kFanVB][KB / W][kFanWin][W];
+    __shared__ int s_max;
+    float *red = &s_y[0][0][0][0][0];  // [KB][256], after the views
+    const int tid = threadIdx.x;
+    const int tx = (tid & (kTile - 1)) - kTile / 2, ty = tid / kTile - kTile / 2;  // relative to the centre pixel
+    const int tiles = a.tps * a.tps;
+    const int segs = a.segs;
+    const int total = a.ngroups * a.F * tiles * segs;
+    const int N = a.N;
+    const float h = 0.5f * (float)(N - 1);
+    const int one = 1 << kFanFrac;
+    if (a.skip && *a.skip) return;
+    for (int item = blockIdx.x; item < total; item += gridDim.x) {  // whole clusters
+        const int seg = item % segs;
+        int t2 = item / segs;
+        const int tile = t2 % tiles;
+        t2 /= tiles;
+        const int f = t2 % a.F;
+        const int grp = t2 / a.F;
+        const int ic = (tile / a.tps) * kTile + kTile / 2, jc = (tile % a.tps) * kTile + kTile / 2;
+        const int k0 = a.kbase + grp * KB;
+        const float x = (float)(jc + tx) - h, y = h - (float)(ic + ty);
+        const float *yg = a.YI + (size_t)(k0 >> 3) * a.yi_stride + (k0 & 7);
+        const int vs = a.fstart[f], vc = a.fcount[f];
+        const int nv = vc > seg ? (vc - seg + segs - 1) / segs : 0;
+        FanSums<KB> acc;
+        acc.clear();
+        for (int cb = 0; cb < nv; cb += kFanCap) {
+            const int nc = min(kFanCap, nv - cb);
+            __syncthreads();
+            if (tid == 0) s_max = 0;
+            __syncthreads();
+            for (int q = tid; q < nc; q += 256) {
+                const int v = vs + seg + (cb + q) * segs;
+                const FanView fv = a.views[v];
+                FanTileView w;
+                w.c = fv.c;
+                w.sn = fv.sn;
+                w.sb0 = fv.sb0;
+                w.iD = fv.iD;
+                w.mode0 = fv.mode0;
+                w.split = fv.split;
+                w.v = v;
+                // (not beyond the image's own one-pixel neighbourhood, where the projection is regular)
+                const float xl = (float)(jc - kTile / 2 - 1) - h, xr = (float)min(jc + kTile / 2, N) - h;
+                const float yt = h - (float)(ic - kTile / 2 - 1), yb = h - (float)min(ic + kTile / 2, N);
+                const float s1 = fan_s(xl, yt, fv.c, fv.sn, fv.iD), s2 = fan_s(xr, yt, fv.c, fv.sn, fv.iD);
+                const float s3 = fan_s(xl, yb, fv.c, fv.sn, fv.iD), s4 = fan_s(xr, yb, fv.c, fv.sn, fv.iD);
+                const int lo = max(0, (int)floorf(fminf(fminf(s1, s2), fminf(s3, s4)) - fv.sb0 - 0.1f));
+                const int hi = min(a.B - 1, (int)ceilf(fmaxf(fmaxf(s1, s2), fmaxf(s3, s4)) - fv.sb0 + 0.1f));
+                w.start = lo;
+                w.count = max(0, hi - lo + 1);
+                s_view[q] = w;
+                if (w.count > 0) atomicMax(&s_max, (w.count + kFanWin - 1) / kFanWin);
+            }
+            __syncthreads();
+            const int nwin = s_max;  // windows of kFanWin rays (one unless the tile is close to the source)
+            const int nblk = (nc + kFanVB - 1) / kFanVB;
+            // one staged ray per thread and block
+            const int sq = tid / kFanWin, sr = tid % kFanWin;
+            FanLine<float> line;
+            bool have = false;
+            auto fetch = [&](int u, int buf) {  // block u: window u / nblk of views (u % nblk) * kFanVB ...
+                const int q = (u % nblk) * kFanVB + sq, off = (u / nblk) * kFanWin + sr;
+                have = q < nc && off < s_view[min(q, nc - 1)].count;
+                if (!have) return;
+                const FanTileView &w = s_view[q];
+                const size_t bin = (size_t)w.v * a.B + w.start + off;
+                line = a.lines[bin];
+                const float *src = yg + bin * 8;
+                const unsigned dst = (unsigned)__cvta_generic_to_shared(&s_y[buf][sq][0][sr][0]);
+                if constexpr (KB >= 4) {
+#pragma unroll
+                    for (int g = 0; g < KB / 4; ++g)
+                        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(dst + 16 * kFanWin * g),
+                                     "l"(src + 4 * g)
+                                     : "memory");
+                } else {
+                    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;\n" ::"r"(dst), "l"(src), "n"(4 * KB)
+                                 : "memory");
+                }
+            };
+            auto store = [&](int u, int buf) {
+                if (!have) return;
+                const FanTileView &w = s_view[(u % nblk) * kFanVB + sq];
+                const int bin = w.start + (u / nblk) * kFanWin + sr;
+                const int mode = bin < w.split ? w.mode0 : 1 - w.mode0;
+                const int r = mode ? jc : ic, m = mode ? ic : jc;
+                const long long Q = line.Qc + (long long)(2 * r - (N - 1)) * line.Qh - ((long long)m << kFracBits);
+                // rays that pass the tile at a distance are held at 20 pixels, out of reach of its pixels
+                const long long far = 20LL << kFanFrac;
+                FanTileRay R;
+                R.P = (int)min(max((Q + (1LL << (kFracBits - kFanFrac - 1))) >> (kFracBits - kFanFrac), -far), far);
+                R.S = (int)((2 * line.Qh + (1LL << (kFracBits - kFanFrac - 1))) >> (kFracBits - kFanFrac));
+                R.w = line.w;
+                R.pad = 0;
+                s_ray[buf][sq][sr] = R;
+            };
+            const int nu = nblk * nwin;
+            if (nu > 0) fetch(0, 0);
+            cp_async_commit();
+            for (int u = 0; u < nu; ++u) {
+                const int buf = u & 1;
+                store(u, buf);
+                cp_async_wait0();
+                // block u is staged, and every thread has finished block u - 1
+                __syncthreads();
+                if (u + 1 < nu) fetch(u + 1, buf ^ 1);
+                cp_async_commit();
+                const int q0 = (u % nblk) * kFanVB, w0 = (u / nblk) * kFanWin;
+                for (int qq = 0; qq < kFanVB && q0 + qq < nc; ++qq) {
+                    const FanTileView &w = s_view[q0 + qq];
+                    const int wlo = w.start + w0, whi = min(w.start + w.count, wlo + kFanWin);  // rays staged
+                    if (wlo >= whi) continue;
+                    const float num = fmaf(x, w.c, y * w.sn), den = fmaf(fmaf(y, w.c, -x * w.sn), w.iD, 1.0f);
+                    const float cD = w.c * w.iD, sD = w.sn * w.iD;
+                    // rays marched along rows that sample row i inside (x - 1, x + 1), then rays
+                    // marched along columns that sample column j inside (y - 1, y + 1)
+#pragma unroll
+                    for (int pass = 0; pass < 2; ++pass) {
+                        const int mlo = max(wlo, w.mode0 == pass ? 0 : w.split);
+                        const int mhi = min(whi, w.mode0 == pass ? w.split : a.B);
+                        if (mlo >= mhi) continue;  // uniform
+                        const float dn = pass == 0 ? w.c : w.sn, dd = pass == 0 ? -sD : cD;
+                        const float s1 = __fdividef(num - dn, den - dd), s2 = __fdividef(num + dn, den + dd);
+                        // margin 0.05 bins: the FP32 detector coordinates are off by < 0.01 bins for N <= 4096
+                        const int blo = max(mlo, (int)ceilf(fminf(s1, s2) - w.sb0 - 0.05f));
+                        const int bhi = min(mhi - 1, (int)floorf(fmaxf(s1, s2) - w.sb0 + 0.05f));
+                        const int along = pass == 0 ? ty : tx, across = (pass == 0 ? tx : ty) * one;
+                        for (int b = blo; b <= bhi; ++b) {
+                            const FanTileRay R = s_ray[buf][qq][b - wlo];
+                            const int d = abs(R.P + along * R.S - across);
+                            if (d < one) {
+                                const float g = __int_as_float((d >> (kFanFrac - 23)) | 0x3F800000);  // 1 + distance
+                                acc.add(R.w * (2.0f - g), &s_y[buf][qq][0][b - wlo][0]);
+                            }
+                        }
+                    }
+                }
+            }
+            cp_async_wait0();  // the last group is empty
+        }
+        __syncthreads();  // every thread is done with the staged bins
+#pragma unroll
+        for (int k = 0; k < KB; ++k) red[k * 256 + tid] = acc.get(k);
+        cg::cluster_group cl = cg::this_cluster();
+        if (segs > 1) cl.sync();
+        else __syncthreads();
+        // this CTA's share of the pixels, the segments added in order
+        constexpr int OUT = KB * 256;
+#pragma unroll 1
+        for (int u = OUT / 32 * seg / segs * 32 + tid; u < OUT / 32 * (seg + 1) / segs * 32; u += 256) {
+            float s;
+            if (segs == 1) {
+                s = red[u];
+            } else {
+                float part[kMaxSegs];
+#pragma unroll
+                for (int q = 0; q < kMaxSegs; ++q) part[q] = q < segs ? *cl.map_shared_rank(red + u, q) : 0.0f;
+                s = part[0];
+#pragma unroll
+                for (int q = 1; q < kMaxSegs; ++q)
+                    if (q < segs) s += part[q];
+            }
+            const int k = u >> 8, p = u & 255;
+            const int i = ic - kTile / 2 + p / kTile, j = jc - kTile / 2 + p % kTile;
+            if (i < N && j < N) a.X[(size_t)(k0 + k) * a.img_stride + (size_t)f * N * N + (size_t)i * N + j] = s;
+        }
+        if (segs > 1) cl.sync();
+        else __syncthreads();
+    }
+}
+
 struct AdjFanArgs {
     const int *fstart, *fcount;
     int N, B, F, tps, Pb, kbase, ngroups;
@@ -421,7 +645,7 @@ template <typename T, int KB> __device__ __forceinline__ void load_bin(const T *
     }
 }
 
-// One CTA = one 16 x 16 pixel tile of one frame and KB sinograms, SPLIT
+// FP64: one CTA = one 16 x 16 pixel tile of one frame and KB sinograms, SPLIT
 // thread groups of 256: group g of a pixel sums the views vs + g, vs + g +
 // SPLIT, ... of its frame in order; the groups' sums are added in group
 // order in shared memory.
@@ -555,21 +779,13 @@ size_t fan_view_bytes() { return sizeof(FanView); }
 cudaError_t launch_fan_rays(const Handle &h, const int *skip)
 {
     const long long n = (long long)h.V * h.B;
-    const int grid = (int)std::max<long long>(1, std::min<long long>((n + 255) / 256, 4LL * h.num_sms));
-    const int vgrid = (h.V + 7) / 8;
-    if (h.precision) {
-        k_fan_rays<double><<<grid, 256, 0, h.stream>>>(h.d_views, h.V, h.B, h.N, h.fan_D,
-                                                       (FanRay<double> *)h.d_rays, fan_lines<double>(h.d_rays, n),
-                                                       skip);
-        k_fan_views<double><<<vgrid, 256, 0, h.stream>>>(h.d_views, h.V, h.B, h.fan_D,
-                                                         (const FanRay<double> *)h.d_rays, (FanView *)h.d_fanview,
-                                                         skip);
-    } else {
-        k_fan_rays<float><<<grid, 256, 0, h.stream>>>(h.d_views, h.V, h.B, h.N, h.fan_D, (FanRay<float> *)h.d_rays,
-                                                      fan_lines<float>(h.d_rays, n), skip);
-        k_fan_views<float><<<vgrid, 256, 0, h.stream>>>(h.d_views, h.V, h.B, h.fan_D, (const FanRay<float> *)h.d_rays,
-                                                        (FanView *)h.d_fanview, skip);
-    }
+    const int grid = std::min(h.V, 16 * h.num_sms);
+    if (h.precision)
+        k_fan_table<double><<<grid, 128, 0, h.stream>>>(h.d_views, h.V, h.B, h.N, h.fan_D, (FanRay<double> *)h.d_rays,
+                                                        fan_lines<double>(h.d_rays, n), (FanView *)h.d_fanview, skip);
+    else
+        k_fan_table<float><<<grid, 128, 0, h.stream>>>(h.d_views, h.V, h.B, h.N, h.fan_D, (FanRay<float> *)h.d_rays,
+                                                       fan_lines<float>(h.d_rays, n), (FanView *)h.d_fanview, skip);
     return cudaGetLastError();
 }
 
@@ -594,18 +810,20 @@ cudaError_t run_fan_ray(const Handle &h, const RayArgs<T> &a, int mode, int kb, 
 
 // kb: sinograms per thread (the candidate search of a pixel and view is
 // shared by them); split: thread groups per pixel (view subsets).
-template <typename T>
-cudaError_t launch_fan_adjoint(const Handle &h, T *X, int batch, int kb, int split, const int *skip)
+cudaError_t fan_adjoint32(const Handle &h, float *X, int batch, int kb, int split, const int *skip)
 {
-    AdjFanArgs a{};
+    FanTileArgs a{};
+    a.lines = fan_lines<float>(h.d_rays, (long long)h.V * h.B);
+    a.views = (const FanView *)h.d_fanview;
     a.fstart = h.d_fstart;
     a.fcount = h.d_fcount;
     a.N = h.N;
     a.B = h.B;
     a.F = h.F;
     a.tps = (h.N + kTile - 1) / kTile;
-    a.Pb = h.Pb;
-    a.ysino_stride = (long long)h.V * h.B;  // per block of 8 interleaved sinograms, in bins
+    a.YI = (const float *)h.d_yi;
+    a.yi_stride = 8LL * h.V * h.B;
+    a.X = X;
     a.img_stride = (long long)h.F * h.N * h.N;
     a.skip = skip;
     int k = 0;
@@ -615,17 +833,56 @@ cudaError_t launch_fan_adjoint(const Handle &h, T *X, int batch, int kb, int spl
         if (groups == 0) continue;
         a.kbase = k;
         a.ngroups = groups;
+        a.segs = adj_segs(h, (long long)groups * h.F * a.tps * a.tps, split, 8);
         cudaError_t e;
         switch (width) {
-        case 1: e = run_adj_fan_split<T, 1>(h, a, X, split); break;
-        case 2: e = run_adj_fan_split<T, 2>(h, a, X, split); break;
-        case 4: e = run_adj_fan_split<T, 4>(h, a, X, split); break;
-        default: e = run_adj_fan_split<T, 8>(h, a, X, split); break;
+        case 1: e = launch_cluster(k_adj_fan_tile<1>, a, h, 0); break;
+        case 2: e = launch_cluster(k_adj_fan_tile<2>, a, h, 0); break;
+        case 4: e = launch_cluster(k_adj_fan_tile<4>, a, h, 0); break;
+        default: e = launch_cluster(k_adj_fan_tile<8>, a, h, 0); break;
         }
         if (e != cudaSuccess) return e;
         k += groups * width;
     }
     return cudaSuccess;
+}
+
+template <typename T>
+cudaError_t launch_fan_adjoint(const Handle &h, T *X, int batch, int kb, int split, const int *skip)
+{
+    if constexpr (std::is_same<T, float>::value) {
+        return fan_adjoint32(h, X, batch, kb, split, skip);
+    } else {
+        AdjFanArgs a{};
+        a.fstart = h.d_fstart;
+        a.fcount = h.d_fcount;
+        a.N = h.N;
+        a.B = h.B;
+        a.F = h.F;
+        a.tps = (h.N + kTile - 1) / kTile;
+        a.Pb = h.Pb;
+        a.ysino_stride = (long long)h.V * h.B;  // per block of 8 interleaved sinograms, in bins
+        a.img_stride = (long long)h.F * h.N * h.N;
+        a.skip = skip;
+        int k = 0;
+        for (int width : {8, 4, 2, 1}) {
+            if (width > kb) continue;
+            const int groups = (batch - k) / width;
+            if (groups == 0) continue;
+            a.kbase = k;
+            a.ngroups = groups;
+            cudaError_t e;
+            switch (width) {
+            case 1: e = run_adj_fan_split<double, 1>(h, a, X, split); break;
+            case 2: e = run_adj_fan_split<double, 2>(h, a, X, split); break;
+            case 4: e = run_adj_fan_split<double, 4>(h, a, X, split); break;
+            default: e = run_adj_fan_split<double, 8>(h, a, X, split); break;
+            }
+            if (e != cudaSuccess) return e;
+            k += groups * width;
+        }
+        return cudaSuccess;
+    }
 }
 
 template <typename T> cudaError_t launch_fan_sino(const Handle &h, const T *Y, int nsino, const int *skip)

@@ -467,40 +467,6 @@ __device__ __forceinline__ void taps_interleaved(const float *__restrict__ q, lo
     }
 }
 
-// Element indices (cell + 2, clamped to the row's zero padding) and fractions
-// of U consecutive rows from the exact line value Q at the first.  FP32: the
-// rows are walked relative to the first one's cell with 55 fractional bits (the
-// 48 of the line, shifted), so the high word holds the cell offset in its top
-// 9 bits and the 23 bits of the fraction below them: one shift, one logic
-// operation and one add-and-clamp a row, where the full-range line needs a
-// two-word shift, two clamps and a second shift (the integer pipe was the bound
-// of one image per lane: 74 % busy, now 58).  The same bits as cell_of and
-// frac_of.  One image of 2048^2, 120 views: 362 -> 282 us; 256^2 / 180 views:
-// 18.6 -> 16.3.
-template <typename T, int U>
-__device__ __forceinline__ void ray_cells(long long Q, long long dQ, unsigned lim, unsigned (&idx)[U], T (&f)[U])
-{
-    if constexpr (std::is_same<T, float>::value) {
-        static_assert(kFracBits == 48 && U <= 16, "cell offsets of a block fit 9 bits");
-        const unsigned base = (unsigned)(cell_of(Q) + 2);
-        const long long L0 = (long long)(((unsigned long long)Q << 16) >> 9), dL = dQ << 7;
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const int hi = (int)((L0 + (long long)u * dL) >> 32);
-            // (a negative index is a large unsigned one)
-            idx[u] = __viaddmin_u32((unsigned)(hi >> 23), base, lim);
-            f[u] = __int_as_float((hi & 0x7FFFFF) | 0x3F800000) - 1.0f;
-        }
-    } else {
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const long long Qu = Q + (long long)u * dQ;
-            idx[u] = min((unsigned)(cell_of(Qu) + 2), lim);
-            f[u] = frac_of(Qu, T());
-        }
-    }
-}
-
 // QL (FP32): the images come from the interleaved layout; the taps, the
 // fractions and the order of the sums are those of the pair form, so both
 // give the same bits.
