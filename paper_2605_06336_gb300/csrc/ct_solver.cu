@@ -167,7 +167,7 @@ template <typename T> struct Solver {
         SV_TRY(alloc(dots, kKMax + 2));
         SV_TRY(alloc(part_gram, (size_t)gram_blocks * kGramPairs));
         SV_TRY(alloc(part_dot, (size_t)kRedBlocks * (kKMax + 2)));
-        SV_TRY(alloc(part_n, (size_t)kRedBlocks * 3));
+        SV_TRY(alloc(part_n, (size_t)kRedBlocks * 4));
         SV_TRY(alloc(norms, 3));
         SV_TRY(alloc(norms2, 3));
         SV_TRY(alloc(scal, kScalCount));
@@ -258,11 +258,15 @@ template <typename T> struct Solver {
                 k_gram_psi_pipe8<1, kP8Threads><<<gram_blocks, kP8Threads, gram_p8_smem(k, epp, 1), h.stream>>>(
                     V, n, k, w, h.N, h.F, o.temporal, part_gram, stop);
         } else {
+            // at least 128 pairs (one chain in flight on each FP64 pipe) per CTA, and CTAs
+            // for every SM where the tiles leave some idle
+            const int shares = std::max(1, std::min((k * (k + 1) / 2 + 127) / 128, 4 * h.num_sms / gram_blocks));
+            const dim3 grid(gram_blocks, shares);
             if (k <= kKSmem)
-                k_gram_psi<T, 4, gram_slots(kKSmem)><<<gram_blocks, kThreads, gram_smem(k, tm, 4), h.stream>>>(
+                k_gram_psi<T, 4, gram_slots(kKSmem)><<<grid, kThreads, gram_smem(k, tm, 4), h.stream>>>(
                     V, n, k, w, h.N, h.F, o.temporal, part_gram, stop);
             else
-                k_gram_psi<T, 1, gram_slots(kKLimit)><<<gram_blocks, kThreads, gram_smem(k, tm, 1), h.stream>>>(
+                k_gram_psi<T, 1, gram_slots(kKLimit)><<<grid, kThreads, gram_smem(k, tm, 1), h.stream>>>(
                     V, n, k, w, h.N, h.F, o.temporal, part_gram, stop);
         }
         k_gram_reduce<<<gram_reduce_blocks(k), 32 * kGramReduceWarps, 0, h.stream>>>(part_gram, gram_blocks, k, GP,
@@ -278,12 +282,27 @@ template <typename T> struct Solver {
     int dots_into(const T *A, long long len, int k, const T *x, const T *x2, double *out, const int *stop)
     {
         const int nblk = red_blocks(len);
-        k_dots<T><<<nblk, kThreads, 0, h.stream>>>(A, len, len, k, x, x2, part_dot, stop);
         const int kk = k + (x2 ? 1 : 0);
+        dots_partials(A, len, k, x, x2, stop);
         k_dots_reduce<<<(kk + kDotsReduceWarps - 1) / kDotsReduceWarps, 32 * kDotsReduceWarps, 0, h.stream>>>(
             part_dot, nblk, kk, out, stop);
         SV_CUDA(cudaGetLastError());
         return CT_OK;
+    }
+
+    void dots_partials(const T *A, long long len, int k, const T *x, const T *x2, const int *stop)
+    {
+        const int kk = k + (x2 ? 1 : 0);
+        const dim3 grid(red_blocks(len), (kk + kDotCols - 1) / kDotCols);
+        k_dots<T><<<grid, kThreads, 0, h.stream>>>(A, len, len, k, x, x2, part_dot, stop);
+    }
+
+    // row kc of (HV)^T HV and entry kc of (HV)^T b; with ctl_end, the end of an Enlarge step
+    void gh_row(int kc, const int *stop, int *ctl_end)
+    {
+        dots_partials(HV, m, kc + 1, col(HV, m, kc), b, stop);
+        k_gh_append<<<1, kGhThreads, 0, h.stream>>>(part_dot, red_blocks(m), kc, GH, cvec, ctl_end,
+                                                    ctl_end ? d_stop : nullptr);
     }
 
     // norms3 of (a, b): {|a|^2, |a-b|^2, |b|^2}
@@ -411,37 +430,42 @@ template <typename T> struct Solver {
     }
 
     // ---- one predicated Enlarge step with kc basis columns ------------------
+    // (w holds the MM weights of u_old: begin_enlarge's before the first step, the
+    // previous step's after that)
     int enlarge_step(const double *theta, int kc)
     {
         const int *stop = ctl + kStop;
-        // P^2 from the previous iterate
-        k_weights<T><<<grid_for(ne), kThreads, 0, h.stream>>>(uold, w, h.N, h.F, o.temporal, o.eps, stop);
         // G_P = (P Psi V)^T (P Psi V)
         SV_TRY(gram_psi(kc, stop));
         // lambda and the reduced solution
         const double target = (o.tau * noise) * (o.tau * noise);
         small_solve(kc, target, o.lam_fix, o.lam_lo, o.lam_hi, o.lam_iters, y, scal, ctl);
         // u = V y ; res = (HV) y - b
-        k_gemv<T><<<grid_for(n), kThreads, 0, h.stream>>>(V, n, n, kc, y, u, T(0), T(1), nullptr, T(0), stop);
-        k_gemv<T><<<grid_for(m), kThreads, 0, h.stream>>>(HV, m, m, kc, y, res, T(0), T(1), b, T(-1), stop);
+        k_gemv_pair<T><<<grid_for(n) + grid_for(m), kThreads, 0, h.stream>>>(V, n, HV, m, kc, y, u, res, b,
+                                                                             grid_for(n), stop);
         SV_CUDA(cudaGetLastError());
         // r = H^T res + lambda Psi^T P^2 Psi u, written straight into the next basis column
         T *r = col(V, n, kc);
         SV_TRY(backproject(theta, res, r, stop));
         k_add_reg<T><<<grid_for(n), kThreads, 0, h.stream>>>(r, u, w, scal, h.N, h.F, o.temporal, stop);
         SV_TRY(cgs2(r, kc, stop));
-        SV_TRY(norms3(r, nullptr, n, norms2, stop));        // |r|^2
-        SV_TRY(norms3(u, uold, n, norms, stop));            // |u|^2, |u - u_old|^2, |u_old|^2
-        k_step_decide<<<1, 1, 0, h.stream>>>(norms2, norms, o.tol1, ctl, scal);
+        // |r|^2; |u|^2, |u - u_old|^2, |u_old|^2; u_old = u; the next step's weights
+        const int nblk = red_blocks(n);
+        k_step_norms<T><<<dim3(nblk, 3), kThreads, 0, h.stream>>>(r, u, uold, n, w, h.N, h.F, o.temporal, o.eps,
+                                                                  part_n, stop);
+        k_step_decide<<<1, 128, 0, h.stream>>>(part_n, nblk, o.tol1, norms2, ctl, scal);
         k_normalize<T><<<grid_for(n), kThreads, 0, h.stream>>>(r, n, norms2, stop);
         // H v_new and the new row of (HV)^T HV, (HV)^T b
         SV_TRY(project(theta, kc, 1, stop));
-        SV_TRY(dots_into(HV, m, kc + 1, col(HV, m, kc), b, dots, stop));
-        k_gh_append<<<1, kKMax + 2, 0, h.stream>>>(dots, kc, GH, cvec, stop);
-        SV_CUDA(cudaMemcpyAsync(uold, u, sizeof(T) * n, cudaMemcpyDeviceToDevice, h.stream));  // (u_old = u)
-        k_step_commit<<<1, 1, 0, h.stream>>>(ctl, d_stop);
+        gh_row(kc, stop, ctl);
         SV_CUDA(cudaGetLastError());
         return CT_OK;
+    }
+
+    // The weights the first step of an Enlarge reads
+    void begin_enlarge()
+    {
+        k_weights<T><<<grid_for(ne), kThreads, 0, h.stream>>>(uold, w, h.N, h.F, o.temporal, o.eps, nullptr);
     }
 
     // One Enlarge step: replay the captured graph for this basis size (capture
@@ -476,8 +500,7 @@ template <typename T> struct Solver {
     {
         // (HV)^T HV and (HV)^T b from scratch
         for (int j = 0; j < kc; ++j) {
-            SV_TRY(dots_into(HV, m, j + 1, col(HV, m, j), b, dots, nullptr));
-            k_gh_append<<<1, kKMax + 2, 0, h.stream>>>(dots, j, GH, cvec, nullptr);
+            gh_row(j, nullptr, nullptr);
         }
         SV_CUDA(cudaGetLastError());
         return CT_OK;
@@ -759,6 +782,7 @@ template <typename T> struct Solver {
         SV_CUDA(cudaStreamSynchronize(h.stream));
         *(volatile int *)h_stop = 0;
         const int s_steps = o.k_max - o.k_min;
+        begin_enlarge();
         for (int step = 0; step < s_steps && kc + step + 1 < KC; ++step) {
             if (step >= 2) {
                 SV_CUDA(cudaEventSynchronize(ev[step & 1]));
@@ -922,6 +946,7 @@ template <typename T> struct Solver {
             SV_CUDA(cudaStreamSynchronize(h.stream));
             *(volatile int *)h_stop = 0;
             // Enlarge: predicated steps issued one step ahead of the device's stop decision
+            begin_enlarge();
             for (int step = 0; step < s && kc + step + 1 < KC; ++step) {
                 if (step >= 2) {
                     SV_CUDA(cudaEventSynchronize(ev[step & 1]));

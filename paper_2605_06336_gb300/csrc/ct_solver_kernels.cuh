@@ -72,14 +72,13 @@ inline long long psi_edges(int N, int F, int temporal)
 }
 
 template <typename T>
-__global__ void k_weights(const T *__restrict__ u, T *__restrict__ w, int N, int F, int temporal, double eps,
-                          const int *stop)
+__device__ __forceinline__ void weights_range(const T *__restrict__ u, T *__restrict__ w, int N, int F, int temporal,
+                                              double eps, long long e0, long long stride)
 {
-    if (stopped(stop)) return;
     const long long nx = (long long)F * N * (N - 1);
     const long long ne = 2 * nx + (temporal && F > 1 ? (long long)(F - 1) * N * N : 0);
     const T e2 = (T)(eps * eps);
-    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < ne; e += (long long)gridDim.x * blockDim.x) {
+    for (long long e = e0; e < ne; e += stride) {
         T z;
         if (e < nx) {
             const long long f = e / ((long long)N * (N - 1));
@@ -100,6 +99,15 @@ __global__ void k_weights(const T *__restrict__ u, T *__restrict__ w, int N, int
         }
         w[e] = rsqrt_t<T>(z * z + e2);
     }
+}
+
+template <typename T>
+__global__ void k_weights(const T *__restrict__ u, T *__restrict__ w, int N, int F, int temporal, double eps,
+                          const int *stop)
+{
+    if (stopped(stop)) return;
+    weights_range(u, w, N, F, temporal, eps, blockIdx.x * (long long)blockDim.x + threadIdx.x,
+                  (long long)gridDim.x * blockDim.x);
 }
 
 // r += lambda Psi^T P^2 Psi u  (lambda = scal[kLam])
@@ -142,7 +150,11 @@ __global__ void k_add_reg(T *__restrict__ r, const T *__restrict__ u, const T *_
 // neighbour of every pixel) of all k columns are formed in shared memory,
 // each thread sums its (a, b) entries over the tile's edges in T and adds the
 // tile sum to an FP64 register accumulator.  Per-CTA FP64 partials;
-// k_gram_reduce sums them in order.
+// k_gram_reduce sums them in order.  blockIdx.y takes a share of the (a, b)
+// pairs: a pair's sum over a tile is one chain of FP64 multiply-adds, and a
+// small image has too few tiles to fill the chip with them (64^2, 25 columns:
+// 32 tiles; 29.7 -> 22 us, with the square roots of the weights taken once
+// per edge instead of once per edge and column).
 // ---------------------------------------------------------------------------
 constexpr int kGramPairs = kKMax * (kKMax + 1) / 2;
 // register slots per thread of k_gram_psi: (pairs of a basis of kc columns) / 256
@@ -163,6 +175,9 @@ __global__ void __launch_bounds__(256) k_gram_psi(const T *__restrict__ V, long 
     const int ntiles = tiles_x * tiles_y * F;
     const long long nx = (long long)F * N * (N - 1);
     const int np = k * (k + 1) / 2;
+    const int share = (np + gridDim.y - 1) / gridDim.y;
+    const int p0 = blockIdx.y * share, p1 = min(np, p0 + share);
+    __shared__ T sw[3][TP];  // square roots of the tile's weights
     double acc[kGramSlots];
 #pragma unroll
     for (int q = 0; q < kGramSlots; ++q) acc[q] = 0.0;
@@ -174,6 +189,18 @@ __global__ void __launch_bounds__(256) k_gram_psi(const T *__restrict__ V, long 
         const T *wy = w + nx + (long long)f * (N - 1) * N;
         const T *wt = w + 2 * nx + (long long)f * N * N;  // temporal edges of frames (f, f + 1)
         __syncthreads();
+        for (int idx = threadIdx.x; idx < EPP * TP; idx += blockDim.x) {
+            const int e = idx / TP, pix = idx % TP;
+            const int i = i0 + pix / 32, j = j0 + pix % 32;
+            T v = T(0);
+            if (i < N && j < N) {
+                if (e == 0 && j < N - 1) v = sqrt(wx[i * (N - 1) + j]);
+                if (e == 1 && i < N - 1) v = sqrt(wy[i * N + j]);
+                if (e == 2 && f < F - 1) v = sqrt(wt[(size_t)i * N + j]);
+            }
+            sw[e][pix] = v;
+        }
+        __syncthreads();
         for (int idx = threadIdx.x; idx < k * TP; idx += blockDim.x) {
             const int a = idx / TP, pix = idx % TP;
             const int i = i0 + pix / 32, j = j0 + pix % 32;
@@ -181,10 +208,9 @@ __global__ void __launch_bounds__(256) k_gram_psi(const T *__restrict__ V, long 
             if (i < N && j < N) {
                 const T *va = V + (long long)a * n + (long long)f * N * N;
                 const T c = va[(size_t)i * N + j];
-                if (j < N - 1) ex = (va[(size_t)i * N + j + 1] - c) * sqrt(wx[i * (N - 1) + j]);
-                if (i < N - 1) ey = (va[(size_t)(i + 1) * N + j] - c) * sqrt(wy[i * N + j]);
-                if (EPP == 3 && f < F - 1)
-                    et = (va[(size_t)N * N + (size_t)i * N + j] - c) * sqrt(wt[(size_t)i * N + j]);
+                if (j < N - 1) ex = (va[(size_t)i * N + j + 1] - c) * sw[0][pix];
+                if (i < N - 1) ey = (va[(size_t)(i + 1) * N + j] - c) * sw[1][pix];
+                if (EPP == 3 && f < F - 1) et = (va[(size_t)N * N + (size_t)i * N + j] - c) * sw[2][pix];
             }
             E[a * EP + EPP * pix] = ex;
             E[a * EP + EPP * pix + 1] = ey;
@@ -193,8 +219,8 @@ __global__ void __launch_bounds__(256) k_gram_psi(const T *__restrict__ V, long 
         __syncthreads();
 #pragma unroll
         for (int q = 0; q < kGramSlots; ++q) {
-            const int p = threadIdx.x + 256 * q;
-            if (p >= np) break;
+            const int p = p0 + threadIdx.x + 256 * q;
+            if (p >= p1) break;
             // p -> (a, b) with a <= b, row-major over the upper triangle
             int a = 0, rem = p;
             while (rem >= k - a) {
@@ -211,8 +237,8 @@ __global__ void __launch_bounds__(256) k_gram_psi(const T *__restrict__ V, long 
     }
 #pragma unroll
     for (int q = 0; q < kGramSlots; ++q) {
-        const int p = threadIdx.x + 256 * q;
-        if (p < np) part[(long long)blockIdx.x * kGramPairs + p] = acc[q];
+        const int p = p0 + threadIdx.x + 256 * q;
+        if (p < p1) part[(long long)blockIdx.x * kGramPairs + p] = acc[q];
     }
 }
 
@@ -662,84 +688,86 @@ __global__ void __launch_bounds__(32 * kGramReduceWarps) k_gram_reduce(const dou
 // with column stride lda); x2 (nullable) adds out[k] = x . x2 .
 // kRedBlocks CTAs each own a contiguous slice; partials reduced in order.
 // ---------------------------------------------------------------------------
-// Columns are taken 16 at a time.  Every thread sums its elements of the 16
-// products: in FP64 for T = double; for T = float in FP32 over runs of 16
-// elements, each run then added in FP64 (the products are FP32 to begin with,
-// and the FP64 pipe of this part is narrow: at 2048^2 per-element FP64 adds
-// bound the kernel).  The 256 per-thread sums of a column are then added
-// through shared memory: 16 threads per column sum 16 values each (strided)
-// and combine them in a 16-lane tree, far fewer FP64 instructions than a
-// shuffle tree per warp.  Fixed order throughout.
+// blockIdx.y takes 8 columns, blockIdx.x a slice of the vectors (a column's
+// sums do not depend on the grid's second dimension).  Every thread sums its
+// elements of the 8 products: in FP64 for T = double; for T = float in FP32
+// over runs of 16 elements, each run then added in FP64 (the products are FP32
+// to begin with, and the FP64 pipe of this part is narrow: at 2048^2
+// per-element FP64 adds bound the kernel).  The 256 per-thread sums of a column
+// are then added through shared memory: 16 threads per column sum 16 values
+// each (strided) and combine them in a 16-lane tree, far fewer FP64
+// instructions than a shuffle tree per warp.  Fixed order throughout.  The
+// FP64 sums are most of the time on short vectors, so the columns go to
+// different CTAs (256^2, 25 columns: 15 us with all of them in one CTA,
+// 10.7 now).
+constexpr int kDotCols = 8;
 template <typename T>
 __global__ void __launch_bounds__(256) k_dots(const T *__restrict__ A, long long len, long long lda, int k,
                                               const T *__restrict__ x, const T *__restrict__ x2,
                                               double *__restrict__ part, const int *stop)
 {
     if (stopped(stop)) return;
-    constexpr int G = 16;
+    constexpr int G = kDotCols;
     __shared__ double sh[G][257];
     const long long per = (len + gridDim.x - 1) / gridDim.x;
     const long long lo = blockIdx.x * per, hi = min(len, lo + per);
     const int kk = k + (x2 ? 1 : 0);
-    for (int a0 = 0; a0 < kk; a0 += G) {
-        const int na = min(G, kk - a0);
-        const T *cols[G];
+    const int a0 = blockIdx.y * G;
+    const int na = min(G, kk - a0);
+    const T *cols[G];
 #pragma unroll
-        for (int q = 0; q < G; ++q) {
-            const int a = min(a0 + q, kk - 1);
-            cols[q] = (a < k) ? A + (long long)a * lda : x2;
-        }
-        double s[G];
-#pragma unroll
-        for (int q = 0; q < G; ++q) s[q] = 0.0;
-        if constexpr (std::is_same<T, float>::value) {
-            // FP32 fused multiply-adds over runs of 16 of the thread's
-            // elements, each run added to the FP64 sum
-            float fr[G];
-#pragma unroll
-            for (int q = 0; q < G; ++q) fr[q] = 0.0f;
-            int run = 0;
-            for (long long i = lo + threadIdx.x; i < hi; i += blockDim.x) {
-                const float xi = x[i];
-#pragma unroll
-                for (int q = 0; q < G; ++q)
-                    if (q < na) fr[q] = fmaf(cols[q][i], xi, fr[q]);
-                if (++run == 16) {
-#pragma unroll
-                    for (int q = 0; q < G; ++q) {
-                        s[q] += (double)fr[q];
-                        fr[q] = 0.0f;
-                    }
-                    run = 0;
-                }
-            }
-#pragma unroll
-            for (int q = 0; q < G; ++q) s[q] += (double)fr[q];
-        } else {
-            for (long long i = lo + threadIdx.x; i < hi; i += blockDim.x) {
-                const T xi = x[i];
-#pragma unroll
-                for (int q = 0; q < G; ++q)
-                    if (q < na) s[q] = fma(cols[q][i], xi, s[q]);
-            }
-        }
-#pragma unroll
-        for (int q = 0; q < G; ++q)
-            if (q < na) sh[q][threadIdx.x] = s[q];
-        __syncthreads();
-        {
-            const int q = threadIdx.x >> 4, seg = threadIdx.x & 15;
-            double t = 0.0;
-            if (q < na) {
-#pragma unroll
-                for (int e = 0; e < 16; ++e) t += sh[q][seg + 16 * e];  // conflict-free
-            }
-#pragma unroll
-            for (int o = 8; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-            if (seg == 0 && q < na) part[(long long)blockIdx.x * (kKMax + 2) + a0 + q] = t;
-        }
-        __syncthreads();
+    for (int q = 0; q < G; ++q) {
+        const int a = min(a0 + q, kk - 1);
+        cols[q] = (a < k) ? A + (long long)a * lda : x2;
     }
+    double s[G];
+#pragma unroll
+    for (int q = 0; q < G; ++q) s[q] = 0.0;
+    if constexpr (std::is_same<T, float>::value) {
+        // FP32 fused multiply-adds over runs of 16 of the thread's
+        // elements, each run added to the FP64 sum
+        float fr[G];
+#pragma unroll
+        for (int q = 0; q < G; ++q) fr[q] = 0.0f;
+        int run = 0;
+        for (long long i = lo + threadIdx.x; i < hi; i += blockDim.x) {
+            const float xi = x[i];
+#pragma unroll
+            for (int q = 0; q < G; ++q)
+                if (q < na) fr[q] = fmaf(cols[q][i], xi, fr[q]);
+            if (++run == 16) {
+#pragma unroll
+                for (int q = 0; q < G; ++q) {
+                    s[q] += (double)fr[q];
+                    fr[q] = 0.0f;
+                }
+                run = 0;
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < G; ++q) s[q] += (double)fr[q];
+    } else {
+        for (long long i = lo + threadIdx.x; i < hi; i += blockDim.x) {
+            const T xi = x[i];
+#pragma unroll
+            for (int q = 0; q < G; ++q)
+                if (q < na) s[q] = fma(cols[q][i], xi, s[q]);
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < G; ++q)
+        if (q < na) sh[q][threadIdx.x] = s[q];
+    __syncthreads();
+    const int q = threadIdx.x >> 4, seg = threadIdx.x & 15;
+    if (q >= G) return;  // whole warps
+    double t = 0.0;
+    if (q < na) {
+#pragma unroll
+        for (int e = 0; e < 16; ++e) t += sh[q][seg + 16 * e];  // conflict-free
+    }
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    if (seg == 0 && q < na) part[(long long)blockIdx.x * (kKMax + 2) + a0 + q] = t;
 }
 
 // out[a] = sum_c part[c][a] for a < kk: one warp per output, lanes over the
@@ -759,6 +787,22 @@ __global__ void __launch_bounds__(32 * kDotsReduceWarps) k_dots_reduce(const dou
     if (lane == 0) out[a] = s;
 }
 
+// sum_a A[a][i] * y[a], added in column order, 16 columns' loads in flight
+template <typename T>
+__device__ __forceinline__ T gemv_row(const T *__restrict__ A, long long lda, int k, const T *ys, long long i)
+{
+    T s = T(0);
+    for (int a0 = 0; a0 < k; a0 += 16) {
+        T v[16];
+#pragma unroll
+        for (int q = 0; q < 16; ++q) v[q] = a0 + q < k ? A[(long long)(a0 + q) * lda + i] : T(0);
+#pragma unroll
+        for (int q = 0; q < 16; ++q)
+            if (a0 + q < k) s = fma(v[q], ys[a0 + q], s);
+    }
+    return s;
+}
+
 // out[i] = beta*out[i] + sgn * sum_a A[a][i] * y[a]  (+ bias[i] * bsgn)
 template <typename T>
 __global__ void k_gemv(const T *__restrict__ A, long long len, long long lda, int k, const double *__restrict__ y,
@@ -769,12 +813,31 @@ __global__ void k_gemv(const T *__restrict__ A, long long len, long long lda, in
     for (int a = threadIdx.x; a < k; a += blockDim.x) ys[a] = (T)y[a];
     __syncthreads();
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < len; i += (long long)gridDim.x * blockDim.x) {
-        T s = T(0);
-        for (int a = 0; a < k; ++a) s = fma(A[(long long)a * lda + i], ys[a], s);
+        const T s = gemv_row(A, lda, k, ys, i);
         T o = beta == T(0) ? T(0) : beta * out[i];
         o = fma(sgn, s, o);
         if (bias) o = fma(bsgn, bias[i], o);
         out[i] = o;
+    }
+}
+
+// u = V y and res = (HV) y - b in one launch: the first g1 CTAs the image, the others the data
+template <typename T>
+__global__ void k_gemv_pair(const T *__restrict__ V, long long n, const T *__restrict__ HV, long long m, int k,
+                            const double *__restrict__ y, T *__restrict__ u, T *__restrict__ res,
+                            const T *__restrict__ b, int g1, const int *stop)
+{
+    if (stopped(stop)) return;
+    __shared__ T ys[kKMax];
+    for (int a = threadIdx.x; a < k; a += blockDim.x) ys[a] = (T)y[a];
+    __syncthreads();
+    if ((int)blockIdx.x < g1) {
+        for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)g1 * blockDim.x)
+            u[i] = fma(T(1), gemv_row(V, n, k, ys, i), T(0));
+    } else {
+        const int blk = blockIdx.x - g1, g2 = gridDim.x - g1;
+        for (long long i = blk * (long long)blockDim.x + threadIdx.x; i < m; i += (long long)g2 * blockDim.x)
+            res[i] = fma(T(-1), b[i], fma(T(1), gemv_row(HV, m, k, ys, i), T(0)));
     }
 }
 
@@ -842,54 +905,131 @@ __global__ void k_norms3_reduce(const double *__restrict__ part, int nblk, doubl
 }
 
 // ---------------------------------------------------------------------------
-// Enlarge step bookkeeping: normalise the new direction, decide whether the
-// step is the last one (tol_1 test or a vanished residual).
-//   scal[kRnorm2] = |r|^2, norms3 = {|u|^2, |u - u_old|^2, |u_old|^2}
+// Enlarge step bookkeeping
 // ---------------------------------------------------------------------------
+// The vector work at the end of a step in one launch, by blockIdx.y: 0 the
+// partials of |r|^2; 1 those of |u|^2, |u - u_old|^2, |u_old|^2, then u_old = u;
+// 2 the MM weights of u for the next step.
 template <typename T>
-__global__ void k_normalize(T *__restrict__ r, long long len, const double *__restrict__ rn2, const int *stop)
+__global__ void __launch_bounds__(256) k_step_norms(const T *__restrict__ r, const T *__restrict__ u, T *uold,
+                                                    long long n, T *__restrict__ w, int N, int F, int temporal,
+                                                    double eps, double *__restrict__ part, const int *stop)
 {
     if (stopped(stop)) return;
-    const double nr = sqrt(*rn2);
-    const T inv = nr > 0.0 ? (T)(1.0 / nr) : T(0);
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < len; i += (long long)gridDim.x * blockDim.x)
-        r[i] *= inv;
+    const long long i0 = blockIdx.x * (long long)blockDim.x + threadIdx.x, stride = (long long)gridDim.x * blockDim.x;
+    if (blockIdx.y == 2) {
+        weights_range(u, w, N, F, temporal, eps, i0, stride);
+        return;
+    }
+    __shared__ double sh[33];
+    if (blockIdx.y == 0) {
+        double s0 = 0.0;
+        for (long long i = i0; i < n; i += stride) {
+            const double x = (double)r[i];
+            s0 += x * x;
+        }
+        s0 = block_sum(s0, sh);
+        if (threadIdx.x == 0) part[3 * gridDim.x + blockIdx.x] = s0;
+        return;
+    }
+    double s0 = 0.0, s1 = 0.0, s2 = 0.0;
+    for (long long i = i0; i < n; i += stride) {
+        const T ui = u[i];
+        const double x = (double)ui;
+        const double y = (double)uold[i];
+        s0 += x * x;
+        s1 += (x - y) * (x - y);
+        s2 += y * y;
+        uold[i] = ui;
+    }
+    s0 = block_sum(s0, sh);
+    s1 = block_sum(s1, sh);
+    s2 = block_sum(s2, sh);
+    if (threadIdx.x == 0) {
+        part[blockIdx.x * 3 + 0] = s0;
+        part[blockIdx.x * 3 + 1] = s1;
+        part[blockIdx.x * 3 + 2] = s2;
+    }
 }
 
-__global__ void k_step_decide(const double *__restrict__ rn2, const double *__restrict__ norms3, double tol1,
-                              int *__restrict__ ctl, double *__restrict__ scal)
+// Sums of the partials (one warp each: lanes over the partials, a fixed tree),
+// then the decision whether the step is the last one (tol_1 test or a
+// vanished residual).  One CTA of 4 warps; rn2 receives |r|^2.
+__global__ void __launch_bounds__(128) k_step_decide(const double *__restrict__ part, int nblk, double tol1,
+                                                     double *__restrict__ rn2, int *__restrict__ ctl,
+                                                     double *__restrict__ scal)
 {
     if (ctl[kStop]) return;
-    const double uold2 = norms3[2];
-    const bool small = uold2 > 0.0 && sqrt(norms3[1]) <= tol1 * sqrt(uold2);
-    const bool vanished = !(*rn2 > 0.0);
+    __shared__ double sum[4];  // |u|^2, |u - u_old|^2, |u_old|^2, |r|^2
+    const int q = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    double s = 0.0;
+    for (int c = lane; c < nblk; c += 32) s += q < 3 ? part[c * 3 + q] : part[3 * nblk + c];
+    s = warp_sum(s);
+    if (lane == 0) sum[q] = s;
+    __syncthreads();
+    if (threadIdx.x != 0) return;
+    const double uold2 = sum[2];
+    const bool small = uold2 > 0.0 && sqrt(sum[1]) <= tol1 * sqrt(uold2);
+    const bool vanished = !(sum[3] > 0.0);
+    *rn2 = sum[3];
     ctl[kSteps] += 1;
-    scal[kDu2] = norms3[1];
+    scal[kDu2] = sum[1];
     scal[kU2] = uold2;
     ctl[kStopNext] = (small || vanished) ? 1 : 0;
     if (vanished) ctl[kBreakdown] = 1;
 }
 
-// Append row/column kc of (HV)^T HV and entry kc of (HV)^T b from
-// dots = {HV[:, j] . h_new for j <= kc, b . h_new}.
-__global__ void k_gh_append(const double *__restrict__ dots, int kc, double *__restrict__ GH,
-                            double *__restrict__ cvec, const int *stop)
+// (the FP64 square root and division once per CTA: done by every thread they
+// were half of the kernel's time)
+template <typename T>
+__global__ void k_normalize(T *__restrict__ r, long long len, const double *__restrict__ rn2, const int *stop)
 {
     if (stopped(stop)) return;
-    const int j = threadIdx.x;
-    if (j <= kc) {
-        GH[kc * kKMax + j] = dots[j];
-        GH[j * kKMax + kc] = dots[j];
+    __shared__ T s_inv;
+    if (threadIdx.x == 0) {
+        const double nr = sqrt(*rn2);
+        s_inv = nr > 0.0 ? (T)(1.0 / nr) : T(0);
     }
-    if (j == 0) cvec[kc] = dots[kc + 1];
+    __syncthreads();
+    const T inv = s_inv;
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < len; i += (long long)gridDim.x * blockDim.x)
+        r[i] *= inv;
 }
 
-// Ends a step: raises the stop flag when the step decided so, and mirrors
-// it to host-mapped memory (nullable) for the host's issue loop.
-__global__ void k_step_commit(int *__restrict__ ctl, volatile int *__restrict__ stop_mirror)
+// Append row/column kc of (HV)^T HV and entry kc of (HV)^T b from the partials
+// of {HV[:, j] . h_new for j <= kc, b . h_new} (one warp per sum, lanes over the
+// partials, a fixed tree).  With ctl, this also ends a step: the stop flag is
+// raised when the step decided so, and mirrored to host-mapped memory
+// (nullable) for the host's issue loop.  One CTA, so that no part of the launch
+// can see the flag it raises.
+constexpr int kGhThreads = 1024;
+__global__ void __launch_bounds__(kGhThreads) k_gh_append(const double *__restrict__ part, int nblk, int kc,
+                                                          double *__restrict__ GH, double *__restrict__ cvec,
+                                                          int *__restrict__ ctl, volatile int *__restrict__ stop_mirror)
 {
-    if (!ctl[kStop] && ctl[kStopNext]) ctl[kStop] = 1;
-    if (stop_mirror) *stop_mirror = ctl[kStop];
+    const bool stop = ctl && ctl[kStop];
+    const int lane = threadIdx.x & 31;
+    if (!stop) {
+        for (int j = threadIdx.x >> 5; j <= kc + 1; j += kGhThreads / 32) {
+            double s = 0.0;
+            for (int c = lane; c < nblk; c += 32) s += part[(long long)c * (kKMax + 2) + j];
+            s = warp_sum(s);
+            if (lane == 0) {
+                if (j <= kc) {
+                    GH[kc * kKMax + j] = s;
+                    GH[j * kKMax + kc] = s;
+                } else {
+                    cvec[kc] = s;
+                }
+            }
+        }
+    }
+    if (!ctl) return;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        if (!stop && ctl[kStopNext]) ctl[kStop] = 1;
+        if (stop_mirror) *stop_mirror = ctl[kStop];
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -1129,30 +1269,68 @@ __device__ void ldlt_fwd(double *L, double *inv, double *rhs, int k, int *bad)
     __syncthreads();
 }
 
-// v := L^{-1} v for the unit factor (warp 0, lanes over rows)
+// The substitutions keep a vector in the registers of warp 0 (row i in lane
+// i % 32, register i / 32) and broadcast each entry as it is final: a shuffle
+// where a vector in shared memory takes a store, a barrier and a load per entry.
+// v := L^{-1} v for the unit factor
 template <int kLd>
 __device__ void fwd_subst_warp(const double *L, double *v, int k)
 {
+    constexpr int NR = (kLd - 1) / 32;
     const int lane = threadIdx.x & 31;
-    for (int j = 0; j < k; ++j) {
-        const double zj = v[j];
-        for (int i = j + 1 + lane; i < k; i += 32) v[i] -= L[i * kLd + j] * zj;
-        __syncwarp();
+    double x[NR];
+#pragma unroll
+    for (int r = 0; r < NR; ++r) x[r] = lane + 32 * r < k ? v[lane + 32 * r] : 0.0;
+#pragma unroll
+    for (int rj = 0; rj < NR; ++rj) {
+        const int n = min(32, k - 32 * rj);
+#pragma unroll 4
+        for (int j0 = 0; j0 < n; ++j0) {
+            const int j = 32 * rj + j0;
+            const double zj = __shfl_sync(0xffffffffu, x[rj], j0);
+#pragma unroll
+            for (int r = rj; r < NR; ++r) {
+                const int i = lane + 32 * r;
+                if (i > j && i < k) x[r] = fma(-L[i * kLd + j], zj, x[r]);
+            }
+        }
     }
+#pragma unroll
+    for (int r = 0; r < NR; ++r)
+        if (lane + 32 * r < k) v[lane + 32 * r] = x[r];
+    __syncwarp();
 }
 
-// v := L^{-T} D^{-1} v (warp 0): the second half of an L D L^T solve
+// v := L^{-T} D^{-1} v: the second half of an L D L^T solve
 template <int kLd>
 __device__ void back_subst_warp(const double *L, const double *inv, double *v, int k)
 {
+    constexpr int NR = (kLd - 1) / 32;
     const int lane = threadIdx.x & 31;
-    for (int i = lane; i < k; i += 32) v[i] *= inv[i];
-    __syncwarp();
-    for (int j = k - 1; j >= 0; --j) {
-        const double yj = v[j];
-        for (int i = lane; i < j; i += 32) v[i] -= L[j * kLd + i] * yj;
-        __syncwarp();
+    double x[NR];
+#pragma unroll
+    for (int r = 0; r < NR; ++r) {
+        const int i = lane + 32 * r;
+        x[r] = i < k ? v[i] * inv[i] : 0.0;
     }
+#pragma unroll
+    for (int rj = NR - 1; rj >= 0; --rj) {
+        const int n = min(32, k - 32 * rj);
+#pragma unroll 4
+        for (int j0 = n - 1; j0 >= 0; --j0) {
+            const int j = 32 * rj + j0;
+            const double yj = __shfl_sync(0xffffffffu, x[rj], j0);
+#pragma unroll
+            for (int r = 0; r <= rj; ++r) {
+                const int i = lane + 32 * r;
+                if (i < j) x[r] = fma(-L[j * kLd + i], yj, x[r]);
+            }
+        }
+    }
+#pragma unroll
+    for (int r = 0; r < NR; ++r)
+        if (lane + 32 * r < k) v[lane + 32 * r] = x[r];
+    __syncwarp();
 }
 
 // KM = kKSmem: the work area in dynamic shared memory; KM = kKMax: in `work`
