@@ -247,6 +247,7 @@ template <int KB> constexpr size_t adj_smem(bool reduce)
 template <int KB>
 __global__ void __launch_bounds__(256, KB <= 2 ? 6 : 0) k_adj_tile(AdjArgs a)
 {
+    chain_wait();
     constexpr int VB = adj_vb<KB>();
     constexpr int VIEW = KB * kAdjWin;  // floats per staged view
     constexpr int NCH = VIEW / 4;       // 16-byte copies per staged view
@@ -438,6 +439,7 @@ __device__ __forceinline__ double clamp0(double x)  // max(0, x) of a number, on
 template <int KB>
 __global__ void __launch_bounds__(256) k_adj64(Adj64Args a)
 {
+    chain_wait();
     __shared__ Adj64View s_view[kAdj64Cap];
     __shared__ double red[KB][256];
     const int tid = threadIdx.x;
@@ -591,6 +593,7 @@ template <typename T> struct __align__(16) Operands {
 template <typename T, int KB, int SPLIT>
 __global__ void __launch_bounds__(32 * kSmallWarps) k_adj_small(SmallArgs<T> a)
 {
+    chain_wait();
     constexpr bool F32 = std::is_same<T, float>::value;
     constexpr int PER = kSmallViews / kSmallWarps;  // views a warp prepares
     __shared__ T s_c[kSmallCap], s_s[kSmallCap], s_w[kSmallCap], s_w1[kSmallCap], s_f[kSmallCap];
@@ -708,9 +711,9 @@ template <typename T, int KB> cudaError_t launch_small(const SmallArgs<T> &a, co
     const long long items = (long long)a.ngroups * a.F * a.tps * a.tps * (kTile / kSmallRows);
     constexpr int NT = 32 * kSmallWarps;
     if (split > 2)
-        k_adj_small<T, KB, 4><<<persistent_grid(k_adj_small<T, KB, 4>, NT, 0, items, h.num_sms), NT, 0, h.stream>>>(a);
+        launch_chained(k_adj_small<T, KB, 4>, persistent_grid(k_adj_small<T, KB, 4>, NT, 0, items, h.num_sms), NT, 0, h.stream, a);
     else
-        k_adj_small<T, KB, 2><<<persistent_grid(k_adj_small<T, KB, 2>, NT, 0, items, h.num_sms), NT, 0, h.stream>>>(a);
+        launch_chained(k_adj_small<T, KB, 2>, persistent_grid(k_adj_small<T, KB, 2>, NT, 0, items, h.num_sms), NT, 0, h.stream, a);
     return cudaGetLastError();
 }
 

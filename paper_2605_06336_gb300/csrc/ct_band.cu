@@ -50,6 +50,7 @@ template <int PENDING> __device__ __forceinline__ void cp_async_wait()
 template <int MODE, bool OFFS, int KB, int VW, int RB, int NS>
 __global__ void __launch_bounds__(32 * VW) k_ray_band(RayArgs<float> a)
 {
+    chain_wait();
     constexpr int IMG = RB * kBandMax;  // pairs per image in one buffer
     constexpr int NACC = (MODE == kFwd) ? KB : 3;
     constexpr int NT = 32 * VW;
@@ -286,6 +287,7 @@ __global__ void __launch_bounds__(32 * VW) k_ray_band(RayArgs<float> a)
 __global__ void k_fwd_combine(const ViewGeo *__restrict__ vg, float *__restrict__ Y, const float *__restrict__ P,
                               int segs, long long stride, int V, int B, long long total, const int *__restrict__ skip)
 {
+    chain_wait();
     if (skip && *skip) return;
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total;
          e += (long long)gridDim.x * blockDim.x) {
@@ -309,7 +311,7 @@ cudaError_t launch_band(const Handle &h, const RayArgs<float> &a)
     }
     const long long items = (long long)a.ngroups * ((a.V + VW - 1) / VW) * a.nchunks * (MODE == kFwd ? a.segs : 1);
     const int grid = persistent_grid(kern, 32 * VW, smem, items, h.num_sms);
-    kern<<<grid, 32 * VW, smem, h.stream>>>(a);
+    launch_chained(kern, grid, 32 * VW, smem, h.stream, a);
     return cudaGetLastError();
 }
 
@@ -338,7 +340,7 @@ cudaError_t launch_fwd_combine(const Handle &h, float *Y, const float *P, int se
     if (total == 0) return cudaSuccess;
     const int threads = 256;
     const long long blocks = std::min<long long>((total + threads - 1) / threads, (long long)h.num_sms * 8);
-    k_fwd_combine<<<(int)blocks, threads, 0, h.stream>>>(h.d_views, Y, P, segs, stride, h.V, h.B, total, skip);
+    launch_chained(k_fwd_combine, (int)blocks, threads, 0, h.stream, h.d_views, Y, P, segs, stride, h.V, h.B, total, skip);
     return cudaGetLastError();
 }
 

@@ -87,6 +87,7 @@ __global__ void __launch_bounds__(128) k_fan_table(const ViewGeo *__restrict__ v
                                                    FanRay<T> *__restrict__ rays, FanLine<T> *__restrict__ lines,
                                                    FanView *__restrict__ views, const int *__restrict__ skip)
 {
+    chain_wait();
     if (skip && *skip) return;
     __shared__ int s_mode0, s_split;
     const double h = 0.5 * (N - 1);
@@ -180,6 +181,7 @@ __global__ void __launch_bounds__(128) k_fan_table(const ViewGeo *__restrict__ v
 template <typename T, int MODE, int KB, int SPLIT, bool OFFS>
 __global__ void __launch_bounds__(32 * SPLIT) k_ray_fan(RayArgs<T> a, const FanRay<T> *__restrict__ rays)
 {
+    chain_wait();
     using P2 = pair_t<T>;
     constexpr int NACC = (MODE == kFwd) ? KB : (OFFS ? 3 : 2);
     __shared__ T red[SPLIT > 1 ? SPLIT : 1][NACC][32];
@@ -338,6 +340,7 @@ template <typename T>
 __global__ void k_fan_sino(const T *__restrict__ Y, T *__restrict__ YI, long long m, int nsino,
                            const int *__restrict__ skip)
 {
+    chain_wait();
     if (skip && *skip) return;
     const long long total = (long long)nsino * m;
     for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < total;
@@ -434,6 +437,7 @@ template <> struct FanSums<8> : FanSumsPacked<8> {};
 template <int KB>
 __global__ void __launch_bounds__(256) k_adj_fan_tile(FanTileArgs a)
 {
+    chain_wait();
     namespace cg = cooperative_groups;
     __shared__ FanTileView s_view[kFanCap];
     __shared__ FanTileRay s_ray[2][kFanVB][kFanWin];
@@ -654,6 +658,7 @@ __global__ void __launch_bounds__(256 * SPLIT) k_adj_fan(AdjFanArgs a, const Fan
                                                          const FanView *__restrict__ views,
                                                          const T *__restrict__ YI, T *__restrict__ X)
 {
+    chain_wait();
     __shared__ T red[SPLIT > 1 ? SPLIT - 1 : 1][KB][256];
     const int pix = threadIdx.x & 255, grp_v = threadIdx.x >> 8;
     const int tx = pix & (kTile - 1), ty = pix / kTile;
@@ -737,7 +742,7 @@ cudaError_t run_fan(const Handle &h, const RayArgs<T> &a)
     auto kern = k_ray_fan<T, MODE, KB, SPLIT, OFFS>;
     const long long items = (long long)a.ngroups * a.V * a.nchunks;
     const int grid = persistent_grid(kern, 32 * SPLIT, 0, items, h.num_sms);
-    kern<<<grid, 32 * SPLIT, 0, h.stream>>>(a, (const FanRay<T> *)h.d_rays);
+    launch_chained(kern, grid, 32 * SPLIT, 0, h.stream, a, (const FanRay<T> *)h.d_rays);
     return cudaGetLastError();
 }
 
@@ -756,7 +761,7 @@ template <typename T, int KB, int SPLIT> cudaError_t run_adj_fan(const Handle &h
     auto kern = k_adj_fan<T, KB, SPLIT>;
     const long long items = (long long)a.ngroups * a.F * a.tps * a.tps;
     const int grid = persistent_grid(kern, 256 * SPLIT, 0, items, h.num_sms);
-    kern<<<grid, 256 * SPLIT, 0, h.stream>>>(a, fan_lines<T>(h.d_rays, (long long)h.V * h.B),
+    launch_chained(kern, grid, 256 * SPLIT, 0, h.stream, a, fan_lines<T>(h.d_rays, (long long)h.V * h.B),
                                              (const FanView *)h.d_fanview, (const T *)h.d_yi, X);
     return cudaGetLastError();
 }
@@ -781,10 +786,10 @@ cudaError_t launch_fan_rays(const Handle &h, const int *skip)
     const long long n = (long long)h.V * h.B;
     const int grid = std::min(h.V, 16 * h.num_sms);
     if (h.precision)
-        k_fan_table<double><<<grid, 128, 0, h.stream>>>(h.d_views, h.V, h.B, h.N, h.fan_D, (FanRay<double> *)h.d_rays,
+        launch_chained(k_fan_table<double>, grid, 128, 0, h.stream, h.d_views, h.V, h.B, h.N, h.fan_D, (FanRay<double> *)h.d_rays,
                                                         fan_lines<double>(h.d_rays, n), (FanView *)h.d_fanview, skip);
     else
-        k_fan_table<float><<<grid, 128, 0, h.stream>>>(h.d_views, h.V, h.B, h.N, h.fan_D, (FanRay<float> *)h.d_rays,
+        launch_chained(k_fan_table<float>, grid, 128, 0, h.stream, h.d_views, h.V, h.B, h.N, h.fan_D, (FanRay<float> *)h.d_rays,
                                                        fan_lines<float>(h.d_rays, n), (FanView *)h.d_fanview, skip);
     return cudaGetLastError();
 }
@@ -890,7 +895,7 @@ template <typename T> cudaError_t launch_fan_sino(const Handle &h, const T *Y, i
     const long long m = (long long)h.V * h.B;
     const long long total = (long long)nsino * m;
     const int grid = (int)std::max<long long>(1, std::min<long long>((total + 255) / 256, 8LL * h.num_sms));
-    k_fan_sino<T><<<grid, 256, 0, h.stream>>>(Y, (T *)h.d_yi, m, nsino, skip);
+    launch_chained(k_fan_sino<T>, grid, 256, 0, h.stream, Y, (T *)h.d_yi, m, nsino, skip);
     return cudaGetLastError();
 }
 

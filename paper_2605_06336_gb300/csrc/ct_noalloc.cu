@@ -17,6 +17,7 @@
 #include <mutex>
 
 #include "../../include/ctgb.h"
+#include "ct_device.cuh"
 #include "ct_internal.cuh"
 
 namespace {
@@ -70,6 +71,7 @@ cudaError_t scratch_base(void **out)
 __global__ void k_mark_nonfinite(const double *__restrict__ theta, const double *__restrict__ delta, int V,
                                  double *__restrict__ gtheta, double *__restrict__ gdelta)
 {
+    ctgb::chain_wait();
     for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < V; v += gridDim.x * blockDim.x) {
         if (isfinite(theta[v]) && (!delta || isfinite(delta[v]))) continue;
         gtheta[v] = __longlong_as_double(0x7ff8000000000000LL);
@@ -118,7 +120,7 @@ extern "C" int ct_jacT_noalloc(int32_t N, int32_t B, int32_t n_views, const doub
     if (ctgb::launch_view_setup(h, theta, delta) != cudaSuccess) return CT_ERR_CUDA;
     if (ctgb::launch_pairs_img<float>(h, x, 1) != cudaSuccess) return CT_ERR_CUDA;
     if (ctgb::launch_vjp<float>(h, r, gtheta, gdelta, h.tune.der_split, 1, 0) != cudaSuccess) return CT_ERR_CUDA;
-    k_mark_nonfinite<<<(n_views + 255) / 256, 256, 0, h.stream>>>(theta, delta, n_views, gtheta, gdelta);
+    ctgb::launch_chained(k_mark_nonfinite, (n_views + 255) / 256, 256, 0, h.stream, theta, delta, n_views, gtheta, gdelta);
     if (cudaGetLastError() != cudaSuccess) return CT_ERR_CUDA;
     return CT_OK;
 }

@@ -192,6 +192,7 @@ __device__ void build_order(const ViewPrep &p, unsigned long long *key)
 
 __global__ void __launch_bounds__(1024) k_view_prep(ViewPrep p, const int *__restrict__ skip)
 {
+    chain_wait();
     __shared__ unsigned long long key[kOrderMaxV];
     if (skip && *skip) return;
     view_prep_block(p, key);
@@ -201,6 +202,7 @@ __global__ void __launch_bounds__(1024) k_view_prep(ViewPrep p, const int *__res
 // (*changed = 1 when a view was rebuilt), then k_view_order in one CTA.
 __global__ void k_view_setup_many(ViewPrep p, int *changed, const int *__restrict__ skip)
 {
+    chain_wait();
     if (skip && *skip) return;
     int mine = 0;
     for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < p.V; v += gridDim.x * blockDim.x)
@@ -210,6 +212,7 @@ __global__ void k_view_setup_many(ViewPrep p, int *changed, const int *__restric
 
 __global__ void __launch_bounds__(1024) k_view_order(ViewPrep p, int *changed, const int *__restrict__ skip)
 {
+    chain_wait();
     __shared__ unsigned long long key[kOrderMaxV];
     if (skip && *skip) return;
     const int ch = *changed;
@@ -232,6 +235,7 @@ __global__ void __launch_bounds__(256) k_pairs_img(const T *__restrict__ X, pair
                                                    pair_t<T> *__restrict__ PT, int N, int Pp, int nimg, ViewPrep p,
                                                    const int *__restrict__ skip)
 {
+    chain_wait();
     extern __shared__ unsigned long long prep_key[];
     if (skip && *skip) return;
     if (p.on && blockIdx.x == gridDim.x - 1) {
@@ -284,6 +288,7 @@ __global__ void __launch_bounds__(256) k_interleave_img(const float *__restrict_
                                                         float *__restrict__ QT, int N, int Pp, int F, int K,
                                                         ViewPrep p, const int *__restrict__ skip)
 {
+    chain_wait();
     extern __shared__ unsigned long long prep_key[];
     if (skip && *skip) return;
     if (p.on && blockIdx.x == gridDim.x - 1) {
@@ -342,6 +347,7 @@ __global__ void k_interleaved_to_pairs(const float *__restrict__ QX, const float
                                        float2 *__restrict__ PX, float2 *__restrict__ PT, int N, int Pp, int F,
                                        int K, int nimg)
 {
+    chain_wait();
     const long long per = (long long)F * N * Pp;  // elements per image
     const long long total = (long long)nimg * per;
     for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < total;
@@ -363,6 +369,7 @@ __global__ void k_interleaved_to_pairs(const float *__restrict__ QX, const float
 __global__ void k_pairs_sino(const double *__restrict__ Y, double2 *__restrict__ YP, int B, int Pb, long long total,
                              ViewPrep p, const int *__restrict__ skip)
 {
+    chain_wait();
     extern __shared__ unsigned long long prep_key[];
     if (skip && *skip) return;
     const int nblk = gridDim.x - (p.on ? 1 : 0);
@@ -393,6 +400,7 @@ __global__ void __launch_bounds__(256) k_interleave_sino(const float *__restrict
                                                          int kb, long long rows, ViewPrep p,
                                                          const int *__restrict__ skip)
 {
+    chain_wait();
     extern __shared__ unsigned long long prep_key[];
     if (skip && *skip) return;
     const int nblk = gridDim.x - (p.on ? 1 : 0);
@@ -473,6 +481,7 @@ __device__ __forceinline__ void taps_interleaved(const float *__restrict__ q, lo
 template <typename T, int MODE, bool OFFS, int KB, int SPLIT, bool QL = false>
 __global__ void __launch_bounds__(512) k_ray(RayArgs<T> a)
 {
+    chain_wait();
     using P2 = pair_t<T>;
     constexpr bool F32 = std::is_same<T, float>::value;
     constexpr int NACC = (MODE == kFwd) ? KB : 3 * KB;
@@ -619,6 +628,7 @@ __global__ void __launch_bounds__(64) k_finalize(const double *__restrict__ part
                                                  double *out2, double scale2, double *out3,
                                                  const int *__restrict__ view_mask, const int *__restrict__ skip)
 {
+    chain_wait();
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     const int o = t >> 2, q = t & 3;
     const int nout = sum ? 1 : nimg;
@@ -678,7 +688,7 @@ cudaError_t run_ray(const Handle &h, const RayArgs<T> &a)
     const size_t smem = SPLIT > 1 ? (size_t)a.VW * SPLIT * NACC * 32 * sizeof(T) : 0;
     const long long items = (long long)a.ngroups * ((a.V + a.VW - 1) / a.VW) * a.nchunks;
     const int grid = persistent_grid(kern, threads, smem, items, h.num_sms);
-    kern<<<grid, threads, smem, h.stream>>>(a);
+    launch_chained(kern, grid, threads, smem, h.stream, a);
     return cudaGetLastError();
 }
 
@@ -753,7 +763,7 @@ template <auto Kernel> cudaError_t allow_prep_smem()
 
 cudaError_t launch_view_setup(const Handle &h, const double *theta, const double *delta, const int *skip)
 {
-    k_view_prep<<<1, 1024, 0, h.stream>>>(view_prep_args(h, theta, delta), skip);
+    launch_chained(k_view_prep, 1, 1024, 0, h.stream, view_prep_args(h, theta, delta), skip);
     if (h.fan_D > 0.0 && theta) {
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
@@ -767,8 +777,8 @@ cudaError_t launch_view_setup_wide(const Handle &h, const double *theta, const d
 {
     const ViewPrep p = view_prep_args(h, theta, delta);
     const int grid = std::max(1, std::min((h.V + 127) / 128, 4 * h.num_sms));
-    k_view_setup_many<<<grid, 128, 0, h.stream>>>(p, changed, skip);
-    k_view_order<<<1, 1024, 0, h.stream>>>(p, changed, skip);
+    launch_chained(k_view_setup_many, grid, 128, 0, h.stream, p, changed, skip);
+    launch_chained(k_view_order, 1, 1024, 0, h.stream, p, changed, skip);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     if (h.fan_D > 0.0) return launch_fan_rays(h, skip);
@@ -783,7 +793,7 @@ cudaError_t launch_pairs_img(const Handle &h, const T *X, int nimg, const int *s
     cudaError_t e = allow_prep_smem<k_pairs_img<T>>();
     if (e != cudaSuccess) return e;
     dim3 grid((h.Pp + 31) / 32 + (p.on ? 1 : 0), (h.N + 31) / 32, std::max(1, std::min(nimg, 65535)));
-    k_pairs_img<T><<<grid, 256, prep_smem(p), h.stream>>>(X, (pair_t<T> *)h.d_px, (pair_t<T> *)h.d_pt, h.N, h.Pp,
+    launch_chained(k_pairs_img<T>, grid, 256, prep_smem(p), h.stream, X, (pair_t<T> *)h.d_px, (pair_t<T> *)h.d_pt, h.N, h.Pp,
                                                           nimg, p, skip);
     if (h.fan_D > 0.0 && theta) {
         e = cudaGetLastError();
@@ -810,7 +820,7 @@ cudaError_t launch_interleave_img(const Handle &h, const float *X, int batch, co
     const int n4 = batch & ~3, rem = batch - n4;
     const int ngroups = n4 / 4 + (rem >= 2 ? 1 : 0) + (rem & 1);
     dim3 grid((h.Pp + 31) / 32 + (p.on ? 1 : 0), (h.N + 31) / 32, std::max(1, std::min(2 * h.F * ngroups, 65535)));
-    k_interleave_img<<<grid, 256, prep_smem(p), h.stream>>>(X, h.d_qx, h.d_qt, h.N, h.Pp, h.F, batch, p, skip);
+    launch_chained(k_interleave_img, grid, 256, prep_smem(p), h.stream, X, h.d_qx, h.d_qt, h.N, h.Pp, h.F, batch, p, skip);
     return cudaGetLastError();
 }
 
@@ -819,7 +829,7 @@ cudaError_t launch_interleaved_to_pairs(const Handle &h, int batch)
     if (!h.d_qx || h.precision != 0 || batch < 1 || batch > h.max_batch) return cudaErrorInvalidValue;
     const long long total = (long long)batch * h.F * h.N * h.Pp;
     const long long blocks = std::min<long long>((total + 255) / 256, (long long)h.num_sms * 16);
-    k_interleaved_to_pairs<<<(int)std::max<long long>(1, blocks), 256, 0, h.stream>>>(
+    launch_chained(k_interleaved_to_pairs, (int)std::max<long long>(1, blocks), 256, 0, h.stream, 
         h.d_qx, h.d_qt, (float2 *)h.d_px, (float2 *)h.d_pt, h.N, h.Pp, h.F, batch, batch);
     return cudaGetLastError();
 }
@@ -845,7 +855,7 @@ cudaError_t launch_sino_layout(const Handle &h, const T *Y, int nsino, int kb, c
         if (e != cudaSuccess) return e;
         const long long rows = (long long)groups * h.V;
         const int blocks = (int)std::min<long long>(rows, (long long)h.num_sms * 16);
-        k_interleave_sino<<<blocks + (p.on ? 1 : 0), 256, prep_smem(p), h.stream>>>(
+        launch_chained(k_interleave_sino, blocks + (p.on ? 1 : 0), 256, prep_smem(p), h.stream, 
             Y, (float *)h.d_yp, h.d_rowflag, h.B, sino_pitch(h.B), h.V, nsino, kb, rows, p, skip);
     } else {
         cudaError_t e = allow_prep_smem<k_pairs_sino>();
@@ -853,7 +863,7 @@ cudaError_t launch_sino_layout(const Handle &h, const T *Y, int nsino, int kb, c
         const long long total = (long long)nsino * h.V * h.Pb;
         const int threads = 256;
         const long long blocks = std::min<long long>((total + threads - 1) / threads, (long long)h.num_sms * 16);
-        k_pairs_sino<<<(int)std::max<long long>(1, blocks) + (p.on ? 1 : 0), threads, prep_smem(p), h.stream>>>(
+        launch_chained(k_pairs_sino, (int)std::max<long long>(1, blocks) + (p.on ? 1 : 0), threads, prep_smem(p), h.stream, 
             Y, (double2 *)h.d_yp, h.B, h.Pb, total, p, skip);
     }
     return cudaGetLastError();
@@ -1005,7 +1015,7 @@ cudaError_t launch_vjp(const Handle &h, const T *R, double *gtheta, double *gdel
                            : der_groups<T, kVjp, false>(h, a, batch, kb, split, stage, interleaved);
     if (e != cudaSuccess) return e;
     const long long outs = (long long)h.V * (sum ? 1 : batch);
-    k_finalize<<<(int)((4 * outs + 63) / 64), 64, 0, h.stream>>>(h.d_partial, h.V, h.nchunks, batch, a.part_stride,
+    launch_chained(k_finalize, (int)((4 * outs + 63) / 64), 64, 0, h.stream, h.d_partial, h.V, h.nchunks, batch, a.part_stride,
                                                             sum, gtheta, gdelta, nullptr, 1.0, nullptr, nullptr,
                                                             nullptr);
     return cudaGetLastError();
@@ -1028,7 +1038,7 @@ cudaError_t launch_gn(const Handle &h, const T *bdata, T *res, double *grad, dou
     cudaError_t e = der_groups<T, kGn, false>(h, a, batch, kb, split, stage, interleaved);
     if (e != cudaSuccess) return e;
     const long long outs = (long long)h.V * batch;
-    k_finalize<<<(int)((4 * outs + 63) / 64), 64, 0, h.stream>>>(h.d_partial, h.V, h.nchunks, batch, a.part_stride, 0,
+    launch_chained(k_finalize, (int)((4 * outs + 63) / 64), 64, 0, h.stream, h.d_partial, h.V, h.nchunks, batch, a.part_stride, 0,
                                                             grad, jnorm2, fval, 0.5, rscale, view_mask, skip);
     return cudaGetLastError();
 }

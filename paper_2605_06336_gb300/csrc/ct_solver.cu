@@ -218,20 +218,20 @@ template <typename T> struct Solver {
                      double *scal_out, int *ctl_out)
     {
         if (k <= kKSmem)
-            k_small_solve<kKSmem><<<1, kSolveThreads, sizeof(SolveShared<kKSmem>), h.stream>>>(
+            launch_chained(k_small_solve<kKSmem>, 1, kSolveThreads, sizeof(SolveShared<kKSmem>), h.stream, 
                 GH, cvec, GP, k, bnorm2, target, lam_fix, lam_lo, lam_hi, lam_iters, yout, scal_out, ctl_out, nullptr);
         else
-            k_small_solve<kKMax><<<1, kSolveThreads, 0, h.stream>>>(GH, cvec, GP, k, bnorm2, target, lam_fix, lam_lo,
+            launch_chained(k_small_solve<kKMax>, 1, kSolveThreads, 0, h.stream, GH, cvec, GP, k, bnorm2, target, lam_fix, lam_lo,
                                                                      lam_hi, lam_iters, yout, scal_out, ctl_out,
                                                                      small_work);
     }
     void compress_basis(int k, int keep)
     {
         if (k <= kKSmem)
-            k_compress_basis<kKSmem><<<1, 256, sizeof(SmallShared<kKSmem>), h.stream>>>(GH, GP, k, scal, keep, W,
+            launch_chained(k_compress_basis<kKSmem>, 1, 256, sizeof(SmallShared<kKSmem>), h.stream, GH, GP, k, scal, keep, W,
                                                                                        nullptr);
         else
-            k_compress_basis<kKMax><<<1, 256, 0, h.stream>>>(GH, GP, k, scal, keep, W, small_work);
+            launch_chained(k_compress_basis<kKMax>, 1, 256, 0, h.stream, GH, GP, k, scal, keep, W, small_work);
     }
 
     // k columns of the edges of one tile of TR x 32 pixels: 2 per pixel, 3 with the temporal edge (ANISO-TV)
@@ -249,13 +249,13 @@ template <typename T> struct Solver {
             if (k <= 32 && gram_pipe_smem(k, epp) <= kGramPipeSmemMax && gram_rb_threads(k) == 256)
                 // 4 x 4 blocks over 4-row tiles for small bases (above 32 columns the 8 x 8 blocks
                 // measured faster: C5 streaming 6.98 -> 6.78 s per pass)
-                k_gram_psi_pipe<<<gram_blocks, kThreads, gram_pipe_smem(k, epp), h.stream>>>(
+                launch_chained(k_gram_psi_pipe, gram_blocks, kThreads, gram_pipe_smem(k, epp), h.stream, 
                     V, n, k, w, h.N, h.F, o.temporal, part_gram, stop);
             else if (gram_p8_rows(k, epp) == 2)  // larger bases: 2-row tiles, 8 x 8 blocks
-                k_gram_psi_pipe8<2, kP8Threads><<<gram_blocks, kP8Threads, gram_p8_smem(k, epp, 2), h.stream>>>(
+                launch_chained(k_gram_psi_pipe8<2, kP8Threads>, gram_blocks, kP8Threads, gram_p8_smem(k, epp, 2), h.stream, 
                     V, n, k, w, h.N, h.F, o.temporal, part_gram, stop);
             else  // 1-row tiles (fits up to the largest basis)
-                k_gram_psi_pipe8<1, kP8Threads><<<gram_blocks, kP8Threads, gram_p8_smem(k, epp, 1), h.stream>>>(
+                launch_chained(k_gram_psi_pipe8<1, kP8Threads>, gram_blocks, kP8Threads, gram_p8_smem(k, epp, 1), h.stream, 
                     V, n, k, w, h.N, h.F, o.temporal, part_gram, stop);
         } else {
             // at least 128 pairs (one chain in flight on each FP64 pipe) per CTA, and CTAs
@@ -263,13 +263,13 @@ template <typename T> struct Solver {
             const int shares = std::max(1, std::min((k * (k + 1) / 2 + 127) / 128, 4 * h.num_sms / gram_blocks));
             const dim3 grid(gram_blocks, shares);
             if (k <= kKSmem)
-                k_gram_psi<T, 4, gram_slots(kKSmem)><<<grid, kThreads, gram_smem(k, tm, 4), h.stream>>>(
+                launch_chained(k_gram_psi<T, 4, gram_slots(kKSmem)>, grid, kThreads, gram_smem(k, tm, 4), h.stream, 
                     V, n, k, w, h.N, h.F, o.temporal, part_gram, stop);
             else
-                k_gram_psi<T, 1, gram_slots(kKLimit)><<<grid, kThreads, gram_smem(k, tm, 1), h.stream>>>(
+                launch_chained(k_gram_psi<T, 1, gram_slots(kKLimit)>, grid, kThreads, gram_smem(k, tm, 1), h.stream, 
                     V, n, k, w, h.N, h.F, o.temporal, part_gram, stop);
         }
-        k_gram_reduce<<<gram_reduce_blocks(k), 32 * kGramReduceWarps, 0, h.stream>>>(part_gram, gram_blocks, k, GP,
+        launch_chained(k_gram_reduce, gram_reduce_blocks(k), 32 * kGramReduceWarps, 0, h.stream, part_gram, gram_blocks, k, GP,
                                                                                      stop);
         SV_CUDA(cudaGetLastError());
         return CT_OK;
@@ -284,7 +284,7 @@ template <typename T> struct Solver {
         const int nblk = red_blocks(len);
         const int kk = k + (x2 ? 1 : 0);
         dots_partials(A, len, k, x, x2, stop);
-        k_dots_reduce<<<(kk + kDotsReduceWarps - 1) / kDotsReduceWarps, 32 * kDotsReduceWarps, 0, h.stream>>>(
+        launch_chained(k_dots_reduce, (kk + kDotsReduceWarps - 1) / kDotsReduceWarps, 32 * kDotsReduceWarps, 0, h.stream, 
             part_dot, nblk, kk, out, stop);
         SV_CUDA(cudaGetLastError());
         return CT_OK;
@@ -294,14 +294,14 @@ template <typename T> struct Solver {
     {
         const int kk = k + (x2 ? 1 : 0);
         const dim3 grid(red_blocks(len), (kk + kDotCols - 1) / kDotCols);
-        k_dots<T><<<grid, kThreads, 0, h.stream>>>(A, len, len, k, x, x2, part_dot, stop);
+        launch_chained(k_dots<T>, grid, kThreads, 0, h.stream, A, len, len, k, x, x2, part_dot, stop);
     }
 
     // row kc of (HV)^T HV and entry kc of (HV)^T b; with ctl_end, the end of an Enlarge step
     void gh_row(int kc, const int *stop, int *ctl_end)
     {
         dots_partials(HV, m, kc + 1, col(HV, m, kc), b, stop);
-        k_gh_append<<<1, kGhThreads, 0, h.stream>>>(part_dot, red_blocks(m), kc, GH, cvec, ctl_end,
+        launch_chained(k_gh_append, 1, kGhThreads, 0, h.stream, part_dot, red_blocks(m), kc, GH, cvec, ctl_end,
                                                     ctl_end ? d_stop : nullptr);
     }
 
@@ -309,8 +309,8 @@ template <typename T> struct Solver {
     int norms3(const T *a, const T *bb, long long len, double *out, const int *stop)
     {
         const int nblk = red_blocks(len);
-        k_norms3<T><<<nblk, kThreads, 0, h.stream>>>(a, bb, len, part_n, stop);
-        k_norms3_reduce<<<1, 32, 0, h.stream>>>(part_n, nblk, out, stop);
+        launch_chained(k_norms3<T>, nblk, kThreads, 0, h.stream, a, bb, len, part_n, stop);
+        launch_chained(k_norms3_reduce, 1, 32, 0, h.stream, part_n, nblk, out, stop);
         SV_CUDA(cudaGetLastError());
         return CT_OK;
     }
@@ -321,7 +321,7 @@ template <typename T> struct Solver {
         if (k == 0) return CT_OK;
         for (int pass = 0; pass < 2; ++pass) {
             SV_TRY(dots_into(V, n, k, r, nullptr, dots, stop));
-            k_gemv<T><<<grid_for(n), kThreads, 0, h.stream>>>(V, n, n, k, dots, r, T(1), T(-1), nullptr, T(0),
+            launch_chained(k_gemv<T>, grid_for(n), kThreads, 0, h.stream, V, n, n, k, dots, r, T(1), T(-1), nullptr, T(0),
                                                                 stop);
         }
         SV_CUDA(cudaGetLastError());
@@ -420,13 +420,13 @@ template <typename T> struct Solver {
     // small elementwise helpers (host-known scalars)
     void scale(T *x, long long len, double s)
     {
-        k_gemv<T><<<grid_for(len), kThreads, 0, h.stream>>>(x, len, len, 0, y, x, (T)s, T(0), nullptr, T(0),
+        launch_chained(k_gemv<T>, grid_for(len), kThreads, 0, h.stream, x, len, len, 0, y, x, (T)s, T(0), nullptr, T(0),
                                                               nullptr);
     }
     // x = a*x + c*z
     void axpby(T *x, const T *z, long long len, double a, double c)
     {
-        k_gemv<T><<<grid_for(len), kThreads, 0, h.stream>>>(x, len, len, 0, y, x, (T)a, T(0), z, (T)c, nullptr);
+        launch_chained(k_gemv<T>, grid_for(len), kThreads, 0, h.stream, x, len, len, 0, y, x, (T)a, T(0), z, (T)c, nullptr);
     }
 
     // ---- one predicated Enlarge step with kc basis columns ------------------
@@ -441,20 +441,20 @@ template <typename T> struct Solver {
         const double target = (o.tau * noise) * (o.tau * noise);
         small_solve(kc, target, o.lam_fix, o.lam_lo, o.lam_hi, o.lam_iters, y, scal, ctl);
         // u = V y ; res = (HV) y - b
-        k_gemv_pair<T><<<grid_for(n) + grid_for(m), kThreads, 0, h.stream>>>(V, n, HV, m, kc, y, u, res, b,
+        launch_chained(k_gemv_pair<T>, grid_for(n) + grid_for(m), kThreads, 0, h.stream, V, n, HV, m, kc, y, u, res, b,
                                                                              grid_for(n), stop);
         SV_CUDA(cudaGetLastError());
         // r = H^T res + lambda Psi^T P^2 Psi u, written straight into the next basis column
         T *r = col(V, n, kc);
         SV_TRY(backproject(theta, res, r, stop));
-        k_add_reg<T><<<grid_for(n), kThreads, 0, h.stream>>>(r, u, w, scal, h.N, h.F, o.temporal, stop);
+        launch_chained(k_add_reg<T>, grid_for(n), kThreads, 0, h.stream, r, u, w, scal, h.N, h.F, o.temporal, stop);
         SV_TRY(cgs2(r, kc, stop));
         // |r|^2; |u|^2, |u - u_old|^2, |u_old|^2; u_old = u; the next step's weights
         const int nblk = red_blocks(n);
-        k_step_norms<T><<<dim3(nblk, 3), kThreads, 0, h.stream>>>(r, u, uold, n, w, h.N, h.F, o.temporal, o.eps,
+        launch_chained(k_step_norms<T>, dim3(nblk, 3), kThreads, 0, h.stream, r, u, uold, n, w, h.N, h.F, o.temporal, o.eps,
                                                                   part_n, stop);
-        k_step_decide<<<1, 128, 0, h.stream>>>(part_n, nblk, o.tol1, norms2, ctl, scal);
-        k_normalize<T><<<grid_for(n), kThreads, 0, h.stream>>>(r, n, norms2, stop);
+        launch_chained(k_step_decide, 1, 128, 0, h.stream, part_n, nblk, o.tol1, norms2, ctl, scal);
+        launch_chained(k_normalize<T>, grid_for(n), kThreads, 0, h.stream, r, n, norms2, stop);
         // H v_new and the new row of (HV)^T HV, (HV)^T b
         SV_TRY(project(theta, kc, 1, stop));
         gh_row(kc, stop, ctl);
@@ -465,7 +465,7 @@ template <typename T> struct Solver {
     // The weights the first step of an Enlarge reads
     void begin_enlarge()
     {
-        k_weights<T><<<grid_for(ne), kThreads, 0, h.stream>>>(uold, w, h.N, h.F, o.temporal, o.eps, nullptr);
+        launch_chained(k_weights<T>, grid_for(ne), kThreads, 0, h.stream, uold, w, h.N, h.F, o.temporal, o.eps, nullptr);
     }
 
     // One Enlarge step: replay the captured graph for this basis size (capture
@@ -514,7 +514,7 @@ template <typename T> struct Solver {
             SV_CUDA(launch_pairs_img<T>(h, uimg, h.F, nullptr, th_n, delta));
             SV_CUDA(launch_gn<T>(h, b, nullptr, g, j2, f0, h.tune.der_split, h.tune.der_vw, h.tune.der_stage,
                                  nullptr, nullptr, 1, 1, rho));
-            k_gn_direction<<<1, 1024, 0, h.stream>>>(g, j2, rho, h.V, o.mu_rel, o.alpha0, armijo_u(), th_n, d, alpha,
+            launch_chained(k_gn_direction, 1, 1024, 0, h.stream, g, j2, rho, h.V, o.mu_rel, o.alpha0, armijo_u(), th_n, d, alpha,
                                                      th_t, active, ctl);
             // Trial rounds run predicated on ctl[kArmijoDone] (set by k_armijo when no
             // view searches any more); the host reads the flag after rounds 1, 3, 7, 15
@@ -526,7 +526,7 @@ template <typename T> struct Solver {
                 SV_CUDA(launch_view_setup_wide(h, th_t, delta, ctl + kViewChanged, done));
                 SV_CUDA(launch_gn<T>(h, b, nullptr, scratch_v, scratch_v, ft, h.tune.der_split, h.tune.der_vw,
                                      h.tune.der_stage, active, done));
-                k_armijo<<<1, 1024, 0, h.stream>>>(f0, ft, g, d, rho, th_n, h.V, o.c1, o.beta, armijo_u(), alpha,
+                launch_chained(k_armijo, 1, 1024, 0, h.stream, f0, ft, g, d, rho, th_n, h.V, o.c1, o.beta, armijo_u(), alpha,
                                                    th_t, active, ctl, hv == o.max_halvings ? 1 : 0);
                 if (hv + 1 == next_check || hv == o.max_halvings || o.plain) {
                     SV_TRY(sync_ctl());
@@ -552,21 +552,21 @@ template <typename T> struct Solver {
             SV_CUDA(launch_pairs_img<T>(h, uimg, h.F, nullptr, th_n, delta));
             SV_CUDA(launch_gn<T>(h, b, nullptr, g, j2, f0, h.tune.der_split, h.tune.der_vw, h.tune.der_stage,
                                  nullptr, nullptr, 1, 1, rho));
-            k_view_sums<<<1, 1024, 0, h.stream>>>(g, j2, f0, rho, h.V, part_n);
+            launch_chained(k_view_sums, 1, 1024, 0, h.stream, g, j2, f0, rho, h.V, part_n);
             double s4[4];
             SV_TRY(read_doubles(part_n, 4, s4));
             const double G = s4[0], JJ = s4[1], F = s4[2], R = s4[3];
             const double dp = -G / (JJ + o.mu_rel * std::max(JJ, 1e-300));
-            k_fill<double><<<grid_for(h.V), kThreads, 0, h.stream>>>(d, h.V, dp);
+            launch_chained(k_fill<double>, grid_for(h.V), kThreads, 0, h.stream, d, h.V, dp);
             bool accepted = false;
             double alpha = o.alpha0;
             for (int hv = 0; hv <= o.max_halvings; ++hv) {
                 if (alpha * std::fabs(G * dp) < armijo_u() * R) break;  // noise floor: no step
-                k_theta_step<<<grid_for(h.V), kThreads, 0, h.stream>>>(th_n, d, alpha, h.V, th_t);
+                launch_chained(k_theta_step, grid_for(h.V), kThreads, 0, h.stream, th_n, d, alpha, h.V, th_t);
                 SV_CUDA(launch_view_setup_wide(h, th_t, delta, ctl + kViewChanged, nullptr));
                 SV_CUDA(launch_gn<T>(h, b, nullptr, scratch_v, scratch_v, ft, h.tune.der_split, h.tune.der_vw,
                                      h.tune.der_stage));
-                k_view_sums<<<1, 1024, 0, h.stream>>>(ft, nullptr, nullptr, nullptr, h.V, part_n);
+                launch_chained(k_view_sums, 1, 1024, 0, h.stream, ft, nullptr, nullptr, nullptr, h.V, part_n);
                 double fsum[1];
                 SV_TRY(read_doubles(part_n, 1, fsum));
                 if (fsum[0] <= F + o.c1 * alpha * G * dp) {
@@ -596,7 +596,7 @@ template <typename T> struct Solver {
         SV_TRY(alloc(vp_scal, kScalCount));
         SV_TRY(alloc(vp_rho, 3));
         SV_TRY(alloc(vp_ctl, kCtlCount));
-        k_fill<double><<<grid_for(v_all), kThreads, 0, h.stream>>>(vp_ones, v_all, 1.0);
+        launch_chained(k_fill<double>, grid_for(v_all), kThreads, 0, h.stream, vp_ones, v_all, 1.0);
         SV_CUDA(cudaMemsetAsync(vp_ctl, 0, sizeof(int) * kCtlCount, h.stream));
         SV_CUDA(cudaMemsetAsync(vp_scal, 0, sizeof(double) * kScalCount, h.stream));
         SV_CUDA(cudaFuncSetAttribute(k_varpro_direction, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -612,10 +612,10 @@ template <typename T> struct Solver {
         SV_CUDA(cudaMemsetAsync(GH, 0, sizeof(double) * kKMax * kKMax, h.stream));
         SV_TRY(full_gram(k));
         small_solve(k, 1.0, lam, 0.0, 0.0, 1, y, vp_scal, vp_ctl);
-        k_gemv<T><<<grid_for(n), kThreads, 0, h.stream>>>(V, n, n, k, y, vp_u, T(0), T(1), nullptr, T(0), nullptr);
-        k_gemv<T><<<grid_for(m), kThreads, 0, h.stream>>>(HV, m, m, k, y, res, T(0), T(1), b, T(-1), nullptr);
+        launch_chained(k_gemv<T>, grid_for(n), kThreads, 0, h.stream, V, n, n, k, y, vp_u, T(0), T(1), nullptr, T(0), nullptr);
+        launch_chained(k_gemv<T>, grid_for(m), kThreads, 0, h.stream, HV, m, m, k, y, res, T(0), T(1), b, T(-1), nullptr);
         SV_TRY(norms3(res, nullptr, m, norms, nullptr));
-        k_varpro_value<<<1, 1, 0, h.stream>>>(norms, GP, y, k, lam, fslot);
+        launch_chained(k_varpro_value, 1, 1, 0, h.stream, norms, GP, y, k, lam, fslot);
         SV_CUDA(cudaGetLastError());
         return CT_OK;
     }
@@ -639,12 +639,12 @@ template <typename T> struct Solver {
             SV_TRY(varpro_eval(th_n, k, lam, vp_scal + kTmp0));
             {  // rounding scale of f's data term at theta (Armijo noise floor)
                 const int nblk = red_blocks(m);
-                k_round_scale<T><<<nblk, kThreads, 0, h.stream>>>(res, b, m, part_n);
-                k_norms3_reduce<<<1, 32, 0, h.stream>>>(part_n, nblk, vp_rho, nullptr);
+                launch_chained(k_round_scale<T>, nblk, kThreads, 0, h.stream, res, b, m, part_n);
+                launch_chained(k_norms3_reduce, 1, 32, 0, h.stream, part_n, nblk, vp_rho, nullptr);
             }
             SV_CUDA(launch_pairs_img<T>(h, vp_u, h.F, nullptr, th_n, delta));
             SV_CUDA(launch_jvp<T>(h, vp_ones, nullptr, vp_a, h.tune.der_split, h.tune.der_vw, h.tune.der_stage));
-            k_view_dots<T><<<std::min(h.V, 8 * h.num_sms), 128, 0, h.stream>>>(HV, m, k, vp_a, res, h.V, h.B, vp_E,
+            launch_chained(k_view_dots<T>, std::min(h.V, 8 * h.num_sms), 128, 0, h.stream, HV, m, k, vp_a, res, h.V, h.B, vp_E,
                                                                                j2, g);
             // G[c][j] = (H_j V_c)^T r: the basis columns in batches of max_batch, one
             // batched VJP against the shared residual per batch
@@ -654,7 +654,7 @@ template <typename T> struct Solver {
                 SV_CUDA(launch_vjp<T>(h, res, vp_G + (size_t)c * h.V, nullptr, h.tune.der_split, h.tune.der_vw,
                                       h.tune.der_stage, nb, h.tune.der_kb, 0, 0));
             }
-            k_varpro_direction<<<1, 1024, sizeof(VpShared), h.stream>>>(GH, GP, lam, vp_E, vp_G, j2, g, k, h.V,
+            launch_chained(k_varpro_direction, 1, 1024, sizeof(VpShared), h.stream, GH, GP, lam, vp_E, vp_G, j2, g, k, h.V,
                                                                         o.mu_rel, vp_Y, vp_idel, d, vp_scal + kTmp1,
                                                                         ctl);
             SV_CUDA(cudaGetLastError());
@@ -669,7 +669,7 @@ template <typename T> struct Solver {
             if (gd < 0.0) {
                 for (int hv = 0; hv <= o.max_halvings; ++hv) {
                     if (alpha * std::fabs(gd) < armijo_u() * rho0) break;  // noise floor: no step
-                    k_theta_step<<<grid_for(h.V), kThreads, 0, h.stream>>>(th_n, d, alpha, h.V, th_t);
+                    launch_chained(k_theta_step, grid_for(h.V), kThreads, 0, h.stream, th_n, d, alpha, h.V, th_t);
                     SV_TRY(varpro_eval(th_t, k, lam, vp_scal + kRnorm2));
                     double ft;
                     SV_TRY(read_doubles(vp_scal + kRnorm2, 1, &ft));
@@ -706,7 +706,7 @@ template <typename T> struct Solver {
         }
         if (o.shared_offset) return update_param_shared(u);
         if (!o.varpro) return update_param(u);
-        k_weights<T><<<grid_for(ne), kThreads, 0, h.stream>>>(u, w, h.N, h.F, o.temporal, o.eps, nullptr);
+        launch_chained(k_weights<T>, grid_for(ne), kThreads, 0, h.stream, u, w, h.N, h.F, o.temporal, o.eps, nullptr);
         double lam;
         SV_TRY(read_doubles(scal + kLam, 1, &lam));
         return varpro_update(th_k, kc, lam, th_n, nullptr);
@@ -728,16 +728,16 @@ template <typename T> struct Solver {
         SV_CUDA(cudaMemsetAsync(GH, 0, sizeof(double) * kKMax * kKMax, h.stream));
         SV_TRY(full_gram(k));
         if (u_w) {
-            k_weights<T><<<grid_for(ne), kThreads, 0, h.stream>>>(u_w, w, h.N, h.F, o.temporal, o.eps, nullptr);
+            launch_chained(k_weights<T>, grid_for(ne), kThreads, 0, h.stream, u_w, w, h.N, h.F, o.temporal, o.eps, nullptr);
         } else {
-            k_fill<T><<<grid_for(ne), kThreads, 0, h.stream>>>(w, ne, T(1));
+            launch_chained(k_fill<T>, grid_for(ne), kThreads, 0, h.stream, w, ne, T(1));
         }
         SV_TRY(gram_psi(k, nullptr));
         small_solve(k, 1.0, lam, 0.0, 0.0, 1, y, scal, ctl);
-        k_gemv<T><<<grid_for(n), kThreads, 0, h.stream>>>(V, n, n, k, y, u, T(0), T(1), nullptr, T(0), nullptr);
-        k_gemv<T><<<grid_for(m), kThreads, 0, h.stream>>>(HV, m, m, k, y, res, T(0), T(1), b, T(-1), nullptr);
+        launch_chained(k_gemv<T>, grid_for(n), kThreads, 0, h.stream, V, n, n, k, y, u, T(0), T(1), nullptr, T(0), nullptr);
+        launch_chained(k_gemv<T>, grid_for(m), kThreads, 0, h.stream, HV, m, m, k, y, res, T(0), T(1), b, T(-1), nullptr);
         SV_TRY(norms3(res, nullptr, m, norms, nullptr));
-        k_varpro_value<<<1, 1, 0, h.stream>>>(norms, GP, y, k, lam, fval);
+        launch_chained(k_varpro_value, 1, 1, 0, h.stream, norms, GP, y, k, lam, fval);
         SV_CUDA(cudaGetLastError());
         if (grad) {
             SV_CUDA(launch_pairs_img<T>(h, u, h.F, nullptr, theta, delta));
@@ -796,8 +796,8 @@ template <typename T> struct Solver {
         const int k_used = kc + steps_out - 1;
         SV_TRY(compress(k_used, kc));
         SV_TRY(param_update(kc));
-        k_norms3<double><<<red_blocks(h.V), kThreads, 0, h.stream>>>(th_n, th_k, h.V, part_n, nullptr);
-        k_norms3_reduce<<<1, 32, 0, h.stream>>>(part_n, red_blocks(h.V), norms, nullptr);
+        launch_chained(k_norms3<double>, red_blocks(h.V), kThreads, 0, h.stream, th_n, th_k, h.V, part_n, nullptr);
+        launch_chained(k_norms3_reduce, 1, 32, 0, h.stream, part_n, red_blocks(h.V), norms, nullptr);
         double dth3[3], lam_now[1];
         SV_TRY(read_doubles(norms, 3, dth3));
         SV_TRY(read_doubles(scal + kLam, 1, lam_now));
@@ -815,11 +815,11 @@ template <typename T> struct Solver {
         const int keep = std::min(o.k_min - 1, k_used);
         compress_basis(k_used, keep);
         for (int c0 = 0; c0 < keep; c0 += 16)  // 16 output columns per pass over V
-            k_gemm_small<T><<<grid_for(n), kThreads, 0, h.stream>>>(V, n, n, k_used, W + c0,
+            launch_chained(k_gemm_small<T>, grid_for(n), kThreads, 0, h.stream, V, n, n, k_used, W + c0,
                                                                     std::min(16, keep - c0), col(Vtmp, n, c0), n);
         SV_CUDA(cudaMemcpyAsync(V, Vtmp, sizeof(T) * n * keep, cudaMemcpyDeviceToDevice, h.stream));
         SV_TRY(dots_into(V, n, keep, u, nullptr, dots, nullptr));
-        k_gemv<T><<<grid_for(n), kThreads, 0, h.stream>>>(V, n, n, keep, dots, col(V, n, keep), T(0), T(-1), u,
+        launch_chained(k_gemv<T>, grid_for(n), kThreads, 0, h.stream, V, n, n, keep, dots, col(V, n, keep), T(0), T(-1), u,
                                                             T(1), nullptr);
         SV_TRY(norms3(col(V, n, keep), u, n, norms, nullptr));
         double nu[3];
@@ -963,12 +963,12 @@ template <typename T> struct Solver {
             // parameter update
             SV_TRY(param_update(kc));
             // residual of the normal equations at H_k, new weights, appended to V
-            k_weights<T><<<grid_for(ne), kThreads, 0, h.stream>>>(u, w, h.N, h.F, o.temporal, o.eps, nullptr);
+            launch_chained(k_weights<T>, grid_for(ne), kThreads, 0, h.stream, u, w, h.N, h.F, o.temporal, o.eps, nullptr);
             SV_CUDA(launch_prep_forward<T>(h, u, h.F, nullptr, th_k, delta));
             SV_CUDA(launch_forward<T>(h, res, 1, h.tune.fwd_kb, h.tune.fwd_split, h.tune.fwd_vw, h.tune.fwd_stage));
             axpby(res, b, m, 1.0, -1.0);
             SV_TRY(backproject(th_k, res, col(V, n, kc), nullptr));
-            k_add_reg<T><<<grid_for(n), kThreads, 0, h.stream>>>(col(V, n, kc), u, w, scal, h.N, h.F, o.temporal,
+            launch_chained(k_add_reg<T>, grid_for(n), kThreads, 0, h.stream, col(V, n, kc), u, w, scal, h.N, h.F, o.temporal,
                                                                 nullptr);
             SV_TRY(cgs2(col(V, n, kc), kc, nullptr));
             SV_TRY(norms3(col(V, n, kc), nullptr, n, norms2, nullptr));
@@ -982,8 +982,8 @@ template <typename T> struct Solver {
                 scale(col(V, n, kc), n, 1.0 / std::sqrt(dr[0]));
                 kc += 1;
             }
-            k_norms3<double><<<red_blocks(h.V), kThreads, 0, h.stream>>>(th_n, th_k, h.V, part_n, nullptr);
-            k_norms3_reduce<<<1, 32, 0, h.stream>>>(part_n, red_blocks(h.V), norms, nullptr);
+            launch_chained(k_norms3<double>, red_blocks(h.V), kThreads, 0, h.stream, th_n, th_k, h.V, part_n, nullptr);
+            launch_chained(k_norms3_reduce, 1, 32, 0, h.stream, part_n, red_blocks(h.V), norms, nullptr);
             double dth3[3];
             SV_TRY(read_doubles(norms, 3, dth3));
             double rre = -1.0;
@@ -1240,10 +1240,10 @@ int nlrmm_varpro_update(ct_handle *H, const void *b, double *theta_inout, const 
         SV_TRY(s.setup());
         SV_CUDA(cudaMemcpyAsync(s.V, V, sizeof(T) * s.n * k, cudaMemcpyDeviceToDevice, ps));
         if (u_w) {
-            k_weights<T><<<s.grid_for(s.ne), kThreads, 0, ps>>>((const T *)u_w, s.w, h.N, h.F, o.temporal, o.eps,
+            launch_chained(k_weights<T>, s.grid_for(s.ne), kThreads, 0, ps, (const T *)u_w, s.w, h.N, h.F, o.temporal, o.eps,
                                                                    nullptr);
         } else {
-            k_fill<T><<<s.grid_for(s.ne), kThreads, 0, ps>>>(s.w, s.ne, T(1));
+            launch_chained(k_fill<T>, s.grid_for(s.ne), kThreads, 0, ps, s.w, s.ne, T(1));
         }
         SV_CUDA(cudaGetLastError());
         return s.varpro_update(theta_inout, k, lam, theta_inout, f_hist);

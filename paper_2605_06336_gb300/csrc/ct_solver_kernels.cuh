@@ -105,6 +105,7 @@ template <typename T>
 __global__ void k_weights(const T *__restrict__ u, T *__restrict__ w, int N, int F, int temporal, double eps,
                           const int *stop)
 {
+    chain_wait();
     if (stopped(stop)) return;
     weights_range(u, w, N, F, temporal, eps, blockIdx.x * (long long)blockDim.x + threadIdx.x,
                   (long long)gridDim.x * blockDim.x);
@@ -115,6 +116,7 @@ template <typename T>
 __global__ void k_add_reg(T *__restrict__ r, const T *__restrict__ u, const T *__restrict__ w,
                           const double *__restrict__ scal, int N, int F, int temporal, const int *stop)
 {
+    chain_wait();
     if (stopped(stop)) return;
     const long long n = (long long)F * N * N;
     const long long nx = (long long)F * N * (N - 1);
@@ -165,6 +167,7 @@ __global__ void __launch_bounds__(256) k_gram_psi(const T *__restrict__ V, long 
                                                   const T *__restrict__ w, int N, int F, int temporal,
                                                   double *__restrict__ part, const int *stop)
 {
+    chain_wait();
     if (stopped(stop)) return;
     extern __shared__ unsigned char smem_raw[];
     constexpr int TP = TR * 32;                  // pixels per tile
@@ -293,6 +296,7 @@ __global__ void __launch_bounds__(256) k_gram_psi_pipe(const float *__restrict__
                                                        const float *__restrict__ w, int N, int F, int temporal,
                                                        double *__restrict__ part, const int *stop)
 {
+    chain_wait();
     if (stopped(stop)) return;
     extern __shared__ float4 rb_smem[];
     const int EPP = (temporal && F > 1) ? 3 : 2;
@@ -481,6 +485,7 @@ __global__ void __launch_bounds__(NT, 1) k_gram_psi_pipe8(const float *__restric
                                                           const float *__restrict__ w, int N, int F, int temporal,
                                                           double *__restrict__ part, const int *stop)
 {
+    chain_wait();
     if (stopped(stop)) return;
     extern __shared__ float4 p8_smem[];
     constexpr int TPIX = TR * 32;
@@ -662,6 +667,7 @@ __global__ void __launch_bounds__(32 * kGramReduceWarps) k_gram_reduce(const dou
                                                                        int k, double *__restrict__ G,
                                                                        const int *stop)
 {
+    chain_wait();
     if (stopped(stop)) return;
     const int np = k * (k + 1) / 2;
     const int lane = threadIdx.x & 31;
@@ -706,6 +712,7 @@ __global__ void __launch_bounds__(256) k_dots(const T *__restrict__ A, long long
                                               const T *__restrict__ x, const T *__restrict__ x2,
                                               double *__restrict__ part, const int *stop)
 {
+    chain_wait();
     if (stopped(stop)) return;
     constexpr int G = kDotCols;
     __shared__ double sh[G][257];
@@ -777,6 +784,7 @@ __global__ void __launch_bounds__(32 * kDotsReduceWarps) k_dots_reduce(const dou
                                                                        int kk, double *__restrict__ out,
                                                                        const int *stop)
 {
+    chain_wait();
     if (stopped(stop)) return;
     const int a = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
@@ -808,6 +816,7 @@ template <typename T>
 __global__ void k_gemv(const T *__restrict__ A, long long len, long long lda, int k, const double *__restrict__ y,
                        T *__restrict__ out, T beta, T sgn, const T *__restrict__ bias, T bsgn, const int *stop)
 {
+    chain_wait();
     if (stopped(stop)) return;
     __shared__ T ys[kKMax];
     for (int a = threadIdx.x; a < k; a += blockDim.x) ys[a] = (T)y[a];
@@ -827,6 +836,7 @@ __global__ void k_gemv_pair(const T *__restrict__ V, long long n, const T *__res
                             const double *__restrict__ y, T *__restrict__ u, T *__restrict__ res,
                             const T *__restrict__ b, int g1, const int *stop)
 {
+    chain_wait();
     if (stopped(stop)) return;
     __shared__ T ys[kKMax];
     for (int a = threadIdx.x; a < k; a += blockDim.x) ys[a] = (T)y[a];
@@ -846,6 +856,7 @@ template <typename T>
 __global__ void k_gemm_small(const T *__restrict__ A, long long len, long long lda, int k,
                              const double *__restrict__ W, int kc, T *__restrict__ out, long long ldo)
 {
+    chain_wait();
     __shared__ T Ws[kKMax * 16];
     for (int idx = threadIdx.x; idx < k * kc; idx += blockDim.x) Ws[idx] = (T)W[(idx / kc) * kKMax + idx % kc];
     __syncthreads();
@@ -870,6 +881,7 @@ template <typename T>
 __global__ void k_norms3(const T *__restrict__ a, const T *__restrict__ b, long long len, double *__restrict__ part,
                          const int *stop)
 {
+    chain_wait();
     if (stopped(stop)) return;
     __shared__ double sh[33];
     double s0 = 0.0, s1 = 0.0, s2 = 0.0;
@@ -894,6 +906,7 @@ __global__ void k_norms3(const T *__restrict__ a, const T *__restrict__ b, long 
 __global__ void k_norms3_reduce(const double *__restrict__ part, int nblk, double *__restrict__ out3,
                                 const int *stop)
 {
+    chain_wait();
     if (stopped(stop)) return;
     if (threadIdx.x >= 32) return;
     for (int q = 0; q < 3; ++q) {
@@ -915,6 +928,7 @@ __global__ void __launch_bounds__(256) k_step_norms(const T *__restrict__ r, con
                                                     long long n, T *__restrict__ w, int N, int F, int temporal,
                                                     double eps, double *__restrict__ part, const int *stop)
 {
+    chain_wait();
     if (stopped(stop)) return;
     const long long i0 = blockIdx.x * (long long)blockDim.x + threadIdx.x, stride = (long long)gridDim.x * blockDim.x;
     if (blockIdx.y == 2) {
@@ -959,6 +973,7 @@ __global__ void __launch_bounds__(128) k_step_decide(const double *__restrict__ 
                                                      double *__restrict__ rn2, int *__restrict__ ctl,
                                                      double *__restrict__ scal)
 {
+    chain_wait();
     if (ctl[kStop]) return;
     __shared__ double sum[4];  // |u|^2, |u - u_old|^2, |u_old|^2, |r|^2
     const int q = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -984,6 +999,7 @@ __global__ void __launch_bounds__(128) k_step_decide(const double *__restrict__ 
 template <typename T>
 __global__ void k_normalize(T *__restrict__ r, long long len, const double *__restrict__ rn2, const int *stop)
 {
+    chain_wait();
     if (stopped(stop)) return;
     __shared__ T s_inv;
     if (threadIdx.x == 0) {
@@ -1007,6 +1023,7 @@ __global__ void __launch_bounds__(kGhThreads) k_gh_append(const double *__restri
                                                           double *__restrict__ GH, double *__restrict__ cvec,
                                                           int *__restrict__ ctl, volatile int *__restrict__ stop_mirror)
 {
+    chain_wait();
     const bool stop = ctl && ctl[kStop];
     const int lane = threadIdx.x & 31;
     if (!stop) {
@@ -1348,6 +1365,7 @@ __global__ void __launch_bounds__(kSolveThreads) k_small_solve(const double *__r
                                                                double *__restrict__ scal, int *__restrict__ ctl,
                                                                double *work)
 {
+    chain_wait();
     if (ctl[kStop]) return;
     extern __shared__ unsigned char smem_raw[];
     constexpr int kLd = SolveShared<KM>::kLd;
@@ -1471,6 +1489,7 @@ __global__ void __launch_bounds__(256) k_compress_basis(const double *__restrict
                                                         int k, const double *__restrict__ scal, int keep,
                                                         double *__restrict__ W, double *work)
 {
+    chain_wait();
     extern __shared__ unsigned char smem_raw[];
     constexpr int kLd = SmallShared<KM>::kLd;
     SmallShared<KM> &S = *reinterpret_cast<SmallShared<KM> *>(KM > kKSmem ? (unsigned char *)work : smem_raw);
@@ -1515,6 +1534,7 @@ template <typename T>
 __global__ void k_round_scale(const T *__restrict__ r, const T *__restrict__ b, long long len,
                               double *__restrict__ part)
 {
+    chain_wait();
     __shared__ double sh[33];
     double s0 = 0.0;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < len; i += (long long)gridDim.x * blockDim.x) {
@@ -1533,6 +1553,7 @@ __global__ void k_round_scale(const T *__restrict__ r, const T *__restrict__ b, 
 __global__ void k_varpro_value(const double *__restrict__ norms3_res, const double *__restrict__ GP,
                                const double *__restrict__ y, int k, double lam, double *__restrict__ fval)
 {
+    chain_wait();
     double q = 0.0;
     for (int i = 0; i < k; ++i)
         for (int j = 0; j < k; ++j) q += y[i] * GP[i * kKMax + j] * y[j];
@@ -1541,6 +1562,7 @@ __global__ void k_varpro_value(const double *__restrict__ norms3_res, const doub
 
 template <typename T> __global__ void k_fill(T *__restrict__ x, long long len, T value)
 {
+    chain_wait();
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < len; i += (long long)gridDim.x * blockDim.x)
         x[i] = value;
 }
@@ -1560,6 +1582,7 @@ __global__ void k_gn_direction(const double *__restrict__ g, const double *__res
                                const double *__restrict__ theta, double *__restrict__ d, double *__restrict__ alpha,
                                double *__restrict__ theta_trial, int *__restrict__ active, int *__restrict__ ctl)
 {
+    chain_wait();
     __shared__ int cnt[32];
     __shared__ double sh[40];
     double mx = 0.0;
@@ -1602,6 +1625,7 @@ __global__ void k_view_sums(const double *__restrict__ a0, const double *__restr
                             const double *__restrict__ a2, const double *__restrict__ a3, int V,
                             double *__restrict__ out)
 {
+    chain_wait();
     __shared__ double sh[40];
     const double *a[4] = {a0, a1, a2, a3};
     for (int q = 0; q < 4; ++q) {
@@ -1624,6 +1648,7 @@ __global__ void k_armijo(const double *__restrict__ f0, const double *__restrict
                          double *__restrict__ alpha, double *__restrict__ theta_trial, int *__restrict__ active,
                          int *__restrict__ ctl, int last)
 {
+    chain_wait();
     __shared__ int cnt[32];
     if (ctl[kArmijoDone]) return;
     int mine = 0;
@@ -1683,6 +1708,7 @@ __global__ void __launch_bounds__(128) k_view_dots(const T *__restrict__ HV, lon
                                                    double *__restrict__ E, double *__restrict__ j2,
                                                    double *__restrict__ g)
 {
+    chain_wait();
     __shared__ double red[4];
     for (int j = blockIdx.x; j < V; j += gridDim.x) {
         const size_t off = (size_t)j * B;
@@ -1727,6 +1753,7 @@ __global__ void __launch_bounds__(1024) k_varpro_direction(const double *__restr
                                                            double *__restrict__ d, double *__restrict__ gd_out,
                                                            int *__restrict__ ctl)
 {
+    chain_wait();
     extern __shared__ unsigned char smem_raw[];
     VpShared &S = *reinterpret_cast<VpShared *>(smem_raw);
     constexpr int kLd = VpShared::kLd;
@@ -1861,6 +1888,7 @@ __global__ void __launch_bounds__(1024) k_varpro_direction(const double *__restr
 __global__ void k_theta_step(const double *__restrict__ theta, const double *__restrict__ d, double alpha, int V,
                              double *__restrict__ out)
 {
+    chain_wait();
     for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < V; v += gridDim.x * blockDim.x)
         out[v] = theta[v] + alpha * d[v];
 }
