@@ -74,6 +74,31 @@ __device__ __forceinline__ double warp_sum(double x)
     return x;
 }
 
+// Sums of NQ (a power of two) values over the warp, each by the tree of
+// warp_sum: while more than one is left, the lanes at each level keep half of
+// them and hand the other half over, so that four sums take 6
+// additions a lane instead of 20 (an FP64 addition occupies the pipe for 64
+// cycles; the same additions, so the same bits).  Lane l returns the sum of
+// value l / (32 / NQ).
+template <int NQ, int O = 16> __device__ __forceinline__ double warp_sums(double (&x)[NQ], int lane)
+{
+    if constexpr (O == 0) {
+        return x[0];
+    } else if constexpr (NQ > 1) {
+        double h[NQ / 2];
+        const bool up = lane & O;
+#pragma unroll
+        for (int i = 0; i < NQ / 2; ++i) {
+            const double send = up ? x[i] : x[i + NQ / 2], keep = up ? x[i + NQ / 2] : x[i];
+            h[i] = keep + __shfl_xor_sync(0xffffffffu, send, O);
+        }
+        return warp_sums<NQ / 2, O / 2>(h, lane);
+    } else {
+        x[0] += __shfl_xor_sync(0xffffffffu, x[0], O);
+        return warp_sums<1, O / 2>(x, lane);
+    }
+}
+
 // floor(t) and t - floor(t) in [0, 1] for |t| < 2^22 without a conversion
 // instruction: t - 1/2 is rounded to an integer by the 1.5 * 2^23 shift.
 // When t is an integer the rounding may land on t - 1, giving f = 1, which
@@ -226,8 +251,11 @@ __device__ __forceinline__ void ray_epilogue(const RayArgs<T> &a, const ViewGeo 
                 if (k0 + k < a.kend) a.Y[(size_t)(k0 + k) * a.sino_stride + (size_t)v * a.B + b] = wv * acc[k];
         }
     } else {
-        // image k of the group: acc[3k] interpolated sum, acc[3k+1] slope x dq/dtheta, acc[3k+2] slopes
+        // image k of the group: acc[3k] interpolated sum, acc[3k+1] slope x dq/dtheta, acc[3k+2] slopes;
+        // VJP / GN: NQ quantities per image, reduced over the warp together
+        constexpr int NQ = MODE == kGn ? 4 : (OFFS ? 2 : 1);
         const size_t vb = (size_t)v * a.B + b;
+        [[maybe_unused]] double part[KB * NQ];
 #pragma unroll
         for (int k = 0; k < KB; ++k) {
             const size_t img = (size_t)(k0 + k);
@@ -246,13 +274,8 @@ __device__ __forceinline__ void ray_epilogue(const RayArgs<T> &a, const ViewGeo 
                     pt = (double)(r * jt);
                     if (OFFS) pd = (double)(r * jd);
                 }
-                pt = warp_sum(pt);
-                if (OFFS) pd = warp_sum(pd);
-                if (lane == 0) {
-                    double *p = a.partial + img * a.part_stride + ((size_t)v * a.nchunks + chunk) * 4;
-                    p[0] = pt;
-                    p[1] = pd;
-                }
+                part[k * NQ] = pt;
+                if constexpr (OFFS) part[k * NQ + 1] = pd;
             } else {  // kGn
                 // pr: the rounding scale |r| (|H x| + |b|) of the misfit (Armijo noise floor)
                 double pg = 0.0, pj = 0.0, pf = 0.0, pr = 0.0;
@@ -266,17 +289,18 @@ __device__ __forceinline__ void ray_epilogue(const RayArgs<T> &a, const ViewGeo 
                     pf = (double)rr * (double)rr;
                     pr = fabs((double)rr) * (fabs((double)hx) + fabs((double)bb));
                 }
-                pg = warp_sum(pg);
-                pj = warp_sum(pj);
-                pf = warp_sum(pf);
-                pr = warp_sum(pr);
-                if (lane == 0) {
-                    double *p = a.partial + img * a.part_stride + ((size_t)v * a.nchunks + chunk) * 4;
-                    p[0] = pg;
-                    p[1] = pj;
-                    p[2] = pf;
-                    p[3] = pr;
-                }
+                part[k * NQ] = pg;
+                part[k * NQ + 1] = pj;
+                part[k * NQ + 2] = pf;
+                part[k * NQ + 3] = pr;
+            }
+        }
+        if constexpr (MODE != kJvp) {
+            constexpr int PER = 32 / (KB * NQ);  // lanes holding one sum
+            const double s = warp_sums(part, lane);
+            if (lane % PER == 0) {
+                const int q = lane / PER;
+                a.partial[(size_t)(k0 + q / NQ) * a.part_stride + ((size_t)v * a.nchunks + chunk) * 4 + q % NQ] = s;
             }
         }
     }
