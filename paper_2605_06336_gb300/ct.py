@@ -146,7 +146,8 @@ def _check(rc: int, what: str):
 
 
 def _p(t):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+    """The device address of a tensor (ctypes turns the int into a pointer; None is NULL)."""
+    return None if t is None else t.data_ptr()
 
 
 def _stream_ptr(stream=None):
@@ -180,11 +181,15 @@ def ct_destroy(h):
 
 
 def ct_forward(h, theta, delta, X, Y, batch):
-    _check(load_library().ct_forward(h, _p(theta), _p(delta), _p(X), _p(Y), int(batch)), "ct_forward")
+    rc = load_library().ct_forward(h, _p(theta), _p(delta), _p(X), _p(Y), int(batch))
+    if rc != CT_OK:
+        raise CTError(rc, "ct_forward")
 
 
 def ct_adjoint(h, theta, delta, Y, X, batch):
-    _check(load_library().ct_adjoint(h, _p(theta), _p(delta), _p(Y), _p(X), int(batch)), "ct_adjoint")
+    rc = load_library().ct_adjoint(h, _p(theta), _p(delta), _p(Y), _p(X), int(batch))
+    if rc != CT_OK:
+        raise CTError(rc, "ct_adjoint")
 
 
 def ct_measure_peaks():
@@ -417,17 +422,11 @@ class CTOperator:
         self.dtype = dtype
         self.device = torch.device(device)
         self.source_distance = source_distance
+        self.n = self.F * self.N * self.N  # elements of an image
+        self.m = self.V * self.B           # elements of a sinogram
         with torch.cuda.device(self.device):
             self.h = ct_init(N, B, n_views, views_per_frame, max_batch, 1 if dtype == torch.float64 else 0,
                              source_distance=source_distance or 0.0)
-
-    @property
-    def n(self):
-        return self.F * self.N * self.N
-
-    @property
-    def m(self):
-        return self.V * self.B
 
     def close(self):
         if getattr(self, "h", None) is not None:
@@ -459,19 +458,26 @@ class CTOperator:
         if X is None:
             K = int(batch or 1)
             shape = (self.m,) if batch is None else (K, self.m)
-            dev = theta.device
         else:
             self._chk(X, self.n, "X")
-            K = 1 if X.dim() == 1 else X.shape[0]
-            shape, dev = X.shape[:-1] + (self.m,), X.device
-        Y = out if out is not None else torch.empty(shape, dtype=self.dtype, device=dev)
+            d = X.dim()
+            K = 1 if d == 1 else X.size(0)
+            Y = out
+            if Y is None:
+                Y = X.new_empty((K, self.m) if d == 2 else X.shape[:-1] + (self.m,))
+            ct_forward(self.h, self._ang(theta, "theta"), self._ang(delta, "delta"), X, Y, K)
+            return Y
+        Y = out if out is not None else torch.empty(shape, dtype=self.dtype, device=theta.device)
         ct_forward(self.h, self._ang(theta, "theta"), self._ang(delta, "delta"), X, Y, K)
         return Y
 
     def adjoint(self, Y, theta, delta=None, out=None):
         self._chk(Y, self.m, "Y")
-        K = 1 if Y.dim() == 1 else Y.shape[0]
-        X = out if out is not None else torch.empty(Y.shape[:-1] + (self.n,), dtype=self.dtype, device=Y.device)
+        d = Y.dim()
+        K = 1 if d == 1 else Y.size(0)
+        X = out
+        if X is None:
+            X = Y.new_empty((K, self.n) if d == 2 else Y.shape[:-1] + (self.n,))
         ct_adjoint(self.h, self._ang(theta, "theta"), self._ang(delta, "delta"), Y, X, K)
         return X
 
