@@ -554,7 +554,7 @@ int ct_init(const ct_geom *g, void *cuda_stream, ct_handle **out)
                   cudaMalloc(&h.d_fov, sizeof(int) * h.V) == cudaSuccess &&
                   cudaMalloc(&h.d_fstart, sizeof(int) * h.F) == cudaSuccess &&
                   cudaMalloc(&h.d_fcount, sizeof(int) * h.F) == cudaSuccess &&
-                  cudaMalloc(&h.d_flag, sizeof(int)) == cudaSuccess &&
+                  cudaMalloc(&h.d_flag, 2 * sizeof(int)) == cudaSuccess &&
                   cudaMalloc(&h.d_order, sizeof(int) * h.V) == cudaSuccess &&
                   cudaMalloc(&h.d_px, img_pairs * pair_bytes) == cudaSuccess &&
                   cudaMalloc(&h.d_pt, img_pairs * pair_bytes) == cudaSuccess &&
@@ -575,7 +575,7 @@ int ct_init(const ct_geom *g, void *cuda_stream, ct_handle **out)
         e = cudaMemcpy(h.d_fov, fov.data(), sizeof(int) * h.V, cudaMemcpyHostToDevice);
         if (e == cudaSuccess) e = cudaMemcpy(h.d_fstart, fstart.data(), sizeof(int) * h.F, cudaMemcpyHostToDevice);
         if (e == cudaSuccess) e = cudaMemcpy(h.d_fcount, fcount.data(), sizeof(int) * h.F, cudaMemcpyHostToDevice);
-        if (e == cudaSuccess) e = cudaMemset(h.d_flag, 0, sizeof(int));
+        if (e == cudaSuccess) e = cudaMemset(h.d_flag, 0, 2 * sizeof(int));
         if (e == cudaSuccess) e = cudaMemset(h.d_views, 0, sizeof(ctgb::ViewGeo) * h.V);
         if (e == cudaSuccess) e = cudaMemset(h.d_px, 0, img_pairs * pair_bytes);
         if (e == cudaSuccess) e = cudaMemset(h.d_pt, 0, img_pairs * pair_bytes);

@@ -151,7 +151,7 @@ struct Handle {
     int *d_fov = nullptr;     // frame of each view
     int *d_fstart = nullptr;  // first view of each frame
     int *d_fcount = nullptr;  // views of each frame
-    int *d_flag = nullptr;    // device-side status bits
+    int *d_flag = nullptr;    // device-side status bits, then the arrival count of the view-table step
     int *d_order = nullptr;   // view order of the ray kernels (sorted by axis and slope)
     void *d_px = nullptr;     // pair images, rows of X:   (max_batch + 1) * F * N * Pp pairs
     void *d_pt = nullptr;     // pair images, rows of X^T: (max_batch + 1) * F * N * Pp pairs
@@ -188,17 +188,11 @@ struct Handle {
 // `skip` (nullable, device) lets a caller that runs a fixed launch sequence
 // (the solver's predicated Enlarge steps) turn a launch into a no-op: when
 // *skip != 0 the kernel returns at once.
+// The view-table step of a call on its own.
 cudaError_t launch_view_setup(const Handle &h, const double *theta, const double *delta,
                               const int *skip = nullptr);
-// The same step with the per-view constants spread over many CTAs (for large
-// view counts) and the view order rebuilt by one more CTA when a view
-// changed; *changed (device, zero on entry) is the flag between the two and
-// is zero again afterwards.
-cudaError_t launch_view_setup_wide(const Handle &h, const double *theta, const double *delta, int *changed,
-                                   const int *skip = nullptr);
-
 // Layout kernels.  With theta non-null the same launch also runs the view-table
-// step of the call (what launch_view_setup does), in one extra CTA.
+// step of the call (what launch_view_setup does), in extra CTAs.
 template <typename T>
 cudaError_t launch_pairs_img(const Handle &h, const T *X, int nimg, const int *skip = nullptr,
                              const double *theta = nullptr, const double *delta = nullptr);

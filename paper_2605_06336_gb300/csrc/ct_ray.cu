@@ -129,98 +129,124 @@ __device__ bool view_setup_one(int v, const double *__restrict__ theta, const do
     return true;
 }
 
-// Per-view setup and view order in one single-CTA launch.  The view order
-// of the ray kernels sorts the views by frame, then by marching axis, then
-// by ray slope qr (ties by index), so that consecutive entries read the same
-// image and sweep nearly the same band of it; it is rebuilt only when a view
-// changed.  Without an order buffer (nullable) only the constants are built.
+// The view-table step of a call: the per-view constants of the views whose
+// angle or offset changed, then the view order.  The order of the ray kernels
+// sorts the views by frame, then by marching axis, then by ray slope qr (ties
+// by index), so that consecutive entries read the same image and sweep nearly
+// the same band of it; it is rebuilt only when a view changed.  Without an
+// order buffer (nullable) only the constants are built.
+//
+// The constants are FP64: some hundred dependent operations of ~63 cycles a
+// view, one warp per scheduler filling the pipe, so the step is spread over
+// ceil(V / 256) CTAs and the last one to finish sorts.  In one CTA, ranking by
+// counting, the layout kernel that carries the step waited for it when the
+// angles were new: 120 us instead of 31 us at 1200 views (first call of a
+// 16-frame block of 8 images: 585 us; 503 us spread).  Up to 256 views one CTA
+// does it, as the arrival costs 0.6 us of every call (28.5 us instead of
+// 27.9 us for a one-image block of 180 views, 128 views per CTA).
 constexpr int kOrderMaxV = 4096;
+constexpr int kOrderRankMaxV = 256;   // rank counting up to here, sorting above
+constexpr int kPrepViews = 256;       // views per CTA of the view-table step, one per thread
 
 // What the view-table step of an operator call needs; `on` = 0: no step.
 struct ViewPrep {
     const double *theta, *delta;
     const int *fov;
-    int V, N, B, on;
+    int V, N, B, on;  // on: CTAs of the step
     ViewGeo *vg;
-    int *flag;
+    int *flag;           // flag[0]: bad input, flag[1]: arrivals of the step's CTAs (0 between calls)
     int *order;  // nullable: constants only
 };
 
 __device__ void build_order(const ViewPrep &p, unsigned long long *key);
 
-// The view-table step, run by one whole CTA; key: shared memory for
-// min(V, kOrderMaxV) 64-bit keys.
-__device__ void view_prep_block(const ViewPrep &p, unsigned long long *key)
+// CTA `part` of the p.on CTAs of the view-table step (kPrepViews threads);
+// key: shared memory of prep_smem bytes.  No CTA waits for another: each adds
+// itself, and whether it rebuilt a view, to the arrival count, and the last
+// one builds the order and clears the count.
+__device__ void view_prep_block(const ViewPrep &p, int part, unsigned long long *key)
 {
-    __shared__ int s_changed;
-    if (threadIdx.x == 0) s_changed = 0;
-    __syncthreads();
+    __shared__ int s_build;
     int mine = 0;
-    for (int v = threadIdx.x; v < p.V; v += blockDim.x)
+    for (int v = part * kPrepViews + threadIdx.x; v < p.V; v += p.on * kPrepViews)
         mine |= view_setup_one(v, p.theta, p.delta, p.fov, p.N, p.B, p.vg, p.flag);
-    if (mine) s_changed = 1;  // every writer stores the same value
-    __syncthreads();
-    if (!p.order || !s_changed) return;
-    build_order(p, key);
+    mine = __syncthreads_or(mine);
+    if (!p.order) return;
+    if (p.on > 1) {
+        if (threadIdx.x == 0) {
+            const int add = mine ? 0x10001 : 1;
+            __threadfence();
+            const int all = atomicAdd(p.flag + 1, add) + add;
+            const bool last = (all & 0xffff) == p.on;
+            if (last) p.flag[1] = 0;
+            s_build = last && (all >> 16);
+            __threadfence();
+        }
+        __syncthreads();
+        mine = s_build;
+    }
+    if (mine) build_order(p, key);
 }
 
-// The view order of a CTA from the current view records (see view_prep_block).
+// The view order, by one CTA, from the current view records.
 __device__ void build_order(const ViewPrep &p, unsigned long long *key)
 {
-    if (p.V > kOrderMaxV) {
-        for (int i = threadIdx.x; i < p.V; i += blockDim.x) p.order[i] = i;
+    const int V = p.V;
+    if (V > kOrderMaxV) {
+        for (int i = threadIdx.x; i < V; i += blockDim.x) p.order[i] = i;
         return;
     }
-    // One unsigned 64-bit key per view orders by (frame, axis, slope): the
-    // fixed-point slope |Qh| < 2^47 is offset into 48 bits, the axis and the
-    // frame sit above it.  The rank of a view counts the keys below it (ties by
-    // index); integer compares, as the FP64 pipe of this part is narrow.
-    for (int i = threadIdx.x; i < p.V; i += blockDim.x)
-        key[i] = ((unsigned long long)p.vg[i].frame << 49) | ((unsigned long long)p.vg[i].mode << 48) |
-                 (unsigned long long)(p.vg[i].Qh + (1LL << 47));
+    // One unsigned 64-bit key per view orders by (frame, axis, slope, index):
+    // 12 bits of the frame, the axis, the leading 39 bits of the fixed-point
+    // slope |Qh| < 2^47 (offset into 48 bits) and 12 bits of the index, so that
+    // no two are alike; integer compares, as the FP64 pipe of this part is narrow.
+    int P = V;
+    if (V > kOrderRankMaxV)
+        for (P = 2 * kOrderRankMaxV; P < V;) P *= 2;
+    for (int i = threadIdx.x; i < P; i += blockDim.x)
+        key[i] = i < V ? ((unsigned long long)(p.vg[i].frame & 0xfff) << 52) |
+                             ((unsigned long long)p.vg[i].mode << 51) |
+                             ((unsigned long long)(p.vg[i].Qh + (1LL << 47)) >> 9 << 12) | i
+                       : ~0ULL;
     __syncthreads();
-    for (int i = threadIdx.x; i < p.V; i += blockDim.x) {
-        const unsigned long long ki = key[i];
-        int rank = 0;
-        for (int j = 0; j < p.V; ++j) {
-            const unsigned long long kj = key[j];
-            rank += (kj < ki || (kj == ki && j < i)) ? 1 : 0;
+    // Up to one view per thread the rank of a view counts the keys below it (V
+    // steps); above, a bitonic sort: 1200 views in 66 steps of 4 exchanges a
+    // thread instead of 5 x 1200 compares, 512 views in 45 instead of 2 x 512.
+    if (V <= kOrderRankMaxV) {
+        for (int i = threadIdx.x; i < V; i += blockDim.x) {
+            const unsigned long long ki = key[i];
+            int rank = 0;
+            for (int j = 0; j < V; ++j) rank += key[j] < ki ? 1 : 0;
+            p.order[rank] = i;
         }
-        p.order[rank] = i;
+        return;
     }
+    for (int size = 2; size <= P; size *= 2) {
+        for (int stride = size / 2; stride > 0; stride /= 2) {
+            for (int t = threadIdx.x; t < P / 2; t += blockDim.x) {
+                const int i = 2 * t - (t & (stride - 1)), j = i + stride;
+                const unsigned long long a = key[i], b = key[j];
+                if ((a > b) == ((i & size) == 0)) {
+                    key[i] = b;
+                    key[j] = a;
+                }
+            }
+            // exchanges over at most 32 stay within the 64 keys of a warp
+            if (stride > 32 || (stride == 1 && size > 32))
+                __syncthreads();
+            else
+                __syncwarp();
+        }
+    }
+    for (int i = threadIdx.x; i < V; i += blockDim.x) p.order[i] = (int)(key[i] & 0xfff);
 }
 
-__global__ void __launch_bounds__(1024) k_view_prep(ViewPrep p, const int *__restrict__ skip)
+__global__ void __launch_bounds__(256) k_view_prep(ViewPrep p, const int *__restrict__ skip)
 {
     chain_wait();
-    __shared__ unsigned long long key[kOrderMaxV];
+    extern __shared__ unsigned long long prep_key[];
     if (skip && *skip) return;
-    view_prep_block(p, key);
-}
-
-// The same step spread over many CTAs: the per-view constants in parallel
-// (*changed = 1 when a view was rebuilt), then k_view_order in one CTA.
-__global__ void k_view_setup_many(ViewPrep p, int *changed, const int *__restrict__ skip)
-{
-    chain_wait();
-    if (skip && *skip) return;
-    int mine = 0;
-    for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < p.V; v += gridDim.x * blockDim.x)
-        mine |= view_setup_one(v, p.theta, p.delta, p.fov, p.N, p.B, p.vg, p.flag);
-    if (mine) *changed = 1;  // every writer stores the same value
-}
-
-__global__ void __launch_bounds__(1024) k_view_order(ViewPrep p, int *changed, const int *__restrict__ skip)
-{
-    chain_wait();
-    __shared__ unsigned long long key[kOrderMaxV];
-    if (skip && *skip) return;
-    const int ch = *changed;
-    __syncthreads();  // every thread has read the flag before it is cleared below
-    if (!ch || !p.order) return;
-    build_order(p, key);
-    __syncthreads();
-    if (threadIdx.x == 0) *changed = 0;
+    view_prep_block(p, blockIdx.x, prep_key);
 }
 
 // ---------------------------------------------------------------------------
@@ -228,8 +254,8 @@ __global__ void __launch_bounds__(1024) k_view_order(ViewPrep p, int *changed, c
 // ---------------------------------------------------------------------------
 // Tile of 32 rows x 32 pairs.  PX[img][r][cp] = (X[r][c], X[r][c+1]) and
 // PT[img][r][cp] = (X[c][r], X[c+1][r]) with c = cp - 2, zero outside.
-// With p.on, one extra column of CTAs is launched and its first CTA runs the
-// view-table step of the call (the two are independent).
+// With p.on, extra columns of CTAs are launched and their first p.on CTAs run
+// the view-table step of the call (the two are independent).
 template <typename T>
 __global__ void __launch_bounds__(256) k_pairs_img(const T *__restrict__ X, pair_t<T> *__restrict__ PX,
                                                    pair_t<T> *__restrict__ PT, int N, int Pp, int nimg, ViewPrep p,
@@ -238,8 +264,9 @@ __global__ void __launch_bounds__(256) k_pairs_img(const T *__restrict__ X, pair
     chain_wait();
     extern __shared__ unsigned long long prep_key[];
     if (skip && *skip) return;
-    if (p.on && blockIdx.x == gridDim.x - 1) {
-        if (blockIdx.y == 0 && blockIdx.z == 0) view_prep_block(p, prep_key);
+    if (blockIdx.x >= (Pp + 31) / 32) {
+        const int part = ((blockIdx.x - (Pp + 31) / 32) * gridDim.z + blockIdx.z) * gridDim.y + blockIdx.y;
+        if (part < p.on) view_prep_block(p, part, prep_key);
         return;
     }
     __shared__ T a[32][34];   // a[i][j] = X[r0 + i][c0 + j]
@@ -282,7 +309,7 @@ __global__ void __launch_bounds__(256) k_pairs_img(const T *__restrict__ X, pair
 // X -> interleaved images of X and X^T (FP32): each CTA writes a 32 x 32
 // element tile of one orientation, of one frame of one group, with the
 // group's images staged together so that every element is written as one
-// vector of w floats.  With p.on the last column of CTAs carries the
+// vector of w floats.  With p.on the last columns of CTAs carry the
 // view-table step, as in k_pairs_img.
 __global__ void __launch_bounds__(256) k_interleave_img(const float *__restrict__ X, float *__restrict__ QX,
                                                         float *__restrict__ QT, int N, int Pp, int F, int K,
@@ -291,8 +318,9 @@ __global__ void __launch_bounds__(256) k_interleave_img(const float *__restrict_
     chain_wait();
     extern __shared__ unsigned long long prep_key[];
     if (skip && *skip) return;
-    if (p.on && blockIdx.x == gridDim.x - 1) {
-        if (blockIdx.y == 0 && blockIdx.z == 0) view_prep_block(p, prep_key);
+    if (blockIdx.x >= (Pp + 31) / 32) {
+        const int part = ((blockIdx.x - (Pp + 31) / 32) * gridDim.z + blockIdx.z) * gridDim.y + blockIdx.y;
+        if (part < p.on) view_prep_block(p, part, prep_key);
         return;
     }
     // rows of X:    t[j][i][e] = X_j[r0 + i][e0 - 2 + e]
@@ -365,19 +393,19 @@ __global__ void k_interleaved_to_pairs(const float *__restrict__ QX, const float
 }
 
 // FP64: YP[row][bp] = (Y[row][bp - 2], Y[row][bp - 1]), zero outside [0, B).
-// With p.on, the last CTA runs the view-table step of the call instead.
+// With p.on, the first p.on CTAs run the view-table step of the call instead.
 __global__ void k_pairs_sino(const double *__restrict__ Y, double2 *__restrict__ YP, int B, int Pb, long long total,
                              ViewPrep p, const int *__restrict__ skip)
 {
     chain_wait();
     extern __shared__ unsigned long long prep_key[];
     if (skip && *skip) return;
-    const int nblk = gridDim.x - (p.on ? 1 : 0);
-    if (p.on && blockIdx.x == nblk) {
-        view_prep_block(p, prep_key);
+    const int nblk = gridDim.x - p.on, blk = blockIdx.x - p.on;
+    if (blk < 0) {
+        view_prep_block(p, blockIdx.x, prep_key);
         return;
     }
-    for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < total;
+    for (long long idx = blk * (long long)blockDim.x + threadIdx.x; idx < total;
          idx += (long long)nblk * blockDim.x) {
         const long long row = idx / Pb;
         const int bp = (int)(idx - row * Pb);
@@ -393,8 +421,8 @@ __global__ void k_pairs_sino(const double *__restrict__ Y, double2 *__restrict__
 // FP32: the interleaved sinograms of the transpose (ct_internal.cuh).  A CTA
 // takes rows (group, view): each thread reads its bin of the group's sinograms
 // (coalesced over the bins) and writes them side by side; the row's flag says
-// whether it holds a non-finite value.  With p.on, the last CTA runs the
-// view-table step of the call instead.
+// whether it holds a non-finite value.  With p.on, the first p.on CTAs
+// run the view-table step of the call instead.
 __global__ void __launch_bounds__(256) k_interleave_sino(const float *__restrict__ Y, float *__restrict__ YI,
                                                          int *__restrict__ rowflag, int B, int Pq, int V, int nsino,
                                                          int kb, long long rows, ViewPrep p,
@@ -403,12 +431,12 @@ __global__ void __launch_bounds__(256) k_interleave_sino(const float *__restrict
     chain_wait();
     extern __shared__ unsigned long long prep_key[];
     if (skip && *skip) return;
-    const int nblk = gridDim.x - (p.on ? 1 : 0);
-    if (p.on && blockIdx.x == nblk) {
-        view_prep_block(p, prep_key);
+    const int nblk = gridDim.x - p.on, blk = blockIdx.x - p.on;
+    if (blk < 0) {
+        view_prep_block(p, blockIdx.x, prep_key);
         return;
     }
-    for (long long row = blockIdx.x; row < rows; row += nblk) {
+    for (long long row = blk; row < rows; row += nblk) {
         const int grp = (int)(row / V), v = (int)(row - (long long)grp * V);
         const int k0 = grp * kb, live = min(kb, nsino - k0);
         int w = 1;
@@ -740,14 +768,25 @@ ViewPrep view_prep_args(const Handle &h, const double *theta, const double *delt
     p.V = h.V;
     p.N = h.N;
     p.B = h.B;
-    p.on = theta != nullptr;
+    p.on = theta ? std::min((h.V + kPrepViews - 1) / kPrepViews, 1024) : 0;
     p.vg = h.d_views;
     p.flag = h.d_flag;
     p.order = h.d_order;
     return p;
 }
 
-size_t prep_smem(const ViewPrep &p) { return p.on ? sizeof(unsigned long long) * std::min(p.V, kOrderMaxV) : 0; }
+// Shared memory for the keys of the order: a power of two where they are sorted.
+size_t prep_smem(const ViewPrep &p)
+{
+    if (!p.on || !p.order || p.V > kOrderMaxV) return 0;
+    size_t keys = p.V;
+    if (p.V > kOrderRankMaxV)
+        for (keys = 2 * kOrderRankMaxV; keys < (size_t)p.V;) keys *= 2;
+    return sizeof(unsigned long long) * keys;
+}
+
+// Columns of CTAs that an image layout launch adds for the step.
+unsigned prep_columns(const ViewPrep &p, dim3 grid) { return (p.on + grid.y * grid.z - 1) / (grid.y * grid.z); }
 
 // The layout kernels may carry the view-table step in up to 32 KB of dynamic shared memory.
 template <auto Kernel> cudaError_t allow_prep_smem()
@@ -764,26 +803,14 @@ template <auto Kernel> cudaError_t allow_prep_smem()
 
 cudaError_t launch_view_setup(const Handle &h, const double *theta, const double *delta, const int *skip)
 {
-    launch_chained(k_view_prep, 1, 1024, 0, h.stream, view_prep_args(h, theta, delta), skip);
+    const ViewPrep p = view_prep_args(h, theta, delta);
+    launch_chained(k_view_prep, p.on, 256, prep_smem(p), h.stream, p, skip);
     if (h.fan_D > 0.0 && theta) {
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
         return launch_fan_rays(h, skip);
     }
     return cudaGetLastError();
-}
-
-cudaError_t launch_view_setup_wide(const Handle &h, const double *theta, const double *delta, int *changed,
-                                   const int *skip)
-{
-    const ViewPrep p = view_prep_args(h, theta, delta);
-    const int grid = std::max(1, std::min((h.V + 127) / 128, 4 * h.num_sms));
-    launch_chained(k_view_setup_many, grid, 128, 0, h.stream, p, changed, skip);
-    launch_chained(k_view_order, 1, 1024, 0, h.stream, p, changed, skip);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    if (h.fan_D > 0.0) return launch_fan_rays(h, skip);
-    return cudaSuccess;
 }
 
 template <typename T>
@@ -793,7 +820,8 @@ cudaError_t launch_pairs_img(const Handle &h, const T *X, int nimg, const int *s
     const ViewPrep p = view_prep_args(h, theta, delta);
     cudaError_t e = allow_prep_smem<k_pairs_img<T>>();
     if (e != cudaSuccess) return e;
-    dim3 grid((h.Pp + 31) / 32 + (p.on ? 1 : 0), (h.N + 31) / 32, std::max(1, std::min(nimg, 65535)));
+    dim3 grid((h.Pp + 31) / 32, (h.N + 31) / 32, std::max(1, std::min(nimg, 65535)));
+    grid.x += prep_columns(p, grid);
     launch_chained(k_pairs_img<T>, grid, 256, prep_smem(p), h.stream, X, (pair_t<T> *)h.d_px, (pair_t<T> *)h.d_pt, h.N, h.Pp,
                                                           nimg, p, skip);
     if (h.fan_D > 0.0 && theta) {
@@ -820,7 +848,8 @@ cudaError_t launch_interleave_img(const Handle &h, const float *X, int batch, co
     if (e != cudaSuccess) return e;
     const int n4 = batch & ~3, rem = batch - n4;
     const int ngroups = n4 / 4 + (rem >= 2 ? 1 : 0) + (rem & 1);
-    dim3 grid((h.Pp + 31) / 32 + (p.on ? 1 : 0), (h.N + 31) / 32, std::max(1, std::min(2 * h.F * ngroups, 65535)));
+    dim3 grid((h.Pp + 31) / 32, (h.N + 31) / 32, std::max(1, std::min(2 * h.F * ngroups, 65535)));
+    grid.x += prep_columns(p, grid);
     launch_chained(k_interleave_img, grid, 256, prep_smem(p), h.stream, X, h.d_qx, h.d_qt, h.N, h.Pp, h.F, batch, p, skip);
     return cudaGetLastError();
 }
@@ -856,7 +885,7 @@ cudaError_t launch_sino_layout(const Handle &h, const T *Y, int nsino, int kb, c
         if (e != cudaSuccess) return e;
         const long long rows = (long long)groups * h.V;
         const int blocks = (int)std::min<long long>(rows, (long long)h.num_sms * 16);
-        launch_chained(k_interleave_sino, blocks + (p.on ? 1 : 0), 256, prep_smem(p), h.stream, 
+        launch_chained(k_interleave_sino, blocks + p.on, 256, prep_smem(p), h.stream, 
             Y, (float *)h.d_yp, h.d_rowflag, h.B, sino_pitch(h.B), h.V, nsino, kb, rows, p, skip);
     } else {
         cudaError_t e = allow_prep_smem<k_pairs_sino>();
@@ -864,7 +893,7 @@ cudaError_t launch_sino_layout(const Handle &h, const T *Y, int nsino, int kb, c
         const long long total = (long long)nsino * h.V * h.Pb;
         const int threads = 256;
         const long long blocks = std::min<long long>((total + threads - 1) / threads, (long long)h.num_sms * 16);
-        launch_chained(k_pairs_sino, (int)std::max<long long>(1, blocks) + (p.on ? 1 : 0), threads, prep_smem(p), h.stream, 
+        launch_chained(k_pairs_sino, (int)std::max<long long>(1, blocks) + p.on, threads, prep_smem(p), h.stream, 
             Y, (double2 *)h.d_yp, h.B, h.Pb, total, p, skip);
     }
     return cudaGetLastError();

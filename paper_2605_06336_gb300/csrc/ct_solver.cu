@@ -523,7 +523,7 @@ template <typename T> struct Solver {
             const int *done = ctl + kArmijoDone;
             int next_check = 1;
             for (int hv = 0; hv <= o.max_halvings; ++hv) {
-                SV_CUDA(launch_view_setup_wide(h, th_t, delta, ctl + kViewChanged, done));
+                SV_CUDA(launch_view_setup(h, th_t, delta, done));
                 SV_CUDA(launch_gn<T>(h, b, nullptr, scratch_v, scratch_v, ft, h.tune.der_split, h.tune.der_vw,
                                      h.tune.der_stage, active, done));
                 launch_chained(k_armijo, 1, 1024, 0, h.stream, f0, ft, g, d, rho, th_n, h.V, o.c1, o.beta, armijo_u(), alpha,
@@ -563,7 +563,7 @@ template <typename T> struct Solver {
             for (int hv = 0; hv <= o.max_halvings; ++hv) {
                 if (alpha * std::fabs(G * dp) < armijo_u() * R) break;  // noise floor: no step
                 launch_chained(k_theta_step, grid_for(h.V), kThreads, 0, h.stream, th_n, d, alpha, h.V, th_t);
-                SV_CUDA(launch_view_setup_wide(h, th_t, delta, ctl + kViewChanged, nullptr));
+                SV_CUDA(launch_view_setup(h, th_t, delta));
                 SV_CUDA(launch_gn<T>(h, b, nullptr, scratch_v, scratch_v, ft, h.tune.der_split, h.tune.der_vw,
                                      h.tune.der_stage));
                 launch_chained(k_view_sums, 1, 1024, 0, h.stream, ft, nullptr, nullptr, nullptr, h.V, part_n);
