@@ -252,12 +252,16 @@ __global__ void __launch_bounds__(256) k_view_prep(ViewPrep p, const int *__rest
 // ---------------------------------------------------------------------------
 // pair layouts
 // ---------------------------------------------------------------------------
-// Tile of 32 rows x 32 pairs.  PX[img][r][cp] = (X[r][c], X[r][c+1]) and
-// PT[img][r][cp] = (X[c][r], X[c+1][r]) with c = cp - 2, zero outside.
+// PX[img][r][cp] = (X[r][c], X[r][c + 1]) and PT[img][c][rp] = (X[r][c],
+// X[r + 1][c]) with cp = c + 2, rp = r + 2 and zero outside the image: the
+// 33 x 33 elements of X from (r0, c0) on, both from -2 in steps of 32, hold a
+// 32 x 32 tile of each, so that X is read once.  Bound by
+// memory (2048^2, one image: 84 MB, 12.4 us at the copy rate): 35 us reading X
+// once per orientation, 17.4 us so; 48 registers (5 CTAs an SM) instead of 64.
 // With p.on, extra columns of CTAs are launched and their first p.on CTAs run
 // the view-table step of the call (the two are independent).
 template <typename T>
-__global__ void __launch_bounds__(256) k_pairs_img(const T *__restrict__ X, pair_t<T> *__restrict__ PX,
+__global__ void __launch_bounds__(256, 5) k_pairs_img(const T *__restrict__ X, pair_t<T> *__restrict__ PX,
                                                    pair_t<T> *__restrict__ PT, int N, int Pp, int nimg, ViewPrep p,
                                                    const int *__restrict__ skip)
 {
@@ -269,49 +273,55 @@ __global__ void __launch_bounds__(256) k_pairs_img(const T *__restrict__ X, pair
         if (part < p.on) view_prep_block(p, part, prep_key);
         return;
     }
-    __shared__ T a[32][34];   // a[i][j] = X[r0 + i][c0 + j]
-    __shared__ T bt[33][33];  // bt[i][j] = X[c0 + i][r0 + j]
+    __shared__ T t[33][33];  // t[i][j] = X[r0 + i][c0 + j]
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-    const int cp0 = blockIdx.x * 32, r0 = blockIdx.y * 32, c0 = cp0 - 2;
+    const int r0 = blockIdx.y * 32 - 2, c0 = blockIdx.x * 32 - 2;
     for (int img = blockIdx.z; img < nimg; img += gridDim.z) {
         const T *src = X + (size_t)img * N * N;
-        __syncthreads();
-        for (int i = ty; i < 32; i += 8) {
-            const int r = r0 + i;
-            for (int j = tx; j < 33; j += 32) {
-                const int c = c0 + j;
-                a[i][j] = (r < N && c >= 0 && c < N) ? src[(size_t)r * N + c] : T(0);
-            }
-        }
-        for (int i = ty; i < 33; i += 8) {
-            const int rr = c0 + i, cc = r0 + tx;
-            bt[i][tx] = (rr >= 0 && rr < N && cc < N) ? src[(size_t)rr * N + cc] : T(0);
-        }
+        auto at = [&](int i, int j) {
+            const int r = r0 + i, c = c0 + j;
+            return (r >= 0 && r < N && c >= 0 && c < N) ? src[(size_t)r * N + c] : T(0);
+        };
+        T x[4];
+#pragma unroll
+        for (int m = 0; m < 4; ++m) x[m] = at(ty + 8 * m, tx);
+        const T edge = ty == 0 ? at(32, tx) : (ty == 1 ? at(tx, 32) : T(0));  // the corner (32, 32) is not used
+        __syncthreads();  // the previous image's tile has been read
+#pragma unroll
+        for (int m = 0; m < 4; ++m) t[ty + 8 * m][tx] = x[m];
+        if (ty == 0) t[32][tx] = edge;
+        if (ty == 1) t[tx][32] = edge;
         __syncthreads();
         pair_t<T> *px = PX + (size_t)img * N * Pp;
         pair_t<T> *pt = PT + (size_t)img * N * Pp;
-        for (int i = ty; i < 32; i += 8) {
-            const int r = r0 + i, cp = cp0 + tx;
-            if (r < N && cp < Pp) {
-                pair_t<T> p;
-                p.x = a[i][tx];
-                p.y = a[i][tx + 1];
-                px[(size_t)r * Pp + cp] = p;
+#pragma unroll
+        for (int m = 0; m < 4; ++m) {
+            const int i = ty + 8 * m;
+            if (r0 + i >= 0 && r0 + i < N && c0 + tx + 2 < Pp) {
                 pair_t<T> q;
-                q.x = bt[tx][i];
-                q.y = bt[tx + 1][i];
-                pt[(size_t)r * Pp + cp] = q;
+                q.x = x[m];
+                q.y = t[i][tx + 1];
+                px[(size_t)(r0 + i) * Pp + c0 + tx + 2] = q;
+            }
+            if (c0 + i >= 0 && c0 + i < N && r0 + tx + 2 < Pp) {
+                pair_t<T> q;
+                q.x = t[tx][i];
+                q.y = t[tx + 1][i];
+                pt[(size_t)(c0 + i) * Pp + r0 + tx + 2] = q;
             }
         }
     }
 }
 
-// X -> interleaved images of X and X^T (FP32): each CTA writes a 32 x 32
-// element tile of one orientation, of one frame of one group, with the
-// group's images staged together so that every element is written as one
-// vector of w floats.  With p.on the last columns of CTAs carry the
-// view-table step, as in k_pairs_img.
-__global__ void __launch_bounds__(256) k_interleave_img(const float *__restrict__ X, float *__restrict__ QX,
+// X -> interleaved images of X and X^T (FP32): each CTA reads a 32 x 32 tile
+// of the images of one group, of one frame, from (r0, c0) on (both from -2 in
+// steps of 32), once; a thread has the group's images at its elements side by
+// side and writes them as one vector of w floats to the image of X, and
+// through shared memory to that of X^T.  Bound by memory (16
+// frames of 256^2, 8 images: 100 MB, 15 us at the copy rate): 31 us with a CTA
+// and a read of X per orientation, 20 us so.
+// With p.on the last columns of CTAs carry the view-table step, as in k_pairs_img.
+__global__ void __launch_bounds__(256, 5) k_interleave_img(const float *__restrict__ X, float *__restrict__ QX,
                                                         float *__restrict__ QT, int N, int Pp, int F, int K,
                                                         ViewPrep p, const int *__restrict__ skip)
 {
@@ -323,48 +333,50 @@ __global__ void __launch_bounds__(256) k_interleave_img(const float *__restrict_
         if (part < p.on) view_prep_block(p, part, prep_key);
         return;
     }
-    // rows of X:    t[j][i][e] = X_j[r0 + i][e0 - 2 + e]
-    // columns of X: t[j][e][i] = X_j[e0 - 2 + e][r0 + i]
-    __shared__ float t[4][32][33];
+    __shared__ float t[4][32][33];  // t[j][i][e] = X_j[r0 + i][c0 + e]
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-    const int e0 = blockIdx.x * 32, r0 = blockIdx.y * 32;
+    const int r0 = blockIdx.y * 32 - 2, c0 = blockIdx.x * 32 - 2;
     const int n4 = K & ~3, rem = K - n4;
     const int ngroups = n4 / 4 + (rem >= 2 ? 1 : 0) + (rem & 1);
-    for (int z = blockIdx.z; z < 2 * F * ngroups; z += gridDim.z) {
-        const int trans = z & 1, gf = z >> 1;
-        const int gi = gf / F, f = gf - gi * F;
+    for (int z = blockIdx.z; z < F * ngroups; z += gridDim.z) {
+        const int gi = z / F, f = z - gi * F;
         int k0, w;
         interleave_group(gi < n4 / 4 ? 4 * gi : (gi == n4 / 4 && rem >= 2 ? n4 : K - 1), K, k0, w);
-        __syncthreads();
+        float x[4][4];  // [m][j]
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-            if (j < w) {
-                const float *src = X + ((size_t)(k0 + j) * F + f) * N * N;
+            const float *src = X + ((size_t)(k0 + j) * F + f) * N * N;
 #pragma unroll
-                for (int m = 0; m < 4; ++m) {
-                    const int i = ty + 8 * m;
-                    const int rr = trans ? e0 - 2 + i : r0 + i, cc = trans ? r0 + tx : e0 - 2 + tx;
-                    t[j][i][tx] = (rr >= 0 && rr < N && cc >= 0 && cc < N) ? src[(size_t)rr * N + cc] : 0.0f;
-                }
+            for (int m = 0; m < 4; ++m) {
+                const int r = r0 + ty + 8 * m, c = c0 + tx;
+                x[m][j] = (j < w && r >= 0 && r < N && c >= 0 && c < N) ? src[(size_t)r * N + c] : 0.0f;
             }
         }
-        __syncthreads();
-        float *Q = (trans ? QT : QX) + (size_t)k0 * F * N * Pp;
-#pragma unroll
-        for (int m = 0; m < 4; ++m) {
-            const int i = ty + 8 * m;
-            const int r = r0 + i, e = e0 + tx;
-            if (r >= N || e >= Pp) continue;
-            float v[4];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) v[j] = trans ? t[j][tx][i] : t[j][i][tx];
-            float *q = Q + (((size_t)f * N + r) * Pp + e) * w;
+        auto put = [&](float *Q, int row, int e, const float (&v)[4]) {
+            if (row < 0 || row >= N || e >= Pp) return;
+            float *q = Q + (size_t)k0 * F * N * Pp + (((size_t)f * N + row) * Pp + e) * w;
             if (w == 4)
                 *reinterpret_cast<float4 *>(q) = make_float4(v[0], v[1], v[2], v[3]);
             else if (w == 2)
                 *reinterpret_cast<float2 *>(q) = make_float2(v[0], v[1]);
             else
                 *q = v[0];
+        };
+        __syncthreads();  // the previous group's tile has been read
+#pragma unroll
+        for (int m = 0; m < 4; ++m) {
+            put(QX, r0 + ty + 8 * m, c0 + tx + 2, x[m]);
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                if (j < w) t[j][ty + 8 * m][tx] = x[m][j];
+        }
+        __syncthreads();
+#pragma unroll
+        for (int m = 0; m < 4; ++m) {
+            float v[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) v[j] = t[j][tx][ty + 8 * m];
+            put(QT, c0 + ty + 8 * m, r0 + tx + 2, v);
         }
     }
 }
@@ -820,7 +832,7 @@ cudaError_t launch_pairs_img(const Handle &h, const T *X, int nimg, const int *s
     const ViewPrep p = view_prep_args(h, theta, delta);
     cudaError_t e = allow_prep_smem<k_pairs_img<T>>();
     if (e != cudaSuccess) return e;
-    dim3 grid((h.Pp + 31) / 32, (h.N + 31) / 32, std::max(1, std::min(nimg, 65535)));
+    dim3 grid((h.Pp + 31) / 32, (h.Pp + 31) / 32, std::max(1, std::min(nimg, 65535)));
     grid.x += prep_columns(p, grid);
     launch_chained(k_pairs_img<T>, grid, 256, prep_smem(p), h.stream, X, (pair_t<T> *)h.d_px, (pair_t<T> *)h.d_pt, h.N, h.Pp,
                                                           nimg, p, skip);
@@ -848,7 +860,7 @@ cudaError_t launch_interleave_img(const Handle &h, const float *X, int batch, co
     if (e != cudaSuccess) return e;
     const int n4 = batch & ~3, rem = batch - n4;
     const int ngroups = n4 / 4 + (rem >= 2 ? 1 : 0) + (rem & 1);
-    dim3 grid((h.Pp + 31) / 32, (h.N + 31) / 32, std::max(1, std::min(2 * h.F * ngroups, 65535)));
+    dim3 grid((h.Pp + 31) / 32, (h.Pp + 31) / 32, std::max(1, std::min(h.F * ngroups, 65535)));
     grid.x += prep_columns(p, grid);
     launch_chained(k_interleave_img, grid, 256, prep_smem(p), h.stream, X, h.d_qx, h.d_qt, h.N, h.Pp, h.F, batch, p, skip);
     return cudaGetLastError();
