@@ -317,13 +317,13 @@ __global__ void __launch_bounds__(256, 5) k_pairs_img(const T *__restrict__ X, p
 // of the images of one group, of one frame, from (r0, c0) on (both from -2 in
 // steps of 32), once; a thread has the group's images at its elements side by
 // side and writes them as one vector of w floats to the image of X, and
-// through shared memory to that of X^T.  Bound by memory (16
-// frames of 256^2, 8 images: 100 MB, 15 us at the copy rate): 31 us with a CTA
-// and a read of X per orientation, 20 us so.
+// through shared memory to that of X^T.  Bound by memory (16 frames of 256^2,
+// 8 images: 100 MB, 15 us at the copy rate): 31 us with a CTA and a read of X
+// per orientation, 20 us so.
 // With p.on the last columns of CTAs carry the view-table step, as in k_pairs_img.
 __global__ void __launch_bounds__(256, 5) k_interleave_img(const float *__restrict__ X, float *__restrict__ QX,
-                                                        float *__restrict__ QT, int N, int Pp, int F, int K,
-                                                        ViewPrep p, const int *__restrict__ skip)
+                                                           float *__restrict__ QT, int N, int Pp, int F, int K,
+                                                           ViewPrep p, const int *__restrict__ skip)
 {
     chain_wait();
     extern __shared__ unsigned long long prep_key[];
@@ -430,15 +430,56 @@ __global__ void k_pairs_sino(const double *__restrict__ Y, double2 *__restrict__
     }
 }
 
+// One row of a group of W sinograms, `live` of them given: U bins of every
+// sinogram in flight per thread.  The loads carry no condition (their
+// addresses are clamped into the row, what lies outside is replaced by zero
+// afterwards): with one around each the compiler kept them one after another.
+template <int W, int U>
+__device__ __forceinline__ int interleave_row(const float *__restrict__ in, float *__restrict__ out, long long pitch,
+                                              int live, int B, int Pq)
+{
+    int bad = 0;
+    for (int b0 = threadIdx.x; b0 < Pq; b0 += U * blockDim.x) {
+        float y[U][W];
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+#pragma unroll
+            for (int k = 0; k < W; ++k)
+                y[u][k] = __ldg(in + min(k, live - 1) * pitch + min(b0 + u * (int)blockDim.x, B - 1));
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int b = b0 + u * blockDim.x;
+#pragma unroll
+            for (int k = 0; k < W; ++k) {
+                if (k >= live || b >= B) y[u][k] = 0.0f;
+                bad |= !isfinite(y[u][k]);
+            }
+            if (b >= Pq) continue;
+            float *o = out + (size_t)b * W;
+            if constexpr (W == 1)
+                *o = y[u][0];
+            else if constexpr (W == 2)
+                *reinterpret_cast<float2 *>(o) = make_float2(y[u][0], y[u][1]);
+            else
+#pragma unroll
+                for (int k = 0; k < W; k += 4)
+                    *reinterpret_cast<float4 *>(o + k) = make_float4(y[u][k], y[u][k + 1], y[u][k + 2], y[u][k + 3]);
+        }
+    }
+    return bad;
+}
+
 // FP32: the interleaved sinograms of the transpose (ct_internal.cuh).  A CTA
-// takes rows (group, view): each thread reads its bin of the group's sinograms
-// (coalesced over the bins) and writes them side by side; the row's flag says
-// whether it holds a non-finite value.  With p.on, the first p.on CTAs
-// run the view-table step of the call instead.
-__global__ void __launch_bounds__(256) k_interleave_sino(const float *__restrict__ Y, float *__restrict__ YI,
-                                                         int *__restrict__ rowflag, int B, int Pq, int V, int nsino,
-                                                         int kb, long long rows, ViewPrep p,
-                                                         const int *__restrict__ skip)
+// takes rows (group, view): each thread reads its bins of the group's
+// sinograms (coalesced over the bins) and writes them side by side; the row's
+// flag says whether it holds a non-finite value.  Bound by memory latency
+// (1200 views x 363 bins, 8 sinograms, 28 MB, 4 us at the copy rate: 20 us with a
+// condition around each load, 9 us so; 2901 bins, 120 views, one: 9.5 -> 4.6 us).
+// With p.on, the first p.on CTAs run the view-table step of the call instead.
+__global__ void __launch_bounds__(256, 5) k_interleave_sino(const float *__restrict__ Y, float *__restrict__ YI,
+                                                            int *__restrict__ rowflag, int B, int Pq, int V,
+                                                            int nsino, int kb, long long rows, ViewPrep p,
+                                                            const int *__restrict__ skip)
 {
     chain_wait();
     extern __shared__ unsigned long long prep_key[];
@@ -455,25 +496,13 @@ __global__ void __launch_bounds__(256) k_interleave_sino(const float *__restrict
         while (w < live) w *= 2;
         float *out = YI + ((size_t)k0 * V + (size_t)v * w) * Pq;
         const float *in = Y + ((size_t)k0 * V + v) * B;
+        const long long pitch = (long long)V * B;
         int bad = 0;
-        auto value = [&](int k, int b) {
-            const float y = (k < live && b < B) ? in[(size_t)k * V * B + b] : 0.0f;
-            bad |= !isfinite(y);
-            return y;
-        };
-        for (int b = threadIdx.x; b < Pq; b += blockDim.x) {
-            if (w == 1) {
-                out[b] = value(0, b);
-            } else if (w == 2) {
-                reinterpret_cast<float2 *>(out)[b] = make_float2(value(0, b), value(1, b));
-            } else {
-                float y[8];
-#pragma unroll
-                for (int k = 0; k < 8; ++k) y[k] = k < w ? value(k, b) : 0.0f;
-                float4 *o = reinterpret_cast<float4 *>(out + (size_t)b * w);
-                o[0] = make_float4(y[0], y[1], y[2], y[3]);
-                if (w == 8) o[1] = make_float4(y[4], y[5], y[6], y[7]);
-            }
+        switch (w) {
+        case 1: bad = interleave_row<1, 8>(in, out, pitch, live, B, Pq); break;
+        case 2: bad = interleave_row<2, 4>(in, out, pitch, live, B, Pq); break;
+        case 4: bad = interleave_row<4, 4>(in, out, pitch, live, B, Pq); break;
+        default: bad = interleave_row<8, 2>(in, out, pitch, live, B, Pq); break;
         }
         bad = __syncthreads_or(bad);
         if (threadIdx.x == 0) rowflag[row] = bad;
