@@ -49,8 +49,8 @@ NUM_SMS = 152
 SM_MAX_MHZ_NOMINAL = 2070.0
 
 # DRAM traffic of the dominant kernels per byte of the layout they read (the
-# images' pairs or the interleaved images for the forward, the sinograms' pairs
-# for the transpose):
+# images' pairs or the interleaved images for the forward, the interleaved
+# sinograms for the transpose):
 # ncu's dram__bytes_read.sum + dram__bytes_write.sum of one launch (cold
 # cache) divided by that launch's pair footprint.  The traffic reported for a
 # launch is this ratio times its own footprint (the ray kernels read each pair
@@ -61,8 +61,8 @@ TRAFFIC_PER_FOOTPRINT = {
     "forward_staged": 8.58e6 / (2 * 8 * 256 * 260 * 8),  # k_ray_band
     # k_ray<float, kFwd, ..., interleaved>: 4.30 MB for 4.26 MB of interleaved X and X^T
     "forward_interleaved": 4.30e6 / (2 * 8 * 256 * 260 * 4),
-    "adjoint": 3.95e6 / (8 * 180 * 368 * 8),            # k_adjoint: 3.95 MB for 4.24 MB of sinogram pairs
-    "adjoint_staged": 4.04e6 / (8 * 180 * 368 * 8),      # k_adj_band
+    # k_adj_tile: 1.99 MB for 2.10 MB of interleaved sinograms
+    "adjoint_staged": 1.99e6 / (8 * 180 * 364 * 4),
 }
 
 
@@ -571,19 +571,19 @@ class OperatorStep:
         gather_bytes = 2.0 * esz * K * steps_img
         out = {}
         for name in ("forward", "adjoint"):
-            staged = (t[7] > 0) if name == "forward" else (t[9] > 0)
-            staged = staged and esz == 4
+            # the FP32 transpose above 64^2 reads staged sinograms from shared memory
+            staged = esz == 4 and (w.N > 64 if name == "adjoint" else t[7] > 0)
             # the forward on interleaved images reads one float per pixel and image, not a pair
             inter = name == "forward" and len(t) > 11 and t[11] == 1 and esz == 4
             # the L1-gather forward misses L1 and hits L2; the staged kernels read shared
-            # memory; the L1-gather transpose mostly hits L1, which shares shared memory's data path
+            # memory; the FP64 transpose mostly hits L1, which shares shared memory's data path
             level = "smem" if staged else ("l2" if name == "forward" else "l1")
             pk = l2_gbs if level == "l2" else smem_gbs
             ach = gather_bytes / (kernel_ms[name] * 1e-3) / 1e9
             if name == "forward":
                 footprint = 2.0 * K * w.F * w.N * (w.N + 4) * (1 if inter else 2) * esz
             else:
-                footprint = float(K * w.V * ((w.B + 5) & ~1) * 2 * esz)
+                footprint = float(K * w.V * (((w.B + 3) & ~3) * esz if staged else ((w.B + 5) & ~1) * 2 * esz))
             fam = name + ("_staged" if staged else ("_interleaved" if inter else ""))
             ratio = TRAFFIC_PER_FOOTPRINT.get(fam) if esz == 4 else None
             out[name] = {"level": level, "achieved": ach, "peak": pk, "unit": "GB/s", "frac": ach / pk,

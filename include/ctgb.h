@@ -87,8 +87,9 @@ typedef struct ct_handle ct_handle;
  * Create a handle: copies the geometry, allocates the workspaces it needs
  * on the current device (per-view tables; zero-padded "pair" copies of
  * max_batch images, of their transposes and of max_batch sinograms, about
- * 4 x 8 bytes per pixel and 8 bytes per sample and image in float32; the
- * reduction partials) and binds it to cuda_stream (a cudaStream_t; NULL =
+ * 4 x 8 bytes per pixel and 8 bytes per sample and image in float32, and 8
+ * bytes per pixel more for the interleaved images of handles that start with
+ * them, see ct_set_tuning; the reduction partials) and binds it to cuda_stream (a cudaStream_t; NULL =
  * legacy default stream).  *out receives the handle.
  */
 int ct_init(const ct_geom *g, void *cuda_stream, ct_handle **out);
@@ -104,9 +105,10 @@ void ct_destroy(ct_handle *h);
  *
  * Image reuse (this call, ct_jac, ct_jacT, ct_gn_terms and the batched
  * forms): every call that takes images lays them out in the handle (pairs
- * of neighbouring pixels along rows and along columns; for this call, with
- * tuning value [11] = 1 on an FP32 parallel-beam handle, the images
- * interleaved in groups of 4 instead, see ct_set_tuning).  Passing X (x) =
+ * of neighbouring pixels along rows and along columns; with tuning value
+ * [11] = 1 on an FP32 parallel-beam handle, batches of two or more of this
+ * call and of the unstaged batched Jacobian products are interleaved in
+ * groups of 4 instead, see ct_set_tuning).  Passing X (x) =
  * NULL uses the layouts of the previous such call on the handle again,
  * i.e. that call's first `batch` images, at this call's angles and offsets:
  * the Jacobian and its transpose at one image (a Gauss-Newton step, an
@@ -260,7 +262,9 @@ int ct_autotune(ct_handle *h);
  *   images interleaved in groups of 4 (FP32 parallel-beam handles, forward
  *   staging 0, [0] 4 or 8; the forward then reads both taps of 4 images with
  *   two 16-byte loads; a later call that passes X = NULL to a Jacobian
- *   product converts them to pair images first).  Layout 1 allocates two
+ *   product converts them to pair images first).  1 is what FP32
+ *   parallel-beam handles with [0] of 4 or 8 start with, where the memory is
+ *   there.  Layout 1 allocates two
  *   buffers of max_batch x n_frames x N x (N + 4) floats the first time
  *   (CT_ERR_OOM if that fails; CT_ERR_ARG on an FP64 or fan-beam handle).
  * [0]..[6] are powers of two, at most 8 (view groups at most 4), warps per
