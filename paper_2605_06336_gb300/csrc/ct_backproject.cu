@@ -37,6 +37,13 @@ namespace {
 
 namespace cg = cooperative_groups;
 
+// A tile's first bin from a 64-bit cell.  A view shifted far off the detector
+// stays off it: cells beyond 32 bits are held short of their range (with room
+// for the in-tile offset), not wrapped back onto the bins.
+__device__ __forceinline__ int far_cell(long long cell)
+{
+    return (int)max(min(cell, 0x7fff0000LL), -0x7fff0000LL);
+}
 
 // ---------------------------------------------------------------------------
 // FP32
@@ -293,7 +300,7 @@ __global__ void __launch_bounds__(256, KB <= 2 ? 6 : 0) k_adj_tile(AdjArgs a)
                 // bin coordinate of the anchor pixel, the only FP64 step per tile and view
                 const double bt = g.beta0 + (double)(j0 + kAdjTile / 2) * g.c - (double)(i0 + kAdjTile / 2) * g.s;
                 const long long fx = __double2ll_rn(bt * (double)(1 << kAdjFrac));
-                const int ix = (int)(fx >> kAdjFrac);
+                const int ix = far_cell(fx >> kAdjFrac);
                 const int frac = (int)(fx & ((1 << kAdjFrac) - 1));
                 const float w = GeoT<float>::w(g);
                 AdjView av;
@@ -481,7 +488,7 @@ __global__ void __launch_bounds__(256) k_adj64(Adj64Args a)
                 av.w2 = w * w;
                 av.wa = w + av.w2;
                 av.wb = w - 2.0 * av.w2;
-                av.ix = (int)fl + 2;
+                av.ix = far_cell((long long)fl) + 2;
                 av.row = v * a.Pb;
                 s_view[q] = av;
             }
@@ -635,7 +642,7 @@ __global__ void __launch_bounds__(32 * kSmallWarps) k_adj_small(SmallArgs<T> a)
                 s_w[q] = GeoT<T>::w(g);
                 s_w1[q] = T(1) - s_w[q];
                 s_f[q] = (T)(bt - fl);
-                s_idx[q] = make_int2((int)fl, vs + base + q);
+                s_idx[q] = make_int2(far_cell((long long)fl), vs + base + q);
             }
             __syncthreads();
             for (int blk = 0; blk < nv; blk += kSmallViews) {

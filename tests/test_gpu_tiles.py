@@ -96,6 +96,23 @@ def test_transpose_keeps_a_non_finite_sample_to_its_pixels(K):
     assert np.abs(got[k][far] - ref[k][far]).max() <= 1e-4
 
 
+@pytest.mark.parametrize("dtype", [torch.float32, torch.float64])
+@pytest.mark.parametrize("K", [1, 2, 8])
+@pytest.mark.parametrize("N", [40, 70])
+def test_transpose_of_views_shifted_off_the_detector(N, K, dtype):
+    """Offsets beyond 32-bit bin numbers, and beyond 64-bit fixed point: such a view adds nothing."""
+    far = [2.0 ** 31 + 3, -(2.0 ** 32) + 5.5, 2.0 ** 32 - 9.25, 3e9, 1e12, -1e12, 1e300, -1e300]
+    V = len(far) + 4
+    op, g, theta, delta, _, Y, _ = _setup(N, synth.n_bins(N), [V], K, dtype, 3 * N + K)
+    Y = Y.reshape(K, V, g.B)
+    zeroed = Y.copy()
+    zeroed[:, :len(far)] = 0.0
+    ref = oracle.adjoint(g, theta, zeroed.reshape(K, -1), delta)
+    delta[:len(far)] = far
+    got = host(op.adjoint(dev(Y.reshape(K, -1), dtype), dev(theta), dev(delta)))
+    assert rel(got, ref) <= TOL[dtype]
+
+
 # N, views, batch: the order of the views (counted, sorted, none) and the CTAs of the view table
 VIEWS = [(16, 255, 1), (16, 256, 2), (16, 257, 1), (8, 512, 1), (8, 513, 4), (8, 1200, 1), (8, 4096, 1), (8, 4097, 2)]
 
