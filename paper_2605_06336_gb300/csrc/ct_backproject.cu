@@ -425,7 +425,7 @@ struct Adj64Args {
     int N, B, F, tps, Pb;
     const double2 *YP;         // pair sinograms
     long long ysino_stride;    // pairs per batch element (V * Pb)
-    int kbase, ngroups;
+    int kbase, ngroups, kend;
     double *X;
     long long img_stride;
     int segs;
@@ -543,7 +543,8 @@ __global__ void __launch_bounds__(256) k_adj64(Adj64Args a)
             }
             const int k = u >> 8, p = u & 255;
             const int i = i0 + p / kTile, j = j0 + p % kTile;
-            if (i < N && j < N) a.X[(size_t)(k0 + k) * a.img_stride + (size_t)f * N * N + (size_t)i * N + j] = s;
+            if (i < N && j < N && k0 + k < a.kend)
+                a.X[(size_t)(k0 + k) * a.img_stride + (size_t)f * N * N + (size_t)i * N + j] = s;
         }
         if (segs > 1) cl.sync();
         else __syncthreads();  // red[] is rewritten by the next item
@@ -780,6 +781,8 @@ cudaError_t adjoint32(const Handle &h, float *X, int batch, int kb, int split, i
     a.skip = skip;
     SinoGroup g[2];
     const int ng = sino_groups(layout_batch, kb, g);
+    // (the form and the CTAs per tile follow the laid-out batch: the first sinograms
+    // of a larger one get the bits they got in its own product)
     for (int q = 0; q < ng; ++q) {
         if (g[q].k0 >= batch) break;
         a.kbase = g[q].k0;
@@ -788,7 +791,7 @@ cudaError_t adjoint32(const Handle &h, float *X, int batch, int kb, int split, i
         a.YI = (const float *)h.d_yp + (size_t)g[q].k0 * h.V * a.Pq;
         a.rowflag = h.d_rowflag + (size_t)g[q].first * h.V;
         cudaError_t e;
-        if (small_image(h, a.ngroups)) {
+        if (small_image(h, g[q].count)) {
             SmallArgs<float> b = small_args<float>(h, X, a.kbase, a.ngroups, batch, skip);
             b.Y = a.YI;
             b.pitch = a.Pq;
@@ -797,7 +800,7 @@ cudaError_t adjoint32(const Handle &h, float *X, int batch, int kb, int split, i
             if (e != cudaSuccess) return e;
             continue;
         }
-        a.segs = adj_segs(h, (long long)a.ngroups * h.F * a.tps * a.tps, split, 8);
+        a.segs = adj_segs(h, (long long)g[q].count * h.F * a.tps * a.tps, split, 8);
         switch (g[q].width) {
         case 1: e = launch_cluster(k_adj_tile<1>, a, h, adj_smem<1>(true)); break;
         case 2: e = launch_cluster(k_adj_tile<2>, a, h, adj_smem<2>(true)); break;
@@ -809,7 +812,7 @@ cudaError_t adjoint32(const Handle &h, float *X, int batch, int kb, int split, i
     return cudaSuccess;
 }
 
-cudaError_t adjoint64(const Handle &h, double *X, int batch, int kb, int split, const int *skip)
+cudaError_t adjoint64(const Handle &h, double *X, int batch, int kb, int split, int layout_batch, const int *skip)
 {
     Adj64Args a{};
     a.vg = h.d_views;
@@ -824,17 +827,19 @@ cudaError_t adjoint64(const Handle &h, double *X, int batch, int kb, int split, 
     a.ysino_stride = (long long)h.V * h.Pb;
     a.X = X;
     a.img_stride = (long long)h.F * h.N * h.N;
+    a.kend = batch;
     a.skip = skip;
     int k = 0;
-    for (int width : {8, 4, 2, 1}) {
+    for (int width : {8, 4, 2, 1}) {  // the groups of the laid-out batch, as in adjoint32
         if (width > kb) continue;
-        const int groups = (batch - k) / width;
+        if (k >= batch) break;
+        const int groups = (layout_batch - k) / width;
         if (groups == 0) continue;
         a.kbase = k;
-        a.ngroups = groups;
+        a.ngroups = std::min(groups, (batch - k + width - 1) / width);
         cudaError_t e;
         if (small_image(h, groups)) {
-            SmallArgs<double> b = small_args<double>(h, X, k, groups, batch, skip);
+            SmallArgs<double> b = small_args<double>(h, X, k, a.ngroups, batch, skip);
             b.Y = (const double *)h.d_yp;
             b.pitch = h.Pb;
             b.group_stride = a.ysino_stride;
@@ -861,9 +866,9 @@ cudaError_t adjoint64(const Handle &h, double *X, int batch, int kb, int split, 
 template <typename T>
 cudaError_t launch_adjoint(const Handle &h, T *X, int batch, int kb, int split, int layout_batch, const int *skip)
 {
-    if (h.fan_D > 0.0) return launch_fan_adjoint<T>(h, X, batch, kb, split, skip);
+    if (h.fan_D > 0.0) return launch_fan_adjoint<T>(h, X, batch, kb, split, layout_batch, skip);
     if constexpr (std::is_same<T, float>::value) return adjoint32(h, X, batch, kb, split, layout_batch, skip);
-    else return adjoint64(h, X, batch, kb, split, skip);
+    else return adjoint64(h, X, batch, kb, split, layout_batch, skip);
 }
 
 template cudaError_t launch_adjoint<float>(const Handle &, float *, int, int, int, int, const int *);

@@ -359,7 +359,7 @@ struct FanTileArgs {
     int N, B, F, tps;
     const float *YI;             // [k / 8][V][B][8]
     long long yi_stride;         // floats per block of 8 sinograms
-    int kbase, ngroups;
+    int kbase, ngroups, kend;
     float *X;
     long long img_stride;
     int segs;
@@ -602,7 +602,8 @@ __global__ void __launch_bounds__(256) k_adj_fan_tile(FanTileArgs a)
             }
             const int k = u >> 8, p = u & 255;
             const int i = ic - kTile / 2 + p / kTile, j = jc - kTile / 2 + p % kTile;
-            if (i < N && j < N) a.X[(size_t)(k0 + k) * a.img_stride + (size_t)f * N * N + (size_t)i * N + j] = s;
+            if (i < N && j < N && k0 + k < a.kend)
+                a.X[(size_t)(k0 + k) * a.img_stride + (size_t)f * N * N + (size_t)i * N + j] = s;
         }
         if (segs > 1) cl.sync();
         else __syncthreads();
@@ -808,7 +809,7 @@ cudaError_t run_fan_ray(const Handle &h, const RayArgs<T> &a, int mode, int kb, 
 
 // kb: sinograms per thread (the candidate search of a pixel and view is
 // shared by them); split: thread groups per pixel (view subsets).
-cudaError_t fan_adjoint32(const Handle &h, float *X, int batch, int kb, int split, const int *skip)
+cudaError_t fan_adjoint32(const Handle &h, float *X, int batch, int kb, int split, int layout_batch, const int *skip)
 {
     FanTileArgs a{};
     a.lines = fan_lines<float>(h.d_rays, (long long)h.V * h.B);
@@ -823,14 +824,16 @@ cudaError_t fan_adjoint32(const Handle &h, float *X, int batch, int kb, int spli
     a.yi_stride = 8LL * h.V * h.B;
     a.X = X;
     a.img_stride = (long long)h.F * h.N * h.N;
+    a.kend = batch;
     a.skip = skip;
     int k = 0;
-    for (int width : {8, 4, 2, 1}) {
+    for (int width : {8, 4, 2, 1}) {  // the groups of the laid-out batch
         if (width > kb) continue;
-        const int groups = (batch - k) / width;
+        if (k >= batch) break;
+        const int groups = (layout_batch - k) / width;
         if (groups == 0) continue;
         a.kbase = k;
-        a.ngroups = groups;
+        a.ngroups = std::min(groups, (batch - k + width - 1) / width);
         a.segs = adj_segs(h, (long long)groups * h.F * a.tps * a.tps, split, 8);
         cudaError_t e;
         switch (width) {
@@ -846,10 +849,10 @@ cudaError_t fan_adjoint32(const Handle &h, float *X, int batch, int kb, int spli
 }
 
 template <typename T>
-cudaError_t launch_fan_adjoint(const Handle &h, T *X, int batch, int kb, int split, const int *skip)
+cudaError_t launch_fan_adjoint(const Handle &h, T *X, int batch, int kb, int split, int layout_batch, const int *skip)
 {
     if constexpr (std::is_same<T, float>::value) {
-        return fan_adjoint32(h, X, batch, kb, split, skip);
+        return fan_adjoint32(h, X, batch, kb, split, layout_batch, skip);
     } else {
         AdjFanArgs a{};
         a.fstart = h.d_fstart;
@@ -896,7 +899,7 @@ template cudaError_t launch_fan_sino<float>(const Handle &, const float *, int, 
 template cudaError_t launch_fan_sino<double>(const Handle &, const double *, int, const int *);
 template cudaError_t run_fan_ray<float>(const Handle &, const RayArgs<float> &, int, int, int, bool);
 template cudaError_t run_fan_ray<double>(const Handle &, const RayArgs<double> &, int, int, int, bool);
-template cudaError_t launch_fan_adjoint<float>(const Handle &, float *, int, int, int, const int *);
-template cudaError_t launch_fan_adjoint<double>(const Handle &, double *, int, int, int, const int *);
+template cudaError_t launch_fan_adjoint<float>(const Handle &, float *, int, int, int, int, const int *);
+template cudaError_t launch_fan_adjoint<double>(const Handle &, double *, int, int, int, int, const int *);
 
 }  // namespace ctgb

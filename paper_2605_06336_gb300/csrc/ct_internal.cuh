@@ -220,7 +220,8 @@ cudaError_t launch_interleaved_to_pairs(const Handle &h, int batch);
 template <typename T>
 cudaError_t launch_forward(const Handle &h, T *Y, int batch, int kb, int split, int vw, int stage,
                            const int *skip = nullptr, bool interleaved = false, int layout_batch = 0);
-// The first `batch` of the layout_batch sinograms laid out at kb per group.
+// The first `batch` of the layout_batch sinograms laid out at kb per group,
+// with the bits that a product of all layout_batch gives them.
 template <typename T>
 cudaError_t launch_adjoint(const Handle &h, T *X, int batch, int kb, int split, int layout_batch,
                            const int *skip = nullptr);
@@ -257,6 +258,7 @@ size_t fan_view_bytes();
 template <typename T> cudaError_t launch_fan_sino(const Handle &h, const T *Y, int nsino, const int *skip);
 cudaError_t launch_fan_rays(const Handle &h, const int *skip);
 template <typename T>
-cudaError_t launch_fan_adjoint(const Handle &h, T *X, int batch, int kb, int split, const int *skip);
+cudaError_t launch_fan_adjoint(const Handle &h, T *X, int batch, int kb, int split, int layout_batch,
+                               const int *skip);
 
 }  // namespace ctgb

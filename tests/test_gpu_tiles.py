@@ -113,6 +113,27 @@ def test_transpose_of_views_shifted_off_the_detector(N, K, dtype):
     assert rel(got, ref) <= TOL[dtype]
 
 
+# N, views, laid-out batch, repeated batches: other numbers of tiles, groups cut, groups left out
+REPEAT = [(256, 180, 16, [1, 8, 11, 15]), (130, 90, 9, [3, 8, 9]), (64, 30, 40, [2, 8, 33]), (97, 40, 7, [1, 4, 6])]
+
+
+@pytest.mark.parametrize("fan", [False, True])
+@pytest.mark.parametrize("dtype", [torch.float32, torch.float64])
+@pytest.mark.parametrize("case", REPEAT, ids=lambda c: f"N{c[0]}_K{c[2]}")
+def test_repeated_transpose_of_fewer_sinograms_gives_the_same_bits(case, dtype, fan):
+    from paper_2605_06336_gb300 import ct
+    N, V, K, fewer = case
+    rng = np.random.default_rng(N)
+    op = ct.CTOperator(N, synth.n_bins(N), V, max_batch=K, dtype=dtype, source_distance=2.0 * N if fan else None)
+    Y = dev(rng.standard_normal((K, op.m)), dtype)
+    whole = op.adjoint(Y, dev(rng.uniform(0, np.pi, V))).clone()
+    for k in fewer:
+        X = torch.zeros_like(whole)
+        ct.ct_adjoint_repeat(op.h, X, k)
+        assert torch.equal(X[:k], whole[:k]), k
+        assert not X[k:].any(), k
+
+
 # N, views, batch: the order of the views (counted, sorted, none) and the CTAs of the view table
 VIEWS = [(16, 255, 1), (16, 256, 2), (16, 257, 1), (8, 512, 1), (8, 513, 4), (8, 1200, 1), (8, 4096, 1), (8, 4097, 2)]
 
