@@ -350,7 +350,7 @@ __global__ void k_fan_sino(const T *__restrict__ Y, T *__restrict__ YI, long lon
 constexpr int kFanWin = 64;      // rays of a view staged at a time
 constexpr int kFanVB = 4;        // views per staged block: one staged ray per thread
 constexpr int kFanCap = 128;     // views whose tile constants are staged at a time
-constexpr int kFanFrac = 25;     // fractional bits of a ray's in-tile coordinate
+constexpr int kFanLow = kFracBits - 23;  // bits of a line's fraction below those of the forward's
 
 struct FanTileArgs {
     const FanLine<float> *lines;
@@ -373,11 +373,11 @@ struct __align__(16) FanTileView {
 };
 
 // A ray near the tile: its coordinate at the tile's centre row (column, for
-// column-marched rays) relative to the centre pixel, its slope, its weight.
+// column-marched rays) relative to the centre pixel and its slope, each as the
+// part above the last kFanLow bits and those bits: all 48 bits of the line's
+// fraction in 32-bit words, so that the sum at any row of the tile is exact.
 struct __align__(16) FanTileRay {
-    int P, S;
-    float w;
-    int pad;
+    int ph, pl, sh, sl;
 };
 
 template <int KB> struct FanSums {
@@ -423,10 +423,11 @@ template <> struct FanSums<8> : FanSumsPacked<8> {};
 // took 250 instructions per warp and view, waiting on loads (152 us for 256^2 /
 // 180 views, 8 sinograms).  Here the rays that can touch the tile (between the
 // projections of the corners of its one-pixel neighbourhood) are staged once
-// per tile and view with their lines reduced to 32-bit in-tile coordinates
-// (from the table's fixed-point line, to 2^-25 pixel: closer than the forward's
-// 23-bit fractions), their sinogram bins beside them; the next block's lines
-// are loaded and its bins copied while the current one is read: 92 us.
+// per tile and view with their lines relative to its centre, their sinogram
+// bins beside them; the next block's lines are loaded and its bins copied while
+// the current one is read: 99 us.  The staged lines keep every bit, so the
+// cell, the fraction and the weight are the forward's own (with 25 bits of
+// fraction kept instead of 48: 92 us, weights up to 2^-23 off).
 template <int KB>
 __global__ void __launch_bounds__(256) k_adj_fan_tile(FanTileArgs a)
 {
@@ -434,6 +435,7 @@ __global__ void __launch_bounds__(256) k_adj_fan_tile(FanTileArgs a)
     namespace cg = cooperative_groups;
     __shared__ FanTileView s_view[kFanCap];
     __shared__ FanTileRay s_ray[2][kFanVB][kFanWin];
+    __shared__ float s_w[2][kFanVB][kFanWin];
     // (8 sinograms as two arrays of 4, so that a quarter-warp's 16-byte loads meet no bank twice)
     constexpr int W = KB >= 4 ? 4 : KB;
     __shared__ __align__(16) float s_y[2][kFanVB][KB / W][kFanWin][W];
@@ -446,7 +448,7 @@ __global__ void __launch_bounds__(256) k_adj_fan_tile(FanTileArgs a)
     const int total = a.ngroups * a.F * tiles * segs;
     const int N = a.N;
     const float h = 0.5f * (float)(N - 1);
-    const int one = 1 << kFanFrac;
+    constexpr int one = 1 << (kFracBits - kFanLow), low = (1 << kFanLow) - 1;
     if (a.skip && *a.skip) return;
     for (int item = blockIdx.x; item < total; item += gridDim.x) {  // whole clusters
         const int seg = item % segs;
@@ -526,13 +528,15 @@ __global__ void __launch_bounds__(256) k_adj_fan_tile(FanTileArgs a)
                 const int r = mode ? jc : ic, m = mode ? ic : jc;
                 const long long Q = line.Qc + (long long)(2 * r - (N - 1)) * line.Qh - ((long long)m << kFracBits);
                 // rays that pass the tile at a distance are held at 20 pixels, out of reach of its pixels
-                const long long far = 20LL << kFanFrac;
+                const long long far = 20LL << kFracBits;
+                const long long P = min(max(Q, -far), far), S = 2 * line.Qh;
                 FanTileRay R;
-                R.P = (int)min(max((Q + (1LL << (kFracBits - kFanFrac - 1))) >> (kFracBits - kFanFrac), -far), far);
-                R.S = (int)((2 * line.Qh + (1LL << (kFracBits - kFanFrac - 1))) >> (kFracBits - kFanFrac));
-                R.w = line.w;
-                R.pad = 0;
+                R.ph = (int)(P >> kFanLow);
+                R.pl = (int)P & low;
+                R.sh = (int)(S >> kFanLow);
+                R.sl = (int)S & low;
                 s_ray[buf][sq][sr] = R;
+                s_w[buf][sq][sr] = line.w;
             };
             const int nu = nblk * nwin;
             if (nu > 0) fetch(0, 0);
@@ -567,10 +571,12 @@ __global__ void __launch_bounds__(256) k_adj_fan_tile(FanTileArgs a)
                         const int along = pass == 0 ? ty : tx, across = (pass == 0 ? tx : ty) * one;
                         for (int b = blo; b <= bhi; ++b) {
                             const FanTileRay R = s_ray[buf][qq][b - wlo];
-                            const int d = abs(R.P + along * R.S - across);
-                            if (d < one) {
-                                const float g = __int_as_float((d >> (kFanFrac - 23)) | 0x3F800000);  // 1 + distance
-                                acc.add(R.w * (2.0f - g), &s_y[buf][qq][0][b - wlo][0]);
+                            // the ray's coordinate relative to the pixel, rounded down to 23 bits of fraction:
+                            // exact, as |pl + along * sl| < 2^29 and |ph + along * sh| < 2^29
+                            const int t = R.ph + along * R.sh + ((R.pl + along * R.sl) >> kFanLow) - across;
+                            if (abs(t) < one) {  // (at -1 pixel the weight is 0)
+                                const float g = __int_as_float(abs(t) | 0x3F800000);  // 1 + distance
+                                acc.add(s_w[buf][qq][b - wlo] * (2.0f - g), &s_y[buf][qq][0][b - wlo][0]);
                             }
                         }
                     }

@@ -260,3 +260,21 @@ def test_fan_image_reuse_with_null_x():
     op.forward(Xd, th1)
     assert torch.equal(op.forward(None, th2, dl, batch=2), y_ref)
     op.close()
+
+
+@pytest.mark.parametrize("N,kind", [(16, "near"), (33, "near"), (40, "far")])
+def test_fp32_transpose_holds_the_forwards_own_entries(N, kind):
+    """The columns of the FP32 forward (a pixel each) and the rows of its transpose (a bin each)
+    hold the same bits: a ray samples a pixel in one row or column, so each entry is one rounded weight."""
+    from paper_2605_06336_gb300 import ct
+    B, V = synth.n_bins(N), 5
+    D = 0.75 * max(N, B) + 2.5 if kind == "near" else 40.0 * N
+    rng = np.random.default_rng(N)
+    theta = dev(rng.uniform(-np.pi, np.pi, V))
+    delta = dev(rng.normal(0, 0.6, V))
+    op = ct.CTOperator(N, B, V, max_batch=64, dtype=torch.float32, source_distance=D)
+    n, m = op.n, op.m
+    H = torch.cat([op.forward(torch.eye(n, device="cuda")[k:k + 64].contiguous(), theta, delta) for k in range(0, n, 64)])
+    Ht = torch.cat([op.adjoint(torch.eye(m, device="cuda")[k:k + 64].contiguous(), theta, delta) for k in range(0, m, 64)])
+    assert int((H != 0).sum()) > m
+    assert torch.equal(H, Ht.T)
