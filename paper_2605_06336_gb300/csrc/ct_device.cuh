@@ -211,7 +211,9 @@ __device__ __forceinline__ void warp_rows(const ViewGeo &g, int b, bool active, 
 // two-word shift, two clamps and a second shift (the integer pipe was the bound
 // of one image per lane: 74 % busy, now 58).  The same bits as cell_of and
 // frac_of.  One image of 2048^2, 120 views: 362 -> 282 us; 256^2 / 180 views:
-// 18.6 -> 16.3.
+// 18.6 -> 16.3.  FP64: the indices alone; ray_frac gives a row's fraction when
+// its sum is formed (an FP64 subtraction, not to be spent on the rows past a
+// segment's end).
 template <typename T, int U>
 __device__ __forceinline__ void ray_cells(long long Q, long long dQ, unsigned lim, unsigned (&idx)[U], T (&f)[U])
 {
@@ -229,11 +231,16 @@ __device__ __forceinline__ void ray_cells(long long Q, long long dQ, unsigned li
     } else {
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            const long long Qu = Q + (long long)u * dQ;
-            idx[u] = min((unsigned)(cell_of(Qu) + 2), lim);
-            f[u] = frac_of(Qu, T());
+            idx[u] = min((unsigned)(cell_of(Q + (long long)u * dQ) + 2), lim);
         }
     }
+}
+// Fraction of row u of the block.
+template <typename T, int U>
+__device__ __forceinline__ T ray_frac(long long Q, long long dQ, const T (&f)[U], int u)
+{
+    if constexpr (std::is_same<T, float>::value) return f[u];
+    else return frac_of(Q + (long long)u * dQ, T());
 }
 
 // Per-ray output of a march: the forward stores w * sum for each image, the

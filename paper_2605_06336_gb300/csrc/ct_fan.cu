@@ -183,6 +183,7 @@ __global__ void __launch_bounds__(32 * SPLIT) k_ray_fan(RayArgs<T> a, const FanR
 {
     chain_wait();
     using P2 = pair_t<T>;
+    constexpr bool F32 = std::is_same<T, float>::value;
     constexpr int NACC = (MODE == kFwd) ? KB : (OFFS ? 3 : 2);
     __shared__ T red[SPLIT > 1 ? SPLIT : 1][NACC][32];
     const int lane = threadIdx.x & 31;
@@ -231,15 +232,17 @@ __global__ void __launch_bounds__(32 * SPLIT) k_ray_fan(RayArgs<T> a, const FanR
             }
 #pragma unroll
             for (int u = 0; u < U; ++u) {
+                if (!F32 && !WHOLE && u >= rows) break;  // FP64 products are dear (uniform)
+                const T fu = ray_frac<T, U>(Q, dQ, f, u);
                 if constexpr (MODE == kFwd) {
-                    const T omf = T(1) - f[u];
+                    const T omf = T(1) - fu;
 #pragma unroll
-                    for (int k = 0; k < KB; ++k) acc[k] = fma(omf, p[u][k].x, fma(f[u], p[u][k].y, acc[k]));
+                    for (int k = 0; k < KB; ++k) acc[k] = fma(omf, p[u][k].x, fma(fu, p[u][k].y, acc[k]));
                 } else {
                     // acc[0] = sum of interpolated values, acc[1] = sum slope * dq/dtheta,
                     // acc[2] (offsets) = sum slope * dq/ddelta
                     const T d = p[u][0].y - p[u][0].x;
-                    acc[0] += fma(f[u], d, p[u][0].x);
+                    acc[0] += fma(fu, d, p[u][0].x);
                     acc[1] = fma(d, fma((T)(r + u), R.gr, R.g0), acc[1]);
                     if constexpr (OFFS) acc[NACC - 1] = fma(d, fma((T)(r + u), R.sr, R.s0), acc[NACC - 1]);
                 }
