@@ -243,10 +243,13 @@ void default_tuning(ctgb::Handle &h)
     h.tune.fwd_vw = 2;
     if (h.precision) {
         // the FP64 pipe is the bound: no warp waits for its neighbours, and finer segments
-        // even out the rays (255^2, 181 views, 4 images: 278 -> 255 us); small images keep
-        // theirs (and with them the order of their sums)
+        // even out the rays (255^2, 181 views, 4 images: 278 -> 255 us).  From 128 rows on, or
+        // where 4 segments leave SMs without a warp: shorter ones lose more in their last
+        // rows (96^2, 90 views, 2 images: 20.2 us with 4 segments, 23.9 with 8; 22 views:
+        // 10.8 and 10.2; 128^2, 180 views: 53.6 and 53.2).  Small images keep theirs (and
+        // with them the order of their sums)
         h.tune.fwd_vw = 1;
-        if (h.N > 64 && rays < 16LL * h.num_sms) h.tune.fwd_split = 8;
+        if (h.N > 64 && rays < (h.N >= 128 ? 16LL : 1LL) * h.num_sms) h.tune.fwd_split = 8;
     }
     h.tune.der_vw = rays >= 32LL * h.num_sms ? 2 : 1;
     h.tune.der_kb = std::min(kb, 4);
