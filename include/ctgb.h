@@ -252,8 +252,9 @@ int ct_autotune(ct_handle *h);
  *   [0] forward images per lane, [1] forward warps per ray (row segments),
  *   [2] forward views per CTA, [3] transpose sinograms per thread,
  *   [4] least number of CTAs (view subsets) per transpose pixel tile (the
- *   launch takes more, up to 8, where the tiles alone leave SMs idle; for the
- *   fan beam and for images of side up to 64, thread groups of a CTA),
+ *   launch takes more, up to 8, where the tiles alone leave SMs idle, and 2
+ *   instead of 4 where 4 would leave a CTA fewer than 8 views; for images of
+ *   side up to 64 and for the FP64 fan beam, thread groups of a CTA),
  *   [5] Jacobian warps per ray, [6] Jacobian views per CTA, [7] forward
  *   staging, [8] Jacobian staging, [9] 0, 8 or 16 (kept with the shape; the
  *   transpose has one form), [10] images per lane of the batched Jacobian

@@ -366,32 +366,10 @@ inline int persistent_grid(K kernel, int threads, size_t smem, long long work_bl
 // ---------------------------------------------------------------------------
 // transpose kernels (ct_backproject.cu, ct_fan.cu)
 // ---------------------------------------------------------------------------
-constexpr int kMaxSegs = 8;  // CTAs per tile: the portable cluster size
-
-// CTAs per tile: at least `split` (the launch shape), at most kMaxSegs, such
-// that the SM with most CTAs has least to do: ceil(tiles * segs / SMs) CTAs of
-// (views / segs) views plus `fixed` views' worth of prologue and epilogue
-// each (8 in FP32; 3 in FP64, whose views take longer); an SM with one CTA does not hide its latency and counts as two.  More
-// than 2 CTAs only where each keeps 8 views: below that the prologue is all
-// there is (64^2, 22 views: 6.1 us at any size).
-// Clusters of odd size measured slower (256^2, 180 views, 8 sinograms: 30.7 us
-// at 4 or 6, 34.8 at 5 and 34.9 at 7; one CTA per tile 65.5).
+// CTAs per tile of a frame's views (adj_cluster_size in ct_internal.cuh)
 inline int adj_segs(const Handle &h, long long tiles, int split, int fixed)
 {
-    const int views = std::max(1, h.V / h.F);
-    int best = 1;
-    double best_cost = 1e300;
-    for (int segs : {1, 2, 4, 6, 8}) {
-        if (segs < split) continue;
-        if (segs > 2 && views < 8 * segs) break;
-        const long long ctas = std::max<long long>(2, (tiles * segs + h.num_sms - 1) / h.num_sms);
-        const double cost = (double)ctas * ((views + segs - 1) / segs + fixed);
-        if (cost < best_cost) {
-            best_cost = cost;
-            best = segs;
-        }
-    }
-    return best;
+    return adj_cluster_size(std::max(1, h.V / h.F), tiles, h.num_sms, split, fixed);
 }
 
 // Launch of a transpose kernel: 256 threads, the a.segs CTAs of a tile one cluster.

@@ -142,6 +142,36 @@ inline int sino_groups(int batch, int kb, SinoGroup *g)
 }
 inline int sino_pitch(int B) { return (B + 3) & ~3; }
 
+// CTAs per tile of the tiled transposes: at least `split` (the launch shape) as
+// far as each keeps 8 views, else at least 2 of them where 2 are asked for; at
+// most kMaxSegs; such that the SM with most CTAs has least to do:
+// ceil(tiles * segs / SMs) CTAs of (views / segs) views plus `fixed` views'
+// worth of prologue and epilogue each (8 in FP32; 3 in FP64, whose views take
+// longer); an SM with one CTA does not hide its latency and counts as two.  More
+// than 2 CTAs only where each keeps 8 views: below that the prologue is all
+// there is (64^2, 22 views: 6.1 us at any size).
+// Clusters of odd size measured slower (256^2, 180 views, 8 sinograms: 30.7 us
+// at 4 or 6, 34.8 at 5 and 34.9 at 7; one CTA per tile 65.5).
+constexpr int kMaxSegs = 8;  // the portable cluster size
+inline int adj_cluster_size(int views, long long tiles, int num_sms, int split, int fixed)
+{
+    const int least = views < 8 * split && split > 2 ? 2 : split;
+    int best = least;
+    double best_cost = 1e300;
+    for (int segs : {1, 2, 4, 6, 8}) {
+        if (segs < least) continue;
+        if (segs > 2 && views < 8 * segs) break;
+        long long ctas = (tiles * segs + num_sms - 1) / num_sms;
+        if (ctas < 2) ctas = 2;
+        const double cost = (double)ctas * ((views + segs - 1) / segs + fixed);
+        if (cost < best_cost) {
+            best_cost = cost;
+            best = segs;
+        }
+    }
+    return best;
+}
+
 struct Handle {
     int N = 0, B = 0, V = 0, F = 1, max_batch = 1, precision = 0, device = 0;
     int Pp = 0, Pb = 0;  // pair pitches

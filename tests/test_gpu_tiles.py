@@ -49,7 +49,9 @@ TRANSPOSE = [
     (2, None, [3], 1), (16, None, [5], 2), (33, 21, [7], 4), (63, None, [9, 0, 4], 3), (64, None, [30], 1),
     (64, 91, [12, 5], 8),                      # up to 64^2: the small-image form and its limit of tiles
     (65, None, [11], 1), (96, 97, [6, 0, 13], 5), (97, None, [64], 2), (128, 33, [10], 7), (160, None, [9], 8),
-    (65, 400, [130], 4),                       # detector wider than the image, more views than one staged set
+    (65, 400, [130], 4),                       # detector wider than the image
+    (65, None, [40], 1), (65, None, [60], 4),  # 4 and 6 CTAs a tile
+    (65, None, [1100], 4), (65, 30, [1100], 8),  # more than the 128 views a CTA stages at a time
 ]
 
 
