@@ -800,7 +800,8 @@ cudaError_t adjoint32(const Handle &h, float *X, int batch, int kb, int split, i
             if (e != cudaSuccess) return e;
             continue;
         }
-        a.segs = adj_segs(h, (long long)g[q].count * h.F * a.tps * a.tps, split, 8);
+        const int alone = g[q].width == 1 ? 20 : (g[q].width == 2 ? 12 : 0);  // views (see adj_cluster_size)
+        a.segs = adj_segs(h, (long long)g[q].count * h.F * a.tps * a.tps, split, 8, alone);
         switch (g[q].width) {
         case 1: e = launch_cluster(k_adj_tile<1>, a, h, adj_smem<1>(true)); break;
         case 2: e = launch_cluster(k_adj_tile<2>, a, h, adj_smem<2>(true)); break;

@@ -367,9 +367,9 @@ inline int persistent_grid(K kernel, int threads, size_t smem, long long work_bl
 // transpose kernels (ct_backproject.cu, ct_fan.cu)
 // ---------------------------------------------------------------------------
 // CTAs per tile of a frame's views (adj_cluster_size in ct_internal.cuh)
-inline int adj_segs(const Handle &h, long long tiles, int split, int fixed)
+inline int adj_segs(const Handle &h, long long tiles, int split, int fixed, int alone = 0)
 {
-    return adj_cluster_size(std::max(1, h.V / h.F), tiles, h.num_sms, split, fixed);
+    return adj_cluster_size(std::max(1, h.V / h.F), tiles, h.num_sms, split, fixed, alone);
 }
 
 // Launch of a transpose kernel: 256 threads, the a.segs CTAs of a tile one cluster.

@@ -151,10 +151,14 @@ inline int sino_pitch(int B) { return (B + 3) & ~3; }
 // than 2 CTAs only where each keeps 8 views: below that the prologue is all
 // there is (64^2, 22 views: 6.1 us at any size).
 // Clusters of odd size measured slower (256^2, 180 views, 8 sinograms: 30.7 us
-// at 4 or 6, 34.8 at 5 and 34.9 at 7; one CTA per tile 65.5).
+// at 4 or 6, 34.8 at 5 and 34.9 at 7; one CTA per tile 65.5).  Below `alone`
+// views a tile keeps one CTA unless more are asked for: a cluster's barriers
+// and exchange take 0.7 us, what that CTA takes for its views (128^2, 8 views,
+// one sinogram: 5.3 us with 2 CTAs, 4.8 alone; at 22 views 6.0 and 6.1).
 constexpr int kMaxSegs = 8;  // the portable cluster size
-inline int adj_cluster_size(int views, long long tiles, int num_sms, int split, int fixed)
+inline int adj_cluster_size(int views, long long tiles, int num_sms, int split, int fixed, int alone = 0)
 {
+    if (split == 1 && views < alone) return 1;
     const int least = views < 8 * split && split > 2 ? 2 : split;
     int best = least;
     double best_cost = 1e300;
@@ -170,6 +174,22 @@ inline int adj_cluster_size(int views, long long tiles, int num_sms, int split, 
         }
     }
     return best;
+}
+
+// Sinograms per group that a FP32 parallel-beam handle starts with, kb (1, 2, 4
+// or 8 by its batch) or fewer.  Sinograms share the weights of a pixel, but
+// groups also give CTAs: with little work a SM (batch x 32 x 32 tiles x views
+// over the SMs) the chip is idle with wide groups, and an odd batch then pays
+// another launch for its last one.  Batch of 8, us at 1 / 2 / 4 / 8 per group:
+// 96^2, 22 views (work 10) 6.3 / 7.2 / 9.2 / 12.2; 256^2, 8 (27) 7.6 / 7.4 / 9.2 /
+// 10.7; 256^2, 22 (74) 11.7 / 10.8 / 11.4 / 12.9; 256^2, 45 (152) 18.7 / 16.9 / 15.0 /
+// 14.8; 400^2, 22 (196) 21.6 / 19.9 / 17.9 / 21.7; 400^2, 90 (800) 62 / 57 / 44 / 41.
+inline int adj_group_width(int kb, int batch, long long tiles, int views, int num_sms)
+{
+    const double work = (double)batch * tiles * views / num_sms;
+    if (work < 25.0 || (work < 100.0 && batch % 2)) return 1;
+    const int most = work < 100.0 ? 2 : (work < 300.0 ? 4 : 8);
+    return kb < most ? kb : most;
 }
 
 struct Handle {

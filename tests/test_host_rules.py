@@ -13,9 +13,10 @@ MAIN = r"""
 #include "ct_internal.cuh"
 int main(int argc, char **argv)
 {
-    long long v[6] = {};
-    while (std::scanf("%lld %lld %lld %lld %lld", v, v + 1, v + 2, v + 3, v + 4) == 5)
-        std::printf("%d\n", ctgb::adj_cluster_size((int)v[0], v[1], (int)v[2], (int)v[3], (int)v[4]));
+    long long r, v[6] = {};
+    while (std::scanf("%lld %lld %lld %lld %lld %lld %lld", &r, v, v + 1, v + 2, v + 3, v + 4, v + 5) == 7)
+        std::printf("%d\n", r == 0 ? ctgb::adj_cluster_size((int)v[0], v[1], (int)v[2], (int)v[3], (int)v[4], (int)v[5])
+                                   : ctgb::adj_group_width((int)v[0], (int)v[1], v[2], (int)v[3], (int)v[4]));
 }
 """
 
@@ -31,8 +32,8 @@ def rules(tmp_path_factory):
     subprocess.run([cxx, "-std=c++17", "-w", "-I", inc, "-I", os.path.join(ROOT, "paper_2605_06336_gb300", "csrc"),
                     str(d / "main.cpp"), "-o", str(d / "main")], check=True)
 
-    def run(rows):
-        text = "\n".join(" ".join(map(str, r)) for r in rows)
+    def run(rows, rule=0):
+        text = "\n".join(" ".join(map(str, (rule, *r, *[0] * (6 - len(r))))) for r in rows)
         out = subprocess.run([str(d / "main")], input=text, capture_output=True, text=True, check=True).stdout
         return [int(x) for x in out.split()]
     return run
@@ -55,3 +56,14 @@ def test_sizes_whose_cluster_is_known(rules):
     rows = [(130, tiles(65, 1), 152, 1, 8), (40, tiles(65, 1), 152, 1, 8), (60, tiles(65, 1), 152, 1, 8),
             (1100, tiles(65, 1), 152, 1, 8)]
     assert rules(rows) == [8, 4, 6, 8]
+
+
+def test_few_views_take_one_cta_and_narrow_groups(rules):
+    """Few views: no cluster unless one is asked for, and groups that leave a CTA for every SM; never wider than kb."""
+    assert rules([(8, 16, 152, 1, 8, 20), (8, 16, 152, 2, 8, 20), (8, 16, 152, 4, 8, 20), (22, 16, 152, 1, 8, 20)]) == [1, 2, 2, 2]
+    tiles = lambda N: ((N + 31) // 32) ** 2
+    rows = [(8, 8, tiles(96), 8, 152), (8, 8, tiles(256), 8, 152), (4, 5, tiles(256), 22, 152), (8, 8, tiles(256), 45, 152),
+            (8, 8, tiles(256), 180, 152), (2, 2, tiles(2048), 120, 152)]
+    assert rules(rows, rule=1) == [1, 2, 1, 4, 8, 2]
+    rows = [(kb, K, t, v, 152) for kb, K in ((1, 1), (2, 3), (4, 7), (8, 9)) for t in (9, 64, 4096) for v in (1, 30, 1200)]
+    assert all(1 <= w <= r[0] for w, r in zip(rules(rows, rule=1), rows))
