@@ -87,9 +87,8 @@ typedef struct ct_handle ct_handle;
  * Create a handle: copies the geometry, allocates the workspaces it needs
  * on the current device (per-view tables; zero-padded "pair" copies of
  * max_batch images, of their transposes and of max_batch sinograms, about
- * 4 x 8 bytes per pixel and 8 bytes per sample and image in float32, and 8
- * bytes per pixel more for the interleaved images of handles that start with
- * them, see ct_set_tuning; the reduction partials) and binds it to cuda_stream (a cudaStream_t; NULL =
+ * 4 x 8 bytes per pixel and 8 bytes per sample and image in float32; the
+ * reduction partials) and binds it to cuda_stream (a cudaStream_t; NULL =
  * legacy default stream).  *out receives the handle.
  */
 int ct_init(const ct_geom *g, void *cuda_stream, ct_handle **out);
@@ -113,8 +112,10 @@ void ct_destroy(ct_handle *h);
  * i.e. that call's first `batch` images, at this call's angles and offsets:
  * the Jacobian and its transpose at one image (a Gauss-Newton step, an
  * inner least-squares solve on J) then lay the image out once.  A Jacobian
- * product after a forward on interleaved images first turns them into pair
- * layouts (one more kernel launch); the results are the same either way.
+ * product of fewer images than an interleaved call laid out first makes the
+ * pairs of its images beside them (not repeated by the next such call), or,
+ * above half of max_batch, of all the images (one more kernel launch); the
+ * results are the same either way.
  * CT_ERR_ARG when no layouts are current (none yet, or an error,
  * ct_autotune or a solver call on the handle since) or batch exceeds that
  * call's.  Calls that take no image (ct_adjoint, the repeats) keep them.
@@ -262,12 +263,9 @@ int ct_autotune(ct_handle *h);
  *   image layout: 0 pair images (each pixel stored beside its neighbour), 1
  *   images interleaved in groups of 4 (FP32 parallel-beam handles, forward
  *   staging 0, [0] 4 or 8; the forward then reads both taps of 4 images with
- *   two 16-byte loads; a later call that passes X = NULL to a Jacobian
- *   product converts them to pair images first).  1 is what FP32
- *   parallel-beam handles with [0] of 4 or 8 start with, where the memory is
- *   there.  Layout 1 allocates two
- *   buffers of max_batch x n_frames x N x (N + 4) floats the first time
- *   (CT_ERR_OOM if that fails; CT_ERR_ARG on an FP64 or fan-beam handle).
+ *   two 16-byte loads; the interleaved images take half of the memory of the
+ *   pair images, which they replace).  1 is what FP32 parallel-beam handles
+ *   with [0] of 4 or 8 start with.  CT_ERR_ARG on an FP64 or fan-beam handle.
  * [0]..[6] are powers of two, at most 8 (view groups at most 4), warps per
  * ray x views per CTA at most 16 (unstaged kernels).  Forward / Jacobian
  * staging is 0 (gathers through L1) or 4 / 8 (rows per shared-memory block of

@@ -51,9 +51,6 @@ void free_all(ctgb::Handle &h)
     cudaFree(h.d_rays);
     cudaFree(h.d_fanview);
     cudaFree(h.d_yi);
-    cudaFree(h.d_qx);
-    cudaFree(h.d_qt);
-    h.d_qx = h.d_qt = nullptr;
     h.d_rays = nullptr;
     h.d_fanview = nullptr;
     h.d_yi = nullptr;
@@ -65,46 +62,60 @@ void free_all(ctgb::Handle &h)
     h.d_segpart = nullptr;
 }
 
-// The pair layouts of the call's images and the view table.  X == null: the
-// layouts left by the previous call that took images are current (the caller
-// checked h.img_ready; interleaved ones, left by a forward, are turned into
-// pair layouts first); only the view table is brought up to date.
+// The pair images of the call's `batch` images and the view table.  X == null:
+// the layouts left by the previous call that took images are current (the
+// caller checked h.img_ready).  Interleaved ones get pairs of the images this
+// call reads beside them where the free half of the pairs' memory holds these
+// (in the launch of the view-table step, once for calls of as many images), else
+// all are turned into pairs (one launch more).  A forward of 8 images, 256^2 / 180
+// views, then J^T of one: 67.2 us, 72.1 turning all (80.8 with the forward on
+// pair images).
 template <typename T>
-cudaError_t prep_images(ctgb::Handle &h, const T *X, int nimg, const double *theta, const double *delta)
+cudaError_t prep_images(ctgb::Handle &h, const T *X, int batch, const double *theta, const double *delta,
+                        ctgb::ImgForm *form)
 {
+    *form = ctgb::kPairImages;
     if (X) {
-        h.img_kind = 0;
-        return ctgb::launch_pairs_img<T>(h, X, nimg, nullptr, theta, delta);
+        h.img_kind = h.side_pairs = 0;
+        return ctgb::launch_pairs_img<T>(h, X, batch * h.F, nullptr, theta, delta);
     }
-    if (h.img_kind == 1) {
-        const cudaError_t e = ctgb::launch_interleaved_to_pairs(h, h.img_ready);
-        if (e != cudaSuccess) return e;
-        h.img_kind = 0;
-    }
-    return ctgb::launch_view_setup(h, theta, delta);
+    if (h.img_kind == 0) return ctgb::launch_view_setup(h, theta, delta);
+    const bool made = h.side_pairs >= batch, beside = made || 2 * batch <= h.max_batch + 1;
+    if (beside) *form = ctgb::kSidePairs;
+    if (made) return ctgb::launch_view_setup(h, theta, delta);
+    h.img_kind = beside ? 1 : 0;
+    h.side_pairs = beside ? batch : 0;
+    return ctgb::launch_interleaved_to_pairs(h, h.side_pairs, theta, delta);
 }
 
 // Whether a product that takes `batch` images lays them out interleaved (the
-// tuning asks for it and the handle can: FP32, parallel beam, workspace
-// present).  One image keeps the pair images, which fetch both taps in one
-// load: 58.8 against 77 us for the forward of 16 frames of 256^2 / 1200 views.
+// tuning asks for it: FP32, parallel beam).  One image keeps the pair images,
+// which fetch both taps in one load: 58.8 against 77 us for the forward of 16
+// frames of 256^2 / 1200 views.
 bool can_interleave(const ctgb::Handle &h, int batch)
 {
-    return h.tune.fwd_layout == 1 && h.precision == 0 && h.fan_D == 0.0 && h.d_qx && batch >= 2;
+    return h.tune.fwd_layout == 1 && h.precision == 0 && h.fan_D == 0.0 && batch >= 2;
 }
 
-// The layout of a batched derivative call and the view table; *inter: the
-// interleaved images hold the call's batch (512^2 / 360 views, 4 images, J^T with
-// offsets: 207 us a call against 221 on pair images), else the pair images do.
-template <typename T>
-cudaError_t prep_batch(ctgb::Handle &h, const T *X, int batch, const double *theta, const double *delta, bool *inter)
+cudaError_t interleave(ctgb::Handle &h, const void *X, int batch, const double *theta, const double *delta)
 {
-    *inter = can_interleave(h, batch) && h.tune.der_stage == 0 && h.tune.der_kb == 4 &&
-             (X || (h.img_kind == 1 && h.img_ready == batch));
-    if (!*inter) return prep_images<T>(h, X, batch * h.F, theta, delta);
-    if (!X) return ctgb::launch_view_setup(h, theta, delta);
     h.img_kind = 1;
+    h.side_pairs = 0;
     return ctgb::launch_interleave_img(h, (const float *)X, batch, theta, delta);
+}
+
+// The layout of a batched derivative call and the view table; *form: the
+// interleaved images where they hold the call's batch (512^2 / 360 views, 4 images,
+// J^T with offsets: 207 us a call against 221 on pair images), else pairs.
+template <typename T>
+cudaError_t prep_batch(ctgb::Handle &h, const T *X, int batch, const double *theta, const double *delta,
+                       ctgb::ImgForm *form)
+{
+    const bool inter = can_interleave(h, batch) && h.tune.der_stage == 0 && h.tune.der_kb == 4 &&
+                       (X || (h.img_kind == 1 && h.img_ready == batch));
+    if (!inter) return prep_images<T>(h, X, batch, theta, delta, form);
+    *form = ctgb::kInterleaved;
+    return X ? interleave(h, X, batch, theta, delta) : ctgb::launch_view_setup(h, theta, delta);
 }
 
 template <typename T>
@@ -113,12 +124,12 @@ int do_forward(ctgb::Handle &h, const double *theta, const double *delta, const 
     // X == null reads whichever layout the previous call left
     const bool inter = X ? can_interleave(h, batch) : h.img_kind == 1;
     if (inter && X) {
-        CT_CUDA(ctgb::launch_interleave_img(h, (const float *)X, batch, theta, delta));
-        h.img_kind = 1;
+        CT_CUDA(interleave(h, X, batch, theta, delta));
     } else if (inter) {
         CT_CUDA(ctgb::launch_view_setup(h, theta, delta));
     } else {
-        CT_CUDA(prep_images<T>(h, (const T *)X, batch * h.F, theta, delta));
+        ctgb::ImgForm form;  // the pair images: X is given, or they are current
+        CT_CUDA(prep_images<T>(h, (const T *)X, batch, theta, delta, &form));
     }
     CT_CUDA(ctgb::launch_forward<T>(h, (T *)Y, batch, h.tune.fwd_kb, h.tune.fwd_split, h.tune.fwd_vw, h.tune.fwd_stage,
                                     nullptr, inter, X ? batch : h.img_ready));
@@ -138,8 +149,10 @@ template <typename T>
 int do_jac(ctgb::Handle &h, const double *theta, const double *delta, const void *x, const double *dtheta,
            const double *ddelta, void *dy)
 {
-    CT_CUDA(prep_images<T>(h, (const T *)x, h.F, theta, delta));
-    CT_CUDA(ctgb::launch_jvp<T>(h, dtheta, ddelta, (T *)dy, h.tune.der_split, h.tune.der_vw, h.tune.der_stage));
+    ctgb::ImgForm form;
+    CT_CUDA(prep_images<T>(h, (const T *)x, 1, theta, delta, &form));
+    CT_CUDA(ctgb::launch_jvp<T>(h, dtheta, ddelta, (T *)dy, h.tune.der_split, h.tune.der_vw, h.tune.der_stage, 1, 1, 0,
+                                form));
     return CT_OK;
 }
 
@@ -147,8 +160,10 @@ template <typename T>
 int do_jacT(ctgb::Handle &h, const double *theta, const double *delta, const void *x, const void *r, double *gtheta,
             double *gdelta)
 {
-    CT_CUDA(prep_images<T>(h, (const T *)x, h.F, theta, delta));
-    CT_CUDA(ctgb::launch_vjp<T>(h, (const T *)r, gtheta, gdelta, h.tune.der_split, h.tune.der_vw, h.tune.der_stage));
+    ctgb::ImgForm form;
+    CT_CUDA(prep_images<T>(h, (const T *)x, 1, theta, delta, &form));
+    CT_CUDA(ctgb::launch_vjp<T>(h, (const T *)r, gtheta, gdelta, h.tune.der_split, h.tune.der_vw, h.tune.der_stage, 1,
+                                1, 0, 0, form));
     return CT_OK;
 }
 
@@ -157,10 +172,10 @@ int do_jac_batch(ctgb::Handle &h, const double *theta, const double *delta, cons
                  const double *ddelta, void *dY, int batch, int flags)
 {
     const long long dstride = (flags & CT_BATCH_PER_IMAGE_DIRECTION) ? h.V : 0;
-    bool inter;
-    CT_CUDA(prep_batch<T>(h, (const T *)X, batch, theta, delta, &inter));
+    ctgb::ImgForm form;
+    CT_CUDA(prep_batch<T>(h, (const T *)X, batch, theta, delta, &form));
     CT_CUDA(ctgb::launch_jvp<T>(h, dtheta, ddelta, (T *)dY, h.tune.der_split, h.tune.der_vw, h.tune.der_stage, batch,
-                                h.tune.der_kb, dstride, inter));
+                                h.tune.der_kb, dstride, form));
     return CT_OK;
 }
 
@@ -169,10 +184,10 @@ int do_jacT_batch(ctgb::Handle &h, const double *theta, const double *delta, con
                   double *gtheta, double *gdelta, int batch, int flags)
 {
     const long long rstride = (flags & CT_BATCH_SHARED_R) ? 0 : (long long)h.V * h.B;
-    bool inter;
-    CT_CUDA(prep_batch<T>(h, (const T *)X, batch, theta, delta, &inter));
+    ctgb::ImgForm form;
+    CT_CUDA(prep_batch<T>(h, (const T *)X, batch, theta, delta, &form));
     CT_CUDA(ctgb::launch_vjp<T>(h, (const T *)R, gtheta, gdelta, h.tune.der_split, h.tune.der_vw, h.tune.der_stage,
-                                batch, h.tune.der_kb, rstride, (flags & CT_BATCH_SUM) ? 1 : 0, inter));
+                                batch, h.tune.der_kb, rstride, (flags & CT_BATCH_SUM) ? 1 : 0, form));
     return CT_OK;
 }
 
@@ -180,10 +195,10 @@ template <typename T>
 int do_gn_batch(ctgb::Handle &h, const double *theta, const double *delta, const void *X, const void *bdata,
                 void *res, double *grad, double *jnorm2, double *fval, int batch)
 {
-    bool inter;
-    CT_CUDA(prep_batch<T>(h, (const T *)X, batch, theta, delta, &inter));
+    ctgb::ImgForm form;
+    CT_CUDA(prep_batch<T>(h, (const T *)X, batch, theta, delta, &form));
     CT_CUDA(ctgb::launch_gn<T>(h, (const T *)bdata, (T *)res, grad, jnorm2, fval, h.tune.der_split, h.tune.der_vw,
-                               h.tune.der_stage, nullptr, nullptr, batch, h.tune.der_kb, nullptr, inter));
+                               h.tune.der_stage, nullptr, nullptr, batch, h.tune.der_kb, nullptr, form));
     return CT_OK;
 }
 
@@ -191,9 +206,10 @@ template <typename T>
 int do_gn(ctgb::Handle &h, const double *theta, const double *delta, const void *x, const void *bdata, void *res,
           double *grad, double *jnorm2, double *fval)
 {
-    CT_CUDA(prep_images<T>(h, (const T *)x, h.F, theta, delta));
+    ctgb::ImgForm form;
+    CT_CUDA(prep_images<T>(h, (const T *)x, 1, theta, delta, &form));
     CT_CUDA(ctgb::launch_gn<T>(h, (const T *)bdata, (T *)res, grad, jnorm2, fval, h.tune.der_split, h.tune.der_vw,
-                                  h.tune.der_stage));
+                               h.tune.der_stage, nullptr, nullptr, 1, 1, nullptr, form));
     return CT_OK;
 }
 
@@ -207,23 +223,6 @@ int ensure_seg_partials(ctgb::Handle &h)
     if (cudaMalloc(&h.d_segpart, bytes) != cudaSuccess) {
         cudaGetLastError();
         h.d_segpart = nullptr;
-        return CT_ERR_OOM;
-    }
-    return CT_OK;
-}
-
-// Workspace of the interleaved forward images, allocated the first time that
-// layout is set (FP32 parallel-beam handles).
-int ensure_interleaved(ctgb::Handle &h)
-{
-    if (h.d_qx) return CT_OK;
-    if (h.precision != 0 || h.fan_D > 0.0) return CT_ERR_ARG;
-    const size_t bytes = sizeof(float) * (size_t)h.max_batch * h.F * h.N * h.Pp;
-    if (cudaMalloc(&h.d_qx, bytes) != cudaSuccess || cudaMalloc(&h.d_qt, bytes) != cudaSuccess) {
-        cudaGetLastError();
-        cudaFree(h.d_qx);
-        cudaFree(h.d_qt);
-        h.d_qx = h.d_qt = nullptr;
         return CT_ERR_OOM;
     }
     return CT_OK;
@@ -361,7 +360,7 @@ template <typename T> int autotune_impl(ctgb::Handle &h)
                 }
             }
             // the same shapes reading the interleaved images (FP32 parallel beam, 4 or 8 per lane)
-            if ((kb == 4 || kb == 8) && fp32 && h.fan_D == 0.0 && ensure_interleaved(h) == CT_OK) {
+            if ((kb == 4 || kb == 8) && fp32 && h.fan_D == 0.0) {
                 for (int sp : {1, 2, 4, 8}) {
                     for (int vw : {1, 2, 4, 8}) {
                         if (sp * vw > 16) continue;
@@ -602,9 +601,7 @@ int ct_init(const ct_geom *g, void *cuda_stream, ct_handle **out)
         return rc;
     }
     default_tuning(h);
-    // batches read the interleaved images where their workspace can be had
-    if (h.tune.fwd_kb >= 4 && h.precision == 0 && h.fan_D == 0.0 && ensure_interleaved(h) == CT_OK)
-        h.tune.fwd_layout = 1;
+    if (h.tune.fwd_kb >= 4 && h.precision == 0 && h.fan_D == 0.0) h.tune.fwd_layout = 1;
     *out = H;
     return CT_OK;
 }
@@ -768,10 +765,7 @@ int ct_set_tuning(ct_handle *H, const int32_t *in)
         const int rc = ensure_seg_partials(H->h);
         if (rc != CT_OK) return rc;
     }
-    if (in[11] == 1) {
-        const int rc = ensure_interleaved(H->h);
-        if (rc != CT_OK) return rc;
-    }
+    if (in[11] == 1 && (H->h.precision != 0 || H->h.fan_D > 0.0)) return CT_ERR_ARG;
     ctgb::Tuning &t = H->h.tune;
     t.fwd_kb = in[0];
     t.fwd_split = in[1];

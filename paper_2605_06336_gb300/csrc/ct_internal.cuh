@@ -192,6 +192,10 @@ inline int adj_group_width(int kb, int batch, long long tiles, int views, int nu
     return kb < most ? kb : most;
 }
 
+// Where a derivative product finds its images: the pair images, the
+// interleaved images, or the pairs made beside the interleaved ones.
+enum ImgForm { kPairImages, kInterleaved, kSidePairs };
+
 struct Handle {
     int N = 0, B = 0, V = 0, F = 1, max_batch = 1, precision = 0, device = 0;
     int Pp = 0, Pb = 0;  // pair pitches
@@ -207,8 +211,6 @@ struct Handle {
     void *d_pt = nullptr;     // pair images, rows of X^T: (max_batch + 1) * F * N * Pp pairs
     void *d_yp = nullptr;     // sinograms of the transpose: pairs (FP64) or interleaved (FP32), max_batch * V * Pb pairs
     int *d_rowflag = nullptr; // FP32 transpose: [group][V], the row of the group holds a non-finite value
-    float *d_qx = nullptr;    // interleaved images, rows of X and of X^T: max_batch * F * N * Pp
-    float *d_qt = nullptr;    // floats each, allocated when fwd_layout 1 is set (FP32 handles)
     double *d_partial = nullptr;  // per (image, view, chunk) reduction partials, 4 per item, max_batch images
     void *d_segpart = nullptr;    // segment partials of the staged forward (sinograms):
                                   // 3 * max_batch * max(V * B, F * N * N) floats, allocated
@@ -230,6 +232,14 @@ struct Handle {
     // which lay out images of their own, clear it.
     int img_ready = 0;
     int img_kind = 0;  // the layout holding them: 0 pair images, 1 interleaved images
+    // img_kind 1: the first side_pairs of them are in d_px as pairs too, image k of X at k and of
+    // X^T at side_pairs + k, for the products that read pairs
+    int side_pairs = 0;
+    long long img_elems() const { return (long long)F * N * Pp; }  // of a padded image
+    // Interleaved images (FP32, parallel beam): half the bytes of the pairs, kept in the memory of
+    // the X^T pairs (a call's images are in one of the layouts), the second 16-byte aligned
+    float *qx() const { return (float *)d_pt; }
+    float *qt() const { return (float *)d_pt + ((max_batch * img_elems() + 3) & ~3LL); }
     int num_sms = 0;
     Tuning tune;
 };
@@ -256,16 +266,18 @@ template <typename T>
 cudaError_t launch_prep_forward(const Handle &h, const T *X, int nimg, const int *skip = nullptr,
                                 const double *theta = nullptr, const double *delta = nullptr);
 // Interleaved images of X and X^T for a batch of `batch` images of F frames
-// (into d_qx / d_qt), with the view-table step as in launch_pairs_img.
+// (into qx / qt), with the view-table step as in launch_pairs_img.
 cudaError_t launch_interleave_img(const Handle &h, const float *X, int batch, const double *theta = nullptr,
                                   const double *delta = nullptr, const int *skip = nullptr);
-// The pair images of the first `batch` images from the interleaved ones.
-cudaError_t launch_interleaved_to_pairs(const Handle &h, int batch);
+// Pair images from the img_ready interleaved ones: of the first `side` beside
+// them (2 * side <= max_batch + 1), or, with side 0, of all in their place; with
+// the view-table step.
+cudaError_t launch_interleaved_to_pairs(const Handle &h, int side, const double *theta, const double *delta);
 
 // stage > 0 (FP32 only): rows per shared-memory block of the band-staged
 // march (ct_band.cu); 0: gathers through L1.  interleaved (FP32, parallel
 // beam): the first `batch` images of the interleaved layout of a batch of
-// layout_batch (>= batch) are read from d_qx / d_qt, 8 per lane when kb is 8,
+// layout_batch (>= batch) are read from qx / qt, 8 per lane when kb is 8,
 // else 4 (stage is then ignored).
 template <typename T>
 cudaError_t launch_forward(const Handle &h, T *Y, int batch, int kb, int split, int vw, int stage,
@@ -283,19 +295,19 @@ cudaError_t launch_adjoint(const Handle &h, T *X, int batch, int kb, int split, 
 // one [V] vector summing the images in order.  GN: image k reads
 // bdata + k * V * B and writes [k][V] outputs; rscale (nullable) receives
 // sum_b |r_b| (|(H x)_b| + |b_b|) per view, the rounding scale of the misfit.
-// interleaved (FP32, parallel beam, stage 0): the images are in the interleaved
-// layout of a batch of `batch`, read 4 (then 2, 1) per lane whatever kb is.
+// form: where the images are; kInterleaved (FP32, parallel beam, stage 0): in the
+// interleaved layout of a batch of `batch`, read 4 (then 2, 1) per lane whatever kb is.
 template <typename T>
 cudaError_t launch_jvp(const Handle &h, const double *dtheta, const double *ddelta, T *dY, int split, int vw,
-                       int stage, int batch = 1, int kb = 1, long long dir_stride = 0, bool interleaved = false);
+                       int stage, int batch = 1, int kb = 1, long long dir_stride = 0, ImgForm form = kPairImages);
 template <typename T>
 cudaError_t launch_vjp(const Handle &h, const T *R, double *gtheta, double *gdelta, int split, int vw, int stage,
                        int batch = 1, int kb = 1, long long r_stride = 0, int sum = 0,
-                       bool interleaved = false);
+                       ImgForm form = kPairImages);
 template <typename T>
 cudaError_t launch_gn(const Handle &h, const T *bdata, T *res, double *grad, double *jnorm2, double *fval,
                       int split, int vw, int stage, const int *view_mask = nullptr, const int *skip = nullptr,
-                      int batch = 1, int kb = 1, double *rscale = nullptr, bool interleaved = false);
+                      int batch = 1, int kb = 1, double *rscale = nullptr, ImgForm form = kPairImages);
 
 // Fan beam (ct_fan.cu).  launch_fan_rays rebuilds the per-ray table from the
 // view table; every launcher that brings the view table up to date runs it

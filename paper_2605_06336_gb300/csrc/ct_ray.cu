@@ -382,16 +382,23 @@ __global__ void __launch_bounds__(256, 5) k_interleave_img(const float *__restri
 }
 
 // Pair images of the first nimg images of a batch of K from the interleaved
-// ones: pair e of a row is (element e, element e + 1), zero past the row end.
+// ones of X, and (PT not null) those of X^T: pair e of a row is (element e,
+// element e + 1), zero past the row end.  The first p.on CTAs run the
+// view-table step of the call instead.
 __global__ void k_interleaved_to_pairs(const float *__restrict__ QX, const float *__restrict__ QT,
-                                       float2 *__restrict__ PX, float2 *__restrict__ PT, int N, int Pp, int F,
-                                       int K, int nimg)
+                                       float2 *__restrict__ PX, float2 *__restrict__ PT, long long per, int Pp, int K,
+                                       int nimg, ViewPrep p)
 {
     chain_wait();
-    const long long per = (long long)F * N * Pp;  // elements per image
-    const long long total = (long long)nimg * per;
-    for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < total;
-         idx += (long long)gridDim.x * blockDim.x) {
+    extern __shared__ unsigned long long prep_key[];
+    const int nblk = gridDim.x - p.on, blk = blockIdx.x - p.on;
+    if (blk < 0) {
+        view_prep_block(p, blockIdx.x, prep_key);
+        return;
+    }
+    const long long total = (long long)nimg * per;  // per: elements per image
+    for (long long idx = blk * (long long)blockDim.x + threadIdx.x; idx < total;
+         idx += (long long)nblk * blockDim.x) {
         const int k = (int)(idx / per);
         const long long el = idx - k * per;
         const int e = (int)(el % Pp);
@@ -400,7 +407,29 @@ __global__ void k_interleaved_to_pairs(const float *__restrict__ QX, const float
         const size_t o = (size_t)k0 * per + (size_t)el * w + (k - k0);
         const bool last = e + 1 >= Pp;
         PX[idx] = make_float2(QX[o], last ? 0.0f : QX[o + w]);
-        PT[idx] = make_float2(QT[o], last ? 0.0f : QT[o + w]);
+        if (PT) PT[idx] = make_float2(QT[o], last ? 0.0f : QT[o + w]);
+    }
+}
+
+// Pair images of X^T from those of X, by 33 x 33 elements as k_pairs_img.
+__global__ void __launch_bounds__(256) k_transpose_pairs(const float2 *__restrict__ PX, float2 *__restrict__ PT, int N,
+                                                         int Pp, int nimg)
+{
+    chain_wait();
+    __shared__ float t[33][33];
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    const int r0 = blockIdx.y * 32 - 2, c0 = blockIdx.x * 32;
+    for (int img = blockIdx.z; img < nimg; img += gridDim.z) {
+        const float2 *px = PX + (size_t)img * N * Pp;
+        __syncthreads();  // the previous image's tile has been read
+        for (int i = ty; i < 33; i += 8) {
+            const int r = r0 + i, c = c0 + tx;
+            t[i][tx] = (r >= 0 && r < N && c < N) ? px[(size_t)r * Pp + c + 2].x : 0.0f;
+        }
+        __syncthreads();
+        for (int i = ty; i < 32; i += 8)
+            if (c0 + i < N && r0 + tx + 2 < Pp)
+                PT[((size_t)img * N + c0 + i) * Pp + r0 + tx + 2] = make_float2(t[tx][i], t[tx + 1][i]);
     }
 }
 
@@ -728,7 +757,7 @@ __global__ void __launch_bounds__(64) k_finalize(const double *__restrict__ part
 // ---------------------------------------------------------------------------
 // launch helpers
 // ---------------------------------------------------------------------------
-template <typename T> RayArgs<T> base_args(const Handle &h)
+template <typename T> RayArgs<T> base_args(const Handle &h, ImgForm form = kPairImages)
 {
     RayArgs<T> a{};
     a.vg = h.d_views;
@@ -738,8 +767,8 @@ template <typename T> RayArgs<T> base_args(const Handle &h)
     a.nchunks = h.nchunks;
     a.Pp = h.Pp;
     a.PX = (const pair_t<T> *)h.d_px;
-    a.PT = (const pair_t<T> *)h.d_pt;
-    a.pimg_stride = (long long)h.F * h.N * h.Pp;
+    a.pimg_stride = h.img_elems();
+    a.PT = form == kSidePairs ? a.PX + h.side_pairs * a.pimg_stride : (const pair_t<T> *)h.d_pt;
     a.kbase = 0;
     a.ngroups = 1;
     a.sino_stride = (long long)h.V * h.B;
@@ -884,7 +913,7 @@ cudaError_t launch_prep_forward(const Handle &h, const T *X, int nimg, const int
 cudaError_t launch_interleave_img(const Handle &h, const float *X, int batch, const double *theta,
                                   const double *delta, const int *skip)
 {
-    if (!h.d_qx || h.fan_D > 0.0 || batch < 1 || batch > h.max_batch) return cudaErrorInvalidValue;
+    if (h.precision != 0 || h.fan_D > 0.0 || batch < 1 || batch > h.max_batch) return cudaErrorInvalidValue;
     const ViewPrep p = view_prep_args(h, theta, delta);
     cudaError_t e = allow_prep_smem<k_interleave_img>();
     if (e != cudaSuccess) return e;
@@ -892,17 +921,25 @@ cudaError_t launch_interleave_img(const Handle &h, const float *X, int batch, co
     const int ngroups = n4 / 4 + (rem >= 2 ? 1 : 0) + (rem & 1);
     dim3 grid((h.Pp + 31) / 32, (h.Pp + 31) / 32, std::max(1, std::min(h.F * ngroups, 65535)));
     grid.x += prep_columns(p, grid);
-    launch_chained(k_interleave_img, grid, 256, prep_smem(p), h.stream, X, h.d_qx, h.d_qt, h.N, h.Pp, h.F, batch, p, skip);
+    launch_chained(k_interleave_img, grid, 256, prep_smem(p), h.stream, X, h.qx(), h.qt(), h.N, h.Pp, h.F, batch, p, skip);
     return cudaGetLastError();
 }
 
-cudaError_t launch_interleaved_to_pairs(const Handle &h, int batch)
+cudaError_t launch_interleaved_to_pairs(const Handle &h, int side, const double *theta, const double *delta)
 {
-    if (!h.d_qx || h.precision != 0 || batch < 1 || batch > h.max_batch) return cudaErrorInvalidValue;
-    const long long total = (long long)batch * h.F * h.N * h.Pp;
-    const long long blocks = std::min<long long>((total + 255) / 256, (long long)h.num_sms * 16);
-    launch_chained(k_interleaved_to_pairs, (int)std::max<long long>(1, blocks), 256, 0, h.stream, 
-        h.d_qx, h.d_qt, (float2 *)h.d_px, (float2 *)h.d_pt, h.N, h.Pp, h.F, batch, batch);
+    const int K = h.img_ready, nimg = side ? side : K;
+    if (h.precision != 0 || h.fan_D > 0.0 || K < 1 || nimg > K || 2 * side > h.max_batch + 1)
+        return cudaErrorInvalidValue;
+    const long long per = h.img_elems(), total = nimg * per;
+    const int blocks = (int)std::min<long long>((total + 255) / 256, (long long)h.num_sms * 16);
+    float2 *px = (float2 *)h.d_px;
+    const ViewPrep p = view_prep_args(h, theta, delta);
+    launch_chained(k_interleaved_to_pairs, blocks + p.on, 256, prep_smem(p), h.stream, h.qx(), h.qt(), px,
+                   side ? px + side * per : nullptr, per, h.Pp, K, nimg, p);
+    if (!side) {  // the pairs of X^T over the interleaved images, from those of X
+        const dim3 grid((h.N + 31) / 32, (h.Pp + 31) / 32, std::min(K * h.F, 65535));
+        launch_chained(k_transpose_pairs, grid, 256, 0, h.stream, px, (float2 *)h.d_pt, h.N, h.Pp, K * h.F);
+    }
     return cudaGetLastError();
 }
 
@@ -955,10 +992,10 @@ cudaError_t launch_forward(const Handle &h, T *Y, int batch, int kb, int split, 
         // the first `batch` images; images past `batch` in the last of them are read
         // but not written.
         if constexpr (std::is_same<T, float>::value) {
-            if (!h.d_qx || h.fan_D > 0.0 || layout_batch < batch || layout_batch > h.max_batch)
+            if (h.fan_D > 0.0 || layout_batch < batch || layout_batch > h.max_batch)
                 return cudaErrorInvalidValue;
-            a.QX = h.d_qx;
-            a.QT = h.d_qt;
+            a.QX = h.qx();
+            a.QT = h.qt();
             a.qimg_stride = (long long)h.F * h.N * h.Pp;
             a.kend = batch;
             int k = 0;
@@ -1010,16 +1047,16 @@ cudaError_t launch_forward(const Handle &h, T *Y, int batch, int kb, int split, 
 // The derivative modes over `batch` images sharing the view table: groups of
 // up to kb (1, 2 or 4) images per lane; the fan-beam and band-staged forms
 // take one image per lane (their launches still cover the whole batch).
-// interleaved (FP32, parallel beam, stage 0): the images are those of the
+// kInterleaved (FP32, parallel beam, stage 0): the images are those of the
 // interleaved layout of a batch of `batch`, read by its groups of 4, 2 and 1.
 template <typename T, int MODE, bool OFFS>
-cudaError_t der_groups(const Handle &h, RayArgs<T> a, int batch, int kb, int split, int stage, bool interleaved)
+cudaError_t der_groups(const Handle &h, RayArgs<T> a, int batch, int kb, int split, int stage, ImgForm form)
 {
-    if (interleaved) {
+    if (form == kInterleaved) {
         if constexpr (std::is_same<T, float>::value) {
-            if (!h.d_qx || h.fan_D > 0.0 || batch > h.max_batch) return cudaErrorInvalidValue;
-            a.QX = h.d_qx;
-            a.QT = h.d_qt;
+            if (h.fan_D > 0.0 || batch > h.max_batch) return cudaErrorInvalidValue;
+            a.QX = h.qx();
+            a.QT = h.qt();
             a.qimg_stride = (long long)h.F * h.N * h.Pp;
             int k = 0;
             for (int width : {4, 2, 1}) {
@@ -1061,30 +1098,30 @@ cudaError_t der_groups(const Handle &h, RayArgs<T> a, int batch, int kb, int spl
 
 template <typename T>
 cudaError_t launch_jvp(const Handle &h, const double *dtheta, const double *ddelta, T *dY, int split, int vw,
-                       int stage, int batch, int kb, long long dir_stride, bool interleaved)
+                       int stage, int batch, int kb, long long dir_stride, ImgForm form)
 {
-    RayArgs<T> a = base_args<T>(h);
+    RayArgs<T> a = base_args<T>(h, form);
     a.VW = vw;
     a.Y = dY;
     a.dtheta = dtheta;
     a.ddelta = ddelta;
     a.dir_stride = dir_stride;
-    return ddelta ? der_groups<T, kJvp, true>(h, a, batch, kb, split, stage, interleaved)
-                  : der_groups<T, kJvp, false>(h, a, batch, kb, split, stage, interleaved);
+    return ddelta ? der_groups<T, kJvp, true>(h, a, batch, kb, split, stage, form)
+                  : der_groups<T, kJvp, false>(h, a, batch, kb, split, stage, form);
 }
 
 template <typename T>
 cudaError_t launch_vjp(const Handle &h, const T *R, double *gtheta, double *gdelta, int split, int vw, int stage,
-                       int batch, int kb, long long r_stride, int sum, bool interleaved)
+                       int batch, int kb, long long r_stride, int sum, ImgForm form)
 {
-    RayArgs<T> a = base_args<T>(h);
+    RayArgs<T> a = base_args<T>(h, form);
     a.VW = vw;
     a.R = R;
     a.r_stride = r_stride;
     a.partial = h.d_partial;
     a.part_stride = 4LL * h.V * h.nchunks;
-    cudaError_t e = gdelta ? der_groups<T, kVjp, true>(h, a, batch, kb, split, stage, interleaved)
-                           : der_groups<T, kVjp, false>(h, a, batch, kb, split, stage, interleaved);
+    cudaError_t e = gdelta ? der_groups<T, kVjp, true>(h, a, batch, kb, split, stage, form)
+                           : der_groups<T, kVjp, false>(h, a, batch, kb, split, stage, form);
     if (e != cudaSuccess) return e;
     const long long outs = (long long)h.V * (sum ? 1 : batch);
     launch_chained(k_finalize, (int)((4 * outs + 63) / 64), 64, 0, h.stream, h.d_partial, h.V, h.nchunks, batch, a.part_stride,
@@ -1096,9 +1133,9 @@ cudaError_t launch_vjp(const Handle &h, const T *R, double *gtheta, double *gdel
 template <typename T>
 cudaError_t launch_gn(const Handle &h, const T *bdata, T *res, double *grad, double *jnorm2, double *fval, int split,
                       int vw, int stage, const int *view_mask, const int *skip, int batch, int kb, double *rscale,
-                      bool interleaved)
+                      ImgForm form)
 {
-    RayArgs<T> a = base_args<T>(h);
+    RayArgs<T> a = base_args<T>(h, form);
     a.VW = vw;
     a.R = bdata;
     a.r_stride = (long long)h.V * h.B;
@@ -1107,7 +1144,7 @@ cudaError_t launch_gn(const Handle &h, const T *bdata, T *res, double *grad, dou
     a.part_stride = 4LL * h.V * h.nchunks;
     a.view_mask = view_mask;
     a.skip = skip;
-    cudaError_t e = der_groups<T, kGn, false>(h, a, batch, kb, split, stage, interleaved);
+    cudaError_t e = der_groups<T, kGn, false>(h, a, batch, kb, split, stage, form);
     if (e != cudaSuccess) return e;
     const long long outs = (long long)h.V * batch;
     launch_chained(k_finalize, (int)((4 * outs + 63) / 64), 64, 0, h.stream, h.d_partial, h.V, h.nchunks, batch, a.part_stride, 0,
@@ -1124,11 +1161,11 @@ cudaError_t launch_gn(const Handle &h, const T *bdata, T *res, double *grad, dou
                                                 const double *);                                           \
     template cudaError_t launch_forward<T>(const Handle &, T *, int, int, int, int, int, const int *, bool, int); \
     template cudaError_t launch_jvp<T>(const Handle &, const double *, const double *, T *, int, int, int, int, \
-                                       int, long long, bool);                                             \
+                                       int, long long, ImgForm);                                          \
     template cudaError_t launch_vjp<T>(const Handle &, const T *, double *, double *, int, int, int, int, int, \
-                                       long long, int, bool);                                             \
+                                       long long, int, ImgForm);                                          \
     template cudaError_t launch_gn<T>(const Handle &, const T *, T *, double *, double *, double *, int,    \
-                                      int, int, const int *, const int *, int, int, double *, bool);
+                                      int, int, const int *, const int *, int, int, double *, ImgForm);
 
 CTGB_RAY_INSTANTIATE(float)
 CTGB_RAY_INSTANTIATE(double)

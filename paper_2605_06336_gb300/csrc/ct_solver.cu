@@ -341,7 +341,7 @@ template <typename T> struct Solver {
             const int nb = std::min(block(), j0 + cnt - j);
             const double *th = j == j0 ? theta : nullptr;  // the first layout launch also updates the view table
             if constexpr (std::is_same<T, float>::value) {
-                if (nb >= 2 && h.tune.fwd_layout == 1 && h.d_qx && h.fan_D == 0.0) {
+                if (nb >= 2 && h.tune.fwd_layout == 1 && h.fan_D == 0.0) {
                     SV_CUDA(launch_interleave_img(h, col(V, n, j), nb, th, delta, stop));
                     SV_CUDA(launch_forward<T>(h, col(HV, m, j), nb, h.tune.fwd_kb, h.tune.fwd_split, h.tune.fwd_vw,
                                               0, stop, true, nb));

@@ -180,6 +180,74 @@ def test_image_layouts(case, dtype):
         assert all(torch.equal(p, q) for p, q in zip(*out))
 
 
+@pytest.mark.parametrize("max_batch", [2, 3, 7, 8])
+@pytest.mark.parametrize("der_kb", [1, 4])
+def test_products_of_fewer_images_after_an_interleaved_call(max_batch, der_kb):
+    """Any order of products that pass no images after a call that laid out a batch interleaved: one image, some
+    and all of them, then the whole batch again -- the bits that passing the images to another handle gives."""
+    from paper_2605_06336_gb300 import ct
+    N, vpf, K = 37, [7, 5], max_batch
+    V, B = sum(vpf), synth.n_bins(37)
+    rng = np.random.default_rng(max_batch)
+    ops = [ct.CTOperator(N, B, V, vpf, max_batch=K, dtype=torch.float32) for _ in range(2)]
+    for op in ops:
+        op.tuning = [4, 2, 2, 4, 1, 4, 1, 0, 0, 0, der_kb, 1]
+    op, other = ops
+    th, dth, dl = dev(rng.uniform(-3, 3, V)), dev(rng.standard_normal(V)), dev(rng.normal(0, 0.5, V))
+    R = dev(rng.standard_normal((K, op.m)), torch.float32)
+    X0 = [dev(rng.uniform(size=(K, op.n)), torch.float32) for _ in range(2)]
+
+    def fwd(o, X, k):
+        return o.forward(X, th, dl, batch=k) if X is None else o.forward(X[:k], th, dl)
+
+    def jac1(o, X, k):
+        return o.jac(None if X is None else X[0], th, dth, dl)
+
+    def jacT(o, X, k):
+        g = torch.zeros(k, V, dtype=torch.float64, device="cuda")
+        ct.ct_jacT_batch(o.h, th, dl, None if X is None else X[:k].contiguous(), R, g, None, k)
+        return g
+
+    def gn(o, X, k):
+        out = [torch.zeros(k, V, dtype=torch.float64, device="cuda") for _ in range(3)]
+        ct.ct_gn_terms_batch(o.h, th, dl, None if X is None else X[:k].contiguous(), R, None, *out, k)
+        return torch.stack(out)
+
+    calls = [(f, k) for f in (fwd, jac1, jacT, gn) for k in {1, 2, (K + 1) // 2, K}]
+    for trial in range(12):
+        X = X0[trial % 2]
+        first = (fwd, jacT)[trial % 2 if der_kb == 4 else 0]
+        first(op, X, K)
+        for q in rng.permutation(len(calls))[:8]:
+            f, k = calls[q]
+            assert torch.equal(f(op, None, k), f(other, X, k)), (trial, f.__name__, k)
+    for op in ops:
+        op.close()
+
+
+def test_interleaved_images_take_no_memory_of_their_own():
+    """A handle that starts on interleaved images allocates what the pair images, the sinograms and the
+    partials take (in 2 MB pieces), and selecting the layout allocates nothing."""
+    from paper_2605_06336_gb300 import ct
+    N, V, K = 1024, 60, 8
+    B = synth.n_bins(N)
+
+    def used():
+        torch.cuda.synchronize()
+        free, total = torch.cuda.mem_get_info()
+        return total - free
+    ct.CTOperator(64, 91, 8, max_batch=K).close()  # the context and the kernels are loaded
+    before = used()
+    op = ct.CTOperator(N, B, V, max_batch=K, dtype=torch.float32)
+    made = used() - before
+    assert op.tuning[11] == 1
+    pairs, sino, partials = 2 * (K + 1) * N * (N + 4) * 8, K * V * (B + 5) * 8, 32 * K * V * ((B + 31) // 32)
+    assert made <= pairs + sino + partials + 24 * 2 ** 20
+    op.tuning = [4, 2, 2, 4, 1, 4, 1, 0, 0, 0, 1, 1]
+    assert used() - before <= made
+    op.close()
+
+
 # the source as near as the geometry takes it (0.75 max(N, B) + 2): wide ray windows at the far side
 FAN = [(33, [9], 1), (48, [5, 0, 6], 3), (65, [12], 8)]
 
