@@ -211,10 +211,13 @@ __device__ __forceinline__ void warp_rows(const ViewGeo &g, int b, bool active, 
 // two-word shift, two clamps and a second shift (the integer pipe was the bound
 // of one image per lane: 74 % busy, now 58).  The same bits as cell_of and
 // frac_of.  One image of 2048^2, 120 views: 362 -> 282 us; 256^2 / 180 views:
-// 18.6 -> 16.3.  FP64: the indices alone; ray_frac gives a row's fraction when
-// its sum is formed (an FP64 subtraction, not to be spent on the rows past a
-// segment's end).
-template <typename T, int U>
+// 18.6 -> 16.3.  FP64 without FRAC: the indices alone; ray_frac gives a row's
+// fraction when its sum is formed (an FP64 subtraction, not spent on the rows
+// past a segment's end: the fan beam's choice, 130^2 / 180 views, J of 8 images
+// 468 -> 399 us with the sums of those rows left out too; the parallel beam, whose
+// segments end together, is faster with the fractions of a block formed ahead of
+// its loads: 32^2 / 360 views, 4 images, forward 20.4 us against 24.7).
+template <typename T, int U, bool FRAC>
 __device__ __forceinline__ void ray_cells(long long Q, long long dQ, unsigned lim, unsigned (&idx)[U], T (&f)[U])
 {
     if constexpr (std::is_same<T, float>::value) {
@@ -231,7 +234,9 @@ __device__ __forceinline__ void ray_cells(long long Q, long long dQ, unsigned li
     } else {
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            idx[u] = min((unsigned)(cell_of(Q + (long long)u * dQ) + 2), lim);
+            const long long Qu = Q + (long long)u * dQ;
+            idx[u] = min((unsigned)(cell_of(Qu) + 2), lim);
+            if constexpr (FRAC) f[u] = frac_of(Qu, T());
         }
     }
 }

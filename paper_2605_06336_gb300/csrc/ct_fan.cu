@@ -221,7 +221,7 @@ __global__ void __launch_bounds__(32 * SPLIT) k_ray_fan(RayArgs<T> a, const FanR
             unsigned idx[U];
             T f[U];
             P2 p[U][KB];
-            ray_cells<T, U>(Q, dQ, lim, idx, f);
+            ray_cells<T, U, false>(Q, dQ, lim, idx, f);
 #pragma unroll
             for (int u = 0; u < U; ++u) {
 #pragma unroll

@@ -641,7 +641,7 @@ __global__ void __launch_bounds__(512) k_ray(RayArgs<T> a)
                 unsigned idx[U];
                 T f[U];
                 P2 p[U][KB];
-                ray_cells<T, U>(Q, dQ, lim, idx, f);
+                ray_cells<T, U, true>(Q, dQ, lim, idx, f);
 #pragma unroll
                 for (int u = 0; u < U; ++u) {
                     if (WHOLE || u < rows) {
@@ -661,9 +661,9 @@ __global__ void __launch_bounds__(512) k_ray(RayArgs<T> a)
 #pragma unroll
                     for (int u = 0; u < U; ++u) {
                         if (!F32 && !WHOLE && u >= rows) break;  // FP64 products are dear (uniform)
-                        const T fu = ray_frac<T, U>(Q, dQ, f, u), omf = T(1) - fu;
+                        const T omf = T(1) - f[u];
 #pragma unroll
-                        for (int k = 0; k < KB; ++k) acc[k] = fma(omf, p[u][k].x, fma(fu, p[u][k].y, acc[k]));
+                        for (int k = 0; k < KB; ++k) acc[k] = fma(omf, p[u][k].x, fma(f[u], p[u][k].y, acc[k]));
                     }
                 } else {
                     // per image k of the group: acc[3k] = sum of interpolated values,
@@ -672,12 +672,11 @@ __global__ void __launch_bounds__(512) k_ray(RayArgs<T> a)
 #pragma unroll
                     for (int u = 0; u < U; ++u) {
                         if (!F32 && !WHOLE && u >= rows) break;
-                        const T fu = ray_frac<T, U>(Q, dQ, f, u);
                         const T dq = fma(rf + T(u), gr, g0);
 #pragma unroll
                         for (int k = 0; k < KB; ++k) {
                             const T d = p[u][k].y - p[u][k].x;
-                            acc[3 * k] += fma(fu, d, p[u][k].x);
+                            acc[3 * k] += fma(f[u], d, p[u][k].x);
                             acc[3 * k + 1] = fma(d, dq, acc[3 * k + 1]);
                             if (OFFS) acc[3 * k + 2] += d;
                         }
