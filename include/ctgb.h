@@ -265,7 +265,9 @@ int ct_autotune(ct_handle *h);
  *   staging 0, [0] 4 or 8; the forward then reads both taps of 4 images with
  *   two 16-byte loads; the interleaved images take half of the memory of the
  *   pair images, which they replace).  1 is what FP32 parallel-beam handles
- *   with [0] of 4 or 8 start with.  CT_ERR_ARG on an FP64 or fan-beam handle.
+ *   with [0] of 4 or 8 start with; such a handle stores 0 instead where [0]
+ *   or [7] rule it out, any other answers CT_ERR_ARG.  CT_ERR_ARG on an FP64 or
+ *   fan-beam handle.
  * [0]..[6] are powers of two, at most 8 (view groups at most 4), warps per
  * ray x views per CTA at most 16 (unstaged kernels).  Forward / Jacobian
  * staging is 0 (gathers through L1) or 4 / 8 (rows per shared-memory block of

@@ -601,7 +601,8 @@ int ct_init(const ct_geom *g, void *cuda_stream, ct_handle **out)
         return rc;
     }
     default_tuning(h);
-    if (h.tune.fwd_kb >= 4 && h.precision == 0 && h.fan_D == 0.0) h.tune.fwd_layout = 1;
+    h.own_layout = h.tune.fwd_kb >= 4 && h.precision == 0 && h.fan_D == 0.0;
+    h.tune.fwd_layout = h.own_layout;
     *out = H;
     return CT_OK;
 }
@@ -759,13 +760,20 @@ int ct_set_tuning(ct_handle *H, const int32_t *in)
         !pow2(in[5], 8) || !pow2(in[6], 8) || (in[7] == 0 && in[1] * in[2] > 16) ||
         (in[8] == 0 && in[5] * in[6] > 16) || !stage_ok(in[7], in[2]) || !stage_ok(in[8], in[6]) ||
         (in[7] > 0 && in[1] > 4) || (in[9] != 0 && in[9] != 8 && in[9] != 16) || !pow2(in[10], 4) ||
-        (in[11] != 0 && in[11] != 1) || (in[11] == 1 && (in[7] != 0 || in[0] < 4)))
+        (in[11] != 0 && in[11] != 1))
         return CT_ERR_ARG;
+    // Layout 1 needs an unstaged forward of 4 or 8 images per lane.  A handle that started
+    // with it takes it as a wish: its own values with [0] or [7] changed stay valid.
+    int layout = in[11];
+    if (layout == 1 && (in[7] != 0 || in[0] < 4)) {
+        if (!H->h.own_layout) return CT_ERR_ARG;
+        layout = 0;
+    }
     if (in[7] > 0 && in[1] > 1) {
         const int rc = ensure_seg_partials(H->h);
         if (rc != CT_OK) return rc;
     }
-    if (in[11] == 1 && (H->h.precision != 0 || H->h.fan_D > 0.0)) return CT_ERR_ARG;
+    if (layout == 1 && (H->h.precision != 0 || H->h.fan_D > 0.0)) return CT_ERR_ARG;
     ctgb::Tuning &t = H->h.tune;
     t.fwd_kb = in[0];
     t.fwd_split = in[1];
@@ -778,7 +786,7 @@ int ct_set_tuning(ct_handle *H, const int32_t *in)
     t.der_stage = in[8];
     t.adj_stage = in[9];
     t.der_kb = in[10];
-    t.fwd_layout = in[11];
+    t.fwd_layout = layout;
     return CT_OK;
 }
 

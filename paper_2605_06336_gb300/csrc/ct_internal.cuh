@@ -242,6 +242,7 @@ struct Handle {
     float *qt() const { return (float *)d_pt + ((max_batch * img_elems() + 3) & ~3LL); }
     int num_sms = 0;
     Tuning tune;
+    bool own_layout = false;  // fwd_layout 1 was the handle's own choice at ct_init
 };
 
 // Kernel launchers.  All launch on h.stream and return the launch status.

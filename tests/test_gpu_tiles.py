@@ -225,6 +225,27 @@ def test_products_of_fewer_images_after_an_interleaved_call(max_batch, der_kb):
         op.close()
 
 
+def test_one_changed_value_of_a_handles_own_tuning_is_taken():
+    """Handles that start on interleaved images: their values with any one of the forward's changed are valid."""
+    from paper_2605_06336_gb300 import ct
+    N, V, K = 40, 9, 8
+    B = synth.n_bins(N)
+    rng = np.random.default_rng(0)
+    op = ct.CTOperator(N, B, V, max_batch=K, dtype=torch.float32)
+    theta, X = rng.uniform(-3, 3, V), rng.uniform(size=(K, N * N))
+    ref = oracle.forward(oracle.Geometry(N, B, V), theta, X)
+    own = op.tuning
+    assert own[0] >= 4 and own[7] == 0 and own[11] == 1
+    for change, layout in (({0: 1}, 0), ({0: 2}, 0), ({0: 8}, 1), ({2: 8, 7: 8}, 0), ({2: 4, 7: 4, 1: 1}, 0), ({}, 1)):
+        t = list(own)
+        for i, v in change.items():
+            t[i] = v
+        op.tuning = t
+        assert op.tuning == t[:11] + [layout]
+        assert rel(host(op.forward(dev(X, torch.float32), dev(theta))), ref) <= TOL[torch.float32]
+    op.close()
+
+
 def test_interleaved_images_take_no_memory_of_their_own():
     """A handle that starts on interleaved images allocates what the pair images, the sinograms and the
     partials take (in 2 MB pieces), and selecting the layout allocates nothing."""
