@@ -313,6 +313,10 @@ __global__ void __launch_bounds__(256, 5) k_pairs_img(const T *__restrict__ X, p
     }
 }
 
+constexpr size_t kInterleaveTile = sizeof(float) * 4 * 32 * 33;
+static_assert(kInterleaveTile <= 48 * 1024 && sizeof(unsigned long long) * kOrderMaxV + sizeof(double) * 33 * 33 <= 47 * 1024,
+              "tiles and keys fit the shared memory of a launch as they are");
+
 // X -> interleaved images of X and X^T (FP32): each CTA reads a 32 x 32 tile
 // of the images of one group, of one frame, from (r0, c0) on (both from -2 in
 // steps of 32), once; a thread has the group's images at its elements side by
@@ -333,7 +337,9 @@ __global__ void __launch_bounds__(256, 5) k_interleave_img(const float *__restri
         if (part < p.on) view_prep_block(p, part, prep_key);
         return;
     }
-    __shared__ float t[4][32][33];  // t[j][i][e] = X_j[r0 + i][c0 + e]
+    // t[j][i][e] = X_j[r0 + i][c0 + e], where the CTAs of the step have their keys: both
+    // together would pass the 48 KB that a launch may use without asking the device
+    float (*t)[32][33] = reinterpret_cast<float (*)[32][33]>(prep_key);
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
     const int r0 = blockIdx.y * 32 - 2, c0 = blockIdx.x * 32 - 2;
     const int n4 = K & ~3, rem = K - n4;
@@ -858,17 +864,6 @@ size_t prep_smem(const ViewPrep &p)
 // Columns of CTAs that an image layout launch adds for the step.
 unsigned prep_columns(const ViewPrep &p, dim3 grid) { return (p.on + grid.y * grid.z - 1) / (grid.y * grid.z); }
 
-// The layout kernels may carry the view-table step in up to 32 KB of dynamic shared memory.
-template <auto Kernel> cudaError_t allow_prep_smem()
-{
-    static bool done = false;  // one flag per kernel; the attribute is idempotent, so a race is harmless
-    if (done) return cudaSuccess;
-    cudaError_t e = cudaFuncSetAttribute(Kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)(sizeof(unsigned long long) * kOrderMaxV));
-    if (e == cudaSuccess) done = true;
-    return e;
-}
-
 }  // namespace
 
 cudaError_t launch_view_setup(const Handle &h, const double *theta, const double *delta, const int *skip)
@@ -888,14 +883,12 @@ cudaError_t launch_pairs_img(const Handle &h, const T *X, int nimg, const int *s
                              const double *delta)
 {
     const ViewPrep p = view_prep_args(h, theta, delta);
-    cudaError_t e = allow_prep_smem<k_pairs_img<T>>();
-    if (e != cudaSuccess) return e;
     dim3 grid((h.Pp + 31) / 32, (h.Pp + 31) / 32, std::max(1, std::min(nimg, 65535)));
     grid.x += prep_columns(p, grid);
     launch_chained(k_pairs_img<T>, grid, 256, prep_smem(p), h.stream, X, (pair_t<T> *)h.d_px, (pair_t<T> *)h.d_pt, h.N, h.Pp,
                                                           nimg, p, skip);
     if (h.fan_D > 0.0 && theta) {
-        e = cudaGetLastError();
+        const cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
         return launch_fan_rays(h, skip);
     }
@@ -914,13 +907,11 @@ cudaError_t launch_interleave_img(const Handle &h, const float *X, int batch, co
 {
     if (h.precision != 0 || h.fan_D > 0.0 || batch < 1 || batch > h.max_batch) return cudaErrorInvalidValue;
     const ViewPrep p = view_prep_args(h, theta, delta);
-    cudaError_t e = allow_prep_smem<k_interleave_img>();
-    if (e != cudaSuccess) return e;
     const int n4 = batch & ~3, rem = batch - n4;
     const int ngroups = n4 / 4 + (rem >= 2 ? 1 : 0) + (rem & 1);
     dim3 grid((h.Pp + 31) / 32, (h.Pp + 31) / 32, std::max(1, std::min(h.F * ngroups, 65535)));
     grid.x += prep_columns(p, grid);
-    launch_chained(k_interleave_img, grid, 256, prep_smem(p), h.stream, X, h.qx(), h.qt(), h.N, h.Pp, h.F, batch, p, skip);
+    launch_chained(k_interleave_img, grid, 256, std::max(prep_smem(p), kInterleaveTile), h.stream, X, h.qx(), h.qt(), h.N, h.Pp, h.F, batch, p, skip);
     return cudaGetLastError();
 }
 
@@ -959,15 +950,11 @@ cudaError_t launch_sino_layout(const Handle &h, const T *Y, int nsino, int kb, c
         SinoGroup g[2];
         const int ng = sino_groups(nsino, kb, g);
         const int groups = g[ng - 1].first + g[ng - 1].count;
-        cudaError_t e = allow_prep_smem<k_interleave_sino>();
-        if (e != cudaSuccess) return e;
         const long long rows = (long long)groups * h.V;
         const int blocks = (int)std::min<long long>(rows, (long long)h.num_sms * 16);
         launch_chained(k_interleave_sino, blocks + p.on, 256, prep_smem(p), h.stream, 
             Y, (float *)h.d_yp, h.d_rowflag, h.B, sino_pitch(h.B), h.V, nsino, kb, rows, p, skip);
     } else {
-        cudaError_t e = allow_prep_smem<k_pairs_sino>();
-        if (e != cudaSuccess) return e;
         const long long total = (long long)nsino * h.V * h.Pb;
         const int threads = 256;
         const long long blocks = std::min<long long>((total + threads - 1) / threads, (long long)h.num_sms * 16);

@@ -137,7 +137,7 @@ def test_repeated_transpose_of_fewer_sinograms_gives_the_same_bits(case, dtype, 
 
 
 # N, views, batch: the order of the views (counted, sorted, none) and the CTAs of the view table
-VIEWS = [(16, 255, 1), (16, 256, 2), (16, 257, 1), (8, 512, 1), (8, 513, 4), (8, 1200, 1), (8, 4096, 1), (8, 4097, 2)]
+VIEWS = [(16, 255, 1), (16, 256, 2), (16, 257, 1), (8, 512, 1), (8, 513, 4), (8, 1200, 1), (8, 2049, 4), (8, 4096, 1), (8, 4096, 5), (8, 4097, 2)]
 
 
 @pytest.mark.parametrize("dtype", [torch.float32, torch.float64])
