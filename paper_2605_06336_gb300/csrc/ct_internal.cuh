@@ -120,6 +120,18 @@ __host__ __device__ inline void interleave_group(int k, int K, int &k0, int &w)
     }
 }
 
+// Key of view i in the order of the ray kernels: frame, marching axis, ray
+// slope, index.  12 bits of the frame, the axis, the leading 39 of 48 bits of the
+// fixed-point slope |Qh| <= 2^47 (a diagonal's 2^47 taken one lower, where it
+// would carry into the axis) and 12 bits of the index, so that no two of up to
+// 4096 views are alike; integer compares, as the FP64 pipe of this part is narrow.
+__host__ __device__ inline unsigned long long order_key(int frame, int mode, long long Qh, int i)
+{
+    const unsigned long long q = (unsigned long long)(Qh + (1LL << 47)), top = (1ULL << 48) - 1;
+    return ((unsigned long long)(frame & 0xfff) << 52) | ((unsigned long long)mode << 51) |
+           (q < top ? q : top) >> 9 << 12 | (unsigned long long)i;
+}
+
 // Groups of the interleaved sinogram layout of `batch` sinograms at kb per
 // group: up to two runs of `count` groups of one width, run q starting at
 // sinogram k0 and group number `first`.  Returns the number of runs.

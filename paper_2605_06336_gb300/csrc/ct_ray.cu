@@ -196,18 +196,11 @@ __device__ void build_order(const ViewPrep &p, unsigned long long *key)
         for (int i = threadIdx.x; i < V; i += blockDim.x) p.order[i] = i;
         return;
     }
-    // One unsigned 64-bit key per view orders by (frame, axis, slope, index):
-    // 12 bits of the frame, the axis, the leading 39 bits of the fixed-point
-    // slope |Qh| < 2^47 (offset into 48 bits) and 12 bits of the index, so that
-    // no two are alike; integer compares, as the FP64 pipe of this part is narrow.
     int P = V;
     if (V > kOrderRankMaxV)
         for (P = 2 * kOrderRankMaxV; P < V;) P *= 2;
     for (int i = threadIdx.x; i < P; i += blockDim.x)
-        key[i] = i < V ? ((unsigned long long)(p.vg[i].frame & 0xfff) << 52) |
-                             ((unsigned long long)p.vg[i].mode << 51) |
-                             ((unsigned long long)(p.vg[i].Qh + (1LL << 47)) >> 9 << 12) | i
-                       : ~0ULL;
+        key[i] = i < V ? order_key(p.vg[i].frame, p.vg[i].mode, p.vg[i].Qh, i) : ~0ULL;
     __syncthreads();
     // Up to one view per thread the rank of a view counts the keys below it (V
     // steps); above, a bitonic sort: 1200 views in 66 steps of 4 exchanges a

@@ -15,8 +15,9 @@ int main(int argc, char **argv)
 {
     long long r, v[6] = {};
     while (std::scanf("%lld %lld %lld %lld %lld %lld %lld", &r, v, v + 1, v + 2, v + 3, v + 4, v + 5) == 7)
-        std::printf("%d\n", r == 0 ? ctgb::adj_cluster_size((int)v[0], v[1], (int)v[2], (int)v[3], (int)v[4], (int)v[5])
-                                   : ctgb::adj_group_width((int)v[0], (int)v[1], v[2], (int)v[3], (int)v[4]));
+        std::printf("%llu\n", r == 0   ? (unsigned long long)ctgb::adj_cluster_size((int)v[0], v[1], (int)v[2], (int)v[3], (int)v[4], (int)v[5])
+                              : r == 1 ? (unsigned long long)ctgb::adj_group_width((int)v[0], (int)v[1], v[2], (int)v[3], (int)v[4])
+                                       : ctgb::order_key((int)v[0], (int)v[1], v[2], (int)v[3]));
 }
 """
 
@@ -67,3 +68,14 @@ def test_few_views_take_one_cta_and_narrow_groups(rules):
     assert rules(rows, rule=1) == [1, 2, 1, 4, 8, 2]
     rows = [(kb, K, t, v, 152) for kb, K in ((1, 1), (2, 3), (4, 7), (8, 9)) for t in (9, 64, 4096) for v in (1, 30, 1200)]
     assert all(1 <= w <= r[0] for w, r in zip(rules(rows, rule=1), rows))
+
+
+def test_view_keys_sort_by_frame_axis_slope_and_index(rules):
+    """Slopes up to and including the diagonals', whose fixed-point value is 2^47 itself."""
+    h = 1 << 47
+    rows = [(f, mode, q, i) for f in (0, 1, 4095) for mode in (0, 1)
+            for q, i in ((-h, 5), (-h, 9), (-h + 512, 2), (-1, 4095), (0, 7), (h - 1024, 3), (h, 0), (h, 4))]
+    keys = rules(rows, rule=2)
+    assert keys == sorted(keys) and len(set(keys)) == len(keys)
+    for (f, mode, _, i), k in zip(rows, keys):
+        assert (k >> 52, k >> 51 & 1, k & 0xfff) == (f, mode, i)
