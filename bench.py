@@ -73,7 +73,7 @@ def launches_per_step(t):
     layout of the J call and brings the view table up to date (1); the forward
     ray kernel(s) over the 8-image block, the transpose, the JVP, the VJP and
     its per-view reduction; the staged forward with several CTAs per ray adds
-    a combining kernel (the staged transpose combines its CTAs per tile inside
+    a combining kernel (the transpose combines its CTAs per tile inside
     their thread-block cluster)."""
     fkb, fsplit, _, akb, asplit, _, _, fstage, _, astage = t[:10]
     fwd = 0

@@ -27,6 +27,12 @@ template <typename T> using pair_t = typename Pair<T>::type;
 // H^T, four launches: 38.9 -> 29.6 us a pass.  No kernel triggers its successor
 // before it ends: resident early, the successor's CTAs take the places of the
 // predecessor's last ones (42.4 us with the trigger at entry).
+// What this relies on: a kernel reads what its predecessor wrote also through
+// read-only loads (__ldg, const __restrict__), whose data must not change while the
+// kernel runs; these have to stay behind the wait.  The wait is volatile and clobbers
+// memory, it is the first statement of every kernel, and each such load is
+// under a condition or in a loop that comes after it.  A new kernel keeps to
+// that, and none may signal its successor before its last write.
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 template <typename... KA, typename... A>
@@ -109,12 +115,6 @@ __device__ __forceinline__ void floor_split(float t, int &m, float &f)
     const float tr = __fadd_rn(__fsub_rn(t, 0.5f), magic);
     m = __float_as_int(tr) - 0x4B400000;
     f = __fsub_rn(t, __fsub_rn(tr, magic));
-}
-__device__ __forceinline__ void floor_split(double t, int &m, double &f)
-{
-    const double fl = floor(t);
-    m = (int)fl;
-    f = t - fl;
 }
 
 // Per-view derivative constants in the working precision.  The FP64 form

@@ -621,25 +621,15 @@ __global__ void __launch_bounds__(256) k_adj_fan_tile(FanTileArgs a)
 
 struct AdjFanArgs {
     const int *fstart, *fcount;
-    int N, B, F, tps, Pb, kbase, ngroups;
+    int N, B, F, tps, kbase, ngroups;
     long long ysino_stride, img_stride;
     const int *skip;
 };
 
-// The KB values of one bin in the interleaved layout (16-byte loads where the
-// group is 16-byte aligned: FP32 groups of 4 or 8, FP64 groups of 2 or more).
-template <typename T, int KB> __device__ __forceinline__ void load_bin(const T *p, T (&out)[KB])
+// The KB values of one bin in the interleaved layout (16-byte loads from groups of 2 on).
+template <int KB> __device__ __forceinline__ void load_bin(const double *p, double (&out)[KB])
 {
-    if constexpr (std::is_same<T, float>::value && KB % 4 == 0) {
-#pragma unroll
-        for (int q = 0; q < KB / 4; ++q) {
-            const float4 v = __ldg(reinterpret_cast<const float4 *>(p) + q);
-            out[4 * q] = v.x;
-            out[4 * q + 1] = v.y;
-            out[4 * q + 2] = v.z;
-            out[4 * q + 3] = v.w;
-        }
-    } else if constexpr (std::is_same<T, double>::value && KB % 2 == 0) {
+    if constexpr (KB % 2 == 0) {
 #pragma unroll
         for (int q = 0; q < KB / 2; ++q) {
             const double2 v = __ldg(reinterpret_cast<const double2 *>(p) + q);
@@ -656,13 +646,13 @@ template <typename T, int KB> __device__ __forceinline__ void load_bin(const T *
 // thread groups of 256: group g of a pixel sums the views vs + g, vs + g +
 // SPLIT, ... of its frame in order; the groups' sums are added in group
 // order in shared memory.
-template <typename T, int KB, int SPLIT>
-__global__ void __launch_bounds__(256 * SPLIT) k_adj_fan(AdjFanArgs a, const FanLine<T> *__restrict__ rays,
+template <int KB, int SPLIT>
+__global__ void __launch_bounds__(256 * SPLIT) k_adj_fan(AdjFanArgs a, const FanLine<double> *__restrict__ rays,
                                                          const FanView *__restrict__ views,
-                                                         const T *__restrict__ YI, T *__restrict__ X)
+                                                         const double *__restrict__ YI, double *__restrict__ X)
 {
     chain_wait();
-    __shared__ T red[SPLIT > 1 ? SPLIT - 1 : 1][KB][256];
+    __shared__ double red[SPLIT > 1 ? SPLIT - 1 : 1][KB][256];
     const int pix = threadIdx.x & 255, grp_v = threadIdx.x >> 8;
     const int tx = pix & (kTile - 1), ty = pix / kTile;
     const int N = a.N;
@@ -680,16 +670,16 @@ __global__ void __launch_bounds__(256 * SPLIT) k_adj_fan(AdjFanArgs a, const Fan
         const bool inside = i < N && j < N;
         const float x = (float)j - h, y = h - (float)i;
         const long long Qrow = (long long)(2 * i - (N - 1)), Qcol = (long long)(2 * j - (N - 1));
-        T acc[KB];
+        double acc[KB];
 #pragma unroll
-        for (int k = 0; k < KB; ++k) acc[k] = T(0);
+        for (int k = 0; k < KB; ++k) acc[k] = 0.0;
         const int vs = a.fstart[f], vc = a.fcount[f];
         for (int v = vs + grp_v; inside && v < vs + vc; v += SPLIT) {
             const FanView fv = views[v];
-            const FanLine<T> *rv = rays + (size_t)v * a.B;
+            const FanLine<double> *rv = rays + (size_t)v * a.B;
             // the KB sinograms of this group at bin b: KB consecutive values (KB divides 8, and a
             // group starts at a multiple of its width)
-            const T *yv = YI + ((size_t)(k0 >> 3) * a.ysino_stride + (size_t)v * a.B) * 8 + (k0 & 7);
+            const double *yv = YI + ((size_t)(k0 >> 3) * a.ysino_stride + (size_t)v * a.B) * 8 + (k0 & 7);
             // rays marched along rows that sample row i inside (x - 1, x + 1), then
             // rays marched along columns that sample column j inside (y - 1, y + 1)
 #pragma unroll
@@ -708,10 +698,10 @@ __global__ void __launch_bounds__(256 * SPLIT) k_adj_fan(AdjFanArgs a, const Fan
                     const long long Q = rv[b].Qc + Qr * rv[b].Qh;
                     const int cell = cell_of(Q);
                     if (cell != me && cell != me - 1) continue;
-                    const T fr = frac_of(Q, T());
-                    const T wt = rv[b].w * (cell == me ? T(1) - fr : fr);
-                    T yk[KB];
-                    load_bin<T, KB>(yv + (size_t)b * 8, yk);
+                    const double fr = frac_of(Q, 0.0);
+                    const double wt = rv[b].w * (cell == me ? 1.0 - fr : fr);
+                    double yk[KB];
+                    load_bin<KB>(yv + (size_t)b * 8, yk);
 #pragma unroll
                     for (int k = 0; k < KB; ++k) acc[k] = fma(wt, yk[k], acc[k]);
                 }
@@ -759,20 +749,20 @@ cudaError_t run_fan_split(const Handle &h, const RayArgs<T> &a, int split)
     }
 }
 
-template <typename T, int KB, int SPLIT> cudaError_t run_adj_fan(const Handle &h, const AdjFanArgs &a, T *X)
+template <int KB, int SPLIT> cudaError_t run_adj_fan(const Handle &h, const AdjFanArgs &a, double *X)
 {
-    auto kern = k_adj_fan<T, KB, SPLIT>;
+    auto kern = k_adj_fan<KB, SPLIT>;
     const long long items = (long long)a.ngroups * a.F * a.tps * a.tps;
     const int grid = persistent_grid(kern, 256 * SPLIT, 0, items, h.num_sms);
-    launch_chained(kern, grid, 256 * SPLIT, 0, h.stream, a, fan_lines<T>(h.d_rays, (long long)h.V * h.B),
-                                             (const FanView *)h.d_fanview, (const T *)h.d_yi, X);
+    launch_chained(kern, grid, 256 * SPLIT, 0, h.stream, a, fan_lines<double>(h.d_rays, (long long)h.V * h.B),
+                                             (const FanView *)h.d_fanview, (const double *)h.d_yi, X);
     return cudaGetLastError();
 }
 
-template <typename T, int KB> cudaError_t run_adj_fan_split(const Handle &h, const AdjFanArgs &a, T *X, int split)
+template <int KB> cudaError_t run_adj_fan_split(const Handle &h, const AdjFanArgs &a, double *X, int split)
 {
-    return split >= 4 ? run_adj_fan<T, KB, 4>(h, a, X)
-                      : (split >= 2 ? run_adj_fan<T, KB, 2>(h, a, X) : run_adj_fan<T, KB, 1>(h, a, X));
+    return split >= 4 ? run_adj_fan<KB, 4>(h, a, X)
+                      : (split >= 2 ? run_adj_fan<KB, 2>(h, a, X) : run_adj_fan<KB, 1>(h, a, X));
 }
 
 }  // namespace
@@ -870,7 +860,6 @@ cudaError_t launch_fan_adjoint(const Handle &h, T *X, int batch, int kb, int spl
         a.B = h.B;
         a.F = h.F;
         a.tps = (h.N + kTile - 1) / kTile;
-        a.Pb = h.Pb;
         a.ysino_stride = (long long)h.V * h.B;  // per block of 8 interleaved sinograms, in bins
         a.img_stride = (long long)h.F * h.N * h.N;
         a.skip = skip;
@@ -883,10 +872,10 @@ cudaError_t launch_fan_adjoint(const Handle &h, T *X, int batch, int kb, int spl
             a.ngroups = groups;
             cudaError_t e;
             switch (width) {
-            case 1: e = run_adj_fan_split<double, 1>(h, a, X, split); break;
-            case 2: e = run_adj_fan_split<double, 2>(h, a, X, split); break;
-            case 4: e = run_adj_fan_split<double, 4>(h, a, X, split); break;
-            default: e = run_adj_fan_split<double, 8>(h, a, X, split); break;
+            case 1: e = run_adj_fan_split<1>(h, a, X, split); break;
+            case 2: e = run_adj_fan_split<2>(h, a, X, split); break;
+            case 4: e = run_adj_fan_split<4>(h, a, X, split); break;
+            default: e = run_adj_fan_split<8>(h, a, X, split); break;
             }
             if (e != cudaSuccess) return e;
             k += groups * width;

@@ -324,8 +324,7 @@ cudaError_t launch_gn(const Handle &h, const T *bdata, T *res, double *grad, dou
 
 // Fan beam (ct_fan.cu).  launch_fan_rays rebuilds the per-ray table from the
 // view table; every launcher that brings the view table up to date runs it
-// on a fan-beam handle.  The transpose of a fan-beam handle reads the pair
-// sinograms like the parallel-beam one.
+// on a fan-beam handle.
 size_t fan_ray_bytes(int precision);
 size_t fan_view_bytes();
 // YI[k / 8][v][b][k % 8] = Y[k][v][b]: the 8 sinograms of a block at one bin
