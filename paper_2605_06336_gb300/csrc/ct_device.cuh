@@ -31,8 +31,9 @@ template <typename T> using pair_t = typename Pair<T>::type;
 // read-only loads (__ldg, const __restrict__), whose data must not change while the
 // kernel runs; these have to stay behind the wait.  The wait is volatile and clobbers
 // memory, it is the first statement of every kernel, and each such load is
-// under a condition or in a loop that comes after it.  A new kernel keeps to
-// that, and none may signal its successor before its last write.
+// under a condition or in a loop that comes after it, or volatile: a load that
+// the compiler may move but not speculate has nowhere ahead of it to go.  A new
+// kernel keeps to that, and none may signal its successor before its last write.
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 template <typename... KA, typename... A>

@@ -1493,7 +1493,7 @@ __global__ void __launch_bounds__(256) k_compress_basis(const double *__restrict
     extern __shared__ unsigned char smem_raw[];
     constexpr int kLd = SmallShared<KM>::kLd;
     SmallShared<KM> &S = *reinterpret_cast<SmallShared<KM> *>(KM > kKSmem ? (unsigned char *)work : smem_raw);
-    const double lam = scal[kLam];
+    const double lam = *static_cast<const volatile double *>(scal + kLam);  // (not ahead of the wait, see chain_wait)
     for (int idx = threadIdx.x; idx < k * k; idx += blockDim.x) {
         const int i = idx / k, j = idx % k;
         S.A[i * kLd + j] = GH[i * kKMax + j] + lam * GP[i * kKMax + j];
