@@ -739,26 +739,32 @@ __global__ void __launch_bounds__(256) k_dots(const T *__restrict__ A, long long
         int run = 0;
         for (long long i = lo + threadIdx.x; i < hi; i += blockDim.x) {
             const float xi = x[i];
+            float v[G];  // (all loads unconditional, so that they are in flight together)
 #pragma unroll
-            for (int q = 0; q < G; ++q)
-                if (q < na) fr[q] = fmaf(cols[q][i], xi, fr[q]);
+            for (int q = 0; q < G; ++q) v[q] = cols[q][i];
+#pragma unroll
+            for (int q = 0; q < G; ++q) fr[q] = fmaf(v[q], xi, fr[q]);
             if (++run == 16) {
 #pragma unroll
                 for (int q = 0; q < G; ++q) {
-                    s[q] += (double)fr[q];
+                    if (q < na) s[q] += (double)fr[q];  // uniform
                     fr[q] = 0.0f;
                 }
                 run = 0;
             }
         }
 #pragma unroll
-        for (int q = 0; q < G; ++q) s[q] += (double)fr[q];
+        for (int q = 0; q < G; ++q)
+            if (q < na) s[q] += (double)fr[q];
     } else {
         for (long long i = lo + threadIdx.x; i < hi; i += blockDim.x) {
             const T xi = x[i];
+            T v[G];
+#pragma unroll
+            for (int q = 0; q < G; ++q) v[q] = cols[q][i];
 #pragma unroll
             for (int q = 0; q < G; ++q)
-                if (q < na) s[q] = fma(cols[q][i], xi, s[q]);
+                if (q < na) s[q] = fma(v[q], xi, s[q]);
         }
     }
 #pragma unroll
@@ -795,19 +801,26 @@ __global__ void __launch_bounds__(32 * kDotsReduceWarps) k_dots_reduce(const dou
     if (lane == 0) out[a] = s;
 }
 
-// sum_a A[a][i] * y[a], added in column order, 16 columns' loads in flight
+// sum_a A[a][i] * y[a], added in column order, 16 columns' loads in flight and
+// then 4 (no condition around the loads: past the last column they repeat it)
+template <int W, typename T>
+__device__ __forceinline__ T gemv_block(const T *__restrict__ A, long long lda, int a0, int k, const T *ys, long long i, T s)
+{
+    T v[W];
+#pragma unroll
+    for (int q = 0; q < W; ++q) v[q] = A[(long long)min(a0 + q, k - 1) * lda + i];
+#pragma unroll
+    for (int q = 0; q < W; ++q)
+        if (a0 + q < k) s = fma(v[q], ys[a0 + q], s);
+    return s;
+}
 template <typename T>
 __device__ __forceinline__ T gemv_row(const T *__restrict__ A, long long lda, int k, const T *ys, long long i)
 {
     T s = T(0);
-    for (int a0 = 0; a0 < k; a0 += 16) {
-        T v[16];
-#pragma unroll
-        for (int q = 0; q < 16; ++q) v[q] = a0 + q < k ? A[(long long)(a0 + q) * lda + i] : T(0);
-#pragma unroll
-        for (int q = 0; q < 16; ++q)
-            if (a0 + q < k) s = fma(v[q], ys[a0 + q], s);
-    }
+    int a = 0;
+    for (; a + 16 <= k; a += 16) s = gemv_block<16>(A, lda, a, k, ys, i, s);
+    for (; a < k; a += 4) s = gemv_block<4>(A, lda, a, k, ys, i, s);
     return s;
 }
 
