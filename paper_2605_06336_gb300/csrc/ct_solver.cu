@@ -451,7 +451,8 @@ template <typename T> struct Solver {
         SV_TRY(cgs2(r, kc, stop));
         // |r|^2; |u|^2, |u - u_old|^2, |u_old|^2; u_old = u; the next step's weights
         const int nblk = red_blocks(n);
-        launch_chained(k_step_norms<T>, dim3(nblk, 3), kThreads, 0, h.stream, r, u, uold, n, w, h.N, h.F, o.temporal, o.eps,
+        const int wrows = std::max(1, grid_for(ne) / nblk);
+        launch_chained(k_step_norms<T>, dim3(nblk, 2 + wrows), kThreads, 0, h.stream, r, u, uold, n, w, h.N, h.F, o.temporal, o.eps,
                                                                   part_n, stop);
         launch_chained(k_step_decide, 1, 128, 0, h.stream, part_n, nblk, o.tol1, norms2, ctl, scal);
         launch_chained(k_normalize<T>, grid_for(n), kThreads, 0, h.stream, r, n, norms2, stop);

@@ -935,17 +935,20 @@ __global__ void k_norms3_reduce(const double *__restrict__ part, int nblk, doubl
 // ---------------------------------------------------------------------------
 // The vector work at the end of a step in one launch, by blockIdx.y: 0 the
 // partials of |r|^2; 1 those of |u|^2, |u - u_old|^2, |u_old|^2, then u_old = u;
-// 2 the MM weights of u for the next step.
+// from 2 on the MM weights of u for the next step, two or three to a pixel and each
+// with index divisions and a square root, hence several rows of CTAs (2048^2: 169 us
+// with one row and the norms an element at a time, 113 and a copy in launches of
+// their own, 101 so; 16 frames of 256^2: 50, 49 and a copy, 29).
 template <typename T>
-__global__ void __launch_bounds__(256) k_step_norms(const T *__restrict__ r, const T *__restrict__ u, T *uold,
-                                                    long long n, T *__restrict__ w, int N, int F, int temporal,
+__global__ void __launch_bounds__(256) k_step_norms(const T *__restrict__ r, const T *__restrict__ u,
+                                                    T *__restrict__ uold, long long n, T *__restrict__ w, int N, int F, int temporal,
                                                     double eps, double *__restrict__ part, const int *stop)
 {
     chain_wait();
     if (stopped(stop)) return;
     const long long i0 = blockIdx.x * (long long)blockDim.x + threadIdx.x, stride = (long long)gridDim.x * blockDim.x;
-    if (blockIdx.y == 2) {
-        weights_range(u, w, N, F, temporal, eps, i0, stride);
+    if (blockIdx.y >= 2) {
+        weights_range(u, w, N, F, temporal, eps, i0 + (blockIdx.y - 2) * stride, (gridDim.y - 2) * stride);
         return;
     }
     __shared__ double sh[33];
@@ -960,14 +963,25 @@ __global__ void __launch_bounds__(256) k_step_norms(const T *__restrict__ r, con
         return;
     }
     double s0 = 0.0, s1 = 0.0, s2 = 0.0;
-    for (long long i = i0; i < n; i += stride) {
-        const T ui = u[i];
-        const double x = (double)ui;
-        const double y = (double)uold[i];
-        s0 += x * x;
-        s1 += (x - y) * (x - y);
-        s2 += y * y;
-        uold[i] = ui;
+    constexpr int U = 4;  // elements whose loads are ahead of the stores
+    for (long long i = i0; i < n; i += U * stride) {
+        T uv[U], ov[U];
+#pragma unroll
+        for (int q = 0; q < U; ++q) {
+            const long long e = min(i + q * stride, n - 1);
+            uv[q] = u[e];
+            ov[q] = uold[e];
+        }
+#pragma unroll
+        for (int q = 0; q < U; ++q) {
+            if (i + q * stride >= n) break;
+            const double x = (double)uv[q];
+            const double y = (double)ov[q];
+            s0 += x * x;
+            s1 += (x - y) * (x - y);
+            s2 += y * y;
+            uold[i + q * stride] = uv[q];
+        }
     }
     s0 = block_sum(s0, sh);
     s1 = block_sum(s1, sh);
