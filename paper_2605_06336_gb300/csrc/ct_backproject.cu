@@ -228,6 +228,19 @@ template <int KB> struct AdjSumsPacked {
 template <> struct AdjSums<4> : AdjSumsPacked<4> {};
 template <> struct AdjSums<8> : AdjSumsPacked<8> {};
 
+// Four floats at a shared-memory address of CTA `rank` of the cluster (its own included).
+__device__ __forceinline__ float4 ld_cluster4(unsigned addr, int rank)
+{
+    unsigned r;
+    float4 v;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+    asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+                 : "r"(r)
+                 : "memory");
+    return v;
+}
+
 // Views per staged block (two blocks in flight).
 template <int KB> constexpr int adj_vb() { return KB >= 8 ? 8 : 16; }
 template <int KB> constexpr size_t adj_smem(bool reduce)
@@ -383,26 +396,50 @@ __global__ void __launch_bounds__(256, KB <= 2 ? 6 : 0) k_adj_tile(AdjArgs a)
         cg::cluster_group cl = cg::this_cluster();
         if (segs > 1) cl.sync();
         else __syncthreads();
-        // this CTA's share of the pixels, the segments added in order
-        constexpr int OUT = KB * kAdjTile * kAdjTile;
+        // this CTA's share of the pixels, the segments added in order; W pixels of a
+        // row at a time (wide groups have as many values to add as a few views take
+        // time: 256^2, 22 views, 8 sinograms: 12.9 us with one at
+        // a time, 11.1 so; 180 views 30.9 and 29.8)
+        constexpr int W = KB >= 4 ? 4 : 1;
+        constexpr int OUT = KB * kAdjTile * kAdjTile / W;
 #pragma unroll 1
         for (int u = OUT / 32 * seg / segs * 32 + tid; u < OUT / 32 * (seg + 1) / segs * 32; u += 256) {
-            float s;
-            if (segs == 1) {
-                s = red[u];
+            float s[W];
+            if constexpr (W == 4) {
+                const unsigned at = (unsigned)__cvta_generic_to_shared(red + 4 * u);
+#pragma unroll
+                for (int q0 = 0; q0 < kMaxSegs; q0 += 4) {  // four segments' loads in flight
+                    if (q0 >= segs) break;
+                    float4 part[4];
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) part[q] = ld_cluster4(at, min(q0 + q, segs - 1));
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        if (q0 + q >= segs) break;
+                        const float e[4] = {part[q].x, part[q].y, part[q].z, part[q].w};
+#pragma unroll
+                        for (int c = 0; c < 4; ++c) s[c] = q0 + q == 0 ? e[c] : s[c] + e[c];
+                    }
+                }
+            } else if (segs == 1) {
+                s[0] = red[u];
             } else {
                 float part[kMaxSegs];  // all loads in flight
 #pragma unroll
                 for (int q = 0; q < kMaxSegs; ++q) part[q] = q < segs ? *cl.map_shared_rank(red + u, q) : 0.0f;
-                s = part[0];
+                s[0] = part[0];
 #pragma unroll
                 for (int q = 1; q < kMaxSegs; ++q)
-                    if (q < segs) s += part[q];
+                    if (q < segs) s[0] += part[q];
             }
-            const int k = u / (kAdjTile * kAdjTile), p = u % (kAdjTile * kAdjTile);
+            const int k = W * u / (kAdjTile * kAdjTile), p = W * u % (kAdjTile * kAdjTile);
             const int i = i0 + p / kAdjTile, j = j0 + p % kAdjTile;
-            if (i < N && j < N && k0 + k < a.kend)
-                a.X[(size_t)(k0 + k) * a.img_stride + (size_t)f * N * N + (size_t)i * N + j] = s;
+            if (i < N && k0 + k < a.kend) {
+                float *x = a.X + (size_t)(k0 + k) * a.img_stride + (size_t)f * N * N + (size_t)i * N + j;
+#pragma unroll
+                for (int c = 0; c < W; ++c)
+                    if (j + c < N) x[c] = s[c];
+            }
         }
         if (segs > 1) cl.sync();  // the others keep their shared memory until it has been read
     }
@@ -554,7 +591,7 @@ __global__ void __launch_bounds__(256) k_adj64(Adj64Args a)
 // ---------------------------------------------------------------------------
 // small images, both precisions
 // ---------------------------------------------------------------------------
-// Images of side up to kSmallN (kSmallTiles).  Every pixel sums its views in
+// Images of side up to kSmallN.  Every pixel sums its views in
 // two (SPLIT) runs, one after the other, and a whole tile per CTA leaves most
 // SMs idle (64^2, 90 views, one sinogram: 16 CTAs took 14 us in FP32 and 94 in
 // FP64, bound by 16 SMs' FP64 pipes).  The shorter per-segment sums of the other
@@ -738,7 +775,7 @@ template <typename T> cudaError_t launch_small(const SmallArgs<T> &a, const Hand
 bool small_image(const Handle &h, int groups)
 {
     const long long tps = (h.N + kTile - 1) / kTile;
-    return h.N <= kSmallN && (long long)groups * h.F * tps * tps <= kSmallTiles;
+    return h.N <= kSmallN && (long long)groups * h.F * tps * tps * (kTile / kSmallRows) <= 3LL * h.num_sms;
 }
 
 template <typename T> SmallArgs<T> small_args(const Handle &h, T *X, int k0, int groups, int kend, const int *skip)
@@ -863,6 +900,16 @@ cudaError_t adjoint64(const Handle &h, double *X, int batch, int kb, int split, 
 }
 
 }  // namespace
+
+int adj_kb(const Handle &h, int batch)
+{
+    if (h.precision || h.fan_D > 0.0) return h.tune.adj_kb;
+    SinoGroup g[2];
+    sino_groups(batch, h.tune.adj_kb, g);
+    if (small_image(h, g[0].count)) return h.tune.adj_kb;  // the small form's sums are the same at any width
+    const long long tps = (h.N + kAdjTile - 1) / kAdjTile;
+    return adj_group_width(h.tune.adj_kb, batch, tps * tps, h.V, h.num_sms);
+}
 
 template <typename T>
 cudaError_t launch_adjoint(const Handle &h, T *X, int batch, int kb, int split, int layout_batch, const int *skip)
