@@ -139,9 +139,10 @@ int do_forward(ctgb::Handle &h, const double *theta, const double *delta, const 
 template <typename T>
 int do_adjoint(ctgb::Handle &h, const double *theta, const double *delta, const void *Y, void *X, int batch)
 {
-    h.adj_kb_laid = h.tune.adj_kb;
-    CT_CUDA(ctgb::launch_sino_layout<T>(h, (const T *)Y, batch, h.tune.adj_kb, nullptr, theta, delta));
-    CT_CUDA(ctgb::launch_adjoint<T>(h, (T *)X, batch, h.tune.adj_kb, h.tune.adj_split, batch));
+    const int kb = ctgb::adj_kb(h, batch);
+    h.adj_kb_laid = kb;
+    CT_CUDA(ctgb::launch_sino_layout<T>(h, (const T *)Y, batch, kb, nullptr, theta, delta));
+    CT_CUDA(ctgb::launch_adjoint<T>(h, (T *)X, batch, kb, h.tune.adj_split, batch));
     return CT_OK;
 }
 
@@ -235,10 +236,6 @@ void default_tuning(ctgb::Handle &h)
     const int kb = h.max_batch >= 8 ? 8 : (h.max_batch >= 4 ? 4 : (h.max_batch >= 2 ? 2 : 1));
     h.tune.fwd_kb = std::min(kb, 4);
     h.tune.adj_kb = h.precision ? std::min(kb, 4) : kb;
-    if (!h.precision && h.N > 64) {  // (small images sum in a fixed order, one group as good as another)
-        const long long tps = (h.N + 31) / 32;
-        h.tune.adj_kb = ctgb::adj_group_width(kb, h.max_batch, tps * tps, h.V, h.num_sms);
-    }
     const long long rays = (long long)h.V * h.nchunks;  // warps per image
     h.tune.fwd_split = rays >= 16LL * h.num_sms ? 2 : 4;
     h.tune.adj_split = 1;  // the launch raises it where the tiles alone leave SMs idle

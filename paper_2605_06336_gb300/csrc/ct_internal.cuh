@@ -188,20 +188,23 @@ inline int adj_cluster_size(int views, long long tiles, int num_sms, int split, 
     return best;
 }
 
-// Sinograms per group that a FP32 parallel-beam handle starts with, kb (1, 2, 4
-// or 8 by its batch) or fewer.  Sinograms share the weights of a pixel, but
-// groups also give CTAs: with little work a SM (batch x 32 x 32 tiles x views
-// over the SMs) the chip is idle with wide groups, and an odd batch then pays
-// another launch for its last one.  Batch of 8, us at 1 / 2 / 4 / 8 per group:
-// 96^2, 22 views (work 10) 6.3 / 7.2 / 9.2 / 12.2; 256^2, 8 (27) 7.6 / 7.4 / 9.2 /
-// 10.7; 256^2, 22 (74) 11.7 / 10.8 / 11.4 / 12.9; 256^2, 45 (152) 18.7 / 16.9 / 15.0 /
-// 14.8; 400^2, 22 (196) 21.6 / 19.9 / 17.9 / 21.7; 400^2, 90 (800) 62 / 57 / 44 / 41.
+// Sinograms per group of a FP32 parallel-beam product: the launch shape's kb or
+// fewer.  Sinograms share the weights of a pixel, but groups also give CTAs: with
+// little work a SM (batch x 32 x 32 tiles x views over the SMs) the chip is idle
+// with wide groups, and a rest that makes a launch of its own costs as much as
+// the work.  Batch of 8, us at 1 / 2 / 4 / 8 per group: 96^2, 22 views (work 10)
+// 6.3 / 7.2 / 8.1 / 10.2; 256^2, 8 (27) 7.7 / 7.4 / 7.4 / 8.8; 256^2, 22 (74) 11.9 / 10.8 /
+// 9.3 / 11.1; 256^2, 90 (303) 30 / 28 / 19.8 / 19.0; 400^2, 90 (801) 63 / 57 / 38.8 / 38.2.  Batch
+// of 5 at 1 / 4: 256^2, 22 (46) 9.8 / 13.0, 90 (189) 22.4 / 20.6; batch of 3 at 1 / 2: 400^2,
+// 64 (213) 23 / 29, 512^2, 90 (455) 43 / 45.
 inline int adj_group_width(int kb, int batch, long long tiles, int views, int num_sms)
 {
     const double work = (double)batch * tiles * views / num_sms;
-    if (work < 25.0 || (work < 100.0 && batch % 2)) return 1;
-    const int most = work < 100.0 ? 2 : (work < 300.0 ? 4 : 8);
-    return kb < most ? kb : most;
+    if (work < 25.0) return 1;
+    const int most = work < 300.0 ? 4 : 8, width = kb < most ? kb : most;
+    SinoGroup g[2];
+    if (sino_groups(batch, width, g) > 1 && work < (width >= 4 ? 150.0 : 500.0)) return 1;
+    return width;
 }
 
 // Where a derivative product finds its images: the pair images, the
@@ -300,6 +303,8 @@ cudaError_t launch_forward(const Handle &h, T *Y, int batch, int kb, int split, 
 template <typename T>
 cudaError_t launch_adjoint(const Handle &h, T *X, int batch, int kb, int split, int layout_batch,
                            const int *skip = nullptr);
+// Sinograms per group for a product of `batch`: the launch shape's, narrowed by adj_group_width.
+int adj_kb(const Handle &h, int batch);
 // Derivative modes on `batch` images laid out in the pair buffers (kb images
 // per lane: 1, 2 or 4), one launch of the ray kernel plus (VJP, GN) the
 // per-view reduction.  JVP: image k uses dtheta + k * dir_stride (0: one

@@ -65,7 +65,7 @@ def test_few_views_take_one_cta_and_narrow_groups(rules):
     tiles = lambda N: ((N + 31) // 32) ** 2
     rows = [(8, 8, tiles(96), 8, 152), (8, 8, tiles(256), 8, 152), (4, 5, tiles(256), 22, 152), (8, 8, tiles(256), 45, 152),
             (8, 8, tiles(256), 180, 152), (2, 2, tiles(2048), 120, 152)]
-    assert rules(rows, rule=1) == [1, 2, 1, 4, 8, 2]
+    assert rules(rows, rule=1) == [1, 4, 1, 4, 8, 2]
     rows = [(kb, K, t, v, 152) for kb, K in ((1, 1), (2, 3), (4, 7), (8, 9)) for t in (9, 64, 4096) for v in (1, 30, 1200)]
     assert all(1 <= w <= r[0] for w, r in zip(rules(rows, rule=1), rows))
 
