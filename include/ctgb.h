@@ -126,9 +126,11 @@ int ct_forward(ct_handle *h, const double *theta, const double *delta,
 
 /*
  * X = H(theta, delta)^T Y, the exact transpose of ct_forward in gather form
- * (one thread per pixel, no atomics); used in the residual
+ * (every pixel written once, no atomics); used in the residual
  * H^T (H u - b) + lambda Psi^T P^2 Psi u of every MM-GKS step (Eq. (3.6)).
  *   Y [batch][n_views][B]  ->  X [batch][n_frames][N][N]
+ * The order of a sinogram's sums, and with it its last bits, depends on the
+ * launch shape and above 64^2 on the batch it is in.
  */
 int ct_adjoint(ct_handle *h, const double *theta, const double *delta,
                const void *Y, void *X, int batch);
@@ -251,7 +253,8 @@ int ct_autotune(ct_handle *h);
 /*
  * Read / set the launch shapes, CT_TUNING_COUNT values:
  *   [0] forward images per lane, [1] forward warps per ray (row segments),
- *   [2] forward views per CTA, [3] transpose sinograms per thread,
+ *   [2] forward views per CTA, [3] transpose sinograms per thread (fewer where
+ *   a FP32 parallel-beam product has too little work to fill the SMs with that),
  *   [4] least number of CTAs (view subsets) per transpose pixel tile (the
  *   launch takes more, up to 8, where the tiles alone leave SMs idle, and 2
  *   instead of 4 where 4 would leave a CTA fewer than 8 views; for images of
