@@ -687,6 +687,11 @@ __global__ void __launch_bounds__(512) k_ray(RayArgs<T> a)
                 Q += (long long)U * dQ;
             };
             int r = r0;
+            // (4 images a lane on pairs: the second block's loads start before the first's sums, or
+            // a launch of few views waits for each: 256^2, 22 views, 8 images, 2 segments a ray
+            // 37.0 us a call, 31.1 so; one whole ray per warp has warps enough, 49.5 and 64.3)
+            constexpr int UNR = F32 && MODE == kFwd && KB == 4 && !QL && (SPLIT == 2 || SPLIT == 4) ? 2 : 1;
+#pragma unroll UNR
             for (; r + U - 1 <= r1; r += U) block(std::true_type(), U);
             if (r <= r1) block(std::false_type(), r1 - r + 1);
         }

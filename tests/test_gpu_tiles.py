@@ -258,15 +258,18 @@ def test_interleaved_images_take_no_memory_of_their_own():
         free, total = torch.cuda.mem_get_info()
         return total - free
     ct.CTOperator(64, 91, 8, max_batch=K).close()  # the context and the kernels are loaded
-    before = used()
-    op = ct.CTOperator(N, B, V, max_batch=K, dtype=torch.float32)
-    made = used() - before
-    assert op.tuning[11] == 1
+    made, more = [], []
+    for _ in range(4):  # (the smallest of a few: another process may use the device meanwhile)
+        before = used()
+        op = ct.CTOperator(N, B, V, max_batch=K, dtype=torch.float32)
+        made.append(used() - before)
+        assert op.tuning[11] == 1
+        op.tuning = [4, 2, 2, 4, 1, 4, 1, 0, 0, 0, 1, 1]
+        more.append(used() - before - made[-1])
+        op.close()
     pairs, sino, partials = 2 * (K + 1) * N * (N + 4) * 8, K * V * (B + 5) * 8, 32 * K * V * ((B + 31) // 32)
-    assert made <= pairs + sino + partials + 24 * 2 ** 20
-    op.tuning = [4, 2, 2, 4, 1, 4, 1, 0, 0, 0, 1, 1]
-    assert used() - before <= made
-    op.close()
+    assert min(made) <= pairs + sino + partials + 24 * 2 ** 20
+    assert min(more) <= 0
 
 
 # the source as near as the geometry takes it (0.75 max(N, B) + 2): wide ray windows at the far side
