@@ -68,7 +68,7 @@ void free_all(ctgb::Handle &h)
 // call reads beside them where the free half of the pairs' memory holds these
 // (in the launch of the view-table step, once for calls of as many images), else
 // all are turned into pairs (one launch more).  A forward of 8 images, 256^2 / 180
-// views, then J^T of one: 67.2 us, 72.1 turning all (80.8 with the forward on
+// views, then J^T of one: 65.8 us, 69.9 turning all (80.8 with the forward on
 // pair images).
 template <typename T>
 cudaError_t prep_images(ctgb::Handle &h, const T *X, int batch, const double *theta, const double *delta,
